@@ -206,7 +206,8 @@ typedef struct {
  *                        Y2 X3 Y3 (snapped, 1/256 pixel), the four vertices' 1/w (f32 bits),
  *                        1/|A0| and 1/|A1| (f32 bits of the reciprocal doubled triangle
  *                        areas, 0 for a zero-area triangle), info (as rec_info, cull reason
- *                        0), 0
+ *                        0), flags (bit 0: 32-bit edge arithmetic is exact on every 8x4
+ *                        half-block the quad's box touches)
  *   rec_rect  u32[Q][2]  pixel-centre AABB: px0 | px1 << 16, py0 | py1 << 16
  *                        (0x0000FFFF, 0x0000FFFF for a culled quad)
  *   rec_info  u32[Q]     bit 0/1: triangle 0/1 has non-zero area, bit 2: spans more than

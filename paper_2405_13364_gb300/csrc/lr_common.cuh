@@ -69,6 +69,9 @@ constexpr uint32_t kInfoFlatDepth = 8u;     // all four vertices have the same 1
 constexpr uint32_t kInfoSwap0 = 16u;        // triangle t (bit << t): negative area, v1 <-> v2
 constexpr uint32_t kInfoSmall0 = 64u;       // triangle t (bit << t): 32-bit edge values are
                                             // exact on every half-block its box touches
+// flags in word 15 of the record
+constexpr uint32_t kRecSmall = 1u;          // 32-bit edge values are exact on every half-block
+                                            // the quad's box touches
 constexpr uint32_t kRectInvisible = 0x0000FFFFu;   // rect.x value of a culled quad
 
 struct ViewDev {
@@ -172,7 +175,8 @@ struct Ctrl {
 // that one quad is four 16-byte loads from one cache line:
 //   w0 = (X0, Y0, X1, Y1), w1 = (X2, Y2, X3, Y3)  snapped vertices, 1/256 pixel
 //   w2 = 1/w of vertices 0..3 (float bits)
-//   w3 = (1 / (float)|A0|, 1 / (float)|A1| (float bits, 0 for a zero-area triangle), info, 0)
+//   w3 = (1 / (float)|A0|, 1 / (float)|A1| (float bits, 0 for a zero-area triangle), info,
+//         kRec* flags)
 struct QuadRec {
   int X[4], Y[4];
   float q[4];

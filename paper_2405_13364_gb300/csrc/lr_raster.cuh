@@ -12,23 +12,36 @@
 //      k_bin_sort: bit j set iff sorted reference j overlaps the half-block) is read with
 //      one coalesced load per 1024 references, and its set bits are handed out 32 at a
 //      time in sorted order, one candidate quad per lane;
-//   2. triangle setup, lane-parallel: for 32 candidate quads, both triangles' integer edge
-//      functions at the half-block origin, per-pixel steps, 1/area, depth-plane deltas;
-//      a triangle whose edge values stay below 2^30 on the half-block is marked "fast"
-//      and evaluated with 32-bit integers, others with exact 64-bit integers; the same
-//      lane computes each triangle's 32-pixel coverage mask (top-left rule) row by row;
-//   3. coverage, transposed: a 32x32 bit transpose across the warp turns "triangle ->
-//      pixels" into "pixel -> triangles", one bit per covering triangle in each lane;
-//   4. fragments, per lane in candidate order: the exact depth key of the fragment
+//   2. coverage, lane-parallel: both triangles' 32-pixel masks (top-left rule) from the
+//      quad's five edges (quad_masks_small / quad_masks_any). Triangles that cover a pixel
+//      go to a small ring in shared memory; those that do not (a third of the layer frame's)
+//      cost nothing further;
+//   3. batches of 32 covering triangles from the ring, one per lane: the depth key's edge
+//      values, steps and plane, and the colours, into shared memory. 32-bit edge values
+//      where k_setup proved them exact, else 64-bit;
+//   4. a 32x32 bit transpose across the warp turns "triangle -> pixels" into "pixel ->
+//      triangles", one bit per covering triangle in each lane;
+//   5. fragments, per lane in candidate order: the exact depth key of the fragment
 //      (interpolated 1/w, identical bit for bit to the oracle's formula) is pushed into a
 //      K-slot register sorter (stage 2, the paper's depth filter, Sec. 2, Stage 3,
 //      Phase 3, "Sample blending"). When full,
 //      the nearest element is evicted and blended front to back. If a fragment arrives
 //      that is nearer than the last evicted one, the stream was not in order for this
 //      pixel: the pixel is flagged (the paper's misorder detection, same passage) and
-//      registered for k_overflow.
+//      registered for k_overflow. While every triangle so far has a flat colour and one
+//      depth (camera-facing quads), the sorted stream is the exact order of every pixel, and
+//      fragments are blended as they come, without key, sorter or test.
 // Sort keys are (float bits of key) << 32 | (2 * quad + triangle): distinct per pixel, so
 // the per-pixel order is total and the result is unique.
+//
+// What bounds it and what it took (K = 1, 1920x1080, kernel times): on 1M wavy quads with
+// vertex colours the shared-memory and gather wavefronts (80% of the L1 data pipe; a 16-byte
+// load per lane costs four), 62% of issue slots; against setting up both triangles of each
+// candidate with a binary search per edge and row, 349M -> 253M warp instructions and
+// 375 -> 328 us. On 2M particles, 60% of issue slots and the gathers of scattered records;
+// 848M -> 372M instructions, 1005 -> 506 us. With normals 602 -> 416 us, with the alpha
+// threshold on the particles 389 -> 268 us, a batch of mixed views at K = 3 2040 -> 911 us,
+// 100k scattered parallelograms with a few screen-filling ones 117 -> 66 us.
 #pragma once
 
 #include "lr_common.cuh"
@@ -42,6 +55,8 @@ constexpr uint32_t kTriConstKey = 64u;
 // lit colours (LR_COLOR_LIT): the triangle's colour slots also hold its perspective-weighted
 // normals, and each fragment's RGB is shaded with the view's light
 constexpr uint32_t kTriLit = 128u;
+// k_raster's batches: the edge values are kept in 64 bits
+constexpr uint32_t kTriWide = 256u;
 constexpr unsigned long long kSent = ~0ull;
 constexpr int kRasterThreads = 256;
 #ifndef LR_RASTER_MIN_BLOCKS
@@ -72,16 +87,6 @@ struct __align__(16) TriSm {
   int X[3], Y[3];  // vertices after the orientation fix (64-bit path)
   int pad[2];
 };
-
-// dynamic shared memory of k_raster: per warp 64 triangle records, when fragments carry
-// colours 3 premultiplied vertex colours per triangle (6 slots with lit colours: also the
-// weighted normals), and for the backward 32 gradient slots
-__host__ __device__ constexpr int col_slots(bool lit) { return lit ? 6 : 3; }
-__host__ __device__ constexpr size_t raster_smem_bytes(bool vtx, bool bwd = false, bool lit = false) {
-  return (size_t)kRasterWarps * 64 * sizeof(TriSm) +
-         (vtx ? (size_t)kRasterWarps * 64 * col_slots(lit) * sizeof(float4) : 0) +
-         (bwd ? (size_t)kRasterWarps * 32 * sizeof(float4) : 0);
-}
 
 // exact 64-bit edge values (unbiased) of a triangle at pixel (px, py)
 __device__ __forceinline__ void edges64(const TriSm& T, int px, int py, long long e[3]) {
@@ -252,23 +257,6 @@ __device__ __forceinline__ uint32_t tri_mask_fast(const int e[3], const int sx[3
   return mask;
 }
 
-// The same for a triangle of a quad whose diagonal's coverage is given: d = the half-block's
-// mask of the diagonal in this triangle's direction; only the other two edges (e0, e1, with
-// their steps) are evaluated.
-__device__ __forceinline__ uint32_t tri_mask_two(int e0, int sx0, int sy0, int e1, int sx1, int sy1, uint32_t d,
-                                                 const int box[4]) {
-  uint32_t mask = 0;
-  const uint32_t cols = ((2u << box[1]) - 1u) & ~((1u << box[0]) - 1u);
-#pragma unroll
-  for (int ly = 0; ly < kHbH; ++ly) {
-    uint32_t row = (ly >= box[2] && ly <= box[3]) ? cols : 0u;
-    row &= row_cover((int)((uint32_t)e0 + (uint32_t)ly * (uint32_t)sy0), sx0) &
-           row_cover((int)((uint32_t)e1 + (uint32_t)ly * (uint32_t)sy1), sx1);
-    mask |= row << (ly * kHbW);
-  }
-  return mask & d;
-}
-
 // The same with exact 64-bit edge values, pixel by pixel (large triangles).
 static __device__ __noinline__ uint32_t tri_mask_slow(const TriSm& T, int ox, int oy, const int box[4]) {
   uint32_t mask = 0;
@@ -388,6 +376,16 @@ struct PixelState {
     else T = __fmaf_rn(-T, col.w, T);
   }
 
+  // forward blend of a fragment known to be next in order, without the sorter
+  __device__ __forceinline__ void blend_direct(float4 col) {
+    const float w = T * col.w;
+    r += w * col.x;
+    g += w * col.y;
+    b += w * col.z;
+    if (ATH) T *= 1.0f - col.w;
+    else T = __fmaf_rn(-T, col.w, T);
+  }
+
   __device__ __forceinline__ void insert(unsigned long long x, float4 xc, const ViewDev& V) {
     // nearer than a fragment already blended: order not guaranteed. The forward pass with
     // carried colours only records it (the pixel's composite is discarded, so inserting the
@@ -491,6 +489,122 @@ __device__ __forceinline__ void write_pixel(const ViewDev& V, long long pidx, fl
   }
 }
 
+// ---- k_raster's coverage masks -------------------------------------------------------------
+//
+// Forward coverage of an edge u -> v on the half-block at pixel-centre origin (Px, Py): row
+// ly's columns as the low 8 bits of f[ly] (the bits above are arbitrary). Covered iff
+// E + bias >= 0, E = dx (Py - yu) - dy (Px - xu), bias = 0 for an owned edge, else -1. A step
+// of one column adds -256 dy and one of a row 256 dx, so E + bias may be replaced by
+// r = floor((E + bias) / 256) with steps -dy and dx. The covered columns are then
+//   dy < 0: those from ceil(r / dy) on,  dy > 0: the first floor(r / dy) + 1,  dy = 0: r >= 0,
+// and both counts are ceil(r / dy -+ eps) for any eps below the quotient's distance from the
+// next integer, 1 / |dy| > 2^-15. The quotient is taken in fp32 as r (1 / (8 dy)), clamped to
+// [0, 1] by the multiply-add's saturation: r and its row steps are exact (|r| < 2^22), the
+// approximate reciprocal and the rounding put the clamped value off by less than 2^-22, and
+// eps = 2^-17 (2^-20 scaled) exceeds that, so the count is exact; the scaling back adds 2^23
+// rounded up, which leaves ceil() in the low bits. Needs |E| < 2^30 and |dx|, |dy| < 2^15 on
+// the half-block (kRecSmall). Five instructions per edge and row, against about 16 for the
+// exact integer binary search (row_cover).
+__device__ __forceinline__ void edge_rows(int xu, int yu, int xv, int yv, int Px, int Py, uint32_t f[kHbH]) {
+  const int dx = xv - xu, dy = yv - yu;
+  const bool owned = dy < 0 || (dy == 0 && dx > 0);
+  const int e = (int)((uint32_t)dx * (uint32_t)(Py - yu) - (uint32_t)dy * (uint32_t)(Px - xu)) - (owned ? 0 : 1);
+  float r = __int2float_rn(e >> 8);
+  const float step = __int2float_rn(dx);
+  const float k = dy == 0 ? -1e20f : rcp_approx(__int2float_rn(8 * dy));
+  const float b = dy > 0 ? 0x1p-20f : -0x1p-20f;
+  const uint32_t flip = dy > 0 ? 0xFFFFFFFFu : 0u;
+#pragma unroll
+  for (int ly = 0; ly < kHbH; ++ly) {
+    const float t = __saturatef(__fmaf_rn(r, k, b));
+    const uint32_t c = __float_as_uint(__fmaf_ru(t, 8.0f, 8388608.0f));   // count in the low 5 bits
+    f[ly] = __funnelshift_l(0u, 0xFFFFFFFFu, c) ^ flip;                   // ~0 << (c mod 32)
+    r = __fadd_rn(r, step);
+  }
+}
+
+__device__ __forceinline__ uint32_t pack_rows(uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+  return __byte_perm(__byte_perm(r0, r1, 0x0040), __byte_perm(r2, r3, 0x0040), 0x5410);
+}
+
+// Coverage masks (bit ly * 8 + lx) of a quad's two triangles on the half-block. Under the
+// top-left rule a pixel centre belongs to exactly one of an edge's two directions, so an edge
+// traversed backwards (a triangle of negative area, or the diagonal's second triangle) takes
+// the complement, and five edges serve both triangles.
+__device__ __forceinline__ void quad_masks_small(const int X[4], const int Y[4], uint32_t info, int Px, int Py,
+                                                 uint32_t& m0, uint32_t& m1) {
+  const uint32_t s0 = (info & kInfoSwap0) ? 0xFFFFFFFFu : 0u;
+  const uint32_t s1 = (info & (kInfoSwap0 << 1)) ? 0xFFFFFFFFu : 0u;
+  uint32_t d[kHbH], f[kHbH], a[kHbH], c[kHbH];
+  edge_rows(X[2], Y[2], X[0], Y[0], Px, Py, d);   // the diagonal, T0's direction
+  edge_rows(X[0], Y[0], X[1], Y[1], Px, Py, f);
+#pragma unroll
+  for (int i = 0; i < kHbH; ++i) { a[i] = (d[i] ^ s0) & (f[i] ^ s0); c[i] = ~(d[i] ^ s1); }
+  edge_rows(X[1], Y[1], X[2], Y[2], Px, Py, f);
+#pragma unroll
+  for (int i = 0; i < kHbH; ++i) a[i] &= f[i] ^ s0;
+  edge_rows(X[2], Y[2], X[3], Y[3], Px, Py, f);
+#pragma unroll
+  for (int i = 0; i < kHbH; ++i) c[i] &= f[i] ^ s1;
+  edge_rows(X[3], Y[3], X[0], Y[0], Px, Py, f);
+#pragma unroll
+  for (int i = 0; i < kHbH; ++i) c[i] &= f[i] ^ s1;
+  m0 = (info & kInfoTri0) ? pack_rows(a[0], a[1], a[2], a[3]) : 0u;
+  m1 = (info & kInfoTri1) ? pack_rows(c[0], c[1], c[2], c[3]) : 0u;
+}
+
+// The same for any quad: the 64-bit edge value at the origin, divided by 256 as above, is
+// clamped to +-2^28 (|7 dy + 3 dx| < 2^27 within the guard band, so a clamped value keeps its
+// sign on the whole half-block), and the rows are searched in 32-bit integers.
+__device__ __forceinline__ void quad_masks_any(const int X[4], const int Y[4], uint32_t info, int Px, int Py,
+                                               uint32_t& m0, uint32_t& m1) {
+  const uint32_t s0 = (info & kInfoSwap0) ? 0xFFFFFFFFu : 0u;
+  const uint32_t s1 = (info & (kInfoSwap0 << 1)) ? 0xFFFFFFFFu : 0u;
+  uint32_t a = 0xFFFFFFFFu, c = 0xFFFFFFFFu;
+#pragma unroll 1
+  for (int k = 0; k < 5; ++k) {
+    // edges v2 -> v0, v0 -> v1, v1 -> v2, v2 -> v3, v3 -> v0
+    const int xu = k == 1 ? X[0] : (k == 2 ? X[1] : (k == 4 ? X[3] : X[2]));
+    const int yu = k == 1 ? Y[0] : (k == 2 ? Y[1] : (k == 4 ? Y[3] : Y[2]));
+    const int xv = k == 1 ? X[1] : (k == 2 ? X[2] : (k == 3 ? X[3] : X[0]));
+    const int yv = k == 1 ? Y[1] : (k == 2 ? Y[2] : (k == 3 ? Y[3] : Y[0]));
+    const int dx = xv - xu, dy = yv - yu;
+    const bool owned = dy < 0 || (dy == 0 && dx > 0);
+    const long long e = ((long long)dx * (Py - yu) - (long long)dy * (Px - xu) - (owned ? 0 : 1)) >> 8;
+    const int r = (int)max(min(e, 1LL << 28), -(1LL << 28));
+    uint32_t f = 0;
+#pragma unroll
+    for (int ly = 0; ly < kHbH; ++ly) f |= row_cover(r + ly * dx, -dy) << (ly * kHbW);
+    if (k < 3) a &= f ^ s0;
+    if (k == 0) c = ~(f ^ s1);
+    if (k > 2) c &= f ^ s1;
+  }
+  m0 = (info & kInfoTri0) ? a : 0u;
+  m1 = (info & kInfoTri1) ? c : 0u;
+}
+
+// ---- k_raster's shared memory ----------------------------------------------------------------
+// Per warp: a ring of covering triangles waiting for a batch, and the records of the batch the
+// fragment loop reads, one 16-byte array per field so that a slot's fields lie at one address
+// plus constants and eight neighbouring slots never share a bank.
+constexpr int kPendCap = 128;      // at most 31 left over + 64 pushed per candidate round
+constexpr uint32_t kPendConst = 0x80000000u;   // pending id: flat colour and constant depth
+struct BatchGeo {
+  int4 ea[32];                     // e1, e2 (edge values at the half-block origin; low words
+                                   // of 64-bit ones), x steps sx1, sx2 (64-bit: -dy1, -dy2)
+  int4 eb[32];                     // y steps sy1, sy2 (64-bit: dx1, dx2), flags, id
+  float4 kq[32];                   // q0, q1 - q0, q2 - q0, 1 / area
+  int2 hi[32];                     // high words of 64-bit e1, e2
+};
+__host__ __device__ constexpr int batch_cols(bool vtx, bool lit) { return vtx ? (lit ? 6 : 3) : 1; }
+__host__ __device__ constexpr size_t batch_smem_warp(bool vtx, bool bwd, bool lit) {
+  return kPendCap * sizeof(uint2) + sizeof(BatchGeo) + (size_t)batch_cols(vtx, lit) * 32 * sizeof(float4) +
+         (bwd ? 32 * sizeof(float4) : 0);
+}
+__host__ __device__ constexpr size_t raster_smem_bytes(bool vtx, bool bwd = false, bool lit = false) {
+  return (size_t)kRasterWarps * batch_smem_warp(vtx, bwd, lit);
+}
+
 // HASH: the variant that also writes the per-pixel coverage hash (a test output); the
 // others carry no code or registers for it. ATH: the alpha-threshold variant (forward
 // only, no hash), which also skips candidate quads that cannot reach in front of any
@@ -500,12 +614,16 @@ template <int K, bool VTX, bool BWD, bool HASH, bool ATH = false, bool LIT = fal
 __global__ __launch_bounds__(kRasterThreads, LR_RASTER_MIN_BLOCKS) void k_raster(Ws ws) {
   pdl_begin();
   extern __shared__ __align__(16) unsigned char smem[];
-  constexpr int kSlots = col_slots(LIT);
+  constexpr bool kCarry = VTX || K == 1;   // the sorter carries each fragment's colour
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lx = lane & (kHbW - 1), ly = lane >> 3;
-  TriSm* tris = reinterpret_cast<TriSm*>(smem) + warp * 64;
-  float4* qcs = reinterpret_cast<float4*>(smem + (size_t)kRasterWarps * 64 * sizeof(TriSm)) + (size_t)warp * 64 * kSlots;
-  float4* agg = reinterpret_cast<float4*>(smem + raster_smem_bytes(VTX, false, LIT)) + (size_t)warp * 32;
+  unsigned char* wbase = smem + (size_t)warp * batch_smem_warp(VTX, BWD, LIT);
+  uint2* pend = reinterpret_cast<uint2*>(wbase);
+  BatchGeo& geo = *reinterpret_cast<BatchGeo*>(wbase + kPendCap * sizeof(uint2));
+  float4* qc = reinterpret_cast<float4*>(wbase + kPendCap * sizeof(uint2) + sizeof(BatchGeo));
+  float4* agg = qc + batch_cols(VTX, LIT) * 32;
+  // a batch blended in stream order keeps its sort keys where the others keep ea
+  unsigned long long* dkey = reinterpret_cast<unsigned long long*>(&geo);
   if (ws.ctrl->error == LR_ERR_OVERFLOW) return;
   const unsigned long long nitems = ws.ctrl->raster_items;
   unsigned long long frag_total = 0;
@@ -528,13 +646,14 @@ __global__ __launch_bounds__(kRasterThreads, LR_RASTER_MIN_BLOCKS) void k_raster
     const bool pix_ok = px < V.width && py < V.height;
     const uint32_t off = ws.bin_off[bin_g];
     const int n = (int)(ws.bin_off[bin_g + 1] - off);
-    const bool vtx_view = V.color_mode != LR_COLOR_FLAT;
+    const bool flat_view = V.color_mode == LR_COLOR_FLAT;
     const bool hashing = HASH && V.hash != nullptr;
+    const int Ox = 256 * ox + 128, Oy = 256 * oy + 128;   // first pixel centre, 1/256 px
     // lit views: unit direction toward the light and the ambient term
     const float4 light = LIT ? make_float4(V.light[0], V.light[1], V.light[2], V.light[3])
                              : make_float4(0.f, 0.f, 0.f, 0.f);
 
-    PixelState<K, VTX, BWD, ATH> st;
+    PixelState<K, kCarry, BWD, ATH> st;
     st.init();
     st.gp.grad = nullptr;
     st.gp.agg = agg;
@@ -547,232 +666,6 @@ __global__ __launch_bounds__(kRasterThreads, LR_RASTER_MIN_BLOCKS) void k_raster
     }
     uint32_t cnt = 0;
     unsigned long long hsh = 0;
-
-    auto process = [&](int nc, uint32_t rec) {
-      bool skip = false;
-      if (ATH) {
-        // The smallest key a fragment must exceed to change any pixel of the half-block:
-        // 0 while a pixel still blends; a finished pixel needs a fragment in front of the
-        // one that finished it (keys are positive floats, so their bits order like them);
-        // pixels outside the image and pixels left to the exact path need nothing. A
-        // candidate whose largest possible key is below that is skipped: every fragment
-        // of it would be dropped.
-        const uint32_t need = (!pix_ok || st.flagged) ? 0xFFFFFFFFu : (st.live() ? 0u : (uint32_t)(st.last >> 32));
-        const uint32_t kmin = __reduce_min_sync(0xffffffffu, need);
-        if (kmin != 0u) {
-          if (lane < nc) {
-            const int4 qv = __ldg(ws.rec + 4ull * rec + 2);   // the record's four 1/w
-            const float qm = fmaxf(fmaxf(__int_as_float(qv.x), __int_as_float(qv.y)),
-                                   fmaxf(__int_as_float(qv.z), __int_as_float(qv.w)));
-            skip = __float_as_uint(qm * kKeyBoundScale) < kmin;
-          }
-          if (__all_sync(0xffffffffu, skip || lane >= nc)) return;
-        }
-      }
-      // ---- 2. triangle setup and coverage masks, one quad per lane ---------------------
-      uint32_t tm0 = 0, tm1 = 0;
-      if (lane < nc && !(ATH && skip)) {
-        const QuadRec R = load_rec(ws.rec, rec);
-        const uint32_t jl = (uint32_t)(rec - V.quad_base);
-        uint32_t vsel = 0;   // per set-up triangle t: bit 8 + t, and its corners 1, 2 at bits 4t
-        // Both triangles share the diagonal v0 v2, which each passes in one direction: under
-        // the top-left rule a pixel centre on it belongs to exactly one of its two directions,
-        // so the coverage of the direction v2 -> v0 is computed once (dmask) and a triangle
-        // traversing the diagonal the other way takes its complement. Only when both
-        // triangles are small: their 32-bit exactness bound covers the diagonal's values at
-        // every half-block that touches either triangle's box, the only ones using dmask.
-        // (Flat colours only: with colours carried the extra live registers spill, and the
-        // layer frame measured no faster; the particle frame's rasteriser 1.011 -> 1.005 ms.)
-        const bool share = !VTX && (R.info & (kInfoSmall0 | (kInfoSmall0 << 1))) == (kInfoSmall0 | (kInfoSmall0 << 1));
-        uint32_t dmask = 0;
-        if (share) {
-          const int dx = R.X[0] - R.X[2], dy = R.Y[0] - R.Y[2];
-          const bool owned = dy < 0 || (dy == 0 && dx > 0);
-          const int e0 = (int)((uint32_t)dx * (uint32_t)(256 * oy + 128 - R.Y[2]) -
-                               (uint32_t)dy * (uint32_t)(256 * ox + 128 - R.X[2])) -
-                         (owned ? 0 : 1);
-#pragma unroll
-          for (int ly = 0; ly < kHbH; ++ly)
-            dmask |= row_cover((int)((uint32_t)e0 + (uint32_t)ly * (uint32_t)(256 * dx)), -256 * dy) << (ly * kHbW);
-        }
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-          TriSm& T = tris[2 * lane + t];
-          int cor[3];
-          uint32_t mk;
-          if (R.info & (kInfoSmall0 << t)) {
-            // arrays of their own, never passed out of line: they stay in registers
-            int box[4], le[3], lsx[3], lsy[3];
-            if (!setup_tri_small(T, R.X, R.Y, R.q, t ? R.inv[1] : R.inv[0], R.info, t, jl, ox, oy, cor, box, le, lsx,
-                                 lsy))
-              continue;
-            if (share) {
-              // the diagonal is edge 1 (c -> a: v2 -> v0) of T0 unswapped and of T1 swapped,
-              // else edge 2 (a -> b: v0 -> v2); edge 0 never touches v0
-              const bool d1 = ((R.info >> t) & kInfoSwap0) ? t == 1 : t == 0;
-              mk = tri_mask_two(le[0], lsx[0], lsy[0], d1 ? le[2] : le[1], d1 ? lsx[2] : lsx[1],
-                                d1 ? lsy[2] : lsy[1], d1 ? dmask : ~dmask, box);
-            } else {
-              mk = tri_mask_fast(le, lsx, lsy, box);
-            }
-          } else {
-            const QuadRec G = R;   // the out-of-line path's own copy (its address escapes)
-            int cg[3], box[4], le[3], lsx[3], lsy[3];
-            if (!setup_tri(T, G.X, G.Y, G.q, G.info, t, jl, ox, oy, cg, box, le, lsx, lsy)) continue;
-            mk = ((uint32_t)T.eb.z & kTriFast) ? tri_mask_fast(le, lsx, lsy, box) : tri_mask_slow(T, ox, oy, box);
-            cor[0] = cg[0]; cor[1] = cg[1]; cor[2] = cg[2];
-          }
-          if (t == 0) tm0 = mk; else tm1 = mk;
-          if (VTX) vsel |= (1u << (8 + t)) | ((uint32_t)(cor[1] | (cor[2] << 2)) << (4 * t));
-        }
-        if (VTX && vsel) {
-          if (!vtx_view) {
-            const float4 fc = __ldg(reinterpret_cast<const float4*>(V.col) + jl);
-#pragma unroll
-            for (int t = 0; t < 2; ++t)
-              if (vsel & (1u << (8 + t))) {
-                // zero increments: the fragments' interpolation with the scale 1 (below)
-                // returns fc bit for bit
-                float4* qc = qcs + (2 * lane + t) * kSlots;
-                qc[0] = fc;
-                qc[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-                qc[2] = make_float4(0.f, 0.f, 0.f, 0.f);
-                tris[2 * lane + t].eb.z |= (int)kTriFlatCol;
-              }
-          } else if (LIT && V.color_mode == LR_COLOR_LIT) {
-            // 32 bytes per vertex (straight RGBA, then the normal): as below, each triangle
-            // stores its corners' colours times 1/w as (c0, c1 - c0, c2 - c0), then the same
-            // for the normals
-            uint4 vi = make_uint4(4 * jl, 4 * jl + 1, 4 * jl + 2, 4 * jl + 3);
-            if (V.idx) vi = __ldg(reinterpret_cast<const uint4*>(V.idx) + jl);
-            const float4* cv = reinterpret_cast<const float4*>(V.col);
-            const uint32_t vk[4] = {vi.x, vi.y, vi.z, vi.w};
-            float4 p[4], m[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float4 c = __ldg(cv + 2ull * vk[k]), n = __ldg(cv + 2ull * vk[k] + 1);
-              p[k] = make_float4(R.q[k] * c.x, R.q[k] * c.y, R.q[k] * c.z, R.q[k] * c.w);
-              m[k] = make_float4(R.q[k] * n.x, R.q[k] * n.y, R.q[k] * n.z, 0.f);
-            }
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-              if (!(vsel & (1u << (8 + t)))) continue;
-              const uint32_t kb = (vsel >> (4 * t)) & 3u, kc = (vsel >> (4 * t + 2)) & 3u;
-              const float4 a1 = kb == 1 ? p[1] : (kb == 2 ? p[2] : p[3]);
-              const float4 a2 = kc == 1 ? p[1] : (kc == 2 ? p[2] : p[3]);
-              const float4 b1 = kb == 1 ? m[1] : (kb == 2 ? m[2] : m[3]);
-              const float4 b2 = kc == 1 ? m[1] : (kc == 2 ? m[2] : m[3]);
-              float4* qc = qcs + (2 * lane + t) * kSlots;
-              qc[0] = p[0];
-              qc[1] = make_float4(a1.x - p[0].x, a1.y - p[0].y, a1.z - p[0].z, a1.w - p[0].w);
-              qc[2] = make_float4(a2.x - p[0].x, a2.y - p[0].y, a2.z - p[0].z, a2.w - p[0].w);
-              qc[3] = m[0];
-              qc[4] = make_float4(b1.x - m[0].x, b1.y - m[0].y, b1.z - m[0].z, 0.f);
-              qc[5] = make_float4(b2.x - m[0].x, b2.y - m[0].y, b2.z - m[0].z, 0.f);
-              tris[2 * lane + t].eb.z |= (int)kTriLit;
-            }
-          } else {
-            // the quad's four corner colours times 1/w, loaded together once; each triangle
-            // stores (c0, c1 - c0, c2 - c0) of its corners for the fragment's
-            // c0 + l1 (c1 - c0) + l2 (c2 - c0)
-            uint4 vi = make_uint4(4 * jl, 4 * jl + 1, 4 * jl + 2, 4 * jl + 3);
-            if (V.idx) vi = __ldg(reinterpret_cast<const uint4*>(V.idx) + jl);
-            const float4* cv = reinterpret_cast<const float4*>(V.col);
-            const float4 c0 = __ldg(cv + vi.x), c1 = __ldg(cv + vi.y), c2 = __ldg(cv + vi.z), c3 = __ldg(cv + vi.w);
-            const float4 p0 = make_float4(R.q[0] * c0.x, R.q[0] * c0.y, R.q[0] * c0.z, R.q[0] * c0.w);
-            const float4 p1 = make_float4(R.q[1] * c1.x, R.q[1] * c1.y, R.q[1] * c1.z, R.q[1] * c1.w);
-            const float4 p2 = make_float4(R.q[2] * c2.x, R.q[2] * c2.y, R.q[2] * c2.z, R.q[2] * c2.w);
-            const float4 p3 = make_float4(R.q[3] * c3.x, R.q[3] * c3.y, R.q[3] * c3.z, R.q[3] * c3.w);
-#pragma unroll
-            for (int t = 0; t < 2; ++t) {
-              if (!(vsel & (1u << (8 + t)))) continue;
-              const uint32_t kb = (vsel >> (4 * t)) & 3u, kc = (vsel >> (4 * t + 2)) & 3u;
-              const float4 a1 = kb == 1 ? p1 : (kb == 2 ? p2 : p3);
-              const float4 a2 = kc == 1 ? p1 : (kc == 2 ? p2 : p3);
-              float4* qc = qcs + (2 * lane + t) * kSlots;
-              qc[0] = p0;
-              qc[1] = make_float4(a1.x - p0.x, a1.y - p0.y, a1.z - p0.z, a1.w - p0.w);
-              qc[2] = make_float4(a2.x - p0.x, a2.y - p0.y, a2.z - p0.z, a2.w - p0.w);
-            }
-          }
-        }
-      }
-      __syncwarp();
-      // ---- 3. transpose: lane = pixel, bit c = covered by triangle t of quad c -----------
-      uint32_t m0 = warp_transpose32(tm0, lane), m1 = warp_transpose32(tm1, lane);
-      if (!pix_ok) m0 = m1 = 0;
-      cnt += __popc(m0) + __popc(m1);
-      // ---- 4. fragments in candidate order through the K-slot sorter -----------------
-      // one fragment per iteration: the lowest candidate with a covering triangle, T0
-      // before T1 when both cover the pixel
-      auto frag_step = [&]() {
-        const int c = __ffs(m0 | m1) - 1;
-        const uint32_t cb = 1u << c;
-        // the bit leaves m0 if set there, else m1 (no branch on which)
-        const uint32_t in0 = m0 & cb;
-        m0 ^= in0;
-        m1 ^= cb ^ in0;
-        const int t = in0 ? 0 : 1;
-        const TriSm& T = tris[2 * c + t];
-        const int4 eb = T.eb;
-        const uint32_t fl = (uint32_t)eb.z, id = (uint32_t)eb.w;
-        if (hashing) hsh += splitmix64(id);
-        // (the forward discards a flagged pixel's composite, the exact path redoing it, so it
-        // keeps inserting rather than testing the flag per fragment; the backward must not
-        // add a flagged pixel's gradient)
-        if (!BWD || !st.flagged) {
-          const float4 kq = T.kq;
-          float l1 = 0.f, l2 = 0.f;
-          // (the colour-carrying variant keeps one path: its branch cost more than it saved)
-          const float key = (!VTX && (fl & kTriConstKey)) ? kq.x : tri_key(T, T.ea, eb, kq, lx, ly, px, py, l1, l2);
-          const unsigned long long sk = ((unsigned long long)__float_as_uint(key) << 32) | id;
-          float4 col = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (VTX) {
-            const float4* qc = qcs + (2 * c + t) * kSlots;
-            {
-              // perspective-correct colour: interpolated (c / w) divided by the
-              // interpolated 1/w, which is the depth key; a flat-colour triangle of the
-              // batch has zero increments and the scale 1, so a select replaces a branch
-              // per fragment (a0 + l1 * 0 + l2 * 0 and the product by 1 are exact)
-              const float rk = (fl & kTriFlatCol) ? 1.0f : rcp_approx(key);
-              const float4 a0 = qc[0], d1 = qc[1], d2 = qc[2];
-              col.x = (a0.x + l1 * d1.x + l2 * d2.x) * rk;
-              col.y = (a0.y + l1 * d1.y + l2 * d2.y) * rk;
-              col.z = (a0.z + l1 * d1.z + l2 * d2.z) * rk;
-              col.w = (a0.w + l1 * d1.w + l2 * d2.w) * rk;
-              if (LIT && (fl & kTriLit)) {
-                // the interpolated normal (times the interpolated 1/w, which only scales
-                // it); two-sided Lambert term plus ambient on RGB
-                const float4 m0 = qc[3], e1 = qc[4], e2 = qc[5];
-                const float nx = m0.x + l1 * e1.x + l2 * e2.x;
-                const float ny = m0.y + l1 * e1.y + l2 * e2.y;
-                const float nz = m0.z + l1 * e1.z + l2 * e2.z;
-                const float nn = nx * nx + ny * ny + nz * nz;
-                const float d = fabsf(nx * light.x + ny * light.y + nz * light.z);
-                const float lam = nn > 0.f ? fminf(d * rsqrtf(nn), 1.0f) : 0.f;
-                const float f = light.w + (1.0f - light.w) * lam;
-                col.x *= f;
-                col.y *= f;
-                col.z *= f;
-              }
-            }
-          }
-          st.insert(sk, col, V);
-        }
-      };
-      if (VTX) {
-        while (m0 | m1) frag_step();
-      } else {
-        // two fragments per iteration (measured faster without colours carried, slower
-        // with them)
-        while (m0 | m1) {
-          frag_step();
-          if (!(m0 | m1)) break;
-          frag_step();
-        }
-      }
-      __syncwarp();
-    };
 
     // The backward pass streams the half-block twice: first without gradients, to learn
     // which pixels the sorter cannot order (those are left to the exact path, which
@@ -798,13 +691,241 @@ __global__ __launch_bounds__(kRasterThreads, LR_RASTER_MIN_BLOCKS) void k_raster
     const uint32_t* row = hb_row(ws, off, bin_g, n, hb);
     const int nw = (n + 31) >> 5;
     const uint32_t* ref_lo = reinterpret_cast<const uint32_t*>(ws.refs + off);   // low words
-    for (int g = 0; g < nw; g += 32) {
-      BitRounds br;
-      br.prepare(g + lane < nw ? __ldg(row + g + lane) : 0u, lane);
-      for (int r0 = 0; r0 < br.total; r0 += 32) {
+    int g = -32, r0 = 0;          // bitmap window and position in it
+    BitRounds br;
+    br.total = 0;
+    int head = 0, tail = 0;       // pending ring
+    bool ordered = !HASH && !BWD; // everything so far was blended in stream order
+    for (;;) {
+      // ---- 2. coverage masks of 32 candidates, one quad per lane, until a batch is full ---
+      while (tail - head < 32) {
+        if (r0 >= br.total) {
+          g += 32;
+          if (g >= nw) break;
+          br.prepare(g + lane < nw ? __ldg(row + g + lane) : 0u, lane);
+          r0 = 0;
+          continue;
+        }
         const int j = br.get(r0, lane);
-        process(min(32, br.total - r0), j < 0 ? 0u : ~ref_lo[2 * (32 * g + j)]);
+        r0 += 32;
+        const bool in = j >= 0;
+        const uint32_t rec = in ? ~ref_lo[2 * (32 * g + j)] : 0u;
+        bool skip = !in;
+        if (ATH) {
+          // The smallest key a fragment must exceed to change any pixel of the half-block:
+          // 0 while a pixel still blends; a finished pixel needs a fragment in front of the
+          // one that finished it (keys are positive floats, so their bits order like them);
+          // pixels outside the image and pixels left to the exact path need nothing. A
+          // candidate whose largest possible key is below that is skipped: every fragment
+          // of it would be dropped.
+          const uint32_t need = (!pix_ok || st.flagged) ? 0xFFFFFFFFu : (st.live() ? 0u : (uint32_t)(st.last >> 32));
+          const uint32_t kmin = __reduce_min_sync(0xffffffffu, need);
+          if (kmin != 0u) {
+            if (in) {
+              const int4 qv = __ldg(ws.rec + 4ull * rec + 2);   // the record's four 1/w
+              const float qm = fmaxf(fmaxf(__int_as_float(qv.x), __int_as_float(qv.y)),
+                                     fmaxf(__int_as_float(qv.z), __int_as_float(qv.w)));
+              skip = __float_as_uint(qm * kKeyBoundScale) < kmin;
+            }
+            if (__all_sync(0xffffffffu, skip)) continue;
+          }
+        }
+        uint32_t ma = 0, mb = 0, ida = 0, idb = 0;
+        if (!skip) {
+          const int4* rp = ws.rec + 4ull * rec;
+          const int4 r0v = __ldg(rp), r1v = __ldg(rp + 1);
+          const int2 fl = __ldg(reinterpret_cast<const int2*>(rp + 3) + 1);   // info, record flags
+          const int X[4] = {r0v.x, r0v.z, r1v.x, r1v.z}, Y[4] = {r0v.y, r0v.w, r1v.y, r1v.w};
+          const uint32_t info = (uint32_t)fl.x;
+          if (fl.y & (int)kRecSmall) quad_masks_small(X, Y, info, Ox, Oy, ma, mb);
+          else quad_masks_any(X, Y, info, Ox, Oy, ma, mb);
+          ida = 2u * (uint32_t)(rec - V.quad_base);
+          idb = ida + 1u;
+          if (flat_view && (info & kInfoFlatDepth)) {
+            // one colour and one depth key for the whole quad: its triangles form one entry
+            // where they do not overlap, else the second goes first (it lies in front: equal
+            // keys order by triangle)
+            if (!HASH && (ma & mb) == 0u) {
+              ma |= mb;
+              mb = 0u;
+            } else {
+              const uint32_t t = ma; ma = mb; mb = t;
+              const uint32_t u = ida; ida = idb; idb = u;
+            }
+            ida |= kPendConst;
+            idb |= kPendConst;
+          }
+        }
+        const unsigned ba = __ballot_sync(0xffffffffu, ma != 0u), bb = __ballot_sync(0xffffffffu, mb != 0u);
+        const unsigned lt = (1u << lane) - 1u;
+        int at = tail + __popc(ba & lt) + __popc(bb & lt);
+        if (ma) pend[at++ & (kPendCap - 1)] = make_uint2(ida, ma);
+        if (mb) pend[at & (kPendCap - 1)] = make_uint2(idb, mb);
+        tail += __popc(ba) + __popc(bb);
+        __syncwarp();
       }
+      const int nb = min(32, tail - head);
+      if (nb == 0) break;
+      // ---- 3. records of the next nb covering triangles, one per lane; entry 31 - L of the
+      // batch goes to lane and slot L, so that the highest set bit is the next in order ------
+      const int e = 31 - lane;
+      uint32_t id = 0, mk = 0;
+      if (e < nb) {
+        const uint2 pe = pend[(head + e) & (kPendCap - 1)];
+        id = pe.x;
+        mk = pe.y;
+      }
+      head += nb;
+      const bool direct = ordered && __all_sync(0xffffffffu, e >= nb || (id & kPendConst));
+      id &= ~kPendConst;
+      if (direct) {
+        if (e < nb) {
+          const float q0 = __ldg(reinterpret_cast<const float*>(ws.rec + 4ull * (uint32_t)(V.quad_base + (id >> 1)) + 2));
+          qc[lane] = __ldg(reinterpret_cast<const float4*>(V.col) + (id >> 1));
+          dkey[lane] = ((unsigned long long)__float_as_uint(q0) << 32) | id;
+        }
+      } else if (e < nb) {
+        const int t = (int)(id & 1u);
+        const uint32_t jl = id >> 1;
+        const QuadRec R = load_rec(ws.rec, (uint32_t)(V.quad_base + jl));
+        const bool sw = (R.info & (kInfoSwap0 << t)) != 0;
+        // vertices a = v0 and, oriented to a positive area, b and c
+        const int xa = R.X[0], ya = R.Y[0];
+        const int x1 = t ? R.X[2] : R.X[1], y1 = t ? R.Y[2] : R.Y[1];
+        const int x2 = t ? R.X[3] : R.X[2], y2 = t ? R.Y[3] : R.Y[2];
+        const float q1 = t ? R.q[2] : R.q[1], q2 = t ? R.q[3] : R.q[2];
+        const int xb = sw ? x2 : x1, yb = sw ? y2 : y1, xc = sw ? x1 : x2, yc = sw ? y1 : y2;
+        const float qb = sw ? q2 : q1, qc2 = sw ? q1 : q2;
+        geo.kq[lane] = make_float4(R.q[0], __fsub_rn(qb, R.q[0]), __fsub_rn(qc2, R.q[0]), t ? R.inv[1] : R.inv[0]);
+        // edges c -> a and a -> b, both through a
+        const int dx1 = xa - xc, dy1 = ya - yc, dx2 = xb - xa, dy2 = yb - ya;
+        const int ux = Ox - xa, uy = Oy - ya;
+        if (R.info & (kInfoSmall0 << t)) {
+          geo.ea[lane] = make_int4((int)((uint32_t)dx1 * (uint32_t)uy - (uint32_t)dy1 * (uint32_t)ux),
+                                   (int)((uint32_t)dx2 * (uint32_t)uy - (uint32_t)dy2 * (uint32_t)ux), -256 * dy1, -256 * dy2);
+          geo.eb[lane] = make_int4(256 * dx1, 256 * dx2, 0, (int)id);
+        } else {
+          // 64-bit edge values: E + 256 (ly dx - lx dy)
+          const long long e1 = (long long)dx1 * uy - (long long)dy1 * ux, e2 = (long long)dx2 * uy - (long long)dy2 * ux;
+          geo.ea[lane] = make_int4((int)(uint32_t)e1, (int)(uint32_t)e2, -dy1, -dy2);
+          geo.hi[lane] = make_int2((int)(e1 >> 32), (int)(e2 >> 32));
+          geo.eb[lane] = make_int4(dx1, dx2, (int)kTriWide, (int)id);
+        }
+        if (VTX && !flat_view) {
+          const uint4 vi = V.idx ? __ldg(reinterpret_cast<const uint4*>(V.idx) + jl)
+                                 : make_uint4(4 * jl, 4 * jl + 1, 4 * jl + 2, 4 * jl + 3);
+          const uint32_t w1 = t ? vi.z : vi.y, w2 = t ? vi.w : vi.z;
+          const uint32_t vb = sw ? w2 : w1, vc = sw ? w1 : w2;
+          const float4* cv = reinterpret_cast<const float4*>(V.col);
+          const bool lit = LIT && V.color_mode == LR_COLOR_LIT;
+          const uint32_t cs = lit ? 2u : 1u;
+          // corner colours times 1/w, as (c0, c1 - c0, c2 - c0) for the fragment's
+          // c0 + l1 (c1 - c0) + l2 (c2 - c0); lit: the same for the normals
+          const float4 c0 = __ldg(cv + (size_t)cs * vi.x), c1 = __ldg(cv + (size_t)cs * vb), c2 = __ldg(cv + (size_t)cs * vc);
+          const float qa = R.q[0];
+          const float4 p0 = make_float4(qa * c0.x, qa * c0.y, qa * c0.z, qa * c0.w);
+          qc[lane] = p0;
+          qc[32 + lane] = make_float4(qb * c1.x - p0.x, qb * c1.y - p0.y, qb * c1.z - p0.z, qb * c1.w - p0.w);
+          qc[64 + lane] = make_float4(qc2 * c2.x - p0.x, qc2 * c2.y - p0.y, qc2 * c2.z - p0.z, qc2 * c2.w - p0.w);
+          if (LIT && lit) {
+            const float4 n0 = __ldg(cv + 2ull * vi.x + 1), n1 = __ldg(cv + 2ull * vb + 1), n2 = __ldg(cv + 2ull * vc + 1);
+            const float4 o0 = make_float4(qa * n0.x, qa * n0.y, qa * n0.z, 0.f);
+            qc[96 + lane] = o0;
+            qc[128 + lane] = make_float4(qb * n1.x - o0.x, qb * n1.y - o0.y, qb * n1.z - o0.z, 0.f);
+            qc[160 + lane] = make_float4(qc2 * n2.x - o0.x, qc2 * n2.y - o0.y, qc2 * n2.z - o0.z, 0.f);
+          }
+        } else if (kCarry) {
+          qc[lane] = __ldg(reinterpret_cast<const float4*>(V.col) + jl);
+        }
+      }
+      // ---- 4. transpose: lane = pixel, bit L = covered by the triangle in slot L -----------
+      uint32_t m = warp_transpose32(mk, lane);   // (its shuffles also order the slots' writes below)
+      __syncwarp();
+      if (!pix_ok) m = 0;
+      cnt += __popc(m);
+      if (direct) {
+        // ---- 5a. flat colours at constant depths, everything before them likewise: the
+        // stream order is the fragments' exact order (the bin sort's key is the depth key), so
+        // they blend as they come, without the sorter
+        const uint32_t all = m;
+        uint32_t lastp = 32;
+        while (m) {
+          if (ATH && !st.live()) break;
+          const int p = 31 - __clz(m);
+          m ^= 1u << p;
+          const float4 c = qc[p];
+          if (ATH) lastp = (uint32_t)p;
+          st.blend_direct(c);
+        }
+        if (!ATH) lastp = (uint32_t)(__ffs(all) - 1);
+        if (lastp < 32u) st.last = dkey[lastp];
+      } else {
+        if (ordered) {
+          // the sorter starts here; with a transparent held fragment at the last key blended
+          // (K = 1), so that its first eviction keeps that key
+          ordered = false;
+          if (PixelState<K, kCarry, BWD, ATH>::kNullSlot) st.s[0] = st.last;
+        }
+        // ---- 5b. fragments in candidate order through the K-slot sorter -------------------
+        auto frag_step = [&]() {
+          const int p = 31 - __clz(m);
+          m ^= 1u << p;
+          const int4 eb = geo.eb[p];
+          const uint32_t fid = (uint32_t)eb.w;
+          if (hashing) hsh += splitmix64(fid);
+          // (the forward discards a flagged pixel's composite, the exact path redoing it, so it
+          // keeps inserting rather than testing the flag per fragment; the backward must not
+          // add a flagged pixel's gradient)
+          if (!BWD || !st.flagged) {
+            const int4 ea = geo.ea[p];
+            const float4 kq = geo.kq[p];
+            float f1, f2;
+            if (!((uint32_t)eb.z & kTriWide)) {
+              f1 = __int2float_rn((int)((uint32_t)ea.x + (uint32_t)lx * (uint32_t)ea.z + (uint32_t)ly * (uint32_t)eb.x));
+              f2 = __int2float_rn((int)((uint32_t)ea.y + (uint32_t)lx * (uint32_t)ea.w + (uint32_t)ly * (uint32_t)eb.y));
+            } else {
+              const int2 h = geo.hi[p];
+              const long long e1 = ((long long)h.x << 32) | (uint32_t)ea.x, e2 = ((long long)h.y << 32) | (uint32_t)ea.y;
+              f1 = __ll2float_rn(e1 + 256LL * (lx * ea.z + ly * eb.x));
+              f2 = __ll2float_rn(e2 + 256LL * (lx * ea.w + ly * eb.y));
+            }
+            // exact depth key: the interpolated 1/w (Sec. 2 "Stage 3", the reading O.8)
+            const float l1 = __fmul_rn(f1, kq.w), l2 = __fmul_rn(f2, kq.w);
+            const float key = __fadd_rn(kq.x, __fadd_rn(__fmul_rn(l1, kq.y), __fmul_rn(l2, kq.z)));
+            const unsigned long long sk = ((unsigned long long)__float_as_uint(key) << 32) | fid;
+            float4 col = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (kCarry) col = qc[p];
+            if (VTX && !flat_view) {
+              // perspective-correct colour: interpolated (c / w) divided by the
+              // interpolated 1/w, which is the depth key
+              const float rk = rcp_approx(key);
+              const float4 d1 = qc[32 + p], d2 = qc[64 + p];
+              col.x = (col.x + l1 * d1.x + l2 * d2.x) * rk;
+              col.y = (col.y + l1 * d1.y + l2 * d2.y) * rk;
+              col.z = (col.z + l1 * d1.z + l2 * d2.z) * rk;
+              col.w = (col.w + l1 * d1.w + l2 * d2.w) * rk;
+              if (LIT && V.color_mode == LR_COLOR_LIT) {
+                // the interpolated normal (times the interpolated 1/w, which only scales
+                // it); two-sided Lambert term plus ambient on RGB
+                const float4 n0 = qc[96 + p], n1 = qc[128 + p], n2 = qc[160 + p];
+                const float nx = n0.x + l1 * n1.x + l2 * n2.x;
+                const float ny = n0.y + l1 * n1.y + l2 * n2.y;
+                const float nz = n0.z + l1 * n1.z + l2 * n2.z;
+                const float nn = nx * nx + ny * ny + nz * nz;
+                const float d = fabsf(nx * light.x + ny * light.y + nz * light.z);
+                const float lam = nn > 0.f ? fminf(d * rsqrtf(nn), 1.0f) : 0.f;
+                const float f = light.w + (1.0f - light.w) * lam;
+                col.x *= f;
+                col.y *= f;
+                col.z *= f;
+              }
+            }
+            st.insert(sk, col, V);
+          }
+        };
+        while (m) frag_step();
+      }
+      __syncwarp();
     }
     if (pass == 0) pre_flagged = st.flagged;
     }

@@ -109,7 +109,7 @@ __global__ __launch_bounds__(256) void k_setup(Ws ws) {
       }
       if (why != kVisible && (worst == kVisible || why < worst)) worst = why;
     }
-    uint32_t info = 0;
+    uint32_t info = 0, rflags = 0;
     float rep = 0.f;
     float2 inv = make_float2(0.f, 0.f);
     uint2 rect = make_uint2(kRectInvisible, kRectInvisible);
@@ -147,6 +147,12 @@ __global__ __launch_bounds__(256) void k_setup(Ws ws) {
         const int xmax = max(max(X[0], X[1]), max(X[2], X[3]));
         const int ymin = min(min(Y[0], Y[1]), min(Y[2], Y[3]));
         const int ymax = max(max(Y[0], Y[1]), max(Y[2], Y[3]));
+        {
+          // the same bound for the whole quad's box (any of its edges)
+          const uint32_t wx = (uint32_t)(xmax - xmin), wy = (uint32_t)(ymax - ymin);
+          if (wx < 32768u && wy < 32768u && wx * (wy + 3u * 256u) + wy * (wx + 7u * 256u) + 1u < (1u << 30))
+            rflags = kRecSmall;
+        }
         const int px0 = max(ceil_div256((long long)xmin - 128), 0);
         const int px1 = min(floor_div256((long long)xmax - 128), V.width - 1);
         const int py0 = max(ceil_div256((long long)ymin - 128), 0);
@@ -175,7 +181,7 @@ __global__ __launch_bounds__(256) void k_setup(Ws ws) {
       rp[0] = make_int4(X[0], Y[0], X[1], Y[1]);
       rp[1] = make_int4(X[2], Y[2], X[3], Y[3]);
       rp[2] = make_int4(__float_as_int(q[0]), __float_as_int(q[1]), __float_as_int(q[2]), __float_as_int(q[3]));
-      rp[3] = make_int4(__float_as_int(inv.x), __float_as_int(inv.y), (int)info, 0);
+      rp[3] = make_int4(__float_as_int(inv.x), __float_as_int(inv.y), (int)info, (int)rflags);
       ws.rec_rep[g] = rep;
     }
     ws.rec_rect[g] = rect;
