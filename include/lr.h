@@ -96,12 +96,10 @@ typedef struct {
                                 and 16 for dense regions); default 32. Any bin size gives the
                                 same exact image: it changes how many (quad, bin) references
                                 binning makes and how large the per-bin depth sorts are. */
-  int32_t block_h;           /* rows of the rasteriser's work item: 4 (8x4 half-blocks, the
-                                default) or 8 (8x8 blocks, Sec. 2, Stage 3, Phase 2: a quad
-                                meeting both halves is set up once). 8 applies to forward
-                                exact renders with flat or per-vertex colours and sorter_k
-                                1, 2 or 3; other renders of the context use 8x4. The image
-                                is the same either way. */
+  int32_t block_h;           /* 4 (default) or 8. Both take the same kernels, which choose the
+                                rasteriser's work item per bin: 8x8 blocks (Sec. 2, Stage 3,
+                                Phase 2) where a bin holds only flat-colour quads of constant
+                                depth, 8x4 half-blocks elsewhere. */
   int32_t shared_setup;      /* 1: a CTA of 8 warps rasterises a 32x8 strip of a bin (one 8x4
                                 half-block per warp) and sets each candidate triangle up once
                                 for the strip in shared memory (Sec. 2, Stage 3: a bin's
@@ -206,8 +204,9 @@ typedef struct {
  *                        Y2 X3 Y3 (snapped, 1/256 pixel), the four vertices' 1/w (f32 bits),
  *                        1/|A0| and 1/|A1| (f32 bits of the reciprocal doubled triangle
  *                        areas, 0 for a zero-area triangle), info (as rec_info, cull reason
- *                        0), flags (bit 0: 32-bit edge arithmetic is exact on every 8x4
- *                        half-block the quad's box touches)
+ *                        0), flags (bit 0: every edge value is below 2^30 on every 8x4
+ *                        and 8x8 block the quad's box touches; bit 1: the snapped quad is an
+ *                        axis-parallel rectangle)
  *   rec_rect  u32[Q][2]  pixel-centre AABB: px0 | px1 << 16, py0 | py1 << 16
  *                        (0x0000FFFF, 0x0000FFFF for a culled quad)
  *   rec_info  u32[Q]     bit 0/1: triangle 0/1 has non-zero area, bit 2: spans more than

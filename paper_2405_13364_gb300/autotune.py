@@ -1,14 +1,14 @@
 """Autotuner for the rasteriser's launch parameters.
 
 Tunable here: the per-pixel sorter capacity K (the paper's depth-filter size, Sec. 2
-"Sample blending"), the rasteriser's work item (8x4 half-blocks or 8x8 blocks, Sec. 2,
+"Sample blending"), the rasteriser's set-up (per warp, or shared by a CTA, Sec. 2,
 Stage 3), the bin size of the binning stage (16, 32 or 64 pixels; Sec. 2, Stage 2
 uses 32 and Sec. 4 proposes 64 and 16 for sparse and dense regions), the number of
 persistent rasteriser CTAs per SM, and for flat-colour scenes whether the sorter carries
 colours. Every candidate gives the same coverage and the same exact fragment order; K only
 moves pixels between the sorter and the exact overflow path, whose composite sums in a
 different order, so colours agree to fp32 rounding (the tuner checks 1e-5, the accuracy
-bar) rather than bit for bit. The work item is an 8x4 half-block per warp, an 8x8 block per
+bar) rather than bit for bit. The work item is an 8x4 half-block or an 8x8 block per
 warp, or (shared set-up) a 32x8 strip per CTA whose candidates the CTA sets up together.
 
 The tuner renders the workload with every candidate, checks that all candidates produce
@@ -67,7 +67,7 @@ def tune(scene, width: int, height: int, ks=DEFAULT_KS, ctas_per_sm=(0,), reps: 
     """scene: a DeviceScene. Returns {'sorter_k', 'raster_ctas_per_sm', 'carry_colors',
     'bin_size', 'block_h', 'ms', 'table'}. carry: candidates for carrying flat colours in the
     sorter (default: both for flat-colour scenes). bin_sizes: candidate bin sizes (16, 32,
-    64). block_hs: candidate work-item heights (4: 8x4 half-blocks, 8: 8x8 blocks, built
+    64). block_hs: values of lr_config.block_h (4 and 8 take the same kernels; 8 is tried
     for sorter capacities up to 3). shared: whether a CTA sets candidates up once per 32x8
     strip (lr_config.shared_setup; 32-pixel bins, 8x4 half-blocks, capacities up to 3)."""
     from . import Renderer

@@ -46,12 +46,6 @@ LR_DECLARE_RASTER(4)
 LR_DECLARE_RASTER(6)
 LR_DECLARE_RASTER(8)
 LR_DECLARE_RASTER(12)
-#define LR_DECLARE_RASTER8(KK)                                                                    \
-  cudaError_t prepare_raster8_##KK(int* blocks_flat, int* blocks_vtx);                            \
-  cudaError_t launch_raster8_##KK(int mode, const Ws& ws, int grid, cudaStream_t st);
-LR_DECLARE_RASTER8(1)
-LR_DECLARE_RASTER8(2)
-LR_DECLARE_RASTER8(3)
 #define LR_DECLARE_RASTER_STRIP(KK)                                                               \
   cudaError_t prepare_raster_strip_##KK(int* blocks_flat, int* blocks_vtx);                       \
   cudaError_t launch_raster_strip_##KK(int mode, const Ws& ws, int grid, cudaStream_t st);
@@ -67,28 +61,26 @@ __global__ void k_write_views(ViewChunk chunk, ViewDev* dst) {
 
 typedef cudaError_t (*PrepareFn)(int*, int*, int*, int*);
 typedef cudaError_t (*LaunchFn)(int, const Ws&, int, cudaStream_t);   // mode 0 flat, 1 colours, 2 backward
-typedef cudaError_t (*Prepare8Fn)(int*, int*);
+typedef cudaError_t (*PrepareStripFn)(int*, int*);
 
-// A sorter capacity's rasterisers: 8x4 half-blocks (every mode) and, for K <= 3, 8x8 blocks
-// (forward exact renders, flat or carried colours, with or without the coverage hash).
+// A sorter capacity's rasterisers: the one of lr_raster.cuh (every mode) and, for K <= 3, the
+// strip form (forward exact renders, flat or carried colours, with or without the hash).
 struct RasterVariant {
   int k;
   PrepareFn prepare;
   LaunchFn launch;
-  Prepare8Fn prepare8;
-  LaunchFn launch8;
-  Prepare8Fn prepare_strip;   // the per-strip shared set-up (lr_raster_strip.cuh)
+  PrepareStripFn prepare_strip;   // the per-strip shared set-up (lr_raster_strip.cuh)
   LaunchFn launch_strip;
 };
 
 static const RasterVariant kVariants[] = {
-    {1, prepare_raster_1, launch_raster_1, prepare_raster8_1, launch_raster8_1, prepare_raster_strip_1, launch_raster_strip_1},
-    {2, prepare_raster_2, launch_raster_2, prepare_raster8_2, launch_raster8_2, prepare_raster_strip_2, launch_raster_strip_2},
-    {3, prepare_raster_3, launch_raster_3, prepare_raster8_3, launch_raster8_3, prepare_raster_strip_3, launch_raster_strip_3},
-    {4, prepare_raster_4, launch_raster_4, nullptr, nullptr, nullptr, nullptr},
-    {6, prepare_raster_6, launch_raster_6, nullptr, nullptr, nullptr, nullptr},
-    {8, prepare_raster_8, launch_raster_8, nullptr, nullptr, nullptr, nullptr},
-    {12, prepare_raster_12, launch_raster_12, nullptr, nullptr, nullptr, nullptr},
+    {1, prepare_raster_1, launch_raster_1, prepare_raster_strip_1, launch_raster_strip_1},
+    {2, prepare_raster_2, launch_raster_2, prepare_raster_strip_2, launch_raster_strip_2},
+    {3, prepare_raster_3, launch_raster_3, prepare_raster_strip_3, launch_raster_strip_3},
+    {4, prepare_raster_4, launch_raster_4, nullptr, nullptr},
+    {6, prepare_raster_6, launch_raster_6, nullptr, nullptr},
+    {8, prepare_raster_8, launch_raster_8, nullptr, nullptr},
+    {12, prepare_raster_12, launch_raster_12, nullptr, nullptr},
 };
 
 struct Layout {
@@ -97,6 +89,7 @@ struct Layout {
   size_t refs, refs_tmp, ref_hb, ovf_list, total;
   long long total_quads = 0, total_pix = 0, refs_cap = 0;
   int total_bins = 0, total_chunks = 0;
+  int cursors = 0;
 };
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -113,6 +106,7 @@ static Layout make_layout(int n, const long long* Q, const int* W, const int* H,
     L.total_quads += Q[i];
     L.total_pix += (long long)W[i] * H[i];
     L.total_bins += nbx * nby;
+    L.cursors |= nbx * nby > kHistSmemBins;
     L.total_chunks += (int)((Q[i] + kChunkQuads - 1) / kChunkQuads);
   }
   size_t o = 0;
@@ -175,6 +169,8 @@ static Ws make_ws(const Layout& L, void* base, int n_views) {
   w.total_pix = L.total_pix;
   w.refs_cap = L.refs_cap;
   w.bin_log2 = L.bin_log2;
+  w.cursors = L.cursors;
+  w.ticket = 1;
   w.rec = reinterpret_cast<int4*>(b + L.rec);
   w.rec_rect = reinterpret_cast<uint2*>(b + L.rec_rect);
   w.rec_info = reinterpret_cast<uint32_t*>(b + L.rec_info);
@@ -200,7 +196,6 @@ using namespace lr;
 struct VariantState {
   const RasterVariant* v = nullptr;
   int flat = 1, vtx = 1, bwd = 1, lit = 1;
-  int flat8 = 1, vtx8 = 1;     // the 8x8-block kernels (when the capacity has them)
   int flat_s = 1, vtx_s = 1;   // the strip kernels
 };
 
@@ -281,9 +276,8 @@ extern "C" lr_status lr_create(const lr_config* config, lr_ctx** out_ctx) {
     VariantState& V = c->vs[i];
     V.v = &kVariants[i];
     e = V.v->prepare(&V.flat, &V.vtx, &V.bwd, &V.lit);
-    if (e == cudaSuccess && V.v->prepare8 && g.block_h == 8) e = V.v->prepare8(&V.flat8, &V.vtx8);
     if (e == cudaSuccess && V.v->prepare_strip && g.shared_setup) e = V.v->prepare_strip(&V.flat_s, &V.vtx_s);
-    int* all[] = {&V.flat, &V.vtx, &V.bwd, &V.lit, &V.flat8, &V.vtx8, &V.flat_s, &V.vtx_s};
+    int* all[] = {&V.flat, &V.vtx, &V.bwd, &V.lit, &V.flat_s, &V.vtx_s};
     for (int* x : all) {
       if (g.raster_ctas_per_sm > 0) *x = std::min(*x, g.raster_ctas_per_sm);
       *x = std::max(*x, 1);
@@ -589,18 +583,20 @@ static lr_status launch_sequence(lr_ctx* ctx, const Prepared& P, cudaStream_t st
   const int mode = bwd ? 2 : (P.any_lit ? 17 : ((carry ? 1 : 0) | (P.any_hash ? 4 : 0) | (ath ? 8 : 0)));
   ws.t_min = ath ? kAlphaTMin : 0.0f;
   const VariantState& VS = ctx->vs[P.variant];
-  // the strip kernel (32-pixel bins) or 8x8 blocks for forward exact renders of flat or
-  // carried colours, when asked for and built
+  // the strip kernel (32-pixel bins) for forward exact renders of flat or carried colours, when
+  // asked for and built
   const bool strip = ctx->cfg.shared_setup && VS.v->launch_strip && !bwd && !ath && !P.any_lit &&
                      ctx->bin_log2 == kBinLog2Default;
-  const bool blk8 = !strip && ctx->cfg.block_h == 8 && VS.v->launch8 && !bwd && !ath && !P.any_lit;
   cudaError_t e;
   if (strip) {
     e = VS.v->launch_strip(mode, ws, ctx->sms * (carry ? VS.vtx_s : VS.flat_s), st);
-  } else if (blk8) {
-    e = VS.v->launch8(mode, ws, ctx->sms * (carry ? VS.vtx8 : VS.flat8), st);
   } else {
     const int rblocks = bwd ? VS.bwd : (P.any_lit ? VS.lit : (carry ? VS.vtx : VS.flat));
+    // two half-blocks per ticket once every warp gets at least four tickets: a bin blended in
+    // list order needs only one of the two (300k particles at 2560x1440: 106 -> 86 us); with
+    // fewer the queue's tail costs more (four 512x384 views, 35 -> 49 us)
+    const long long warps = (long long)ctx->sms * rblocks * kRasterWarps;
+    if ((long long)L.total_bins * bin_hb(ctx->bin_log2) >= 8 * warps) ws.ticket = 2;
     e = VS.v->launch(mode, ws, ctx->sms * rblocks, st);
   }
   if (e != cudaSuccess) return cuda_fail(ctx, e, "raster launch");

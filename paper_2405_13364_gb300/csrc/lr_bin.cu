@@ -154,8 +154,11 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_count(Ws ws)
   if (smem)
     for (int b = threadIdx.x; b < nb; b += blockDim.x) hist[b] = 0u;
   __syncthreads();
-  for_each_ref<true>(ws, V, q0, q1, [&](long long, int b, int, int, uint2, uint32_t) {
-    if (smem) atomicAdd(&hist[b], 1u);
+  // (the high half of a shared counter counts the references to quads of varying depth; a chunk
+  // makes at most kChunkQuads of either per bin)
+  static_assert(kChunkQuads < 65536, "chunk counters share a word");
+  for_each_ref<true>(ws, V, q0, q1, [&](long long, int b, int, int, uint2, uint32_t info) {
+    if (smem) atomicAdd(&hist[b], (info & kInfoFlatDepth) ? 1u : 0x10001u);
     else atomicAdd(&ws.bin_count[V.bin_base + b], 1u);
   });
   __syncthreads();
@@ -176,8 +179,9 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_count(Ws ws)
   __syncthreads();
   uint2* list = reinterpret_cast<uint2*>(ws.refs_tmp);
   for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-    const uint32_t c = hist[b];
+    const uint32_t c = hist[b] & 0xFFFFu;
     if (!c) continue;
+    if (!ws.cursors && (hist[b] >> 16)) ws.bin_cursor[V.bin_base + b] = 1u;   // not of constant depths
     const uint32_t base = atomicAdd(&ws.bin_count[V.bin_base + b], c);
     const unsigned long long at = (unsigned long long)s_start + atomicAdd(&s_pos, 1u);
     // a list past the reference capacity means the references do not fit either: the scan
@@ -235,7 +239,7 @@ __global__ __launch_bounds__(1024) void k_bin_scan(Ws ws) {
     if (i < n) {
       const unsigned long long excl = incl - c;
       ws.bin_off[i] = (uint32_t)min(excl, (unsigned long long)ws.refs_cap);
-      ws.bin_cursor[i] = (uint32_t)min(excl, (unsigned long long)ws.refs_cap);
+      if (ws.cursors) ws.bin_cursor[i] = (uint32_t)min(excl, (unsigned long long)ws.refs_cap);
     }
     __syncthreads();
     if (tid == 1023) carry = incl;

@@ -70,8 +70,9 @@ constexpr uint32_t kInfoSwap0 = 16u;        // triangle t (bit << t): negative a
 constexpr uint32_t kInfoSmall0 = 64u;       // triangle t (bit << t): 32-bit edge values are
                                             // exact on every half-block its box touches
 // flags in word 15 of the record
-constexpr uint32_t kRecSmall = 1u;          // 32-bit edge values are exact on every half-block
-                                            // the quad's box touches
+constexpr uint32_t kRecSmall = 1u;          // every edge value is below 2^30 on every 8x4 and
+                                            // 8x8 block the quad's box touches
+constexpr uint32_t kRecBox = 2u;            // the snapped quad is an axis-parallel rectangle
 constexpr uint32_t kRectInvisible = 0x0000FFFFu;   // rect.x value of a culled quad
 
 struct ViewDev {
@@ -184,16 +185,40 @@ struct QuadRec {
   uint32_t info;
 };
 
+// 32-byte loads and stores (32-byte aligned): a gather of one record half per lane takes half
+// the L1 data-pipe wavefronts of two 16-byte ones, whose lanes fall on the same banks (records
+// are 64 bytes apart).
+struct __align__(32) Int8 {
+  int v[8];
+};
+__device__ __forceinline__ Int8 ldg32(const void* p) {
+  Int8 r;
+  asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r.v[0]), "=r"(r.v[1]), "=r"(r.v[2]), "=r"(r.v[3]), "=r"(r.v[4]), "=r"(r.v[5]), "=r"(r.v[6]),
+                 "=r"(r.v[7])
+               : "l"(p));
+  return r;
+}
+__device__ __forceinline__ void stg32(void* p, int a, int b, int c, int d, int e, int f, int g, int h) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(a), "r"(b), "r"(c), "r"(d), "r"(e), "r"(f),
+               "r"(g), "r"(h)
+               : "memory");
+}
+
+// the record's first half
+__device__ __forceinline__ void load_rec_xy(const int4* rec, uint32_t i, int X[4], int Y[4]) {
+  const Int8 a = ldg32(rec + 4ull * i);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) { X[k] = a.v[2 * k]; Y[k] = a.v[2 * k + 1]; }
+}
 __device__ __forceinline__ QuadRec load_rec(const int4* rec, uint32_t i) {
-  const int4* p = rec + 4ull * i;
-  const int4 a = p[0], b = p[1], c = p[2], d = p[3];
   QuadRec r;
-  r.X[0] = a.x; r.Y[0] = a.y; r.X[1] = a.z; r.Y[1] = a.w;
-  r.X[2] = b.x; r.Y[2] = b.y; r.X[3] = b.z; r.Y[3] = b.w;
-  r.q[0] = __int_as_float(c.x); r.q[1] = __int_as_float(c.y);
-  r.q[2] = __int_as_float(c.z); r.q[3] = __int_as_float(c.w);
-  r.inv[0] = __int_as_float(d.x); r.inv[1] = __int_as_float(d.y);
-  r.info = (uint32_t)d.z;
+  load_rec_xy(rec, i, r.X, r.Y);
+  const Int8 b = ldg32(rec + 4ull * i + 2);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) r.q[k] = __int_as_float(b.v[k]);
+  r.inv[0] = __int_as_float(b.v[4]); r.inv[1] = __int_as_float(b.v[5]);
+  r.info = (uint32_t)b.v[6];
   return r;
 }
 
@@ -206,6 +231,8 @@ struct Ws {
   long long total_quads;
   long long total_pix;
   long long refs_cap;
+  int cursors;               // a view has more bins than the shared counters hold
+  int ticket;                // half-blocks per ticket of the rasteriser's queue: 1 or 2
   int bin_log2;              // bins of 2^bin_log2 x 2^bin_log2 pixels (the same for every view)
   int4* rec;                 // [4 * total_quads]: the 64-byte quad record (QuadRec)
   uint2* rec_rect;           // [total_quads]: pixel AABB (px0 | px1 << 16, py0 | py1 << 16)
@@ -213,7 +240,8 @@ struct Ws {
   float* rec_rep;            // [total_quads]: representative 1/w over the quad's whole box
   uint32_t* bin_count;       // [total_bins]
   uint32_t* bin_off;         // [total_bins + 1]
-  uint32_t* bin_cursor;      // [total_bins]
+  uint32_t* bin_cursor;      // [total_bins] with `cursors` the scatter's cursors, else 1 where the
+                             // bin holds a reference to a quad that is not of constant depth
   uint2* chunk_span;         // [total_chunks] (start, length) of the chunk's list of (bin, base
                              // of the chunk's range within the bin), kept in refs_tmp
   uint32_t* bin_order;       // [total_bins]: bins by decreasing reference count

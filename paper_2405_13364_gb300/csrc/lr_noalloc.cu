@@ -191,6 +191,8 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
   ws.total_pix = npix;
   ws.refs_cap = cap;
   ws.bin_log2 = kBinLog2Default;
+  ws.cursors = nbins > kHistSmemBins;
+  ws.ticket = 1;
   ws.rec = reinterpret_cast<int4*>(base + o_rec);
   ws.rec_rect = reinterpret_cast<uint2*>(base + o_rect);
   ws.rec_info = reinterpret_cast<uint32_t*>(base + o_info);

@@ -48,23 +48,21 @@
 
 namespace lr {
 
-constexpr uint32_t kTriValid = 1u, kTriFast = 2u, kTriFlatCol = 4u;   // + corr bits 3..5
-// all three vertices at the same 1/w: the depth key is q0 at every pixel (the
-// interpolation adds l1 * 0 + l2 * 0 with l1, l2 >= 0)
-constexpr uint32_t kTriConstKey = 64u;
-// lit colours (LR_COLOR_LIT): the triangle's colour slots also hold its perspective-weighted
-// normals, and each fragment's RGB is shaded with the view's light
-constexpr uint32_t kTriLit = 128u;
 // k_raster's batches: the edge values are kept in 64 bits
 constexpr uint32_t kTriWide = 256u;
 constexpr unsigned long long kSent = ~0ull;
 constexpr int kRasterThreads = 256;
-#ifndef LR_RASTER_MIN_BLOCKS
-// resident CTAs per SM requested from the compiler: 3 caps registers at 80 per thread (24
-// warps per SM, a few spills), measured faster than 2 (128 registers) on both the layer
-// and the particle workloads; without a bound the compiler takes ~160 and one CTA fits
-#define LR_RASTER_MIN_BLOCKS 3
-#endif
+// Resident CTAs per SM requested from the compiler: 3 caps registers at 80 per thread (24 warps
+// per SM), 4 at 64. Neither spills in the forward kernels up to K = 3. With four the layer frame
+// took 307 instead of 315 us and the backward 438 instead of 475, flat layers at K = 3 154
+// instead of 168; with three the particle frame 275 instead of 309, the batch of mixed views at
+// K = 3 833 instead of 868, lit layers 406 instead of 422, flat layers with the alpha threshold
+// 217 instead of 225.
+__host__ __device__ constexpr int raster_min_blocks(int k, bool vtx, bool bwd, bool ath, bool lit) {
+  if (lit || ath || k > 3) return 3;
+  if (bwd) return 4;
+  return vtx ? (k == 1 ? 4 : 3) : (k == 1 ? 3 : 4);
+}
 constexpr int kRasterWarps = kRasterThreads / 32;
 constexpr int kOvfThreads = 128;
 // alpha threshold (LR_FLAG_ALPHA_THRESHOLD, the paper's opt-in early stop, Sec. 2 "Sample
@@ -75,140 +73,6 @@ constexpr float kAlphaTMin = 1.0f / 128.0f;
 // this: the key is a convex combination of three vertex values evaluated with a handful
 // of roundings of relative size 2^-24 each, far inside the 2^-16 margin.
 constexpr float kKeyBoundScale = 1.0f + 1.0f / 65536.0f;
-
-// Per (triangle, half-block) record read by the fragment loop, laid out for three 16-byte
-// shared-memory loads. Edges 1 (v2->v0) and 2 (v0->v1) give the barycentric numerators
-// of the depth key; edge 0 is only needed for coverage, which the masks already hold.
-struct __align__(16) TriSm {
-  int4 ea;         // e1, e2: edge values E at the half-block's first pixel centre; sx1,
-                   // sx2: change per pixel step in x
-  int4 eb;         // sy1, sy2: change per pixel step in y; flags; id (2 * quad + triangle)
-  float4 kq;       // q0 = 1/w at v0, d1 = q1 - q0, d2 = q2 - q0, inv = 1 / (float)area
-  int X[3], Y[3];  // vertices after the orientation fix (64-bit path)
-  int pad[2];
-};
-
-// exact 64-bit edge values (unbiased) of a triangle at pixel (px, py)
-__device__ __forceinline__ void edges64(const TriSm& T, int px, int py, long long e[3]) {
-  const long long Px = 256LL * px + 128, Py = 256LL * py + 128;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const int u = k == 0 ? 1 : (k == 1 ? 2 : 0);
-    const int w = k == 0 ? 2 : (k == 1 ? 0 : 1);
-    e[k] = (long long)(T.X[w] - T.X[u]) * (Py - T.Y[u]) - (long long)(T.Y[w] - T.Y[u]) * (Px - T.X[u]);
-  }
-}
-
-// Builds the per-half-block record of triangle t of a quad; returns false if the triangle
-// has zero area or its pixel AABB misses the half-block (BH rows: 4, or 8 for the 8x8
-// blocks of k_raster8).
-template <int BH = kHbH>
-static __device__ __noinline__ bool setup_tri(TriSm& T, const int X[4], const int Y[4], const float qv[4],
-                                          uint32_t info, int t, uint32_t jl, int ox, int oy,
-                                          int cor[3], int box[4], int le[3], int lsx[3], int lsy[3]) {
-  if (!(info & (t ? kInfoTri1 : kInfoTri0))) return false;
-  // vertices (v0, v1, v2) of T0 or (v0, v2, v3) of T1, chosen with selects (no indexing)
-  int xa = X[0], ya = Y[0];
-  int xb = t ? X[2] : X[1], yb = t ? Y[2] : Y[1];
-  int xc = t ? X[3] : X[2], yc = t ? Y[3] : Y[2];
-  float qa = qv[0], qb = t ? qv[2] : qv[1], qc = t ? qv[3] : qv[2];
-  int ib = t ? 2 : 1, ic = t ? 3 : 2;
-  long long A = area2(xa, ya, xb, yb, xc, yc);
-  if (A < 0) {   // orientation fix: swap v1 and v2
-    int ti = xb; xb = xc; xc = ti;
-    ti = yb; yb = yc; yc = ti;
-    const float tq = qb; qb = qc; qc = tq;
-    ti = ib; ib = ic; ic = ti;
-    A = -A;
-  }
-  const int xmin = min(xa, min(xb, xc)), xmax = max(xa, max(xb, xc));
-  const int ymin = min(ya, min(yb, yc)), ymax = max(ya, max(yb, yc));
-  const int bx0 = ceil_div256((long long)xmin - 128), bx1 = floor_div256((long long)xmax - 128);
-  const int by0 = ceil_div256((long long)ymin - 128), by1 = floor_div256((long long)ymax - 128);
-  if (bx0 > ox + kHbW - 1 || bx1 < ox || by0 > oy + BH - 1 || by1 < oy) return false;
-  box[0] = max(bx0 - ox, 0);
-  box[1] = min(bx1 - ox, kHbW - 1);
-  box[2] = max(by0 - oy, 0);
-  box[3] = min(by1 - oy, BH - 1);
-  cor[0] = 0; cor[1] = ib; cor[2] = ic;
-  T.X[0] = xa; T.X[1] = xb; T.X[2] = xc;
-  T.Y[0] = ya; T.Y[1] = yb; T.Y[2] = yc;
-  T.kq = make_float4(qa, __fsub_rn(qb, qa), __fsub_rn(qc, qa), __fdiv_rn(1.0f, __ll2float_rn(A)));
-  uint32_t flags = kTriValid | ((qb == qa && qc == qa) ? kTriConstKey : 0u);
-  bool fast = true;
-  const long long P0x = 256LL * ox + 128, P0y = 256LL * oy + 128;
-  const long long lim = 1LL << 30;
-  // edges v1->v2, v2->v0, v0->v1
-  const int ux[3] = {xb, xc, xa}, uy[3] = {yb, yc, ya}, wx[3] = {xc, xa, xb}, wy[3] = {yc, ya, yb};
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const long long dx = (long long)wx[k] - ux[k], dy = (long long)wy[k] - uy[k];
-    const bool owned = dy < 0 || (dy == 0 && dx > 0);
-    const long long e0 = dx * (P0y - uy[k]) - dy * (P0x - ux[k]) + (owned ? 0 : -1);
-    const long long sx = -256 * dy, sy = 256 * dx;
-    const long long c1 = e0 + (kHbW - 1) * sx, c2 = e0 + (BH - 1) * sy, c3 = c1 + (BH - 1) * sy;
-    fast &= (e0 > -lim && e0 < lim && c1 > -lim && c1 < lim && c2 > -lim && c2 < lim && c3 > -lim && c3 < lim);
-    le[k] = (int)e0;
-    lsx[k] = (int)sx;
-    lsy[k] = (int)sy;
-    if (!owned) flags |= 1u << (3 + k);
-  }
-  if (fast) flags |= kTriFast;
-  // the key's edge values unbiased (the masks use the biased ones in le)
-  T.ea = make_int4((int)((uint32_t)le[1] + ((flags >> 4) & 1u)), (int)((uint32_t)le[2] + ((flags >> 5) & 1u)), lsx[1],
-                   lsx[2]);
-  T.eb = make_int4(lsy[1], lsy[2], (int)flags, (int)(2u * jl + (uint32_t)t));
-  return true;
-}
-
-// setup_tri for a triangle that k_setup marked small (kInfoSmall0 << t): the orientation
-// and 1/area come precomputed, and every edge value at the pixel centres of the box's rows,
-// up to 7 pixels to either side of the box, fits in 32 bits, so the whole set-up is 32-bit
-// integer arithmetic (a block row outside the box is masked off, whatever its values).
-template <int BH = kHbH>
-__device__ __forceinline__ bool setup_tri_small(TriSm& T, const int X[4], const int Y[4], const float qv[4],
-                                                float inv, uint32_t info, int t, uint32_t jl, int ox, int oy,
-                                                int cor[3], int box[4], int le[3], int lsx[3], int lsy[3]) {
-  if (!(info & (t ? kInfoTri1 : kInfoTri0))) return false;
-  int xa = X[0], ya = Y[0];
-  int xb = t ? X[2] : X[1], yb = t ? Y[2] : Y[1];
-  int xc = t ? X[3] : X[2], yc = t ? Y[3] : Y[2];
-  float qa = qv[0], qb = t ? qv[2] : qv[1], qc = t ? qv[3] : qv[2];
-  int ib = t ? 2 : 1, ic = t ? 3 : 2;
-  if (info & (kInfoSwap0 << t)) {
-    int ti = xb; xb = xc; xc = ti;
-    ti = yb; yb = yc; yc = ti;
-    const float tq = qb; qb = qc; qc = tq;
-    ti = ib; ib = ic; ic = ti;
-  }
-  // pixel-centre box: ceil((min - 128) / 256) .. floor((max - 128) / 256)
-  const int bx0 = (min(xa, min(xb, xc)) + 127) >> 8, bx1 = (max(xa, max(xb, xc)) - 128) >> 8;
-  const int by0 = (min(ya, min(yb, yc)) + 127) >> 8, by1 = (max(ya, max(yb, yc)) - 128) >> 8;
-  if (bx0 > ox + kHbW - 1 || bx1 < ox || by0 > oy + BH - 1 || by1 < oy) return false;
-  box[0] = max(bx0 - ox, 0);
-  box[1] = min(bx1 - ox, kHbW - 1);
-  box[2] = max(by0 - oy, 0);
-  box[3] = min(by1 - oy, BH - 1);
-  cor[0] = 0; cor[1] = ib; cor[2] = ic;
-  T.kq = make_float4(qa, __fsub_rn(qb, qa), __fsub_rn(qc, qa), inv);
-  uint32_t flags = kTriValid | kTriFast | ((qb == qa && qc == qa) ? kTriConstKey : 0u);
-  const int P0x = 256 * ox + 128, P0y = 256 * oy + 128;
-  const int ux[3] = {xb, xc, xa}, uy[3] = {yb, yc, ya}, wx[3] = {xc, xa, xb}, wy[3] = {yc, ya, yb};
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const int dx = wx[k] - ux[k], dy = wy[k] - uy[k];
-    const bool owned = dy < 0 || (dy == 0 && dx > 0);
-    le[k] = (int)((uint32_t)dx * (uint32_t)(P0y - uy[k]) - (uint32_t)dy * (uint32_t)(P0x - ux[k])) - (owned ? 0 : 1);
-    lsx[k] = -256 * dy;
-    lsy[k] = 256 * dx;
-    if (!owned) flags |= 1u << (3 + k);
-  }
-  // the key's edge values unbiased (the masks use the biased ones in le)
-  T.ea = make_int4((int)((uint32_t)le[1] + ((flags >> 4) & 1u)), (int)((uint32_t)le[2] + ((flags >> 5) & 1u)), lsx[1],
-                   lsx[2]);
-  T.eb = make_int4(lsy[1], lsy[2], (int)flags, (int)(2u * jl + (uint32_t)t));
-  return true;
-}
 
 // Backward of the front-to-back composite for one pixel (flat per-quad RGBA). With
 // C = sum_i T_i a_i c_i, T_i = prod_{k<i} (1 - a_k), A = 1 - prod (1 - a_k):
@@ -237,66 +101,6 @@ __device__ __forceinline__ uint32_t row_cover(int r, int sx) {
   cnt += ((int)(g0 + (uint32_t)cnt * sa) < 0) ? 1 : 0;
   cnt += (cnt == 7 && (int)(g0 + 7u * sa) < 0) ? 1 : 0;
   return neg ? (0xFFu >> cnt) : ((0xFFu << cnt) & 0xFFu);
-}
-
-// Coverage of the half-block's 32 pixel centres (bit ly * 8 + lx) by a "fast" triangle:
-// per row the intersection of the three edges' covered columns, limited to the triangle's
-// pixel bounding box.
-__device__ __forceinline__ uint32_t tri_mask_fast(const int e[3], const int sx[3], const int sy[3],
-                                                  const int box[4]) {
-  uint32_t mask = 0;
-  const uint32_t cols = ((2u << box[1]) - 1u) & ~((1u << box[0]) - 1u);
-#pragma unroll
-  for (int ly = 0; ly < kHbH; ++ly) {
-    uint32_t row = (ly >= box[2] && ly <= box[3]) ? cols : 0u;
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-      row &= row_cover((int)((uint32_t)e[k] + (uint32_t)ly * (uint32_t)sy[k]), sx[k]);
-    mask |= row << (ly * kHbW);
-  }
-  return mask;
-}
-
-// The same with exact 64-bit edge values, pixel by pixel (large triangles).
-static __device__ __noinline__ uint32_t tri_mask_slow(const TriSm& T, int ox, int oy, const int box[4]) {
-  uint32_t mask = 0;
-  for (int ly = box[2]; ly <= box[3]; ++ly)
-    for (int lx = box[0]; lx <= box[1]; ++lx) {
-      long long e[3];
-      edges64(T, ox + lx, oy + ly, e);
-      bool cov = true;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const bool owned = !((uint32_t)T.eb.z & (1u << (3 + k)));
-        cov &= e[k] > 0 || (e[k] == 0 && owned);
-      }
-      if (cov) mask |= 1u << (ly * kHbW + lx);
-    }
-  return mask;
-}
-
-
-// Exact depth key (interpolated 1/w, Sec. 2 "Stage 3", the reading O.8 of the depth
-// formula) of a triangle record at pixel (px, py) = (ox + lx, oy + ly) of its half-block;
-// also returns the barycentric weights l1, l2 it used.
-__device__ __forceinline__ float tri_key(const TriSm& T, int4 ea, int4 eb, float4 kq, int lx, int ly, int px,
-                                         int py, float& l1, float& l2) {
-  const uint32_t fl = (uint32_t)eb.z;
-  float f1, f2;
-  if (fl & kTriFast) {
-    const int e1 = (int)((uint32_t)ea.x + (uint32_t)lx * (uint32_t)ea.z + (uint32_t)ly * (uint32_t)eb.x);
-    const int e2 = (int)((uint32_t)ea.y + (uint32_t)lx * (uint32_t)ea.w + (uint32_t)ly * (uint32_t)eb.y);
-    f1 = __int2float_rn(e1);
-    f2 = __int2float_rn(e2);
-  } else {
-    long long e[3];
-    edges64(T, px, py, e);
-    f1 = __ll2float_rn(e[1]);
-    f2 = __ll2float_rn(e[2]);
-  }
-  l1 = __fmul_rn(f1, kq.w);
-  l2 = __fmul_rn(f2, kq.w);
-  return __fadd_rn(kq.x, __fadd_rn(__fmul_rn(l1, kq.y), __fmul_rn(l2, kq.z)));
 }
 
 // ATH: the alpha-threshold variant. Once the transmittance drops to kAlphaTMin nothing
@@ -489,78 +293,85 @@ __device__ __forceinline__ void write_pixel(const ViewDev& V, long long pidx, fl
   }
 }
 
-// ---- k_raster's coverage masks -------------------------------------------------------------
+// ---- coverage masks ------------------------------------------------------------------------
 //
-// Forward coverage of an edge u -> v on the half-block at pixel-centre origin (Px, Py): row
-// ly's columns as the low 8 bits of f[ly] (the bits above are arbitrary). Covered iff
+// An edge u -> v at a block's first pixel centre (Px, Py). A pixel centre is covered iff
 // E + bias >= 0, E = dx (Py - yu) - dy (Px - xu), bias = 0 for an owned edge, else -1. A step
 // of one column adds -256 dy and one of a row 256 dx, so E + bias may be replaced by
-// r = floor((E + bias) / 256) with steps -dy and dx. The covered columns are then
+// r = floor((E + bias) / 256) with steps -dy and dx. A row's covered columns are then
 //   dy < 0: those from ceil(r / dy) on,  dy > 0: the first floor(r / dy) + 1,  dy = 0: r >= 0,
 // and both counts are ceil(r / dy -+ eps) for any eps below the quotient's distance from the
 // next integer, 1 / |dy| > 2^-15. The quotient is taken in fp32 as r (1 / (8 dy)), clamped to
-// [0, 1] by the multiply-add's saturation: r and its row steps are exact (|r| < 2^22), the
+// [0, 1] by the multiply-add's saturation: r and its row steps are exact (below 2^24), the
 // approximate reciprocal and the rounding put the clamped value off by less than 2^-22, and
 // eps = 2^-17 (2^-20 scaled) exceeds that, so the count is exact; the scaling back adds 2^23
 // rounded up, which leaves ceil() in the low bits. Needs |E| < 2^30 and |dx|, |dy| < 2^15 on
-// the half-block (kRecSmall). Five instructions per edge and row, against about 16 for the
+// the block (kRecSmall). Five instructions per edge and row, against about 16 for the
 // exact integer binary search (row_cover).
-__device__ __forceinline__ void edge_rows(int xu, int yu, int xv, int yv, int Px, int Py, uint32_t f[kHbH]) {
-  const int dx = xv - xu, dy = yv - yu;
-  const bool owned = dy < 0 || (dy == 0 && dx > 0);
-  const int e = (int)((uint32_t)dx * (uint32_t)(Py - yu) - (uint32_t)dy * (uint32_t)(Px - xu)) - (owned ? 0 : 1);
-  float r = __int2float_rn(e >> 8);
-  const float step = __int2float_rn(dx);
-  const float k = dy == 0 ? -1e20f : rcp_approx(__int2float_rn(8 * dy));
-  const float b = dy > 0 ? 0x1p-20f : -0x1p-20f;
-  const uint32_t flip = dy > 0 ? 0xFFFFFFFFu : 0u;
-#pragma unroll
-  for (int ly = 0; ly < kHbH; ++ly) {
+struct EdgeRows {
+  float r, k, b, step;
+  uint32_t flip;       // all ones: the count is of covered columns, else of uncovered ones
+  __device__ __forceinline__ EdgeRows(int xu, int yu, int xv, int yv, int Px, int Py) {
+    const int dx = xv - xu, dy = yv - yu;
+    const bool owned = dy < 0 || (dy == 0 && dx > 0);
+    const int e = (int)((uint32_t)dx * (uint32_t)(Py - yu) - (uint32_t)dy * (uint32_t)(Px - xu)) - (owned ? 0 : 1);
+    r = __int2float_rn(e >> 8);
+    step = __int2float_rn(dx);
+    k = dy == 0 ? -1e20f : rcp_approx(__int2float_rn(8 * dy));
+    b = dy > 0 ? 0x1p-20f : -0x1p-20f;
+    flip = dy > 0 ? 0xFFFFFFFFu : 0u;
+  }
+  // the row's columns in the low 8 bits, before the flip (the bits above are arbitrary)
+  __device__ __forceinline__ uint32_t row() const {
     const float t = __saturatef(__fmaf_rn(r, k, b));
-    const uint32_t c = __float_as_uint(__fmaf_ru(t, 8.0f, 8388608.0f));   // count in the low 5 bits
-    f[ly] = __funnelshift_l(0u, 0xFFFFFFFFu, c) ^ flip;                   // ~0 << (c mod 32)
-    r = __fadd_rn(r, step);
+    return __funnelshift_l(0u, 0xFFFFFFFFu, __float_as_uint(__fmaf_ru(t, 8.0f, 8388608.0f)));   // ~0 << (c mod 32)
+  }
+  __device__ __forceinline__ void next() { r = __fadd_rn(r, step); }
+};
+
+// Coverage masks of a quad's two triangles on a block of 8 x ROWS pixels: ROWS = 4, bit
+// ly * 8 + lx of m[0]; ROWS = 8, row ly is byte ly / 2 of m[ly & 1] (even rows, odd rows).
+// Under the top-left rule a pixel centre belongs to exactly one of an edge's two directions,
+// so an edge traversed backwards (a triangle of negative area, or the diagonal's second
+// triangle) takes the complement, and five edges serve both triangles.
+template <int ROWS>
+__device__ __forceinline__ void quad_masks_small(const int X[4], const int Y[4], uint32_t info, int Px, int Py,
+                                                 uint32_t m0[ROWS / 4], uint32_t m1[ROWS / 4]) {
+  const uint32_t s0 = (info & kInfoSwap0) ? 0xFFFFFFFFu : 0u;
+  const uint32_t s1 = (info & (kInfoSwap0 << 1)) ? 0xFFFFFFFFu : 0u;
+  EdgeRows d(X[2], Y[2], X[0], Y[0], Px, Py);   // the diagonal, T0's direction
+  EdgeRows e1(X[0], Y[0], X[1], Y[1], Px, Py), e2(X[1], Y[1], X[2], Y[2], Px, Py);
+  EdgeRows e3(X[2], Y[2], X[3], Y[3], Px, Py), e4(X[3], Y[3], X[0], Y[0], Px, Py);
+  const uint32_t fd0 = d.flip ^ s0, fd1 = ~(d.flip ^ s1), f1 = e1.flip ^ s0, f2 = e2.flip ^ s0;
+  const uint32_t f3 = e3.flip ^ s1, f4 = e4.flip ^ s1;
+#pragma unroll
+  for (int ly = 0; ly < ROWS; ++ly) {
+    const uint32_t rd = d.row();
+    const uint32_t a = (rd ^ fd0) & (e1.row() ^ f1) & (e2.row() ^ f2);
+    const uint32_t c = (rd ^ fd1) & (e3.row() ^ f3) & (e4.row() ^ f4);
+    if (ly + 1 < ROWS) { d.next(); e1.next(); e2.next(); e3.next(); e4.next(); }
+    const int w = ROWS == 4 ? 0 : (ly & 1), at = ROWS == 4 ? ly : ly >> 1;
+    const int sel = at == 1 ? 0x3240 : (at == 2 ? 0x3410 : 0x4210);   // byte at <- the row
+    m0[w] = at == 0 ? a : __byte_perm(m0[w], a, sel);
+    m1[w] = at == 0 ? c : __byte_perm(m1[w], c, sel);
+  }
+#pragma unroll
+  for (int w = 0; w < ROWS / 4; ++w) {
+    if (!(info & kInfoTri0)) m0[w] = 0u;
+    if (!(info & kInfoTri1)) m1[w] = 0u;
   }
 }
 
-__device__ __forceinline__ uint32_t pack_rows(uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
-  return __byte_perm(__byte_perm(r0, r1, 0x0040), __byte_perm(r2, r3, 0x0040), 0x5410);
-}
-
-// Coverage masks (bit ly * 8 + lx) of a quad's two triangles on the half-block. Under the
-// top-left rule a pixel centre belongs to exactly one of an edge's two directions, so an edge
-// traversed backwards (a triangle of negative area, or the diagonal's second triangle) takes
-// the complement, and five edges serve both triangles.
-__device__ __forceinline__ void quad_masks_small(const int X[4], const int Y[4], uint32_t info, int Px, int Py,
-                                                 uint32_t& m0, uint32_t& m1) {
-  const uint32_t s0 = (info & kInfoSwap0) ? 0xFFFFFFFFu : 0u;
-  const uint32_t s1 = (info & (kInfoSwap0 << 1)) ? 0xFFFFFFFFu : 0u;
-  uint32_t d[kHbH], f[kHbH], a[kHbH], c[kHbH];
-  edge_rows(X[2], Y[2], X[0], Y[0], Px, Py, d);   // the diagonal, T0's direction
-  edge_rows(X[0], Y[0], X[1], Y[1], Px, Py, f);
-#pragma unroll
-  for (int i = 0; i < kHbH; ++i) { a[i] = (d[i] ^ s0) & (f[i] ^ s0); c[i] = ~(d[i] ^ s1); }
-  edge_rows(X[1], Y[1], X[2], Y[2], Px, Py, f);
-#pragma unroll
-  for (int i = 0; i < kHbH; ++i) a[i] &= f[i] ^ s0;
-  edge_rows(X[2], Y[2], X[3], Y[3], Px, Py, f);
-#pragma unroll
-  for (int i = 0; i < kHbH; ++i) c[i] &= f[i] ^ s1;
-  edge_rows(X[3], Y[3], X[0], Y[0], Px, Py, f);
-#pragma unroll
-  for (int i = 0; i < kHbH; ++i) c[i] &= f[i] ^ s1;
-  m0 = (info & kInfoTri0) ? pack_rows(a[0], a[1], a[2], a[3]) : 0u;
-  m1 = (info & kInfoTri1) ? pack_rows(c[0], c[1], c[2], c[3]) : 0u;
-}
-
 // The same for any quad: the 64-bit edge value at the origin, divided by 256 as above, is
-// clamped to +-2^28 (|7 dy + 3 dx| < 2^27 within the guard band, so a clamped value keeps its
-// sign on the whole half-block), and the rows are searched in 32-bit integers.
+// clamped to +-2^28 (|7 dy + 7 dx| < 2^27 within the guard band, so a clamped value keeps its
+// sign on the whole block), and the rows are searched in 32-bit integers.
+template <int ROWS>
 __device__ __forceinline__ void quad_masks_any(const int X[4], const int Y[4], uint32_t info, int Px, int Py,
-                                               uint32_t& m0, uint32_t& m1) {
+                                               uint32_t m0[ROWS / 4], uint32_t m1[ROWS / 4]) {
   const uint32_t s0 = (info & kInfoSwap0) ? 0xFFFFFFFFu : 0u;
   const uint32_t s1 = (info & (kInfoSwap0 << 1)) ? 0xFFFFFFFFu : 0u;
-  uint32_t a = 0xFFFFFFFFu, c = 0xFFFFFFFFu;
+#pragma unroll
+  for (int w = 0; w < ROWS / 4; ++w) m0[w] = m1[w] = 0xFFFFFFFFu;
 #pragma unroll 1
   for (int k = 0; k < 5; ++k) {
     // edges v2 -> v0, v0 -> v1, v1 -> v2, v2 -> v3, v3 -> v0
@@ -572,21 +383,73 @@ __device__ __forceinline__ void quad_masks_any(const int X[4], const int Y[4], u
     const bool owned = dy < 0 || (dy == 0 && dx > 0);
     const long long e = ((long long)dx * (Py - yu) - (long long)dy * (Px - xu) - (owned ? 0 : 1)) >> 8;
     const int r = (int)max(min(e, 1LL << 28), -(1LL << 28));
-    uint32_t f = 0;
 #pragma unroll
-    for (int ly = 0; ly < kHbH; ++ly) f |= row_cover(r + ly * dx, -dy) << (ly * kHbW);
-    if (k < 3) a &= f ^ s0;
-    if (k == 0) c = ~(f ^ s1);
-    if (k > 2) c &= f ^ s1;
+    for (int w = 0; w < ROWS / 4; ++w) {
+      uint32_t f = 0;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) f |= row_cover(r + (ROWS == 4 ? i : 2 * i + w) * dx, -dy) << (8 * i);
+      if (k < 3) m0[w] &= f ^ s0;
+      if (k == 0) m1[w] = ~(f ^ s1);
+      if (k > 2) m1[w] &= f ^ s1;
+    }
   }
-  m0 = (info & kInfoTri0) ? a : 0u;
-  m1 = (info & kInfoTri1) ? c : 0u;
+#pragma unroll
+  for (int w = 0; w < ROWS / 4; ++w) {
+    if (!(info & kInfoTri0)) m0[w] = 0u;
+    if (!(info & kInfoTri1)) m1[w] = 0u;
+  }
+}
+
+// Lists the set bits of the warp's words (bit 32 l + b: bit b of lane l's word) in order as
+// 16-bit indices, and returns their number. One step per set bit of the fullest word, for the
+// whole window of 1024 references, where finding the n-th set bit anew for every round of 32
+// candidates took about 45 instructions a round.
+__device__ __forceinline__ int list_bits(uint32_t word, int lane, uint16_t* list) {
+  const int n = __popc(word);
+  int incl = n;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  const int total = __shfl_sync(0xffffffffu, incl, 31);
+  __syncwarp();                       // the window before has been read
+  uint16_t* at = list + (incl - n);
+  const int base = 32 * lane;
+  while (word) {
+    *at++ = (uint16_t)(base + __ffs(word) - 1);
+    word &= word - 1;
+  }
+  __syncwarp();
+  return total;
+}
+
+// Pixel-centre extent of a box-shaped quad (kRecBox) on a block of 8 x rows pixels at (ox, oy):
+// columns [c0, c1) and rows [y0, y1). Under the top-left rule a centre is covered iff
+// xmin <= x < xmax and ymin <= y < ymax.
+struct BoxSpan {
+  int c0, c1, y0, y1;
+  __device__ __forceinline__ BoxSpan(const int X[4], const int Y[4], int ox, int oy, int rows) {
+    // vertices 0 and 2 are opposite corners
+    c0 = min(max(((min(X[0], X[2]) + 127) >> 8) - ox, 0), 8);
+    c1 = min(max(((max(X[0], X[2]) + 127) >> 8) - ox, 0), 8);
+    y0 = min(max(((min(Y[0], Y[2]) + 127) >> 8) - oy, 0), rows);
+    y1 = min(max(((max(Y[0], Y[2]) + 127) >> 8) - oy, 0), rows);
+  }
+  __device__ __forceinline__ uint32_t columns() const { return (0xFFu << c0) & ~(0xFFFFFFFFu << c1); }
+};
+
+// Bytes [a, b) of a word set, 0 <= a, b <= 4.
+__device__ __forceinline__ uint32_t byte_span(int a, int b) {
+  // (funnel shifts by 32 clamp to zero)
+  return __funnelshift_lc(0u, 0xFFFFFFFFu, 8 * a) & ~__funnelshift_lc(0u, 0xFFFFFFFFu, 8 * b);
 }
 
 // ---- k_raster's shared memory ----------------------------------------------------------------
-// Per warp: a ring of covering triangles waiting for a batch, and the records of the batch the
-// fragment loop reads, one 16-byte array per field so that a slot's fields lie at one address
+// Per warp: the candidates of a 1024-reference window, a ring of covering triangles waiting for
+// a batch, and the records of the batch the fragment loop reads, one 16-byte array per field so that a slot's fields lie at one address
 // plus constants and eight neighbouring slots never share a bank.
+constexpr int kWinRefs = 1024;     // references per bitmap window (a word per lane)
 constexpr int kPendCap = 128;      // at most 31 left over + 64 pushed per candidate round
 constexpr uint32_t kPendConst = 0x80000000u;   // pending id: flat colour and constant depth
 struct BatchGeo {
@@ -598,11 +461,237 @@ struct BatchGeo {
 };
 __host__ __device__ constexpr int batch_cols(bool vtx, bool lit) { return vtx ? (lit ? 6 : 3) : 1; }
 __host__ __device__ constexpr size_t batch_smem_warp(bool vtx, bool bwd, bool lit) {
-  return kPendCap * sizeof(uint2) + sizeof(BatchGeo) + (size_t)batch_cols(vtx, lit) * 32 * sizeof(float4) +
+  return kWinRefs * sizeof(uint16_t) + kPendCap * sizeof(uint2) + sizeof(BatchGeo) + (size_t)batch_cols(vtx, lit) * 32 * sizeof(float4) +
          (bwd ? 32 * sizeof(float4) : 0);
 }
 __host__ __device__ constexpr size_t raster_smem_bytes(bool vtx, bool bwd = false, bool lit = false) {
   return (size_t)kRasterWarps * batch_smem_warp(vtx, bwd, lit);
+}
+
+// The record of covering triangle id (2 * quad + triangle of view V) into slot `lane` of the
+// batch: the depth key's two edge values at the block's first pixel centre (Ox, Oy), their
+// steps, its plane, and with colours carried (CARRY) the flat colour or the corner colours
+// times 1/w as (c0, c1 - c0, c2 - c0) for the fragment's c0 + l1 (c1 - c0) + l2 (c2 - c0);
+// lit: the same for the normals.
+template <bool VTX, bool LIT, bool CARRY>
+__device__ __forceinline__ void setup_batch(const Ws& ws, const ViewDev& V, bool flat_view, uint32_t id, int lane, int Ox,
+                                            int Oy, BatchGeo& geo, float4* qc) {
+  const int t = (int)(id & 1u);
+  const uint32_t jl = id >> 1;
+  const QuadRec R = load_rec(ws.rec, (uint32_t)(V.quad_base + jl));
+  const bool sw = (R.info & (kInfoSwap0 << t)) != 0;
+  // vertices a = v0 and, oriented to a positive area, b and c
+  const int xa = R.X[0], ya = R.Y[0];
+  const int x1 = t ? R.X[2] : R.X[1], y1 = t ? R.Y[2] : R.Y[1];
+  const int x2 = t ? R.X[3] : R.X[2], y2 = t ? R.Y[3] : R.Y[2];
+  const float q1 = t ? R.q[2] : R.q[1], q2 = t ? R.q[3] : R.q[2];
+  const int xb = sw ? x2 : x1, yb = sw ? y2 : y1, xc = sw ? x1 : x2, yc = sw ? y1 : y2;
+  const float q_a = R.q[0], q_b = sw ? q2 : q1, q_c = sw ? q1 : q2;
+  geo.kq[lane] = make_float4(q_a, __fsub_rn(q_b, q_a), __fsub_rn(q_c, q_a), t ? R.inv[1] : R.inv[0]);
+  // edges c -> a and a -> b, both through a
+  const int dx1 = xa - xc, dy1 = ya - yc, dx2 = xb - xa, dy2 = yb - ya;
+  const int ux = Ox - xa, uy = Oy - ya;
+  if (R.info & (kInfoSmall0 << t)) {
+    geo.ea[lane] = make_int4((int)((uint32_t)dx1 * (uint32_t)uy - (uint32_t)dy1 * (uint32_t)ux),
+                             (int)((uint32_t)dx2 * (uint32_t)uy - (uint32_t)dy2 * (uint32_t)ux), -256 * dy1, -256 * dy2);
+    geo.eb[lane] = make_int4(256 * dx1, 256 * dx2, 0, (int)id);
+  } else {
+    // 64-bit edge values: E + 256 (ly dx - lx dy)
+    const long long e1 = (long long)dx1 * uy - (long long)dy1 * ux, e2 = (long long)dx2 * uy - (long long)dy2 * ux;
+    geo.ea[lane] = make_int4((int)(uint32_t)e1, (int)(uint32_t)e2, -dy1, -dy2);
+    geo.hi[lane] = make_int2((int)(e1 >> 32), (int)(e2 >> 32));
+    geo.eb[lane] = make_int4(dx1, dx2, (int)kTriWide, (int)id);
+  }
+  if (VTX && !flat_view) {
+    const uint4 vi = V.idx ? __ldg(reinterpret_cast<const uint4*>(V.idx) + jl)
+                           : make_uint4(4 * jl, 4 * jl + 1, 4 * jl + 2, 4 * jl + 3);
+    const uint32_t w1 = t ? vi.z : vi.y, w2 = t ? vi.w : vi.z;
+    const uint32_t vb = sw ? w2 : w1, vc = sw ? w1 : w2;
+    const float4* cv = reinterpret_cast<const float4*>(V.col);
+    const bool lit = LIT && V.color_mode == LR_COLOR_LIT;
+    const uint32_t cs = lit ? 2u : 1u;
+    const float4 c0 = __ldg(cv + (size_t)cs * vi.x), c1 = __ldg(cv + (size_t)cs * vb), c2 = __ldg(cv + (size_t)cs * vc);
+    const float4 p0 = make_float4(q_a * c0.x, q_a * c0.y, q_a * c0.z, q_a * c0.w);
+    qc[lane] = p0;
+    qc[32 + lane] = make_float4(q_b * c1.x - p0.x, q_b * c1.y - p0.y, q_b * c1.z - p0.z, q_b * c1.w - p0.w);
+    qc[64 + lane] = make_float4(q_c * c2.x - p0.x, q_c * c2.y - p0.y, q_c * c2.z - p0.z, q_c * c2.w - p0.w);
+    if (LIT && lit) {
+      const float4 n0 = __ldg(cv + 2ull * vi.x + 1), n1 = __ldg(cv + 2ull * vb + 1), n2 = __ldg(cv + 2ull * vc + 1);
+      const float4 o0 = make_float4(q_a * n0.x, q_a * n0.y, q_a * n0.z, 0.f);
+      qc[96 + lane] = o0;
+      qc[128 + lane] = make_float4(q_b * n1.x - o0.x, q_b * n1.y - o0.y, q_b * n1.z - o0.z, 0.f);
+      qc[160 + lane] = make_float4(q_c * n2.x - o0.x, q_c * n2.y - o0.y, q_c * n2.z - o0.z, 0.f);
+    }
+  } else if (CARRY) {
+    qc[lane] = __ldg(reinterpret_cast<const float4*>(V.col) + jl);
+  }
+}
+
+// Sort key of a triangle of constant depth.
+__device__ __forceinline__ unsigned long long const_key(const Ws& ws, const ViewDev& V, uint32_t id) {
+  const float q0 = __ldg(reinterpret_cast<const float*>(ws.rec + 4ull * (uint32_t)(V.quad_base + (id >> 1)) + 2));
+  return ((unsigned long long)__float_as_uint(q0) << 32) | id;
+}
+
+// Perspective-correct colour of a fragment: c / w interpolated with the weights l1, l2 and
+// divided by the interpolated 1/w, which is the depth key (rk its reciprocal).
+__device__ __forceinline__ float4 interpolate(float4 c0, float4 d1, float4 d2, float l1, float l2, float rk) {
+  return make_float4((c0.x + l1 * d1.x + l2 * d2.x) * rk, (c0.y + l1 * d1.y + l2 * d2.y) * rk,
+                     (c0.z + l1 * d1.z + l2 * d2.z) * rk, (c0.w + l1 * d1.w + l2 * d2.w) * rk);
+}
+
+// Lit views: RGB times the two-sided Lambert term of the interpolated normal (times the
+// interpolated 1/w, which only scales it) plus ambient.
+__device__ __forceinline__ void apply_light(float4& col, float4 n0, float4 n1, float4 n2, float l1, float l2, float4 light) {
+  const float nx = n0.x + l1 * n1.x + l2 * n2.x;
+  const float ny = n0.y + l1 * n1.y + l2 * n2.y;
+  const float nz = n0.z + l1 * n1.z + l2 * n2.z;
+  const float nn = nx * nx + ny * ny + nz * nz;
+  const float d = fabsf(nx * light.x + ny * light.y + nz * light.z);
+  const float lam = nn > 0.f ? fminf(d * rsqrtf(nn), 1.0f) : 0.f;
+  const float f = light.w + (1.0f - light.w) * lam;
+  col.x *= f;
+  col.y *= f;
+  col.z *= f;
+}
+
+// Colour of a fragment of the triangle in slot p, with barycentric weights l1, l2 and depth
+// key `key`.
+template <bool VTX, bool LIT>
+__device__ __forceinline__ float4 shade(const float4* qc, int p, bool flat_view, bool lit, float4 light, float l1, float l2,
+                                        float key) {
+  float4 col = qc[p];
+  if (VTX && !flat_view) {
+    col = interpolate(col, qc[32 + p], qc[64 + p], l1, l2, rcp_approx(key));
+    if (LIT && lit) apply_light(col, qc[96 + p], qc[128 + p], qc[160 + p], l1, l2, light);
+  }
+  return col;
+}
+
+// A bin that holds only flat-colour quads of one depth each (camera-facing sprites and
+// particles; bin_cursor, set by the bin count): the bin's list, sorted by that depth with the
+// tie rule, is every pixel's exact fragment order, so fragments are blended as they come,
+// without depth keys, sorter or exact path. A warp takes an 8x8 block, the half-blocks hb and
+// hb_l below it, with two pixels per lane, one above the other: a record read from shared
+// memory and a step of the loop serve both, and a quad that meets both half-blocks is gathered
+// and masked once. Rectangles (kRecBox) take their masks from two spans. (Blocks of two pixels
+// per lane for quads of other depths measured slower than half-blocks, 340 against 317 us on
+// the layer frame: the pixels' triangles differ too often for the second sorter's registers.)
+// 2M particles at 1920x1080: rasteriser 496 us by half-blocks without the spans, 299 us so.
+template <bool ATH>
+__device__ __forceinline__ unsigned const_block(const Ws& ws, const ViewDev& V, const uint32_t* row_u,
+                                                const uint32_t* row_l, uint32_t off, int n, int ox, int oy, int lane,
+                                                uint16_t* cand, uint2* pend, float4* qc) {
+  const int px = ox + (lane & 7), py = oy + 2 * (lane >> 3);
+  const bool ok_a = px < V.width && py < V.height, ok_b = px < V.width && py + 1 < V.height;
+  const int Ox = 256 * ox + 128, Oy = 256 * oy + 128;
+  const uint32_t* ref_lo = reinterpret_cast<const uint32_t*>(ws.refs + off);   // low words
+  const float4* colors = reinterpret_cast<const float4*>(V.col);
+  const uint32_t quad_base = (uint32_t)V.quad_base;
+  uint32_t* pend_j = reinterpret_cast<uint32_t*>(qc + 32);   // the ring's quads; pend: their masks
+  PixelState<1, true, false, ATH> sa, sb;
+  sa.init();
+  sb.init();
+  uint32_t cnt_a = 0, cnt_b = 0;
+  const int nw = (n + 31) >> 5;
+  int g = -32, r0 = 0, total = 0, head = 0, tail = 0;
+  for (;;) {
+    // masks of 32 candidates, one quad per lane, until a batch of covering quads is full
+    while (tail - head < 32) {
+      if (ATH && !__any_sync(0xffffffffu, (ok_a && sa.live()) || (ok_b && sb.live()))) break;   // all finished
+      if (r0 >= total) {
+        g += 32;
+        if (g >= nw) break;
+        total = list_bits(g + lane < nw ? (__ldg(row_u + g + lane) | __ldg(row_l + g + lane)) : 0u, lane, cand);
+        r0 = 0;
+        continue;
+      }
+      // first entry m, and for triangles that overlap (concave or crossed quads) a second one:
+      // triangle 1 lies in front
+      uint32_t m[2] = {0, 0}, m2[2] = {0, 0}, j = 0;
+      if (r0 + lane < total) {
+        const uint32_t rec = ~ref_lo[2 * (32 * g + (int)cand[r0 + lane])];
+        int X[4], Y[4];
+        load_rec_xy(ws.rec, rec, X, Y);
+        const int2 fl = __ldg(reinterpret_cast<const int2*>(ws.rec + 4ull * rec + 3) + 1);   // info, record flags
+        j = rec - quad_base;
+        if (fl.y & (int)kRecBox) {
+          const BoxSpan B(X, Y, ox, oy, 8);
+          const uint32_t cols = 0x01010101u * B.columns();
+          // even rows 2 i in [y0, y1): i in [(y0 + 1) / 2, (y1 + 1) / 2); odd: [y0 / 2, y1 / 2)
+          m[0] = cols & byte_span((B.y0 + 1) >> 1, (B.y1 + 1) >> 1);
+          m[1] = cols & byte_span(B.y0 >> 1, B.y1 >> 1);
+        } else {
+          if (fl.y & (int)kRecSmall) quad_masks_small<8>(X, Y, (uint32_t)fl.x, Ox, Oy, m2, m);
+          else quad_masks_any<8>(X, Y, (uint32_t)fl.x, Ox, Oy, m2, m);
+          if (((m[0] & m2[0]) | (m[1] & m2[1])) == 0u) {
+            m[0] |= m2[0]; m[1] |= m2[1];
+            m2[0] = m2[1] = 0u;
+          }
+        }
+      }
+      r0 += 32;
+      const bool h1 = (m[0] | m[1]) != 0u, h2 = (m2[0] | m2[1]) != 0u;
+      const unsigned b1 = __ballot_sync(0xffffffffu, h1), b2 = __ballot_sync(0xffffffffu, h2);
+      const unsigned lt = (1u << lane) - 1u;
+      int at = tail + __popc(b1 & lt) + __popc(b2 & lt);
+      if (h1) {
+        pend[at & (kPendCap - 1)] = make_uint2(m[0], m[1]);
+        pend_j[at++ & (kPendCap - 1)] = j;
+      }
+      if (h2) {
+        pend[at & (kPendCap - 1)] = make_uint2(m2[0], m2[1]);
+        pend_j[at & (kPendCap - 1)] = j;
+      }
+      tail += __popc(b1) + __popc(b2);
+      __syncwarp();
+    }
+    const int nb = min(32, tail - head);
+    if (nb == 0) break;
+    // entry 31 - L of the batch goes to lane and slot L: the highest set bit is the next
+    uint2 k = make_uint2(0u, 0u);
+    if (31 - lane < nb) {
+      const int i = (head + 31 - lane) & (kPendCap - 1);
+      k = pend[i];
+      qc[lane] = __ldg(colors + pend_j[i]);
+    }
+    head += nb;
+    uint32_t m_a = warp_transpose32(k.x, lane), m_b = warp_transpose32(k.y, lane);
+    __syncwarp();
+    if (!ok_a) m_a = 0;
+    if (!ok_b) m_b = 0;
+    cnt_a += __popc(m_a);
+    cnt_b += __popc(m_b);
+    while (m_a | m_b) {
+      if (ATH) {
+        if (!sa.live()) m_a = 0;
+        if (!sb.live()) m_b = 0;
+        if (!(m_a | m_b)) break;
+      }
+      const int p = 31 - __clz(m_a | m_b);
+      const uint32_t bit = 1u << p;
+      const float4 c = qc[p];
+      if (m_a & bit) sa.blend_direct(c);
+      if (m_b & bit) sb.blend_direct(c);
+      m_a &= ~bit;
+      m_b &= ~bit;
+    }
+    __syncwarp();
+  }
+  if (V.xmask && lane < 2 && oy + lane * kHbH < V.height) {
+    const uint32_t hbw = ((uint32_t)V.width + kHbW - 1) / kHbW;
+    V.xmask[((uint32_t)oy / kHbH + lane) * hbw + (uint32_t)ox / kHbW] = 0u;
+  }
+  const long long pa = (long long)py * V.width + px;
+  if (ok_a) {
+    if (V.cnt) V.cnt[pa] = cnt_a;
+    write_pixel(V, pa, sa.r, sa.g, sa.b, sa.T);
+  }
+  if (ok_b) {
+    if (V.cnt) V.cnt[pa + V.width] = cnt_b;
+    write_pixel(V, pa + V.width, sb.r, sb.g, sb.b, sb.T);
+  }
+  return cnt_a + cnt_b;
 }
 
 // HASH: the variant that also writes the per-pixel coverage hash (a test output); the
@@ -611,31 +700,39 @@ __host__ __device__ constexpr size_t raster_smem_bytes(bool vtx, bool bwd = fals
 // pixel of the half-block still blending. LIT: the colour-carrying variant that also
 // shades lit views (per-vertex normals, one directional light).
 template <int K, bool VTX, bool BWD, bool HASH, bool ATH = false, bool LIT = false>
-__global__ __launch_bounds__(kRasterThreads, LR_RASTER_MIN_BLOCKS) void k_raster(Ws ws) {
+__global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH, LIT)) void k_raster(Ws ws) {
   pdl_begin();
   extern __shared__ __align__(16) unsigned char smem[];
   constexpr bool kCarry = VTX || K == 1;   // the sorter carries each fragment's colour
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lx = lane & (kHbW - 1), ly = lane >> 3;
   unsigned char* wbase = smem + (size_t)warp * batch_smem_warp(VTX, BWD, LIT);
-  uint2* pend = reinterpret_cast<uint2*>(wbase);
-  BatchGeo& geo = *reinterpret_cast<BatchGeo*>(wbase + kPendCap * sizeof(uint2));
-  float4* qc = reinterpret_cast<float4*>(wbase + kPendCap * sizeof(uint2) + sizeof(BatchGeo));
+  uint16_t* cand = reinterpret_cast<uint16_t*>(wbase);
+  uint2* pend = reinterpret_cast<uint2*>(wbase + kWinRefs * sizeof(uint16_t));
+  BatchGeo& geo = *reinterpret_cast<BatchGeo*>(pend + kPendCap);
+  float4* qc = reinterpret_cast<float4*>(&geo + 1);
   float4* agg = qc + batch_cols(VTX, LIT) * 32;
-  // a batch blended in stream order keeps its sort keys where the others keep ea
+  // a batch blended in stream order keeps its sort keys (alpha threshold) or ids where the
+  // others keep ea
   unsigned long long* dkey = reinterpret_cast<unsigned long long*>(&geo);
+  uint32_t* did = reinterpret_cast<uint32_t*>(&geo);
   if (ws.ctrl->error == LR_ERR_OVERFLOW) return;
-  const unsigned long long nitems = ws.ctrl->raster_items;
+  const uint32_t nitems = (uint32_t)ws.ctrl->raster_items;   // (a batch has less than 2^32 pixels)
   unsigned long long frag_total = 0;
 
-  for (;;) {
-    unsigned long long item = 0;
-    if (lane == 0) item = atomicAdd(&ws.ctrl->raster_head, 1ull);
-    item = __shfl_sync(0xffffffffu, item, 0);
-    if (item >= nitems) break;
+  // the next item: the one after i, or the first of a new ticket (of 1 or 2 items)
+  auto next_item = [&](uint32_t i) {
+    if (i & (uint32_t)(ws.ticket - 1)) return i;
+    unsigned long long k = 0;
+    if (lane == 0) k = atomicAdd(&ws.ctrl->raster_head, (unsigned long long)ws.ticket);
+    return (uint32_t)__shfl_sync(0xffffffffu, (uint32_t)min(k, 0xFFFFFFF0ull), 0);
+  };
+  for (uint32_t item = next_item(0u); item < nitems; item = next_item(item + 1u)) {
     const int lg = ws.bin_log2, hl = bin_hb_log2(lg), cl = bin_hb_cols_log2(lg);
     const int bin_g = (int)ws.bin_order[item >> hl];
-    const int hb = (int)(item & ((1u << hl) - 1u));
+    // items 2 i and 2 i + 1 of a bin: the upper and the lower half-block of its 8x8 block i
+    const int blk = (int)(item & ((1u << hl) - 1u)) >> 1;
+    const int hb = ((2 * (blk >> cl) + (int)(item & 1u)) << cl) + (blk & ((1 << cl) - 1));
     const int v = view_of_bin(ws.views, ws.n_views, bin_g);
     const ViewDev& V = ws.views[v];
     const int b = bin_g - V.bin_base;
@@ -646,7 +743,14 @@ __global__ __launch_bounds__(kRasterThreads, LR_RASTER_MIN_BLOCKS) void k_raster
     const bool pix_ok = px < V.width && py < V.height;
     const uint32_t off = ws.bin_off[bin_g];
     const int n = (int)(ws.bin_off[bin_g + 1] - off);
-    const bool flat_view = V.color_mode == LR_COLOR_FLAT;
+    if (!HASH && !BWD && !ws.cursors && V.color_mode == LR_COLOR_FLAT && ws.bin_cursor[bin_g] == 0u) {
+      // an 8x8 block at its upper half-block; nothing at its lower one
+      if (item & 1u) continue;
+      frag_total += const_block<ATH>(ws, V, hb_row(ws, off, bin_g, n, hb), hb_row(ws, off, bin_g, n, hb + (1 << cl)), off, n,
+                                     ox, oy, lane, cand, pend, reinterpret_cast<float4*>(&geo));
+      continue;
+    }
+    const bool flat_view = V.color_mode == LR_COLOR_FLAT, lit_view = LIT && V.color_mode == LR_COLOR_LIT;
     const bool hashing = HASH && V.hash != nullptr;
     const int Ox = 256 * ox + 128, Oy = 256 * oy + 128;   // first pixel centre, 1/256 px
     // lit views: unit direction toward the light and the ambient term
@@ -691,25 +795,23 @@ __global__ __launch_bounds__(kRasterThreads, LR_RASTER_MIN_BLOCKS) void k_raster
     const uint32_t* row = hb_row(ws, off, bin_g, n, hb);
     const int nw = (n + 31) >> 5;
     const uint32_t* ref_lo = reinterpret_cast<const uint32_t*>(ws.refs + off);   // low words
-    int g = -32, r0 = 0;          // bitmap window and position in it
-    BitRounds br;
-    br.total = 0;
+    int g = -32, r0 = 0, total = 0;   // bitmap window, position in it, its candidates
     int head = 0, tail = 0;       // pending ring
     bool ordered = !HASH && !BWD; // everything so far was blended in stream order
+    uint32_t last_id = 0xFFFFFFFFu;   // ... the last fragment's id
     for (;;) {
       // ---- 2. coverage masks of 32 candidates, one quad per lane, until a batch is full ---
       while (tail - head < 32) {
-        if (r0 >= br.total) {
+        if (r0 >= total) {
           g += 32;
           if (g >= nw) break;
-          br.prepare(g + lane < nw ? __ldg(row + g + lane) : 0u, lane);
+          total = list_bits(g + lane < nw ? __ldg(row + g + lane) : 0u, lane, cand);
           r0 = 0;
           continue;
         }
-        const int j = br.get(r0, lane);
+        const bool in = r0 + lane < total;
+        const uint32_t rec = in ? ~ref_lo[2 * (32 * g + (int)cand[r0 + lane])] : 0u;
         r0 += 32;
-        const bool in = j >= 0;
-        const uint32_t rec = in ? ~ref_lo[2 * (32 * g + j)] : 0u;
         bool skip = !in;
         if (ATH) {
           // The smallest key a fragment must exceed to change any pixel of the half-block:
@@ -732,16 +834,22 @@ __global__ __launch_bounds__(kRasterThreads, LR_RASTER_MIN_BLOCKS) void k_raster
         }
         uint32_t ma = 0, mb = 0, ida = 0, idb = 0;
         if (!skip) {
-          const int4* rp = ws.rec + 4ull * rec;
-          const int4 r0v = __ldg(rp), r1v = __ldg(rp + 1);
-          const int2 fl = __ldg(reinterpret_cast<const int2*>(rp + 3) + 1);   // info, record flags
-          const int X[4] = {r0v.x, r0v.z, r1v.x, r1v.z}, Y[4] = {r0v.y, r0v.w, r1v.y, r1v.w};
+          int X[4], Y[4];
+          load_rec_xy(ws.rec, rec, X, Y);
+          const int2 fl = __ldg(reinterpret_cast<const int2*>(ws.rec + 4ull * rec + 3) + 1);   // info, record flags
           const uint32_t info = (uint32_t)fl.x;
-          if (fl.y & (int)kRecSmall) quad_masks_small(X, Y, info, Ox, Oy, ma, mb);
-          else quad_masks_any(X, Y, info, Ox, Oy, ma, mb);
+          const bool one = flat_view && (info & kInfoFlatDepth);
+          if (!HASH && one && (fl.y & (int)kRecBox)) {
+            const BoxSpan B(X, Y, ox, oy, kHbH);
+            ma = (0x01010101u * B.columns()) & byte_span(B.y0, B.y1);
+          } else if (fl.y & (int)kRecSmall) {
+            quad_masks_small<kHbH>(X, Y, info, Ox, Oy, &ma, &mb);
+          } else {
+            quad_masks_any<kHbH>(X, Y, info, Ox, Oy, &ma, &mb);
+          }
           ida = 2u * (uint32_t)(rec - V.quad_base);
           idb = ida + 1u;
-          if (flat_view && (info & kInfoFlatDepth)) {
+          if (one) {
             // one colour and one depth key for the whole quad: its triangles form one entry
             // where they do not overlap, else the second goes first (it lies in front: equal
             // keys order by triangle)
@@ -780,63 +888,12 @@ __global__ __launch_bounds__(kRasterThreads, LR_RASTER_MIN_BLOCKS) void k_raster
       id &= ~kPendConst;
       if (direct) {
         if (e < nb) {
-          const float q0 = __ldg(reinterpret_cast<const float*>(ws.rec + 4ull * (uint32_t)(V.quad_base + (id >> 1)) + 2));
           qc[lane] = __ldg(reinterpret_cast<const float4*>(V.col) + (id >> 1));
-          dkey[lane] = ((unsigned long long)__float_as_uint(q0) << 32) | id;
+          if (ATH) dkey[lane] = const_key(ws, V, id);
+          else did[lane] = id;
         }
       } else if (e < nb) {
-        const int t = (int)(id & 1u);
-        const uint32_t jl = id >> 1;
-        const QuadRec R = load_rec(ws.rec, (uint32_t)(V.quad_base + jl));
-        const bool sw = (R.info & (kInfoSwap0 << t)) != 0;
-        // vertices a = v0 and, oriented to a positive area, b and c
-        const int xa = R.X[0], ya = R.Y[0];
-        const int x1 = t ? R.X[2] : R.X[1], y1 = t ? R.Y[2] : R.Y[1];
-        const int x2 = t ? R.X[3] : R.X[2], y2 = t ? R.Y[3] : R.Y[2];
-        const float q1 = t ? R.q[2] : R.q[1], q2 = t ? R.q[3] : R.q[2];
-        const int xb = sw ? x2 : x1, yb = sw ? y2 : y1, xc = sw ? x1 : x2, yc = sw ? y1 : y2;
-        const float qb = sw ? q2 : q1, qc2 = sw ? q1 : q2;
-        geo.kq[lane] = make_float4(R.q[0], __fsub_rn(qb, R.q[0]), __fsub_rn(qc2, R.q[0]), t ? R.inv[1] : R.inv[0]);
-        // edges c -> a and a -> b, both through a
-        const int dx1 = xa - xc, dy1 = ya - yc, dx2 = xb - xa, dy2 = yb - ya;
-        const int ux = Ox - xa, uy = Oy - ya;
-        if (R.info & (kInfoSmall0 << t)) {
-          geo.ea[lane] = make_int4((int)((uint32_t)dx1 * (uint32_t)uy - (uint32_t)dy1 * (uint32_t)ux),
-                                   (int)((uint32_t)dx2 * (uint32_t)uy - (uint32_t)dy2 * (uint32_t)ux), -256 * dy1, -256 * dy2);
-          geo.eb[lane] = make_int4(256 * dx1, 256 * dx2, 0, (int)id);
-        } else {
-          // 64-bit edge values: E + 256 (ly dx - lx dy)
-          const long long e1 = (long long)dx1 * uy - (long long)dy1 * ux, e2 = (long long)dx2 * uy - (long long)dy2 * ux;
-          geo.ea[lane] = make_int4((int)(uint32_t)e1, (int)(uint32_t)e2, -dy1, -dy2);
-          geo.hi[lane] = make_int2((int)(e1 >> 32), (int)(e2 >> 32));
-          geo.eb[lane] = make_int4(dx1, dx2, (int)kTriWide, (int)id);
-        }
-        if (VTX && !flat_view) {
-          const uint4 vi = V.idx ? __ldg(reinterpret_cast<const uint4*>(V.idx) + jl)
-                                 : make_uint4(4 * jl, 4 * jl + 1, 4 * jl + 2, 4 * jl + 3);
-          const uint32_t w1 = t ? vi.z : vi.y, w2 = t ? vi.w : vi.z;
-          const uint32_t vb = sw ? w2 : w1, vc = sw ? w1 : w2;
-          const float4* cv = reinterpret_cast<const float4*>(V.col);
-          const bool lit = LIT && V.color_mode == LR_COLOR_LIT;
-          const uint32_t cs = lit ? 2u : 1u;
-          // corner colours times 1/w, as (c0, c1 - c0, c2 - c0) for the fragment's
-          // c0 + l1 (c1 - c0) + l2 (c2 - c0); lit: the same for the normals
-          const float4 c0 = __ldg(cv + (size_t)cs * vi.x), c1 = __ldg(cv + (size_t)cs * vb), c2 = __ldg(cv + (size_t)cs * vc);
-          const float qa = R.q[0];
-          const float4 p0 = make_float4(qa * c0.x, qa * c0.y, qa * c0.z, qa * c0.w);
-          qc[lane] = p0;
-          qc[32 + lane] = make_float4(qb * c1.x - p0.x, qb * c1.y - p0.y, qb * c1.z - p0.z, qb * c1.w - p0.w);
-          qc[64 + lane] = make_float4(qc2 * c2.x - p0.x, qc2 * c2.y - p0.y, qc2 * c2.z - p0.z, qc2 * c2.w - p0.w);
-          if (LIT && lit) {
-            const float4 n0 = __ldg(cv + 2ull * vi.x + 1), n1 = __ldg(cv + 2ull * vb + 1), n2 = __ldg(cv + 2ull * vc + 1);
-            const float4 o0 = make_float4(qa * n0.x, qa * n0.y, qa * n0.z, 0.f);
-            qc[96 + lane] = o0;
-            qc[128 + lane] = make_float4(qb * n1.x - o0.x, qb * n1.y - o0.y, qb * n1.z - o0.z, 0.f);
-            qc[160 + lane] = make_float4(qc2 * n2.x - o0.x, qc2 * n2.y - o0.y, qc2 * n2.z - o0.z, 0.f);
-          }
-        } else if (kCarry) {
-          qc[lane] = __ldg(reinterpret_cast<const float4*>(V.col) + jl);
-        }
+        setup_batch<VTX, LIT, kCarry>(ws, V, flat_view, id, lane, Ox, Oy, geo, qc);
       }
       // ---- 4. transpose: lane = pixel, bit L = covered by the triangle in slot L -----------
       uint32_t m = warp_transpose32(mk, lane);   // (its shuffles also order the slots' writes below)
@@ -858,9 +915,11 @@ __global__ __launch_bounds__(kRasterThreads, LR_RASTER_MIN_BLOCKS) void k_raster
           st.blend_direct(c);
         }
         if (!ATH) lastp = (uint32_t)(__ffs(all) - 1);
-        if (lastp < 32u) st.last = dkey[lastp];
+        if (ATH) { if (lastp < 32u) st.last = dkey[lastp]; }
+        else if (lastp < 32u) last_id = did[lastp];
       } else {
         if (ordered) {
+          if (!ATH && last_id != 0xFFFFFFFFu) st.last = const_key(ws, V, last_id);
           // the sorter starts here; with a transparent held fragment at the last key blended
           // (K = 1), so that its first eviction keeps that key
           ordered = false;
@@ -894,32 +953,7 @@ __global__ __launch_bounds__(kRasterThreads, LR_RASTER_MIN_BLOCKS) void k_raster
             const float key = __fadd_rn(kq.x, __fadd_rn(__fmul_rn(l1, kq.y), __fmul_rn(l2, kq.z)));
             const unsigned long long sk = ((unsigned long long)__float_as_uint(key) << 32) | fid;
             float4 col = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (kCarry) col = qc[p];
-            if (VTX && !flat_view) {
-              // perspective-correct colour: interpolated (c / w) divided by the
-              // interpolated 1/w, which is the depth key
-              const float rk = rcp_approx(key);
-              const float4 d1 = qc[32 + p], d2 = qc[64 + p];
-              col.x = (col.x + l1 * d1.x + l2 * d2.x) * rk;
-              col.y = (col.y + l1 * d1.y + l2 * d2.y) * rk;
-              col.z = (col.z + l1 * d1.z + l2 * d2.z) * rk;
-              col.w = (col.w + l1 * d1.w + l2 * d2.w) * rk;
-              if (LIT && V.color_mode == LR_COLOR_LIT) {
-                // the interpolated normal (times the interpolated 1/w, which only scales
-                // it); two-sided Lambert term plus ambient on RGB
-                const float4 n0 = qc[96 + p], n1 = qc[128 + p], n2 = qc[160 + p];
-                const float nx = n0.x + l1 * n1.x + l2 * n2.x;
-                const float ny = n0.y + l1 * n1.y + l2 * n2.y;
-                const float nz = n0.z + l1 * n1.z + l2 * n2.z;
-                const float nn = nx * nx + ny * ny + nz * nz;
-                const float d = fabsf(nx * light.x + ny * light.y + nz * light.z);
-                const float lam = nn > 0.f ? fminf(d * rsqrtf(nn), 1.0f) : 0.f;
-                const float f = light.w + (1.0f - light.w) * lam;
-                col.x *= f;
-                col.y *= f;
-                col.z *= f;
-              }
-            }
+            if (kCarry) col = shade<VTX, LIT>(qc, p, flat_view, lit_view, light, l1, l2, key);
             st.insert(sk, col, V);
           }
         };

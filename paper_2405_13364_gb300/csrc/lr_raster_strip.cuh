@@ -28,6 +28,94 @@ constexpr int kStripWin = 8;                       // bitmap words (256 referenc
 constexpr int kStripCap = 32 * kStripWin;          // candidate quads per window, at most
 constexpr uint32_t kTriSmall = 256u;               // 32-bit key arithmetic is exact (k_setup's flag)
 
+// flags of a triangle record
+constexpr uint32_t kTriValid = 1u, kTriFast = 2u, kTriFlatCol = 4u;   // + corr bits 3..5
+// all three vertices at the same 1/w: the depth key is q0 at every pixel (the
+// interpolation adds l1 * 0 + l2 * 0 with l1, l2 >= 0)
+constexpr uint32_t kTriConstKey = 64u;
+
+// Per (triangle, half-block) record read by the fragment loop, laid out for three 16-byte
+// shared-memory loads. Edges 1 (v2->v0) and 2 (v0->v1) give the barycentric numerators
+// of the depth key; edge 0 is only needed for coverage, which the masks already hold.
+struct __align__(16) TriSm {
+  int4 ea;         // e1, e2: edge values E at the half-block's first pixel centre; sx1,
+                   // sx2: change per pixel step in x
+  int4 eb;         // sy1, sy2: change per pixel step in y; flags; id (2 * quad + triangle)
+  float4 kq;       // q0 = 1/w at v0, d1 = q1 - q0, d2 = q2 - q0, inv = 1 / (float)area
+  int X[3], Y[3];  // vertices after the orientation fix (64-bit path)
+  int pad[2];
+};
+
+// exact 64-bit edge values (unbiased) of a triangle at pixel (px, py)
+__device__ __forceinline__ void edges64(const TriSm& T, int px, int py, long long e[3]) {
+  const long long Px = 256LL * px + 128, Py = 256LL * py + 128;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int u = k == 0 ? 1 : (k == 1 ? 2 : 0);
+    const int w = k == 0 ? 2 : (k == 1 ? 0 : 1);
+    e[k] = (long long)(T.X[w] - T.X[u]) * (Py - T.Y[u]) - (long long)(T.Y[w] - T.Y[u]) * (Px - T.X[u]);
+  }
+}
+
+// Coverage of the half-block's 32 pixel centres (bit ly * 8 + lx) by a "fast" triangle:
+// per row the intersection of the three edges' covered columns, limited to the triangle's
+// pixel bounding box.
+__device__ __forceinline__ uint32_t tri_mask_fast(const int e[3], const int sx[3], const int sy[3],
+                                                  const int box[4]) {
+  uint32_t mask = 0;
+  const uint32_t cols = ((2u << box[1]) - 1u) & ~((1u << box[0]) - 1u);
+#pragma unroll
+  for (int ly = 0; ly < kHbH; ++ly) {
+    uint32_t row = (ly >= box[2] && ly <= box[3]) ? cols : 0u;
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+      row &= row_cover((int)((uint32_t)e[k] + (uint32_t)ly * (uint32_t)sy[k]), sx[k]);
+    mask |= row << (ly * kHbW);
+  }
+  return mask;
+}
+
+// The same with exact 64-bit edge values, pixel by pixel (large triangles).
+static __device__ __noinline__ uint32_t tri_mask_slow(const TriSm& T, int ox, int oy, const int box[4]) {
+  uint32_t mask = 0;
+  for (int ly = box[2]; ly <= box[3]; ++ly)
+    for (int lx = box[0]; lx <= box[1]; ++lx) {
+      long long e[3];
+      edges64(T, ox + lx, oy + ly, e);
+      bool cov = true;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const bool owned = !((uint32_t)T.eb.z & (1u << (3 + k)));
+        cov &= e[k] > 0 || (e[k] == 0 && owned);
+      }
+      if (cov) mask |= 1u << (ly * kHbW + lx);
+    }
+  return mask;
+}
+
+// Exact depth key (interpolated 1/w, Sec. 2 "Stage 3", the reading O.8 of the depth
+// formula) of a triangle record at pixel (px, py) = (ox + lx, oy + ly) of its half-block;
+// also returns the barycentric weights l1, l2 it used.
+__device__ __forceinline__ float tri_key(const TriSm& T, int4 ea, int4 eb, float4 kq, int lx, int ly, int px,
+                                         int py, float& l1, float& l2) {
+  const uint32_t fl = (uint32_t)eb.z;
+  float f1, f2;
+  if (fl & kTriFast) {
+    const int e1 = (int)((uint32_t)ea.x + (uint32_t)lx * (uint32_t)ea.z + (uint32_t)ly * (uint32_t)eb.x);
+    const int e2 = (int)((uint32_t)ea.y + (uint32_t)lx * (uint32_t)ea.w + (uint32_t)ly * (uint32_t)eb.y);
+    f1 = __int2float_rn(e1);
+    f2 = __int2float_rn(e2);
+  } else {
+    long long e[3];
+    edges64(T, px, py, e);
+    f1 = __ll2float_rn(e[1]);
+    f2 = __ll2float_rn(e[2]);
+  }
+  l1 = __fmul_rn(f1, kq.w);
+  l2 = __fmul_rn(f2, kq.w);
+  return __fadd_rn(kq.x, __fadd_rn(__fmul_rn(l1, kq.y), __fmul_rn(l2, kq.z)));
+}
+
 // shared memory of k_raster_strip: per candidate triangle a TriSm record (its pad words hold
 // the pixel box relative to the strip), 3 colour slots when fragments carry colours; the
 // window's union words, their prefix counts, the compacted candidates and per warp the slots

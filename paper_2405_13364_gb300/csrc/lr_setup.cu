@@ -32,7 +32,10 @@ __global__ void k_init(Ws ws, unsigned long long refs_cap, ViewChunk views, View
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long stride = (long long)gridDim.x * blockDim.x;
   if (i < (long long)(sizeof(Ctrl) / 4)) reinterpret_cast<uint32_t*>(ws.ctrl)[i] = 0u;
-  for (long long b = i; b < ws.total_bins; b += stride) ws.bin_count[b] = 0u;
+  for (long long b = i; b < ws.total_bins; b += stride) {
+    ws.bin_count[b] = 0u;
+    ws.bin_cursor[b] = 0u;
+  }
   __syncthreads();
   if (blockIdx.x == 0 && threadIdx.x == 0) ws.ctrl->refs_cap = refs_cap;
 }
@@ -124,7 +127,8 @@ __global__ __launch_bounds__(256) void k_setup(Ws ws) {
         // orientation, 1/area of the depth interpolation (Sec. 2, "Stage 3"), and whether
         // 32-bit edge arithmetic is exact wherever the triangle is rasterised. A half-block
         // touching the triangle's pixel box holds pixel centres within 7 px (x) and 3 px (y)
-        // of the vertex box, so |E| <= Wx (Wy + 3*256) + Wy (Wx + 7*256) + 1 there.
+        // of the vertex box, so |E| <= Wx (Wy + 3*256) + Wy (Wx + 7*256) + 1 there (and below
+        // 2^31 on an 8x8 block touching the box: 4 px more add less than 2^25).
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
           long long A = t ? a1 : a0;
@@ -148,10 +152,15 @@ __global__ __launch_bounds__(256) void k_setup(Ws ws) {
         const int ymin = min(min(Y[0], Y[1]), min(Y[2], Y[3]));
         const int ymax = max(max(Y[0], Y[1]), max(Y[2], Y[3]));
         {
-          // the same bound for the whole quad's box (any of its edges)
+          // the same bound for the whole quad's box (any of its edges) and blocks of 8x8 pixels
           const uint32_t wx = (uint32_t)(xmax - xmin), wy = (uint32_t)(ymax - ymin);
-          if (wx < 32768u && wy < 32768u && wx * (wy + 3u * 256u) + wy * (wx + 7u * 256u) + 1u < (1u << 30))
+          if (wx < 32768u && wy < 32768u && wx * (wy + 7u * 256u) + wy * (wx + 7u * 256u) + 1u < (1u << 30))
             rflags = kRecSmall;
+          // an axis-parallel rectangle, from any corner and in either winding (its triangles
+          // share a diagonal and do not overlap)
+          if ((X[0] == X[3] && X[1] == X[2] && Y[0] == Y[1] && Y[2] == Y[3]) ||
+              (X[0] == X[1] && X[2] == X[3] && Y[0] == Y[3] && Y[1] == Y[2]))
+            rflags |= kRecBox;
         }
         const int px0 = max(ceil_div256((long long)xmin - 128), 0);
         const int px1 = min(floor_div256((long long)xmax - 128), V.width - 1);
@@ -178,10 +187,9 @@ __global__ __launch_bounds__(256) void k_setup(Ws ws) {
     // culled quad's invisible rectangle keeps it out of every bin), so culled quads skip them
     if (worst == kVisible) {
       int4* rp = ws.rec + 4 * g;
-      rp[0] = make_int4(X[0], Y[0], X[1], Y[1]);
-      rp[1] = make_int4(X[2], Y[2], X[3], Y[3]);
-      rp[2] = make_int4(__float_as_int(q[0]), __float_as_int(q[1]), __float_as_int(q[2]), __float_as_int(q[3]));
-      rp[3] = make_int4(__float_as_int(inv.x), __float_as_int(inv.y), (int)info, (int)rflags);
+      stg32(rp, X[0], Y[0], X[1], Y[1], X[2], Y[2], X[3], Y[3]);
+      stg32(rp + 2, __float_as_int(q[0]), __float_as_int(q[1]), __float_as_int(q[2]), __float_as_int(q[3]),
+            __float_as_int(inv.x), __float_as_int(inv.y), (int)info, (int)rflags);
       ws.rec_rep[g] = rep;
     }
     ws.rec_rect[g] = rect;

@@ -92,3 +92,20 @@ def test_constant_depths_threshold(lr, k):
     got = r.render(lr.DeviceScene.from_scene(s), w, h)["rgba"].cpu().numpy().astype(np.float64)
     r.close()
     assert np.abs(got - ref["rgba"]).max() <= 1e-5
+
+
+@pytest.mark.parametrize("size,bin_size", [((2560, 2048), 16), ((2560, 2048), 32), ((9, 5), 32)])
+def test_constant_depths_sizes(lr, size, bin_size):
+    # more bins than the binning CTAs count in shared memory, two half-blocks per ticket, a
+    # frame smaller than a bin; no pixel takes the exact path
+    w, h = size
+    s = scenegen.gaussian_particles(30_000 if w > 9 else 300, w, h, seed=bin_size)
+    ref = oracle.render(s)
+    r = lr.Renderer(sorter_k=3, bin_size=bin_size)
+    out = r.render(lr.DeviceScene.from_scene(s), w, h, count=True, exact_mask=True)
+    torch.cuda.synchronize()
+    assert np.array_equal(out["count"].cpu().numpy().view(np.uint32), ref["count"])
+    assert np.abs(out["rgba"].cpu().numpy().astype(np.float64) - ref["rgba"]).max() <= 1e-5
+    assert not out["exact_mask"].any()
+    assert r.stats()["fragments"] == int(ref["count"].sum())
+    r.close()
