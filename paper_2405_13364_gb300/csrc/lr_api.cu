@@ -32,7 +32,6 @@ __global__ void k_bin_count(Ws ws);
 __global__ void k_bin_scan(Ws ws);
 __global__ void k_bin_scatter(Ws ws);
 __global__ void k_bin_sort(Ws ws);
-__global__ void k_bin_sort_big(Ws ws);
 cudaError_t overflow_occupancy(int* blocks_per_sm);
 cudaError_t launch_overflow(bool bwd, const Ws& ws, int grid, cudaStream_t st, bool pdl);
 
@@ -285,8 +284,6 @@ extern "C" lr_status lr_create(const lr_config* config, lr_ctx** out_ctx) {
   }
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_bin_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)kSortSmemBytes);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_bin_sort_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)kSortBigSmemBytes);
   if (e == cudaSuccess) e = overflow_occupancy(&c->ovf_blocks);
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&c->host_ctrl), sizeof(Ctrl));
   for (int i = 0; i < 9 && e == cudaSuccess; ++i) e = cudaEventCreate(&c->ev[i]);
@@ -574,8 +571,7 @@ static lr_status launch_sequence(lr_ctx* ctx, const Prepared& P, cudaStream_t st
   rec(ctx, timed, 3, st);
   if (L.total_chunks > 0) launch_pdl(pdl, k_bin_scatter, dim3(L.total_chunks), dim3(kBinThreads), 0, st, ws);
   rec(ctx, timed, 4, st);
-  launch_pdl(pdl, k_bin_sort, dim3(L.total_bins), dim3(256), kSortSmemBytes, st, ws);
-  launch_pdl(pdl, k_bin_sort_big, dim3(ctx->sms), dim3(kSortBigThreads), kSortBigSmemBytes, st, ws);
+  launch_pdl(pdl, k_bin_sort, dim3(ctx->sms), dim3(kSortThreads), kSortSmemBytes, st, ws);
   rec(ctx, timed, 5, st);
   const bool carry = P.any_vertex || P.any_lit || (ctx->cfg.flags & LR_FLAG_CARRY_COLORS);
   const bool ath = !bwd && (ctx->cfg.flags & LR_FLAG_ALPHA_THRESHOLD);   // no hash then (prepare)

@@ -18,16 +18,14 @@
 //                  (~representative 1/w) << 32 | ~record index.
 //   k_bin_sort     Stage-1 depth sort: sorts each bin's references ascending, i.e. front
 //                  to back by a representative depth, ties with the higher quad index
-//                  first. Bins with fewer than 2048 references: one 256-thread CTA per
-//                  bin, a merge sort in shared memory (runs of 64 to 256 keys sorted in
-//                  registers by one warp each, then merge-path levels).
-//   k_bin_sort_big The high-density bins (2048 references or more; the paper's "high"
-//                  category): persistent 1024-thread CTAs take them from the front of the
-//                  size-ordered bin list. Up to 20480 references are bucket-sorted in
-//                  shared memory (about two references per bucket between the bin's depth
-//                  extremes, insertion sort per bucket); bins with a bucket over 64
-//                  references (many equal depths) or longer lists merge-sort runs of up to
-//                  8192 references in shared memory and merge them through a global buffer.
+//                  first, and writes the half-block bitmap. Bucket sorts in shared memory,
+//                  buckets spaced linearly between the list's depth extremes, ranks by
+//                  comparison within a bucket: bins with fewer than 2048 references by a
+//                  quarter of a 1024-thread CTA with the keys in registers, high-density bins
+//                  (the paper's "high" category) of up to 20480 by the whole CTA. A list with a
+//                  bucket over 64 references (many equal depths) or a longer one merge-sorts
+//                  runs in shared memory (up to 2048 and 8192 references), longer ones
+//                  merged through a global buffer.
 #include "lr_common.cuh"
 
 namespace lr {
@@ -341,173 +339,277 @@ __device__ void cta_merge(const unsigned long long* a, int na, const unsigned lo
   }
 }
 
+// Threads that sort one bin together: the whole CTA, or one of its quarters with a named
+// barrier of its own.
+struct Group {
+  int t, n, bar;             // thread index, threads, barrier
+  __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(n) : "memory"); }
+};
+
+// Mask word m of the 8x4 half-blocks of the bin with pixel origin (x0, y0) (bit hy * cols + hx, in
+// mw 32-bit words) that the pixel box rc overlaps.
+__device__ __forceinline__ uint32_t hb_mask_word(uint2 rc, int x0, int y0, int lg, int m) {
+  const int B = 1 << lg, cols = bin_hb_cols(lg), rpw = 32 / cols;   // half-block rows per mask word
+  // bit i * cols for every row i of a word: the row pattern's replication
+  const uint32_t rep = cols == 8 ? 0x01010101u : (cols == 4 ? 0x11111111u : 0x55555555u);
+  const int px0 = max((int)(rc.x & 0xffff), x0) - x0, px1 = min((int)(rc.x >> 16), x0 + B - 1) - x0;
+  const int py0 = max((int)(rc.y & 0xffff), y0) - y0, py1 = min((int)(rc.y >> 16), y0 + B - 1) - y0;
+  if (px0 > px1 || py0 > py1) return 0u;
+  const int hx0 = px0 / kHbW, hx1 = px1 / kHbW, hy0 = py0 / kHbH, hy1 = py1 / kHbH;
+  // the half-block columns hx0..hx1 replicated into the rows hy0..hy1 that fall in mask
+  // word m: a product, since a row's pattern never carries into the next row
+  const uint32_t row = ((2u << hx1) - 1u) & ~((1u << hx0) - 1u);
+  const int a = max(hy0 - m * rpw, 0), c = min(hy1 - m * rpw, rpw - 1);
+  return a <= c ? row * (rep & ((2u << (c * cols)) - 1u) & ~((1u << (a * cols)) - 1u)) : 0u;
+}
+
 // The bin's transposed half-block bitmap (hb_row): for each sorted reference, the mask of
-// the bin's 8x4 half-blocks (bit hy * cols + hx, in mw 32-bit words) that the quad's pixel
-// AABB overlaps, computed one warp per 32 references and transposed across the warp word by
-// word, so that row h, word w holds the bits of references 32 w .. 32 w + 31 for half-block
-// h. The rasteriser then reads a half-block's candidates with one coalesced load per 1024
-// references. When the bitmap fits `stage` (shared memory, stage_words 32-bit words), the
-// transposed words are assembled there and copied out row by row with coalesced stores;
-// otherwise each lane stores its word of a row directly.
+// the bin's 8x4 half-blocks that the quad's pixel AABB overlaps, computed one warp per 32
+// references and transposed across the warp word by word, so that row h, word w holds the
+// bits of references 32 w .. 32 w + 31 for half-block h. The rasteriser then reads a
+// half-block's candidates with one coalesced load per 1024 references. When the bitmap fits
+// `stage` (shared memory, stage_words 32-bit words), the transposed words are assembled there
+// and copied out row by row with coalesced stores; otherwise each lane stores its word of a
+// row directly. Four words' references and boxes are in flight at a time.
 __device__ void write_hb_bitmap(const Ws& ws, const unsigned long long* r, int n, int bin, uint32_t* stage,
-                                int stage_words) {
+                                int stage_words, const Group& G) {
   const int v = view_of_bin(ws.views, ws.n_views, bin);
   const ViewDev& V = ws.views[v];
   const int b = bin - V.bin_base;
-  const int lg = ws.bin_log2, B = 1 << lg;
-  const int cols = bin_hb_cols(lg), mw = bin_mw(lg), mrows = bin_mrows(lg);
-  const int rpw = 32 / cols;                              // half-block rows per mask word
-  // bit i * cols for every row i of a word: the row pattern's replication
-  const uint32_t rep = cols == 8 ? 0x01010101u : (cols == 4 ? 0x11111111u : 0x55555555u);
+  const int lg = ws.bin_log2;
+  const int mw = bin_mw(lg), mrows = bin_mrows(lg);
   const int x0 = (b % V.nbx) << lg, y0 = (b / V.nbx) << lg;
   const int nw = (n + 31) >> 5;
-  const int lane = threadIdx.x & 31;
+  const int lane = G.t & 31, warps = G.n >> 5;
   uint32_t* bm = ws.ref_hb + (size_t)mw * (size_t)(r - ws.refs) + (size_t)mrows * (size_t)bin;
   const bool staged = mrows * nw <= stage_words;
   uint32_t* dst = staged ? stage : bm;
-  for (int w = threadIdx.x >> 5; w < nw; w += blockDim.x >> 5) {
-    const int i = 32 * w + lane;
-    int hx0 = 1, hx1 = 0, hy0 = 1, hy1 = 0;                // empty unless the box meets the bin
-    const uint32_t rec = i < n ? ~(uint32_t)r[i] : 0xFFFFFFFFu;
-    if (rec < (uint64_t)ws.total_quads) {
-      const uint2 rc = ws.rec_rect[rec];
-      const int px0 = max((int)(rc.x & 0xffff), x0) - x0, px1 = min((int)(rc.x >> 16), x0 + B - 1) - x0;
-      const int py0 = max((int)(rc.y & 0xffff), y0) - y0, py1 = min((int)(rc.y >> 16), y0 + B - 1) - y0;
-      if (px0 <= px1 && py0 <= py1) {
-        hx0 = px0 / kHbW; hx1 = px1 / kHbW; hy0 = py0 / kHbH; hy1 = py1 / kHbH;
-      }
+  for (int w0 = G.t >> 5; w0 < nw; w0 += 4 * warps) {
+    uint32_t rec[4];
+    uint2 rc[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = 32 * (w0 + u * warps) + lane;
+      rec[u] = i < n ? ~(uint32_t)r[i] : 0xFFFFFFFFu;
     }
-    // the half-block columns hx0..hx1 replicated into the rows hy0..hy1 that fall in mask
-    // word m: a product, since a row's pattern never carries into the next row
-    const uint32_t row = hx0 <= hx1 ? ((2u << hx1) - 1u) & ~((1u << hx0) - 1u) : 0u;
-    for (int m = 0; m < mw; ++m) {
-      const int a = max(hy0 - m * rpw, 0), c = min(hy1 - m * rpw, rpw - 1);
-      const uint32_t rows = a <= c ? rep & ((2u << (c * cols)) - 1u) & ~((1u << (a * cols)) - 1u) : 0u;
-      dst[(size_t)(32 * m + lane) * nw + w] = warp_transpose32(row * rows, lane);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      rc[u] = rec[u] < (uint64_t)ws.total_quads ? ws.rec_rect[rec[u]] : make_uint2(1u, 1u);   // (an empty box)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int w = w0 + u * warps;
+      if (w >= nw) break;
+      for (int m = 0; m < mw; ++m)
+        dst[(size_t)(32 * m + lane) * nw + w] = warp_transpose32(hb_mask_word(rc[u], x0, y0, lg, m), lane);
     }
   }
   if (staged) {
-    __syncthreads();
-    for (int i = threadIdx.x; i < mrows * nw; i += blockDim.x) bm[i] = stage[i];
+    G.sync();
+    for (int i = G.t; i < mrows * nw; i += G.n) bm[i] = stage[i];
   }
 }
 
-// Block-wide reduction / exclusive scan helpers over all threads of the CTA (blockDim a
-// multiple of 32, at most 1024); red holds 32 words of shared scratch.
-__device__ __forceinline__ uint32_t block_min_u32(uint32_t v, uint32_t* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  __syncthreads();
-  if (lane == 0) red[w] = v;
-  __syncthreads();
-  v = lane < nw ? red[lane] : 0xFFFFFFFFu;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ uint32_t block_max_u32(uint32_t v, uint32_t* red) {
-  return ~block_min_u32(~v, red);
-}
-// exclusive prefix sum of v over threads (in thread order); *total receives the sum
-__device__ __forceinline__ uint32_t block_excl_scan(uint32_t v, uint32_t* red, uint32_t* total) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  uint32_t incl = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
+// Bucket of a key between the depth extremes lo and hi of its list (high words of the keys): linear,
+// hence monotone, so that buckets come out in order.
+struct Buckets {
+  uint32_t lo;
+  float scale;
+  int last;
+  __device__ __forceinline__ Buckets(uint32_t lo_, uint32_t hi_, int nb) : lo(lo_), last(nb - 1) {
+    scale = (float)nb / ((float)(hi_ - lo_) + 1.0f);
   }
-  __syncthreads();
-  if (lane == 31) red[w] = incl;
-  __syncthreads();
-  uint32_t ws = lane < nw ? red[lane] : 0u;
-  uint32_t wincl = ws;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t t = __shfl_up_sync(0xffffffffu, wincl, o);
-    if (lane >= o) wincl += t;
+  __device__ __forceinline__ int of(unsigned long long key) const {
+    return min(last, (int)((float)((uint32_t)(key >> 32) - lo) * scale));
   }
-  *total = __shfl_sync(0xffffffffu, wincl, 31);
-  const uint32_t wbase = __shfl_sync(0xffffffffu, wincl - ws, w);
-  return wbase + incl - v;
+};
+
+// Reductions over the group's warps through red (one word per warp, at most 32), after a sync.
+__device__ __forceinline__ uint32_t red_min(const uint32_t* red, int nw, int lane) {
+  return __reduce_min_sync(0xffffffffu, lane < nw ? red[lane] : 0xFFFFFFFFu);
+}
+__device__ __forceinline__ uint32_t red_max(const uint32_t* red, int nw, int lane) {
+  return __reduce_max_sync(0xffffffffu, lane < nw ? red[lane] : 0u);
 }
 
-// Ascending bucket sort of the 64-bit keys r[0, n) by the whole CTA, through shared memory
-// dst[n] and cnt[2 * NBMAX + 2] (NBMAX a power of two). Keys are bucketed by their high word,
-// linearly between its minimum and maximum over the list (monotone, so buckets come out in
-// order), each bucket is sorted by insertion by one thread, and the result is written back
-// to r. Returns false, with r unchanged, when a bucket would hold more than kMaxBucket keys
-// (many equal or clustered depths); the caller then uses a comparison sort.
-template <int NBMAX>
-__device__ bool cta_bucket_sort(unsigned long long* r, int n, unsigned long long* dst, uint32_t* cnt,
-                                uint32_t* red) {
-  const int T = (int)blockDim.x, tid = threadIdx.x;
-  // about two keys per bucket: a power of two in [32, NBMAX]
-  int NB = 32;
-  while (NB < NBMAX && 2 * NB < n) NB <<= 1;
-  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
-  for (int i = tid; i < n; i += T) {
-    const uint32_t h = (uint32_t)(r[i] >> 32);
-    lo = min(lo, h);
-    hi = max(hi, h);
+// The buckets' counters are 16 bits wide, two to a word (lists are shorter than 2^16): many buckets
+// keep the comparisons within a bucket few where depths cluster, and those, of a warp's fullest
+// bucket, were most of the sort's instructions (2M particles: 4096 buckets for 15,000 keys 84 us,
+// 16384 80 us).
+__device__ __forceinline__ uint32_t count_up(uint32_t* cnt, int b) {   // the count before
+  const int sh = 16 * (b & 1);
+  return (atomicAdd(&cnt[b >> 1], 1u << sh) >> sh) & 0xFFFFu;
+}
+
+// Turns the counts of 2 PER * G.n buckets into exclusive prefix sums, 2 PER consecutive ones per
+// thread; false (counts undefined) when one of them exceeds kMaxBucket. red: 64 words.
+template <int PER>
+__device__ __forceinline__ bool scan_counts(uint32_t* cnt, uint32_t* red, const Group& G) {
+  const int lane = G.t & 31, w = G.t >> 5, nw = G.n >> 5;
+  uint32_t c[PER], sum = 0, mx = 0;
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    c[k] = cnt[PER * G.t + k];
+    sum += (c[k] & 0xFFFFu) + (c[k] >> 16);
+    mx = max(mx, max(c[k] & 0xFFFFu, c[k] >> 16));
   }
-  lo = block_min_u32(lo, red);
-  hi = block_max_u32(hi, red);
-  const float scale = (float)NB / ((float)(hi - lo) + 1.0f);
-  auto bucket = [&](unsigned long long key) {
-    return min(NB - 1, (int)((float)((uint32_t)(key >> 32) - lo) * scale));
+  uint32_t incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += x;
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 31) { red[w] = incl; red[32 + w] = mx; }
+  G.sync();
+  if (red_max(red + 32, nw, lane) > (uint32_t)kMaxBucket) return false;
+  uint32_t at = incl - sum + __reduce_add_sync(0xffffffffu, lane < w ? red[lane] : 0u);
+#pragma unroll
+  for (int k = 0; k < PER; ++k) {
+    const uint32_t odd = at + (c[k] & 0xFFFFu);
+    cnt[PER * G.t + k] = at | (odd << 16);
+    at = odd + (c[k] >> 16);
+  }
+  return true;
+}
+
+// Position of key among the keys [s0, s1) of its bucket.
+__device__ __forceinline__ int bucket_rank(const unsigned long long* keys, int s0, int s1, unsigned long long key) {
+  int c = s0;
+  for (int j = s0; j < s1; ++j) c += keys[j] < key;
+  return c;
+}
+
+// Ascending bucket sort of the 64-bit keys r[0, n), n <= kBucketBigCap, by the whole CTA (1024
+// threads), through shared memory dst[n] and cnt[kBucketsBig / 2]: counts, prefix sums, keys to their
+// buckets, then each key's rank by comparison within its bucket. Returns false, with r unchanged,
+// when a bucket would hold more than kMaxBucket keys (many equal or clustered depths); the caller
+// then uses a comparison sort. The three passes over the list are bound by latency, so four loads
+// are in flight per thread.
+__device__ bool cta_bucket_sort(unsigned long long* r, int n, unsigned long long* dst, uint32_t* cnt, uint32_t* red,
+                                const Group& G) {
+  const int t = G.t, lane = t & 31, w = t >> 5, T = G.n;
+  auto each_key = [&](auto f) {
+    for (int i = t; i < n; i += 4 * T) {
+      unsigned long long k[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) k[u] = i + u * T < n ? r[i + u * T] : 0ull;
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (i + u * T < n) f(k[u]);
+    }
   };
-  uint32_t* start = cnt;            // [NB + 1]
-  uint32_t* cur = cnt + NBMAX + 1;  // [NB]
-  for (int b = tid; b < NB; b += T) start[b] = 0u;
-  __syncthreads();
-  for (int i = tid; i < n; i += T) atomicAdd(&start[bucket(r[i])], 1u);
-  __syncthreads();
-  // each thread owns `per` consecutive buckets (threads past NB own none): the largest
-  // bucket and the buckets' sum
-  const int per = NB >= T ? NB / T : 1;
-  const int mine = tid * per < NB ? per : 0;
-  uint32_t mx = 0u, sum = 0u;
-  for (int k = 0; k < mine; ++k) {
-    const uint32_t c = start[tid * per + k];
-    mx = max(mx, c);
-    sum += c;
+  uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+  each_key([&](unsigned long long k) {
+    lo = min(lo, (uint32_t)(k >> 32));
+    hi = max(hi, (uint32_t)(k >> 32));
+  });
+  constexpr int PER = kBucketsBig / 2 / kSortThreads;
+#pragma unroll
+  for (int k = 0; k < PER; ++k) cnt[t + k * T] = 0u;
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) { red[w] = lo; red[32 + w] = hi; }
+  G.sync();
+  const Buckets bk(red_min(red, T >> 5, lane), red_max(red + 32, T >> 5, lane), kBucketsBig);
+  each_key([&](unsigned long long k) { count_up(cnt, bk.of(k)); });
+  G.sync();
+  if (!scan_counts<PER>(cnt, red, G)) return false;
+  G.sync();
+  each_key([&](unsigned long long k) { dst[count_up(cnt, bk.of(k))] = k; });   // b's end afterwards
+  G.sync();
+  const uint16_t* end = reinterpret_cast<const uint16_t*>(cnt);
+  for (int i = t; i < n; i += T) {
+    const unsigned long long k = dst[i];
+    const int b = bk.of(k);
+    r[bucket_rank(dst, b ? (int)end[b - 1] : 0, (int)end[b], k)] = k;
   }
-  mx = block_max_u32(mx, red);
-  if (mx > (uint32_t)kMaxBucket) return false;
-  uint32_t total = 0;
-  uint32_t base = block_excl_scan(sum, red, &total);
-  __syncthreads();
-  for (int k = 0; k < mine; ++k) {
-    const int b = tid * per + k;
-    const uint32_t c = start[b];
-    start[b] = base;
-    cur[b] = base;
-    base += c;
-  }
-  if (tid == 0) start[NB] = (uint32_t)n;
-  __syncthreads();
-  for (int i = tid; i < n; i += T) {
-    const unsigned long long key = r[i];
-    dst[atomicAdd(&cur[bucket(key)], 1u)] = key;
-  }
-  __syncthreads();
-  for (int b = tid; b < NB; b += T) {
-    const int s0 = (int)start[b], s1 = (int)start[b + 1];
-    for (int i = s0 + 1; i < s1; ++i) {
-      const unsigned long long x = dst[i];
-      int j = i - 1;
-      while (j >= s0 && dst[j] > x) {
-        dst[j + 1] = dst[j];
-        --j;
-      }
-      dst[j + 1] = x;
+  G.sync();
+  return true;
+}
+
+// Shared memory of a quarter CTA sorting one bin of fewer than kSortSmemCap references.
+struct SmallSort {
+  unsigned long long a[kSortSmemCap], b[kSortSmemCap];
+  uint32_t mask[kSortSmemCap];
+  uint32_t cnt[kBucketsSmall / 2 + 4];
+};
+constexpr int kStageWords = (int)(sizeof(SmallSort::a) / 4);   // bitmap assembled in `a`
+
+// The same for n <= KPT * 256 keys by a quarter CTA, the keys in registers,
+// each with its half-block mask (bins of up to 32 pixels: one word), loaded while the keys are
+// counted; the sorted list and its bitmap are written from shared memory.
+template <int KPT>
+__device__ __forceinline__ bool small_bucket_sort(const Ws& ws, unsigned long long* r, int n, int bin, SmallSort& S,
+                                                  uint32_t* red, const Group& G) {
+  const int t = G.t, lane = t & 31, w = t >> 5;
+  constexpr int T = kSortThreads / 4, NB = KPT >= 3 ? kBucketsSmall : 2 * KPT * T, PER = NB / 2 / T;
+  const bool one_word = bin_mw(ws.bin_log2) == 1;
+  const ViewDev& V = ws.views[view_of_bin(ws.views, ws.n_views, bin)];
+  unsigned long long key[KPT];
+  uint32_t at[KPT], mask[KPT], lo = 0xFFFFFFFFu, hi = 0u;
+#pragma unroll
+  for (int k = 0; k < KPT; ++k) key[k] = t + k * T < n ? r[t + k * T] : 0ull;
+#pragma unroll
+  for (int k = 0; k < PER; ++k) S.cnt[t + k * T] = 0u;
+#pragma unroll
+  for (int k = 0; k < KPT; ++k)
+    if (t + k * T < n) {
+      lo = min(lo, (uint32_t)(key[k] >> 32));
+      hi = max(hi, (uint32_t)(key[k] >> 32));
+    }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) { red[w] = lo; red[32 + w] = hi; }
+#pragma unroll
+  for (int k = 0; k < KPT; ++k) mask[k] = 0u;
+  if (one_word) {
+    const int b = bin - V.bin_base, lg = ws.bin_log2;
+    const int x0 = (b % V.nbx) << lg, y0 = (b / V.nbx) << lg;
+#pragma unroll
+    for (int k = 0; k < KPT; ++k) {
+      const uint32_t rec = t + k * T < n ? ~(uint32_t)key[k] : 0xFFFFFFFFu;
+      mask[k] = rec < (uint64_t)ws.total_quads ? hb_mask_word(ws.rec_rect[rec], x0, y0, lg, 0) : 0u;
     }
   }
-  __syncthreads();
-  for (int i = tid; i < n; i += T) r[i] = dst[i];
-  __syncthreads();
+  G.sync();
+  const Buckets bk(red_min(red, T / 32, lane), red_max(red + 32, T / 32, lane), NB);
+#pragma unroll
+  for (int k = 0; k < KPT; ++k)
+    if (t + k * T < n) {
+      const int b = bk.of(key[k]);
+      at[k] = (uint32_t)b | (count_up(S.cnt, b) << 16);
+    }
+  G.sync();
+  if (!scan_counts<PER>(S.cnt, red, G)) return false;
+  if (t == 0) S.cnt[NB / 2] = (uint32_t)n;
+  const uint16_t* start = reinterpret_cast<const uint16_t*>(S.cnt);
+  G.sync();
+#pragma unroll
+  for (int k = 0; k < KPT; ++k)
+    if (t + k * T < n) S.a[start[at[k] & 0xFFFFu] + (at[k] >> 16)] = key[k];
+  G.sync();
+#pragma unroll
+  for (int k = 0; k < KPT; ++k)
+    if (t + k * T < n) {
+      const int b = (int)(at[k] & 0xFFFFu);
+      const int p = bucket_rank(S.a, (int)start[b], (int)start[b + 1], key[k]);
+      S.b[p] = key[k];
+      S.mask[p] = mask[k];
+    }
+  G.sync();
+  for (int i = t; i < n; i += T) r[i] = S.b[i];
+  uint32_t* stage = reinterpret_cast<uint32_t*>(S.a);
+  if (!one_word) {
+    G.sync();
+    write_hb_bitmap(ws, r, n, bin, stage, kStageWords, G);
+    return true;
+  }
+  const int nw = (n + 31) >> 5;
+  uint32_t* bm = ws.ref_hb + (size_t)(r - ws.refs) + (size_t)bin_mrows(ws.bin_log2) * (size_t)bin;
+  for (int i = w; i < nw; i += T / 32)
+    stage[lane * nw + i] = warp_transpose32(32 * i + lane < n ? S.mask[32 * i + lane] : 0u, lane);
+  G.sync();
+  for (int i = t; i < 32 * nw; i += T) bm[i] = stage[i];
   return true;
 }
 
@@ -551,9 +653,9 @@ __device__ __forceinline__ void warp_bitonic(unsigned long long v[KPL], int lane
 // Runs of 32 KPL keys of g[0, n), one warp each, sorted into A (padded with the largest key
 // up to the end of the last run).
 template <int KPL>
-__device__ __forceinline__ void sort_runs(const unsigned long long* g, int n, unsigned long long* A) {
+__device__ __forceinline__ void sort_runs(const unsigned long long* g, int n, unsigned long long* A, const Group& G) {
   constexpr int L = 32 * KPL;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int lane = G.t & 31, warp = G.t >> 5, nw = G.n >> 5;
   for (int r = warp; L * r < n; r += nw) {
     unsigned long long v[KPL];
     const int base = L * r + KPL * lane;
@@ -565,26 +667,26 @@ __device__ __forceinline__ void sort_runs(const unsigned long long* g, int n, un
   }
 }
 
-// Ascending merge sort of g[0, n) (n <= 256 * warps of the CTA) in shared memory by the whole
-// CTA: runs sorted in registers, one per warp (sort_runs), then merge levels between two
+// Ascending merge sort of g[0, n) (n <= 256 * warps of the group) in shared memory by the whole
+// group: runs sorted in registers, one per warp (sort_runs), then merge levels between two
 // shared buffers, each thread producing an equal slice of every level's output (merge path
 // search + a sequential merge of its slice). Runs are 256 keys long when nearly every warp
 // gets one, else 128 or 64 (a warp without a run would wait at the barrier). The keys are
 // padded to a power of two N with the largest key, so every output position from n on
 // holds padding at every level: both buffers are padded once, and the runs and output
 // slices starting at n or later are skipped.
-__device__ __forceinline__ void cta_merge_sort_smem(unsigned long long* g, int n, unsigned long long* A,
-                                    unsigned long long* Bf) {
-  const int T = (int)blockDim.x, t = threadIdx.x, nw = T >> 5;
+__device__ __noinline__ void merge_sort_smem(unsigned long long* g, int n, unsigned long long* A,
+                                             unsigned long long* Bf, const Group G) {
+  const int T = G.n, t = G.t, nw = T >> 5;
   const int run = n > (nw - 1) * 256 ? 256 : (n > (nw - 1) * 128 ? 128 : 64);
   int N = run;
   while (N < n) N <<= 1;
-  if (run == 256) sort_runs<8>(g, n, A);
-  else if (run == 128) sort_runs<4>(g, n, A);
-  else sort_runs<2>(g, n, A);
+  if (run == 256) sort_runs<8>(g, n, A, G);
+  else if (run == 128) sort_runs<4>(g, n, A, G);
+  else sort_runs<2>(g, n, A, G);
   for (int i = ((n + run - 1) / run) * run + t; i < N; i += T) A[i] = ~0ull;
   for (int i = n + t; i < N; i += T) Bf[i] = ~0ull;
-  __syncthreads();
+  G.sync();
   unsigned long long* src = A;
   unsigned long long* dst = Bf;
   for (int w = run; w < N; w <<= 1) {
@@ -606,7 +708,7 @@ __device__ __forceinline__ void cta_merge_sort_smem(unsigned long long* g, int n
         j += !ta;
       }
     }
-    __syncthreads();
+    G.sync();
     unsigned long long* tmp = src; src = dst; dst = tmp;
   }
   for (int i = t; i < n; i += T) g[i] = src[i];
@@ -628,59 +730,47 @@ __device__ __forceinline__ bool bin_owned(const Ws& ws, int bin) {
   return false;
 }
 
-#ifndef LR_SORT_MIN_BLOCKS
-#define LR_SORT_MIN_BLOCKS 5   // resident CTAs per SM (48 registers, no spills)
-#endif
-__global__ __launch_bounds__(256, LR_SORT_MIN_BLOCKS) void k_bin_sort(Ws ws) {
+// One persistent CTA per SM. It takes the high-density bins first, one at a time with all its
+// threads, then its quarters take the other non-empty bins, largest first: while a few CTAs still
+// sort the largest bins, the others have gone on. Bound by latency and issue (46% of the slots). As
+// two kernels one after the other, the small bins merge-sorted: 2M particles 41 + 80 us against
+// 82 us, the layer frame 41 + 4 against 31, a batch of six mixed views 131 against 74.
+__global__ __launch_bounds__(kSortThreads, 1) void k_bin_sort(Ws ws) {
   pdl_begin();
-  extern __shared__ unsigned long long sbuf[];
+  extern __shared__ __align__(16) unsigned char sort_smem[];
+  __shared__ int s_bin[4];
+  __shared__ uint32_t s_red[4][64];
   if (ws.ctrl->error == LR_ERR_OVERFLOW) return;
-  const int bin = blockIdx.x;
-  const uint32_t off = ws.bin_off[bin];
-  const int n = (int)(ws.bin_off[bin + 1] - off);
-  if (n >= kSortSmemCap) return;   // high-density: k_bin_sort_big
-  if (!bin_owned(ws, bin)) return;  // a tile another renderer rasterises
-  unsigned long long* r = ws.refs + off;
-  if (n > 1) {
-    cta_merge_sort_smem(r, n, sbuf, sbuf + kSortSmemCap);
-    __syncthreads();
-  }
-  write_hb_bitmap(ws, r, n, bin, reinterpret_cast<uint32_t*>(sbuf), (int)(kSortSmemBytes / 4));
-}
-
-__global__ __launch_bounds__(kSortBigThreads, 1) void k_bin_sort_big(Ws ws) {
-  pdl_begin();
-  extern __shared__ unsigned long long sbuf[];
-  __shared__ int s_bin;
-  if (ws.ctrl->error == LR_ERR_OVERFLOW) return;
-  const unsigned long long n_big = ws.ctrl->bins_high;
-  for (;;) {
+  const unsigned long long n_big = ws.ctrl->bins_high, n_all = ws.ctrl->bins_nonempty;
+  const Group C{(int)threadIdx.x, kSortThreads, 0};
+  unsigned long long* sbuf = reinterpret_cast<unsigned long long*>(sort_smem);
+  uint32_t* stage = reinterpret_cast<uint32_t*>(sort_smem);
+  while (n_big) {
     if (threadIdx.x == 0) {
       const unsigned long long k = atomicAdd(&ws.ctrl->sort_head, 1ull);
-      s_bin = k < n_big ? (int)ws.bin_order[k] : -1;
+      s_bin[0] = k < n_big ? (int)ws.bin_order[k] : -1;
     }
-    __syncthreads();
-    const int bin = s_bin;
-    __syncthreads();
-    if (bin < 0) return;
-    if (!bin_owned(ws, bin)) continue;
+    C.sync();
+    const int bin = s_bin[0];
+    C.sync();
+    if (bin < 0) break;
+    if (!bin_owned(ws, bin)) continue;  // a tile another renderer rasterises
     const uint32_t off = ws.bin_off[bin];
     const int n = (int)(ws.bin_off[bin + 1] - off);
     unsigned long long* r = ws.refs + off;
-    __shared__ uint32_t red[32];
-    if (n <= kBucketBigCap &&
-        cta_bucket_sort<kBucketsBig>(r, n, sbuf, reinterpret_cast<uint32_t*>(sbuf + kBucketBigCap), red)) {
+    if (n <= kBucketBigCap && cta_bucket_sort(r, n, sbuf, reinterpret_cast<uint32_t*>(sbuf + kBucketBigCap), s_red[0], C)) {
       if (threadIdx.x == 0) atomicAdd(&ws.ctrl->sort_branch[0], 1ull);
-      write_hb_bitmap(ws, r, n, bin, reinterpret_cast<uint32_t*>(sbuf), (int)(kSortBigSmemBytes / 4));
-      __syncthreads();
+      write_hb_bitmap(ws, r, n, bin, stage, (int)(kSortSmemBytes / 4), C);
+      C.sync();
       continue;
     }
     const int run0 = n <= kSortBigCap ? n : kSortBigCap;
     if (threadIdx.x == 0) atomicAdd(&ws.ctrl->sort_branch[n <= kSortBigCap ? 1 : 2], 1ull);
+    C.sync();
     // sort runs of up to kSortBigCap references in shared memory
     for (int s = 0; s < n; s += run0) {
-      cta_merge_sort_smem(r + s, min(run0, n - s), sbuf, sbuf + kSortBigCap);
-      __syncthreads();
+      merge_sort_smem(r + s, min(run0, n - s), sbuf, sbuf + kSortBigCap, C);
+      C.sync();
     }
     // merge the runs through the global buffer (only for more than kSortBigCap)
     unsigned long long* src = r;
@@ -691,16 +781,47 @@ __global__ __launch_bounds__(kSortBigThreads, 1) void k_bin_sort_big(Ws ws) {
         const int nbb = min(run, max(0, n - s - run));
         cta_merge(src + s, na, src + s + na, nbb, dst + s);
       }
-      __syncthreads();
+      C.sync();
       unsigned long long* t = src; src = dst; dst = t;
     }
     if (src != r) {
       for (int i = threadIdx.x; i < n; i += blockDim.x) r[i] = src[i];
     }
-    __syncthreads();
-    write_hb_bitmap(ws, r, n, bin, reinterpret_cast<uint32_t*>(sbuf), (int)(kSortBigSmemBytes / 4));
-    __syncthreads();
+    C.sync();
+    write_hb_bitmap(ws, r, n, bin, stage, (int)(kSortSmemBytes / 4), C);
+    C.sync();
+  }
+  const int q = (int)(threadIdx.x / (kSortThreads / 4));
+  const Group G{(int)(threadIdx.x % (kSortThreads / 4)), kSortThreads / 4, 1 + q};
+  SmallSort& S = reinterpret_cast<SmallSort*>(sort_smem)[q];
+  auto ticket = [&]() { return (int)min(n_big + atomicAdd(&ws.ctrl->sort_small_head, 1ull), n_all); };
+  int k = 0;   // (thread 0 of the quarter; the next ticket is drawn while a bin is sorted)
+  if (G.t == 0) s_bin[q] = ticket();
+  for (;;) {
+    G.sync();
+    const int item = s_bin[q];
+    if (item >= (int)n_all) return;
+    if (G.t == 0) k = ticket();
+    const int bin = (int)ws.bin_order[item];
+    if (bin_owned(ws, bin)) {
+      const uint32_t off = ws.bin_off[bin];
+      const int n = (int)(ws.bin_off[bin + 1] - off);
+      unsigned long long* r = ws.refs + off;
+      const bool done = n <= kSortThreads / 4       ? small_bucket_sort<1>(ws, r, n, bin, S, s_red[q], G)
+                        : n <= 2 * kSortThreads / 4 ? small_bucket_sort<2>(ws, r, n, bin, S, s_red[q], G)
+                        : n <= 3 * kSortThreads / 4 ? small_bucket_sort<3>(ws, r, n, bin, S, s_red[q], G)
+                        : n <= kSortThreads         ? small_bucket_sort<4>(ws, r, n, bin, S, s_red[q], G)
+                                                    : small_bucket_sort<8>(ws, r, n, bin, S, s_red[q], G);
+      if (!done) {
+        merge_sort_smem(r, n, S.a, S.b, G);
+        G.sync();
+        write_hb_bitmap(ws, r, n, bin, reinterpret_cast<uint32_t*>(S.a), kStageWords, G);
+      }
+    }
+    G.sync();
+    if (G.t == 0) s_bin[q] = k;
   }
 }
+static_assert(4 * sizeof(SmallSort) <= kSortSmemBytes, "a quarter of the CTA's shared memory each");
 
 }  // namespace lr

@@ -32,20 +32,18 @@ __host__ __device__ __forceinline__ int bin_mrows_log2(int lg) { return lg < 5 ?
 __host__ __device__ __forceinline__ int bin_mrows(int lg) { return 1 << bin_mrows_log2(lg); }  // 32, 32, 128
 __host__ __device__ __forceinline__ int bin_mw(int lg) { return bin_mrows(lg) >> 5; }         // 1, 1, 4
 constexpr float kGuardPx = 16384.0f;        // guard band, pixels
-constexpr int kSortSmemCap = 2048;          // bins below this many refs: k_bin_sort (256 threads)
-constexpr int kSortBigCap = 8192;           // k_bin_sort_big sorts runs of up to this many refs
-constexpr int kSortBigThreads = 1024;
-// k_bin_sort_big's bucket sort: at most this many buckets per bin, the largest bin sorted
-// this way in shared memory, and the largest bucket sorted by insertion (a bin with a
-// larger bucket, e.g. many equal depths, falls back to the merge sort)
-constexpr int kBucketsBig = 4096;
+constexpr int kSortThreads = 1024;          // k_bin_sort's CTA
+constexpr int kSortSmemCap = 2048;          // bins below this many refs: a quarter of the CTA each
+constexpr int kSortBigCap = 8192;           // the merge sort's runs of a high-density bin, at most
+// the bucket sorts: buckets of a high-density and (at most) of another bin, the largest bin sorted
+// this way in shared memory, and the largest bucket (a bin with a larger one, e.g. many equal
+// depths, falls back to the merge sort)
+constexpr int kBucketsBig = 16384;
+constexpr int kBucketsSmall = 2048;
 constexpr int kBucketBigCap = 20480;
 constexpr int kMaxBucket = 64;
-constexpr size_t kSortSmemBytes = 2 * (size_t)kSortSmemCap * 8;
-constexpr size_t kSortBigSmemBytes =
-    (size_t)kBucketBigCap * 8 + (2 * (size_t)kBucketsBig + 2) * 4 > 2 * (size_t)kSortBigCap * 8
-        ? (size_t)kBucketBigCap * 8 + (2 * (size_t)kBucketsBig + 2) * 4
-        : 2 * (size_t)kSortBigCap * 8;
+constexpr size_t kSortSmemBytes = (size_t)kBucketBigCap * 8 + (size_t)kBucketsBig * 2;
+static_assert(kSortSmemBytes >= 2 * (size_t)kSortBigCap * 8, "two merge buffers");
 constexpr int kHistSmemBins = 8192;         // shared-memory bin counters per CTA (Sec. 2 Stage 2)
 #ifndef LR_CHUNK_QUADS
 #define LR_CHUNK_QUADS 2048
@@ -158,15 +156,15 @@ struct Ctrl {
   unsigned long long raster_items;
   unsigned long long ovf_count;      // pixels registered for the exact path
   unsigned long long ovf_head;
-  unsigned long long sort_head;      // k_bin_sort_big's queue over the high-density bins
+  unsigned long long sort_head;      // k_bin_sort's queue over the high-density bins
   unsigned long long fragments;
-  unsigned long long unused0;
+  unsigned long long sort_small_head;   // ... and over the others
   unsigned long long culled[8];
   unsigned long long bins_nonempty;
   unsigned long long bins_high;
   unsigned long long max_bin;
   unsigned long long chunk_list_head;   // allocation cursor of the chunks' (bin, base) lists
-  // high-density bins by the sort k_bin_sort_big gave them: bucket sort, merge sort in
+  // high-density bins by the sort k_bin_sort gave them: bucket sort, merge sort in
   // shared memory alone, merge sort with runs merged through global memory
   unsigned long long sort_branch[3];
   unsigned long long pad[4];

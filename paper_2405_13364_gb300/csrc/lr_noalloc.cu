@@ -34,7 +34,6 @@ __global__ void k_bin_count(Ws ws);
 __global__ void k_bin_scan(Ws ws);
 __global__ void k_bin_scatter(Ws ws);
 __global__ void k_bin_sort(Ws ws);
-__global__ void k_bin_sort_big(Ws ws);
 cudaError_t prepare_raster_3(int* blocks_flat, int* blocks_vtx, int* blocks_bwd, int* blocks_lit);
 cudaError_t launch_raster_3(int mode, const Ws& ws, int grid, cudaStream_t st);
 cudaError_t overflow_occupancy(int* blocks_per_sm);
@@ -132,9 +131,7 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
           prepare_raster_3(&d.blocks_flat, &d.blocks_vtx, &blocks_bwd, &blocks_lit) != cudaSuccess ||
           overflow_occupancy(&d.ovf_blocks) != cudaSuccess ||
           cudaFuncSetAttribute(k_bin_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kSortSmemBytes) != cudaSuccess ||
-          cudaFuncSetAttribute(k_bin_sort_big, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)kSortBigSmemBytes) != cudaSuccess)
+                               (int)kSortSmemBytes) != cudaSuccess)
         return LR_ERR_CUDA;
       // Load every kernel this entry point can launch now, not at its first launch: with
       // CUDA's lazy module loading a kernel's first launch loads it, which a later call
@@ -218,8 +215,7 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
   if (chunks > 0) k_bin_count<<<chunks, kBinThreads, 0, st>>>(ws);
   k_bin_scan<<<1, 1024, 0, st>>>(ws);
   if (chunks > 0) k_bin_scatter<<<chunks, kBinThreads, 0, st>>>(ws);
-  k_bin_sort<<<(int)nbins, 256, kSortSmemBytes, st>>>(ws);
-  k_bin_sort_big<<<ds.sms, kSortBigThreads, kSortBigSmemBytes, st>>>(ws);
+  k_bin_sort<<<ds.sms, kSortThreads, kSortSmemBytes, st>>>(ws);
   const bool vtx_kernel = Q > 0 && vtx;
   if (launch_raster_3(vtx_kernel ? 1 : 0, ws, ds.sms * (vtx_kernel ? ds.blocks_vtx : ds.blocks_flat), st) != cudaSuccess)
     return LR_ERR_CUDA;
