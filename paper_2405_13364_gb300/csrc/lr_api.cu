@@ -87,7 +87,7 @@ struct Layout {
   size_t ctrl, views, rec, rec_rect, rec_info, rec_rep, bin_count, bin_off, bin_cursor, bin_order, chunk_span;
   size_t refs, refs_tmp, ref_hb, ovf_list, total;
   long long total_quads = 0, total_pix = 0, refs_cap = 0;
-  int total_bins = 0, total_chunks = 0;
+  int total_bins = 0, total_chunks = 0, chunk_quads = kChunkQuads;
   int cursors = 0;
 };
 
@@ -106,8 +106,9 @@ static Layout make_layout(int n, const long long* Q, const int* W, const int* H,
     L.total_pix += (long long)W[i] * H[i];
     L.total_bins += nbx * nby;
     L.cursors |= nbx * nby > kHistSmemBins;
-    L.total_chunks += (int)((Q[i] + kChunkQuads - 1) / kChunkQuads);
   }
+  L.chunk_quads = chunk_quads_for(L.total_quads);
+  for (int i = 0; i < n; ++i) L.total_chunks += (int)((Q[i] + L.chunk_quads - 1) / L.chunk_quads);
   size_t o = 0;
   auto take = [&](size_t bytes) { const size_t at = o; o = align256(o + bytes); return at; };
   L.ctrl = take(sizeof(Ctrl));
@@ -169,6 +170,7 @@ static Ws make_ws(const Layout& L, void* base, int n_views) {
   w.refs_cap = L.refs_cap;
   w.bin_log2 = L.bin_log2;
   w.cursors = L.cursors;
+  w.chunk_quads = L.chunk_quads;
   w.ticket = 1;
   w.rec = reinterpret_cast<int4*>(b + L.rec);
   w.rec_rect = reinterpret_cast<uint2*>(b + L.rec_rect);
@@ -442,7 +444,7 @@ struct Prepared {
 };
 
 static void describe_views(int32_t n_views, const lr_view* views, std::vector<ViewDev>& vd, bool* any_vertex,
-                           bool* any_hash, bool* any_lit, const float* light, int lg) {
+                           bool* any_hash, bool* any_lit, const float* light, int lg, int chunk_quads) {
   const int B = 1 << lg;
   vd.resize(n_views);
   long long qb = 0, pb = 0;
@@ -488,7 +490,7 @@ static void describe_views(int32_t n_views, const lr_view* views, std::vector<Vi
     qb += v.quads.num_quads;
     pb += (long long)v.width * v.height;
     bb += d.nbx * d.nby;
-    cb += (int)((v.quads.num_quads + kChunkQuads - 1) / kChunkQuads);
+    cb += (int)((v.quads.num_quads + chunk_quads - 1) / chunk_quads);
     *any_vertex |= (v.quads.color_mode == LR_COLOR_VERTEX && v.quads.num_quads > 0);
     *any_hash |= v.target.cov_hash != nullptr;
     *any_lit |= (v.quads.color_mode == LR_COLOR_LIT && v.quads.num_quads > 0);
@@ -520,7 +522,8 @@ static lr_status prepare(lr_ctx* ctx, int32_t n_views, const lr_view* views, voi
   if (s != LR_OK) return s;
   set_capacity(P->L, workspace_bytes);
   if (P->L.refs_cap < 1024) return fail(ctx, LR_ERR_OOM, "workspace too small (see lr_workspace_size)%s");
-  describe_views(n_views, views, P->vd, &P->any_vertex, &P->any_hash, &P->any_lit, ctx->light, ctx->bin_log2);
+  describe_views(n_views, views, P->vd, &P->any_vertex, &P->any_hash, &P->any_lit, ctx->light, ctx->bin_log2,
+                 P->L.chunk_quads);
   if (P->any_lit && (P->any_hash || (ctx->cfg.flags & LR_FLAG_ALPHA_THRESHOLD)))
     return fail(ctx, LR_ERR_UNSUPPORTED, "lit colours with coverage hashes or the alpha threshold%s");
   P->ws = make_ws(P->L, workspace, n_views);
@@ -719,7 +722,8 @@ extern "C" lr_status lr_graph_launch(lr_graph* g, const lr_view* views, lr_strea
     std::vector<ViewDev> vd;
     bool any_vertex = false, any_hash = false, any_lit = false;
     // replays keep the light the graph was captured with
-    describe_views(n, views, vd, &any_vertex, &any_hash, &any_lit, g->P.vd[0].light, ctx->bin_log2);
+    describe_views(n, views, vd, &any_vertex, &any_hash, &any_lit, g->P.vd[0].light, ctx->bin_log2,
+                   g->P.L.chunk_quads);
     memcpy(g->staging[b], vd.data(), sizeof(ViewDev) * (size_t)n);
   }
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);

@@ -1,8 +1,8 @@
 // lr_bin.cu -- Stage 2 of the pipeline, quad binning (Sec. 2, "Stage 2: quad binning"),
 // plus the per-bin depth sort that feeds Stage 3.
 //
-//   k_bin_count    Phase 1: per-bin reference counts. Each CTA owns a chunk of 2048 quads
-//                  of one view and counts into shared-memory bin counters (the paper's
+//   k_bin_count    Phase 1: per-bin reference counts. Each CTA owns a chunk of up to 2048
+//                  quads of one view and counts into shared-memory bin counters (the paper's
 //                  5120-entry arrays), then adds its non-zero counters to global memory.
 //                  Quads whose bin rectangle is at most 4x4 bins are counted from their
 //                  AABB; larger quads are tested bin by bin with a conservative
@@ -30,47 +30,32 @@
 
 namespace lr {
 
-// Conservative test whether a triangle of a quad can cover a pixel centre of bin (bx, by):
-// false only if one edge is negative (after the fill-rule bias) at all four corner pixel
-// centres of the bin rectangle clipped to the triangle's pixel AABB and the screen.
-__device__ bool tri_may_touch_bin(const int X[4], const int Y[4], int t, int bx, int by, int W, int H, int lg) {
-  int a = 0, b = t == 0 ? 1 : 2, c = t == 0 ? 2 : 3;
-  long long A = area2(X[a], Y[a], X[b], Y[b], X[c], Y[c]);
-  if (A == 0) return false;
-  if (A < 0) { int tmp = b; b = c; c = tmp; }
-  const int vx[3] = {X[a], X[b], X[c]}, vy[3] = {Y[a], Y[b], Y[c]};
-  const int xmin = min(vx[0], min(vx[1], vx[2])), xmax = max(vx[0], max(vx[1], vx[2]));
-  const int ymin = min(vy[0], min(vy[1], vy[2])), ymax = max(vy[0], max(vy[1], vy[2]));
-  const int x0 = max(max(ceil_div256((long long)xmin - 128), 0), bx << lg);
-  const int x1 = min(min(floor_div256((long long)xmax - 128), W - 1), ((bx + 1) << lg) - 1);
-  const int y0 = max(max(ceil_div256((long long)ymin - 128), 0), by << lg);
-  const int y1 = min(min(floor_div256((long long)ymax - 128), H - 1), ((by + 1) << lg) - 1);
-  if (x0 > x1 || y0 > y1) return false;
-  const long long cx[2] = {256LL * x0 + 128, 256LL * x1 + 128};
-  const long long cy[2] = {256LL * y0 + 128, 256LL * y1 + 128};
+// Conservative test whether triangle t of a quad can cover a pixel centre of bin (bx, by): false
+// only if one edge is negative (after the fill-rule bias) at all four corner pixel centres of the
+// bin rectangle clipped to the triangle's pixel AABB and the screen. An edge value is a sum of a
+// term in x and one in y, so its largest corner value takes the better x and the better y. What
+// does not depend on the bin stays in registers over a quad's bins.
+__device__ __forceinline__ bool tri_may_touch_bin(const int X[4], const int Y[4], uint32_t info, int t, int bx, int by, int W,
+                                                  int H, int lg) {
+  if (!(info & (kInfoTri0 << t))) return false;
+  const bool sw = (info & (kInfoSwap0 << t)) != 0;
+  const int b = sw ? 2 + t : 1 + t, c = sw ? 1 + t : 2 + t;
+  const int vx[3] = {X[0], b == 1 ? X[1] : (b == 2 ? X[2] : X[3]), c == 1 ? X[1] : (c == 2 ? X[2] : X[3])};
+  const int vy[3] = {Y[0], b == 1 ? Y[1] : (b == 2 ? Y[2] : Y[3]), c == 1 ? Y[1] : (c == 2 ? Y[2] : Y[3])};
+  const int x0 = max(max((min(vx[0], min(vx[1], vx[2])) + 127) >> 8, 0), bx << lg);
+  const int x1 = min(min((max(vx[0], max(vx[1], vx[2])) - 128) >> 8, W - 1), ((bx + 1) << lg) - 1);
+  const int y0 = max(max((min(vy[0], min(vy[1], vy[2])) + 127) >> 8, 0), by << lg);
+  const int y1 = min(min((max(vy[0], max(vy[1], vy[2])) - 128) >> 8, H - 1), ((by + 1) << lg) - 1);
+  bool in = x0 <= x1 && y0 <= y1;
 #pragma unroll
   for (int e = 0; e < 3; ++e) {
-    const int u = e == 0 ? 1 : (e == 1 ? 2 : 0);
-    const int w = e == 0 ? 2 : (e == 1 ? 0 : 1);
-    const long long dx = (long long)vx[w] - vx[u], dy = (long long)vy[w] - vy[u];
-    const long long bias = (dy < 0 || (dy == 0 && dx > 0)) ? 0 : -1;
-    bool all_out = true;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const long long ev = dx * (cy[i >> 1] - vy[u]) - dy * (cx[i & 1] - vx[u]) + bias;
-      all_out &= ev < 0;
-    }
-    if (all_out) return false;
+    const int u = e == 2 ? 0 : e + 1, w = e == 0 ? 2 : (e == 1 ? 0 : 1);
+    const int dx = vx[w] - vx[u], dy = vy[w] - vy[u];
+    const int cx = 256 * (dy < 0 ? x1 : x0) + 128, cy = 256 * (dx > 0 ? y1 : y0) + 128;
+    const long long ev = (long long)dx * (cy - vy[u]) - (long long)dy * (cx - vx[u]);
+    in = in && ev >= ((dy < 0 || (dy == 0 && dx > 0)) ? 0 : 1);
   }
-  return true;
-}
-
-__device__ __forceinline__ bool quad_may_touch_bin(const Ws& ws, long long q, uint32_t info, int bx,
-                                                   int by, int W, int H) {
-  const int4 a = ws.rec[4 * q], b = ws.rec[4 * q + 1];
-  const int X[4] = {a.x, a.z, b.x, b.z}, Y[4] = {a.y, a.w, b.y, b.w};
-  return ((info & kInfoTri0) && tri_may_touch_bin(X, Y, 0, bx, by, W, H, ws.bin_log2)) ||
-         ((info & kInfoTri1) && tri_may_touch_bin(X, Y, 1, bx, by, W, H, ws.bin_log2));
+  return in;
 }
 
 // Per-bin representative depth of a quad that spans several bins.
@@ -88,13 +73,35 @@ __device__ __forceinline__ unsigned long long ref_key(float rep, long long q) {
 
 // Shared by count and scatter: for each (visible quad, touched bin) of the CTA's chunk
 // call f(q, local_bin, bx, by). Small quads enumerate their AABB bins in their own
-// thread; large quads are processed by the whole warp, one bin per lane.
+// thread; large quads are processed by the whole warp, one bin per lane, and those whose box
+// spans more than kWarpBins bins by the whole CTA afterwards: one warp walks the 2,040 bins of a
+// screen-filling quad in 64 steps, which took longer than all the rest of the chunk (a frame of
+// 100,000 parallelograms with a few such quads: count 15.5 us, scatter 22.4).
 // PF: the next iteration's rectangle and info are loaded while this one's bins are handled
 // (the count's loop is latency-bound, a dependent load per iteration otherwise: 18.4 -> 17.0
 // µs on the layer frame; the scatter, with more live registers, measured no faster with it).
+constexpr int kWarpBins = 128;
+struct LargeList {
+  uint32_t n;
+  uint16_t at[kChunkQuads];   // offset in the chunk
+};
+template <typename F>
+__device__ __forceinline__ void large_quad_bins(const Ws& ws, const ViewDev& V, long long q, uint2 rect, uint32_t info,
+                                                int first, int step, F&& f) {
+  const int lg = ws.bin_log2, W = V.width, H = V.height;
+  const int bx0 = (int)(rect.x & 0xffff) >> lg, by0 = (int)(rect.y & 0xffff) >> lg;
+  const int bw = ((int)(rect.x >> 16) >> lg) - bx0 + 1, nb = bw * (((int)(rect.y >> 16) >> lg) - by0 + 1);
+  int X[4], Y[4];
+  load_rec_xy(ws.rec, (uint32_t)q, X, Y);
+  for (int i = first; i < nb; i += step) {
+    const int by = by0 + i / bw, bx = bx0 + i - (by - by0) * bw;
+    if (tri_may_touch_bin(X, Y, info, 0, bx, by, W, H, lg) || tri_may_touch_bin(X, Y, info, 1, bx, by, W, H, lg))
+      f(q, by * V.nbx + bx, bx, by, rect, info);
+  }
+}
 template <bool PF, typename F>
 __device__ __forceinline__ void for_each_ref(const Ws& ws, const ViewDev& V, long long q0, long long q1,
-                                             F&& f) {
+                                             LargeList& list, F&& f) {
   const int lane = threadIdx.x & 31;
   const int lg = ws.bin_log2;
   long long base = q0 + (threadIdx.x & ~31);
@@ -115,26 +122,32 @@ __device__ __forceinline__ void for_each_ref(const Ws& ws, const ViewDev& V, lon
       info = ws.rec_info[q];
     }
     const bool vis = in && rect.x != kRectInvisible;
-    const int px0 = rect.x & 0xffff, px1 = rect.x >> 16, py0 = rect.y & 0xffff, py1 = rect.y >> 16;
-    if (vis && !(info & kInfoLarge)) {
-      for (int by = py0 >> lg; by <= (py1 >> lg); ++by)
-        for (int bx = px0 >> lg; bx <= (px1 >> lg); ++bx) f(q, by * V.nbx + bx, bx, by, rect, info);
+    const int bx0 = (int)(rect.x & 0xffff) >> lg, bx1 = (int)(rect.x >> 16) >> lg;
+    const int by0 = (int)(rect.y & 0xffff) >> lg, by1 = (int)(rect.y >> 16) >> lg;
+    bool large = vis && (info & kInfoLarge);
+    if (vis && !large) {
+      for (int by = by0; by <= by1; ++by)
+        for (int bx = bx0; bx <= bx1; ++bx) f(q, by * V.nbx + bx, bx, by, rect, info);
     }
-    unsigned large = __ballot_sync(0xffffffffu, vis && (info & kInfoLarge));
-    while (large) {
-      const int src = __ffs(large) - 1;
-      large &= large - 1;
-      const long long lq = __shfl_sync(0xffffffffu, q, src);
+    if (large && (bx1 - bx0 + 1) * (by1 - by0 + 1) > kWarpBins) {
+      list.at[atomicAdd(&list.n, 1u)] = (uint16_t)(q - q0);
+      large = false;
+    }
+    unsigned todo = __ballot_sync(0xffffffffu, large);
+    while (todo) {
+      const int src = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const long long lq = base + src;
       const uint2 lr = make_uint2(__shfl_sync(0xffffffffu, rect.x, src), __shfl_sync(0xffffffffu, rect.y, src));
       const uint32_t li = __shfl_sync(0xffffffffu, info, src);
-      const int bx0 = (lr.x & 0xffff) >> lg, bx1 = (lr.x >> 16) >> lg;
-      const int by0 = (lr.y & 0xffff) >> lg, by1 = (lr.y >> 16) >> lg;
-      const int bw = bx1 - bx0 + 1, nb = bw * (by1 - by0 + 1);
-      for (int i = lane; i < nb; i += 32) {
-        const int bx = bx0 + i % bw, by = by0 + i / bw;
-        if (quad_may_touch_bin(ws, lq, li, bx, by, V.width, V.height)) f(lq, by * V.nbx + bx, bx, by, lr, li);
-      }
+      large_quad_bins(ws, V, lq, lr, li, lane, 32, f);
     }
+  }
+  __syncthreads();
+  const int n = (int)list.n;
+  for (int i = 0; i < n; ++i) {
+    const long long q = q0 + list.at[i];
+    large_quad_bins(ws, V, q, ws.rec_rect[q], ws.rec_info[q], threadIdx.x, blockDim.x, f);
   }
 }
 
@@ -143,19 +156,21 @@ __device__ __forceinline__ void for_each_ref(const Ws& ws, const ViewDev& V, lon
 __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_count(Ws ws) {
   pdl_begin();
   __shared__ uint32_t hist[kHistSmemBins];
+  __shared__ LargeList large;
   const int v = view_of_chunk(ws.views, ws.n_views, blockIdx.x);
   const ViewDev& V = ws.views[v];
-  const long long q0 = V.quad_base + (long long)(blockIdx.x - V.chunk_base) * kChunkQuads;
-  const long long q1 = min(q0 + kChunkQuads, V.quad_base + V.num_quads);
+  const long long q0 = V.quad_base + (long long)(blockIdx.x - V.chunk_base) * ws.chunk_quads;
+  const long long q1 = min(q0 + ws.chunk_quads, V.quad_base + V.num_quads);
   const int nb = V.nbx * V.nby;
   const bool smem = nb <= kHistSmemBins;
+  if (threadIdx.x == 0) large.n = 0u;
   if (smem)
     for (int b = threadIdx.x; b < nb; b += blockDim.x) hist[b] = 0u;
   __syncthreads();
   // (the high half of a shared counter counts the references to quads of varying depth; a chunk
   // makes at most kChunkQuads of either per bin)
   static_assert(kChunkQuads < 65536, "chunk counters share a word");
-  for_each_ref<true>(ws, V, q0, q1, [&](long long, int b, int, int, uint2, uint32_t info) {
+  for_each_ref<true>(ws, V, q0, q1, large, [&](long long, int b, int, int, uint2, uint32_t info) {
     if (smem) atomicAdd(&hist[b], (info & kInfoFlatDepth) ? 1u : 0x10001u);
     else atomicAdd(&ws.bin_count[V.bin_base + b], 1u);
   });
@@ -285,13 +300,15 @@ __global__ __launch_bounds__(1024) void k_bin_scan(Ws ws) {
 __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_scatter(Ws ws) {
   pdl_begin();
   __shared__ uint32_t hist[kHistSmemBins];
+  __shared__ LargeList large;
   if (ws.ctrl->error == LR_ERR_OVERFLOW) return;
   const int v = view_of_chunk(ws.views, ws.n_views, blockIdx.x);
   const ViewDev& V = ws.views[v];
-  const long long q0 = V.quad_base + (long long)(blockIdx.x - V.chunk_base) * kChunkQuads;
-  const long long q1 = min(q0 + kChunkQuads, V.quad_base + V.num_quads);
+  const long long q0 = V.quad_base + (long long)(blockIdx.x - V.chunk_base) * ws.chunk_quads;
+  const long long q1 = min(q0 + ws.chunk_quads, V.quad_base + V.num_quads);
   const int nb = V.nbx * V.nby;
   const bool smem = nb <= kHistSmemBins;
+  if (threadIdx.x == 0) large.n = 0u;
   if (smem) {
     // the chunk's range in each bin it touches, reserved by k_bin_count
     const uint2 sp = ws.chunk_span[blockIdx.x];
@@ -300,9 +317,9 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_scatter(Ws w
       const uint2 e = list[i];
       hist[e.x] = ws.bin_off[V.bin_base + e.x] + e.y;
     }
-    __syncthreads();
   }
-  for_each_ref<false>(ws, V, q0, q1, [&](long long q, int b, int bx, int by, uint2 rect, uint32_t info) {
+  __syncthreads();
+  for_each_ref<false>(ws, V, q0, q1, large, [&](long long q, int b, int bx, int by, uint2 rect, uint32_t info) {
     const uint32_t slot = smem ? atomicAdd(&hist[b], 1u) : atomicAdd(&ws.bin_cursor[V.bin_base + b], 1u);
     const int lg = ws.bin_log2;
     const int x0 = max((int)(rect.x & 0xffff), bx << lg);

@@ -48,7 +48,16 @@ constexpr int kHistSmemBins = 8192;         // shared-memory bin counters per CT
 #ifndef LR_CHUNK_QUADS
 #define LR_CHUNK_QUADS 2048
 #endif
-constexpr int kChunkQuads = LR_CHUNK_QUADS;  // quads per binning CTA
+constexpr int kChunkQuads = LR_CHUNK_QUADS;  // quads per binning CTA, at most
+constexpr int kChunkQuadsMin = 256;
+// ... and of a render of `quads` quads: halved until there are two CTAs for each of the 152 SMs
+// (the count and the scatter are bound by latency, and 2048 quads each left most SMs idle below
+// 600,000 quads)
+__host__ __forceinline__ int chunk_quads_for(long long quads) {
+  int c = kChunkQuads;
+  while (c > kChunkQuadsMin && quads < 304LL * c) c >>= 1;
+  return c;
+}
 constexpr int kBinThreads = kChunkQuads / 4 < 1024 ? kChunkQuads / 4 : 1024;   // threads per binning CTA
 constexpr int kBinMinBlocks = kBinThreads >= 1024 ? 1 : (kBinThreads >= 512 ? 2 : 5);
 constexpr int kSmallBins = 4;               // AABB-counted up to kSmallBins x kSmallBins bins
@@ -94,7 +103,7 @@ struct ViewDev {
   int width, height;
   int nbx, nby;              // bins per row / column
   int bin_base;              // first bin of this view in the flattened bin space
-  int chunk_base;            // first binning chunk (kChunkQuads quads) of this view
+  int chunk_base;            // first binning chunk (Ws::chunk_quads quads) of this view
   int sub_x, sub_y;          // multisampling: the view's sample offset from the pixel centre
                              // (1/256 px), subtracted from the snapped vertices, so that the
                              // pixel-centre tests of every later stage test the sample
@@ -231,6 +240,7 @@ struct Ws {
   long long refs_cap;
   int cursors;               // a view has more bins than the shared counters hold
   int ticket;                // half-blocks per ticket of the rasteriser's queue: 1 or 2
+  int chunk_quads;           // quads per binning CTA (chunk_quads_for)
   int bin_log2;              // bins of 2^bin_log2 x 2^bin_log2 pixels (the same for every view)
   int4* rec;                 // [4 * total_quads]: the 64-byte quad record (QuadRec)
   uint2* rec_rect;           // [total_quads]: pixel AABB (px0 | px1 << 16, py0 | py1 << 16)

@@ -101,7 +101,8 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
   const size_t o_cnt = o; o = up256(o + 4 * (size_t)nbins);
   const size_t o_off = o; o = up256(o + 4 * ((size_t)nbins + 1));
   const size_t o_cur = o; o = up256(o + 4 * (size_t)nbins);
-  const size_t o_span = o; o = up256(o + 8 * (size_t)((Q + kChunkQuads - 1) / kChunkQuads));
+  const int chunk_quads = chunk_quads_for(Q), chunks = (int)((Q + chunk_quads - 1) / chunk_quads);
+  const size_t o_span = o; o = up256(o + 8 * (size_t)chunks);
   const size_t o_ord = o; o = up256(o + 4 * (size_t)nbins);
   const size_t o_ovf = o; o = up256(o + 4 * (size_t)npix);
   if (o >= (size_t)LR_NOALLOC_SCRATCH_BYTES) return LR_ERR_TOO_LARGE;
@@ -187,6 +188,7 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
   ws.total_quads = Q;
   ws.total_pix = npix;
   ws.refs_cap = cap;
+  ws.chunk_quads = chunk_quads;
   ws.bin_log2 = kBinLog2Default;
   ws.cursors = nbins > kHistSmemBins;
   ws.ticket = 1;
@@ -206,7 +208,6 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
 
   // ---- the pipeline, as lr_render launches it ------------------------------------------
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  const int chunks = (int)((Q + kChunkQuads - 1) / kChunkQuads);
   k_noalloc_view<<<1, 1, 0, st>>>(v, reinterpret_cast<ViewDev*>(base + o_view));
   ViewChunk no_views;
   memset(&no_views, 0, sizeof(no_views));
