@@ -206,11 +206,7 @@ static __device__ void composite_sorted(const Ws& ws, const ViewDev& V, const un
         da -= (gp->gr * (gp->fr - wr) + gp->gg * (gp->fg - wg) + gp->gb * (gp->fb - wb)) * inv;
         da += gp->ga * gp->fT * inv;
       }
-      float* gq = gp->grad + 4ull * j;
-      atomicAdd(gq + 0, gp->gr * w);
-      atomicAdd(gq + 1, gp->gg * w);
-      atomicAdd(gq + 2, gp->gb * w);
-      atomicAdd(gq + 3, da);
+      atomicAdd(reinterpret_cast<float4*>(gp->grad) + j, make_float4(gp->gr * w, gp->gg * w, gp->gb * w, da));
       wT *= om;
     }
   }
@@ -241,10 +237,7 @@ __device__ void overflow_pixel(const Ws& ws, long long pid, unsigned long long* 
   unsigned long long tau = kSent;   // exclusive upper bound of the fragments still to do
   GradPixel gp;
   if (BWD) {
-    const float4 gq = reinterpret_cast<const float4*>(ws.grad_out)[pidx];
-    const float4 fq = reinterpret_cast<const float4*>(ws.fwd)[pidx];
-    gp.gr = gq.x; gp.gg = gq.y; gp.gb = gq.z; gp.ga = gq.w;
-    gp.fr = fq.x; gp.fg = fq.y; gp.fb = fq.z; gp.fT = 1.0f - fq.w;
+    gp.load(ws.grad_out, ws.fwd, pidx);
     gp.grad = ws.grad_col;
   }
   for (;;) {

@@ -46,6 +46,8 @@
 
 #include "lr_common.cuh"
 
+#include <type_traits>
+
 namespace lr {
 
 // k_raster's batches: the edge values are kept in 64 bits
@@ -54,13 +56,12 @@ constexpr unsigned long long kSent = ~0ull;
 constexpr int kRasterThreads = 256;
 // Resident CTAs per SM requested from the compiler: 3 caps registers at 80 per thread (24 warps
 // per SM), 4 at 64. Neither spills in the forward kernels up to K = 3. With four the layer frame
-// took 307 instead of 315 us and the backward 438 instead of 475, flat layers at K = 3 154
-// instead of 168; with three the particle frame 275 instead of 309, the batch of mixed views at
+// took 307 instead of 315 us, flat layers at K = 3 154 instead of 168; with three the particle frame 275 instead of 309, the batch of mixed views at
 // K = 3 833 instead of 868, lit layers 406 instead of 422, flat layers with the alpha threshold
-// 217 instead of 225.
+// 217 instead of 225. The backward's shared memory holds three.
 __host__ __device__ constexpr int raster_min_blocks(int k, bool vtx, bool bwd, bool ath, bool lit) {
   if (lit || ath || k > 3) return 3;
-  if (bwd) return 4;
+  if (bwd) return 3;
   return vtx ? (k == 1 ? 4 : 3) : (k == 1 ? 3 : 4);
 }
 constexpr int kRasterWarps = kRasterThreads / 32;
@@ -79,12 +80,17 @@ constexpr float kKeyBoundScale = 1.0f + 1.0f / 65536.0f;
 //   dC/dc_i = T_i a_i,   dC/da_i = T_i c_i - S_i / (1 - a_i),   dA/da_i = T_final / (1 - a_i)
 // where S_i = C_final - (C accumulated through fragment i) is the colour contributed by the
 // fragments behind i. C_final, T_final come from the forward image; the running sums are
-// recomputed with the forward's operations in the forward's order.
+// recomputed in the forward's order.
 struct GradPixel {
   float gr, gg, gb, ga;      // dL/d(R, G, B, A) of the pixel
   float fr, fg, fb, fT;      // forward colour and transmittance
   float* grad;               // f32[Q][4] of the view
-  float4* agg;               // this warp's 32 shared-memory slots for combining lanes' gradients
+  __device__ __forceinline__ void load(const float* grad_out, const float* fwd, long long pidx) {
+    const float4 g = reinterpret_cast<const float4*>(grad_out)[pidx];
+    const float4 f = reinterpret_cast<const float4*>(fwd)[pidx];
+    gr = g.x; gg = g.y; gb = g.z; ga = g.w;
+    fr = f.x; fg = f.y; fb = f.z; fT = 1.0f - f.w;
+  }
 };
 
 // Columns lx in [0, 8) of one half-block row where an edge is non-negative, as an 8-bit
@@ -106,7 +112,7 @@ __device__ __forceinline__ uint32_t row_cover(int r, int sx) {
 // ATH: the alpha-threshold variant. Once the transmittance drops to kAlphaTMin nothing
 // more is blended and `last` stays at the key of the fragment that got it there, so the
 // misorder test below only flags fragments that belong in front of that one.
-template <int K, bool VTX, bool BWD = false, bool ATH = false>
+template <int K, bool VTX, bool ATH = false>
 struct PixelState {
   // K = 1 with flat colours gathered at blend time: the colour of the fragment held in the
   // slot is loaded when it enters, so the gather overlaps the next fragment's work
@@ -116,13 +122,12 @@ struct PixelState {
   unsigned long long last;
   float r, g, b, T;
   bool flagged;
-  GradPixel gp;
 
-  // K = 1, forward, colours carried: the empty slot holds a fully transparent colour, so
+  // K = 1, colours carried: the empty slot holds a fully transparent colour, so
   // blending it changes nothing (T and the colour stay, last is still kSent) and the in-order
   // insert needs no test for it (layer frame rasteriser 0.409 -> 0.394 ms; the same for the
   // flat colours gathered at blend time made the particle frame's 14% slower)
-  static constexpr bool kNullSlot = VTX && K == 1 && !BWD;
+  static constexpr bool kNullSlot = VTX && K == 1;
 
   __device__ __forceinline__ void init() {
 #pragma unroll
@@ -144,43 +149,14 @@ struct PixelState {
     r += w * col.x;
     g += w * col.y;
     b += w * col.z;
-    if (BWD && gp.grad) {
-      const float om = 1.0f - col.w;
-      float da = gp.gr * T * col.x + gp.gg * T * col.y + gp.gb * T * col.z;
-      if (om > 1e-6f) {
-        const float inv = rcp_approx(om);   // gradients need no correctly rounded divide
-        da -= (gp.gr * (gp.fr - r) + gp.gg * (gp.fg - g) + gp.gb * (gp.fb - b)) * inv;
-        da += gp.ga * gp.fT * inv;
-      }
-      // lanes blending a fragment of the same quad at this point add their contributions
-      // in shared memory first, and one of them issues the four global atomics
-      const int lane = threadIdx.x & 31;
-      const unsigned act = __activemask();
-      const unsigned grp = __match_any_sync(act, j);
-      gp.agg[lane] = make_float4(gp.gr * w, gp.gg * w, gp.gb * w, da);
-      __syncwarp(act);
-      if (lane == __ffs(grp) - 1) {
-        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (unsigned m = grp; m; m &= m - 1) {
-          const float4 c = gp.agg[__ffs(m) - 1];
-          sum.x += c.x; sum.y += c.y; sum.z += c.z; sum.w += c.w;
-        }
-        float* gq = gp.grad + 4ull * j;
-        atomicAdd(gq + 0, sum.x);
-        atomicAdd(gq + 1, sum.y);
-        atomicAdd(gq + 2, sum.z);
-        atomicAdd(gq + 3, sum.w);
-      }
-      __syncwarp(act);
-    }
     // T (1 - a) as one fused T - T a (a rounding, not the product's two, away from it: well
     // inside the colour tolerance); the threshold variant, whose T decides which fragments
-    // blend, and the backward keep the product
-    if (ATH || BWD) T *= 1.0f - col.w;
+    // blend, keeps the product
+    if (ATH) T *= 1.0f - col.w;
     else T = __fmaf_rn(-T, col.w, T);
   }
 
-  // forward blend of a fragment known to be next in order, without the sorter
+  // blend of a fragment known to be next in order, without the sorter
   __device__ __forceinline__ void blend_direct(float4 col) {
     const float w = T * col.w;
     r += w * col.x;
@@ -191,11 +167,11 @@ struct PixelState {
   }
 
   __device__ __forceinline__ void insert(unsigned long long x, float4 xc, const ViewDev& V) {
-    // nearer than a fragment already blended: order not guaranteed. The forward pass with
-    // carried colours only records it (the pixel's composite is discarded, so inserting the
+    // nearer than a fragment already blended: order not guaranteed. With carried colours this
+    // only records it (the pixel's composite is discarded, so inserting the
     // fragment anyway is harmless; measured faster than the branch there, slower for the
     // colours gathered at blend time)
-    if (VTX && !BWD) {
+    if (VTX) {
       flagged |= x > last;
     } else if (x > last) {
       flagged = true;
@@ -214,14 +190,14 @@ struct PixelState {
       c[0] = nearer ? c[0] : xc;
       return;
     }
-    if (VTX && K == 1) {       // one slot (threshold, backward): a branch
+    if (VTX && K == 1) {       // one slot (threshold): a branch
       if (x > s[0]) {          // nearer than the held fragment: blend it at once
         if (live()) {
           blend(x, xc, V);
           last = x;
         }
       } else {
-        if ((kNullSlot || s[0] != kSent) && live()) {
+        if (live()) {   // (the empty slot is transparent)
           blend(s[0], c[0], V);
           last = s[0];
         }
@@ -279,6 +255,140 @@ struct PixelState {
       if (s[i] != kSent && live()) blend(s[i], VTX || kPrefetch ? c[i] : make_float4(0.f, 0.f, 0.f, 0.f), V);
   }
 };
+
+// Backward: one pixel. The sorter's slots hold keys and the fragment's slot in the current batch
+// (kOldSlot: it came with an earlier one). What a blended fragment contributes to its quad's
+// gradient is, with the pixel's g = dL/d(R, G, B), two numbers times quantities of the quad or of
+// the pixel alone: the transmittance T in front of it (dL/dc = a T g) and the rest
+// S = g . (C_final - C through it) - ga T_final (dL/da = T g . c - S / (1 - a)). The warp's pixels
+// record them per batch in shared memory, rank of the fragment in its pixel by pixel, and
+// batch_gradients sums them with one lane per triangle and one vector atomic each. Only fragments
+// blended after their batch (the K last of it) or beyond kGradRanks of a pixel are added one by
+// one. 25M fragments at 1024x1024, K = 1: 435 us and 384M warp instructions when each blended
+// fragment searched the warp for lanes with the same quad and issued four atomics per group;
+// 289 us and 215M so.
+constexpr uint32_t kOldSlot = 32u;
+constexpr int kGradRanks = 12;     // (eight fragments per pixel and batch are ordinary)
+struct GradShared {
+  float4 g[32];                    // per pixel: dL/d(R, G, B), its batch coverage (bits)
+  float4 agg[32];                  // combines lanes' gradients of late fragments
+  float2 ts[kGradRanks][32];       // (T, S) by rank and pixel
+};
+template <int K>
+struct GradState {
+  unsigned long long s[K], last;
+  uint32_t sl[K];
+  float T, r, g, b;                // running transmittance and colour
+  GradPixel gp;
+  uint32_t cover, done;            // the pixel's batch mask and the slots recorded
+  bool flagged;
+
+  __device__ __forceinline__ void init() {
+#pragma unroll
+    for (int i = 0; i < K; ++i) { s[i] = kSent; sl[i] = kOldSlot; }
+    last = kSent;
+    T = 1.f;
+    r = g = b = 0.f;
+    cover = done = 0;
+    flagged = false;
+  }
+
+  __device__ __forceinline__ void blend(unsigned long long key, uint32_t slot, const ViewDev& V, const float4* qc,
+                                        GradShared& G) {
+    const uint32_t j = (uint32_t)key >> 1;
+    float4 c;
+    if (slot < kOldSlot) c = qc[slot];
+    else c = __ldg(reinterpret_cast<const float4*>(V.col) + j);
+    const int lane = threadIdx.x & 31;
+    const float w = T * c.w;
+    r += w * c.x;
+    g += w * c.y;
+    b += w * c.z;
+    const float S = gp.gr * (gp.fr - r) + gp.gg * (gp.fg - g) + gp.gb * (gp.fb - b) - gp.ga * gp.fT;
+    const int rank = __popc((cover >> (slot & 31u)) >> 1);
+    if (slot < kOldSlot && rank < kGradRanks) {
+      G.ts[rank][lane] = make_float2(T, S);
+      done |= 1u << slot;
+    } else {
+      const float om = 1.0f - c.w;
+      const float da = T * (gp.gr * c.x + gp.gg * c.y + gp.gb * c.z) - (om > 1e-6f ? S * rcp_approx(om) : 0.f);
+      // lanes blending a fragment of the same quad at this point add their contributions
+      // in shared memory first, and one of them issues the global atomic
+      const unsigned act = __activemask();
+      const unsigned grp = __match_any_sync(act, j);
+      G.agg[lane] = make_float4(gp.gr * w, gp.gg * w, gp.gb * w, da);
+      __syncwarp(act);
+      if (lane == __ffs(grp) - 1) {
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (unsigned m = grp; m; m &= m - 1) {
+          const float4 x = G.agg[__ffs(m) - 1];
+          sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
+        }
+        atomicAdd(reinterpret_cast<float4*>(gp.grad) + j, sum);
+      }
+      __syncwarp(act);
+    }
+    T *= 1.0f - c.w;
+  }
+
+  // without a gradient (gp.grad null) the order is tested, nothing is blended
+  __device__ __forceinline__ void insert(unsigned long long x, uint32_t slot, const ViewDev& V, const float4* qc,
+                                         GradShared& G) {
+    // nearer than a fragment already blended: order not guaranteed, and the gradient is left to
+    // the exact path
+    if (x > last) {
+      flagged = true;
+      return;
+    }
+    const bool xfirst = x > s[0];
+    const unsigned long long ev = xfirst ? x : s[0], y = xfirst ? s[0] : x;
+    const uint32_t evs = xfirst ? slot : sl[0], ys = xfirst ? sl[0] : slot;
+    // new slots = {s[1..K-1], y} in decreasing order
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      const bool take_next = (i + 1 < K) && (s[i + 1 < K ? i + 1 : i] > y);
+      const bool take_y = (i == 0) || (s[i] > y);
+      const unsigned long long nxt = s[i + 1 < K ? i + 1 : i];
+      const uint32_t nsl = sl[i + 1 < K ? i + 1 : i];
+      sl[i] = take_next ? nsl : (take_y ? ys : sl[i]);
+      s[i] = take_next ? nxt : (take_y ? y : s[i]);
+    }
+    if (ev != kSent) {
+      if (gp.grad) blend(ev, evs, V, qc, G);
+      last = ev;
+    }
+  }
+
+  __device__ __forceinline__ void flush(const ViewDev& V, const float4* qc, GradShared& G) {
+#pragma unroll
+    for (int i = 0; i < K; ++i)
+      if (s[i] != kSent) blend(s[i], sl[i], V, qc, G);
+  }
+};
+
+// Adds what the warp's pixels recorded for the batch: lane = slot, the triangle of quad j.
+__device__ __forceinline__ void batch_gradients(uint32_t done, uint32_t j, float* grad, const float4* qc,
+                                                const GradShared& G) {
+  const int lane = threadIdx.x & 31;
+  uint32_t m = warp_transpose32(done, lane);   // (its shuffles precede the reads below)
+  __syncwarp();
+  if (!m) return;
+  float r = 0.f, g = 0.f, b = 0.f, s = 0.f;
+  while (m) {
+    const int px = __ffs(m) - 1;
+    m &= m - 1;
+    const float4 p = G.g[px];
+    const float2 ts = G.ts[__popc((__float_as_uint(p.w) >> lane) >> 1)][px];
+    r += ts.x * p.x;
+    g += ts.x * p.y;
+    b += ts.x * p.z;
+    s += ts.y;
+  }
+  const float4 c = qc[lane];
+  const float om = 1.0f - c.w;
+  const float da = r * c.x + g * c.y + b * c.z - (om > 1e-6f ? s * rcp_approx(om) : 0.f);
+  atomicAdd(reinterpret_cast<float4*>(grad) + j, make_float4(r * c.w, g * c.w, b * c.w, da));
+}
 
 __device__ __forceinline__ void write_pixel(const ViewDev& V, long long pidx, float r, float g, float b,
                                             float T) {
@@ -449,7 +559,9 @@ __device__ __forceinline__ uint32_t byte_span(int a, int b) {
 // Per warp: the candidates of a 1024-reference window, a ring of covering triangles waiting for
 // a batch, and the records of the batch the fragment loop reads, one 16-byte array per field so that a slot's fields lie at one address
 // plus constants and eight neighbouring slots never share a bank.
-constexpr int kWinRefs = 1024;     // references per bitmap window (a word per lane)
+// references per bitmap window (a word per lane; half of them in the backward, whose shared memory
+// leaves room for three CTAs then)
+__host__ __device__ constexpr int win_refs(bool bwd) { return bwd ? 512 : 1024; }
 constexpr int kPendCap = 128;      // at most 31 left over + 64 pushed per candidate round
 constexpr uint32_t kPendConst = 0x80000000u;   // pending id: flat colour and constant depth
 struct BatchGeo {
@@ -461,8 +573,8 @@ struct BatchGeo {
 };
 __host__ __device__ constexpr int batch_cols(bool vtx, bool lit) { return vtx ? (lit ? 6 : 3) : 1; }
 __host__ __device__ constexpr size_t batch_smem_warp(bool vtx, bool bwd, bool lit) {
-  return kWinRefs * sizeof(uint16_t) + kPendCap * sizeof(uint2) + sizeof(BatchGeo) + (size_t)batch_cols(vtx, lit) * 32 * sizeof(float4) +
-         (bwd ? 32 * sizeof(float4) : 0);
+  return win_refs(bwd) * sizeof(uint16_t) + kPendCap * sizeof(uint2) + sizeof(BatchGeo) +
+         (size_t)batch_cols(vtx, lit) * 32 * sizeof(float4) + (bwd ? sizeof(GradShared) : 0);
 }
 __host__ __device__ constexpr size_t raster_smem_bytes(bool vtx, bool bwd = false, bool lit = false) {
   return (size_t)kRasterWarps * batch_smem_warp(vtx, bwd, lit);
@@ -589,7 +701,7 @@ __device__ __forceinline__ unsigned const_block(const Ws& ws, const ViewDev& V, 
   const float4* colors = reinterpret_cast<const float4*>(V.col);
   const uint32_t quad_base = (uint32_t)V.quad_base;
   uint32_t* pend_j = reinterpret_cast<uint32_t*>(qc + 32);   // the ring's quads; pend: their masks
-  PixelState<1, true, false, ATH> sa, sb;
+  PixelState<1, true, ATH> sa, sb;
   sa.init();
   sb.init();
   uint32_t cnt_a = 0, cnt_b = 0;
@@ -703,15 +815,17 @@ template <int K, bool VTX, bool BWD, bool HASH, bool ATH = false, bool LIT = fal
 __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH, LIT)) void k_raster(Ws ws) {
   pdl_begin();
   extern __shared__ __align__(16) unsigned char smem[];
-  constexpr bool kCarry = VTX || K == 1;   // the sorter carries each fragment's colour
+  // the sorter carries each fragment's colour (backward: the batch holds its triangles' colours)
+  constexpr bool kCarry = VTX || K == 1 || BWD;
+  constexpr int kWin = win_refs(BWD);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lx = lane & (kHbW - 1), ly = lane >> 3;
   unsigned char* wbase = smem + (size_t)warp * batch_smem_warp(VTX, BWD, LIT);
   uint16_t* cand = reinterpret_cast<uint16_t*>(wbase);
-  uint2* pend = reinterpret_cast<uint2*>(wbase + kWinRefs * sizeof(uint16_t));
+  uint2* pend = reinterpret_cast<uint2*>(wbase + kWin * sizeof(uint16_t));
   BatchGeo& geo = *reinterpret_cast<BatchGeo*>(pend + kPendCap);
   float4* qc = reinterpret_cast<float4*>(&geo + 1);
-  float4* agg = qc + batch_cols(VTX, LIT) * 32;
+  GradShared& gs = *reinterpret_cast<GradShared*>(qc + batch_cols(VTX, LIT) * 32);   // (backward)
   // a batch blended in stream order keeps its sort keys (alpha threshold) or ids where the
   // others keep ea
   unsigned long long* dkey = reinterpret_cast<unsigned long long*>(&geo);
@@ -757,16 +871,12 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
     const float4 light = LIT ? make_float4(V.light[0], V.light[1], V.light[2], V.light[3])
                              : make_float4(0.f, 0.f, 0.f, 0.f);
 
-    PixelState<K, kCarry, BWD, ATH> st;
-    st.init();
-    st.gp.grad = nullptr;
-    st.gp.agg = agg;
-    if (BWD && pix_ok) {
-      const long long pidx = (long long)py * V.width + px;
-      const float4 gq = reinterpret_cast<const float4*>(ws.grad_out)[pidx];
-      const float4 fq = reinterpret_cast<const float4*>(ws.fwd)[pidx];
-      st.gp.gr = gq.x; st.gp.gg = gq.y; st.gp.gb = gq.z; st.gp.ga = gq.w;
-      st.gp.fr = fq.x; st.gp.fg = fq.y; st.gp.fb = fq.z; st.gp.fT = 1.0f - fq.w;
+    typename std::conditional<BWD, GradState<K>, PixelState<K, kCarry, ATH>>::type st;
+    if constexpr (BWD) {
+      st.gp = GradPixel();
+      if (pix_ok) st.gp.load(ws.grad_out, ws.fwd, (long long)py * V.width + px);
+    } else {
+      st.init();
     }
     uint32_t cnt = 0;
     unsigned long long hsh = 0;
@@ -784,10 +894,11 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
       first_pass = 1;
     }
     for (int pass = first_pass; pass < 2; ++pass) {
-    if (BWD) {
+    if constexpr (BWD) {
       st.init();
       st.flagged = pre_flagged;
-      st.gp.grad = (pass == 1 && pix_ok) ? ws.grad_col : nullptr;
+      st.gp.grad = pass == 1 ? ws.grad_col : nullptr;
+      gs.g[lane] = make_float4(st.gp.gr, st.gp.gg, st.gp.gb, 0.f);
       cnt = 0;
       hsh = 0;
     }
@@ -795,7 +906,7 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
     const uint32_t* row = hb_row(ws, off, bin_g, n, hb);
     const int nw = (n + 31) >> 5;
     const uint32_t* ref_lo = reinterpret_cast<const uint32_t*>(ws.refs + off);   // low words
-    int g = -32, r0 = 0, total = 0;   // bitmap window, position in it, its candidates
+    int g = -kWin / 32, r0 = 0, total = 0;   // bitmap window, position in it, its candidates
     int head = 0, tail = 0;       // pending ring
     bool ordered = !HASH && !BWD; // everything so far was blended in stream order
     uint32_t last_id = 0xFFFFFFFFu;   // ... the last fragment's id
@@ -803,9 +914,9 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
       // ---- 2. coverage masks of 32 candidates, one quad per lane, until a batch is full ---
       while (tail - head < 32) {
         if (r0 >= total) {
-          g += 32;
+          g += kWin / 32;
           if (g >= nw) break;
-          total = list_bits(g + lane < nw ? __ldg(row + g + lane) : 0u, lane, cand);
+          total = list_bits(lane < kWin / 32 && g + lane < nw ? __ldg(row + g + lane) : 0u, lane, cand);
           r0 = 0;
           continue;
         }
@@ -813,7 +924,7 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
         const uint32_t rec = in ? ~ref_lo[2 * (32 * g + (int)cand[r0 + lane])] : 0u;
         r0 += 32;
         bool skip = !in;
-        if (ATH) {
+        if constexpr (ATH) {
           // The smallest key a fragment must exceed to change any pixel of the half-block:
           // 0 while a pixel still blends; a finished pixel needs a fragment in front of the
           // one that finished it (keys are positive floats, so their bits order like them);
@@ -900,66 +1011,83 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
       __syncwarp();
       if (!pix_ok) m = 0;
       cnt += __popc(m);
-      if (direct) {
-        // ---- 5a. flat colours at constant depths, everything before them likewise: the
-        // stream order is the fragments' exact order (the bin sort's key is the depth key), so
-        // they blend as they come, without the sorter
-        const uint32_t all = m;
-        uint32_t lastp = 32;
-        while (m) {
-          if (ATH && !st.live()) break;
-          const int p = 31 - __clz(m);
-          m ^= 1u << p;
-          const float4 c = qc[p];
-          if (ATH) lastp = (uint32_t)p;
-          st.blend_direct(c);
+      if constexpr (!BWD) {
+        if (direct) {
+          // ---- 5a. flat colours at constant depths, everything before them likewise: the
+          // stream order is the fragments' exact order (the bin sort's key is the depth key), so
+          // they blend as they come, without the sorter
+          const uint32_t all = m;
+          uint32_t lastp = 32;
+          while (m) {
+            if (ATH && !st.live()) break;
+            const int p = 31 - __clz(m);
+            m ^= 1u << p;
+            const float4 c = qc[p];
+            if (ATH) lastp = (uint32_t)p;
+            st.blend_direct(c);
+          }
+          if (!ATH) lastp = (uint32_t)(__ffs(all) - 1);
+          if (ATH) { if (lastp < 32u) st.last = dkey[lastp]; }
+          else if (lastp < 32u) last_id = did[lastp];
+          __syncwarp();
+          continue;
         }
-        if (!ATH) lastp = (uint32_t)(__ffs(all) - 1);
-        if (ATH) { if (lastp < 32u) st.last = dkey[lastp]; }
-        else if (lastp < 32u) last_id = did[lastp];
-      } else {
         if (ordered) {
           if (!ATH && last_id != 0xFFFFFFFFu) st.last = const_key(ws, V, last_id);
           // the sorter starts here; with a transparent held fragment at the last key blended
           // (K = 1), so that its first eviction keeps that key
           ordered = false;
-          if (PixelState<K, kCarry, BWD, ATH>::kNullSlot) st.s[0] = st.last;
+          if (PixelState<K, kCarry, ATH>::kNullSlot) st.s[0] = st.last;
         }
-        // ---- 5b. fragments in candidate order through the K-slot sorter -------------------
-        auto frag_step = [&]() {
-          const int p = 31 - __clz(m);
-          m ^= 1u << p;
-          const int4 eb = geo.eb[p];
-          const uint32_t fid = (uint32_t)eb.w;
-          if (hashing) hsh += splitmix64(fid);
-          // (the forward discards a flagged pixel's composite, the exact path redoing it, so it
-          // keeps inserting rather than testing the flag per fragment; the backward must not
-          // add a flagged pixel's gradient)
-          if (!BWD || !st.flagged) {
-            const int4 ea = geo.ea[p];
-            const float4 kq = geo.kq[p];
-            float f1, f2;
-            if (!((uint32_t)eb.z & kTriWide)) {
-              f1 = __int2float_rn((int)((uint32_t)ea.x + (uint32_t)lx * (uint32_t)ea.z + (uint32_t)ly * (uint32_t)eb.x));
-              f2 = __int2float_rn((int)((uint32_t)ea.y + (uint32_t)lx * (uint32_t)ea.w + (uint32_t)ly * (uint32_t)eb.y));
-            } else {
-              const int2 h = geo.hi[p];
-              const long long e1 = ((long long)h.x << 32) | (uint32_t)ea.x, e2 = ((long long)h.y << 32) | (uint32_t)ea.y;
-              f1 = __ll2float_rn(e1 + 256LL * (lx * ea.z + ly * eb.x));
-              f2 = __ll2float_rn(e2 + 256LL * (lx * ea.w + ly * eb.y));
-            }
-            // exact depth key: the interpolated 1/w (Sec. 2 "Stage 3", the reading O.8)
-            const float l1 = __fmul_rn(f1, kq.w), l2 = __fmul_rn(f2, kq.w);
-            const float key = __fadd_rn(kq.x, __fadd_rn(__fmul_rn(l1, kq.y), __fmul_rn(l2, kq.z)));
-            const unsigned long long sk = ((unsigned long long)__float_as_uint(key) << 32) | fid;
+      } else {
+        st.cover = m;
+        st.done = 0u;
+        gs.g[lane].w = __uint_as_float(m);
+      }
+      // ---- 5b. fragments in candidate order through the K-slot sorter -------------------
+      auto frag_step = [&]() {
+        const int p = 31 - __clz(m);
+        m ^= 1u << p;
+        const int4 eb = geo.eb[p];
+        const uint32_t fid = (uint32_t)eb.w;
+        if (hashing) hsh += splitmix64(fid);
+        // (the forward discards a flagged pixel's composite, the exact path redoing it, so it
+        // keeps inserting rather than testing the flag per fragment; the backward must not
+        // add a flagged pixel's gradient)
+        if (!BWD || !st.flagged) {
+          const int4 ea = geo.ea[p];
+          const float4 kq = geo.kq[p];
+          float f1, f2;
+          if (!((uint32_t)eb.z & kTriWide)) {
+            f1 = __int2float_rn((int)((uint32_t)ea.x + (uint32_t)lx * (uint32_t)ea.z + (uint32_t)ly * (uint32_t)eb.x));
+            f2 = __int2float_rn((int)((uint32_t)ea.y + (uint32_t)lx * (uint32_t)ea.w + (uint32_t)ly * (uint32_t)eb.y));
+          } else {
+            const int2 h = geo.hi[p];
+            const long long e1 = ((long long)h.x << 32) | (uint32_t)ea.x, e2 = ((long long)h.y << 32) | (uint32_t)ea.y;
+            f1 = __ll2float_rn(e1 + 256LL * (lx * ea.z + ly * eb.x));
+            f2 = __ll2float_rn(e2 + 256LL * (lx * ea.w + ly * eb.y));
+          }
+          // exact depth key: the interpolated 1/w (Sec. 2 "Stage 3", the reading O.8)
+          const float l1 = __fmul_rn(f1, kq.w), l2 = __fmul_rn(f2, kq.w);
+          const float key = __fadd_rn(kq.x, __fadd_rn(__fmul_rn(l1, kq.y), __fmul_rn(l2, kq.z)));
+          const unsigned long long sk = ((unsigned long long)__float_as_uint(key) << 32) | fid;
+          if constexpr (BWD) {
+            st.insert(sk, (uint32_t)p, V, qc, gs);
+          } else {
             float4 col = make_float4(0.f, 0.f, 0.f, 0.f);
             if (kCarry) col = shade<VTX, LIT>(qc, p, flat_view, lit_view, light, l1, l2, key);
             st.insert(sk, col, V);
           }
-        };
-        while (m) frag_step();
-      }
+        }
+      };
+      while (m) frag_step();
       __syncwarp();
+      if constexpr (BWD) {
+        if (st.gp.grad) batch_gradients(st.done, id >> 1, st.gp.grad, qc, gs);
+#pragma unroll
+        for (int i = 0; i < K; ++i) st.sl[i] = kOldSlot;
+        __syncwarp();
+      }
     }
     if (pass == 0) pre_flagged = st.flagged;
     }
@@ -974,13 +1102,16 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
         V.xmask[((uint32_t)oy / kHbH) * hbw + (uint32_t)ox / kHbW] = fm;
       }
     }
-    if (!st.flagged) st.flush(V);
+    if (!st.flagged) {
+      if constexpr (BWD) st.flush(V, qc, gs);
+      else st.flush(V);
+    }
     if (pix_ok) {
       const long long pidx = (long long)py * V.width + px;
       if (!BWD && V.cnt) V.cnt[pidx] = cnt;
       if (!BWD && hashing) V.hash[pidx] = hsh;
       if (!st.flagged) {
-        if (!BWD) write_pixel(V, pidx, st.r, st.g, st.b, st.T);
+        if constexpr (!BWD) write_pixel(V, pidx, st.r, st.g, st.b, st.T);
       } else {
         const unsigned long long slot = atomicAdd(&ws.ctrl->ovf_count, 1ull);
         ws.ovf_list[slot] = (uint32_t)(V.pix_base + pidx);

@@ -176,7 +176,6 @@ __global__ __launch_bounds__(kRasterThreads, 3) void k_raster_strip(Ws ws) {
 
     PixelState<K, VTX> st;
     st.init();
-    st.gp.grad = nullptr;
     uint32_t cnt = 0;
     unsigned long long hsh = 0;
 

@@ -26,7 +26,7 @@ def test_large_quads(lr, n, box):
     xy = rng.uniform(0, [w, h], (n, 1, 2)) + rng.uniform(0, 6, (n, 4, 2))
     # m of them span up to box px: random (convex, concave, crossed), and exact rectangles
     big = rng.choice(n, m, replace=False)
-    o = rng.uniform(-20, [w - box[0] + 20, h - box[1] + 20], (m, 1, 2))
+    o = rng.uniform(-100, [w - box[0] + 100, h - box[1] + 100], (m, 1, 2))
     xy[big] = o + rng.uniform(0, 1, (m, 4, 2)) * box
     rect = np.array([[0, 0], [1, 0], [1, 1], [0, 1]]) * np.array(box)
     xy[big[::3]] = np.floor(o[::3] / 32) * 32 + rect

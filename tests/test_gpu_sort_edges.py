@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from tests.scene_helpers import rects_scene
-from tests.test_gpu_sort import _bin_lists, _check, _particles_in_one_bin
+from tests.test_gpu_sort import _bin_lists, _check
 
 pytestmark = pytest.mark.gpu
 
@@ -22,7 +22,12 @@ def lr():
 @pytest.mark.parametrize("n", [1, 31, 32, 33, 255, 256, 257, 511, 512, 513, 768, 769, 1024, 1025, 2046, 2047, 2048,
                                2049, 20479, 20480, 20481])
 def test_list_length(lr, n):
-    s = _particles_in_one_bin(n, seed=60 + n % 13)
+    # squares inside the image at distinct depths
+    rng = np.random.default_rng(n)
+    xy = rng.uniform(2, 20, (n, 2))
+    rects = [(float(x), float(y), float(x + 3.0), float(y + 2.0)) for x, y in xy]
+    s = rects_scene(rects, width=32, height=32, depths=rng.uniform(1.0, 2.0, n),
+                    colors=np.concatenate([rng.random((n, 3)), np.full((n, 1), 0.05)], 1))
     st, bin_off, refs, rect = _bin_lists(lr, s)
     lens = _check(s, st, bin_off, refs, rect)
     assert lens.sum() == n
