@@ -8,6 +8,7 @@
 //   k_bin_scan     Stage 2, Phase 2
 //   k_bin_scatter  Stage 2, Phase 3
 //   k_bin_sort     Stage 3, Phase 2's depth sort of each bin's references (stage 1 of 2)
+//   k_raster_ordered  Stage 3 of the bins whose list is in every pixel's order (flat views)
 //   k_raster       Stage 3: coverage, per-pixel sorter (stage 2 of 2), blending
 //   k_overflow     exact full sort of the pixels the sorter flagged
 //
@@ -32,6 +33,8 @@ __global__ void k_bin_count(Ws ws);
 __global__ void k_bin_scan(Ws ws);
 __global__ void k_bin_scatter(Ws ws);
 __global__ void k_bin_sort(Ws ws);
+cudaError_t prepare_ordered(int* blocks_per_sm);
+cudaError_t launch_ordered(const Ws& ws, int grid, cudaStream_t st, bool pdl);
 cudaError_t overflow_occupancy(int* blocks_per_sm);
 cudaError_t launch_overflow(bool bwd, const Ws& ws, int grid, cudaStream_t st, bool pdl);
 
@@ -171,7 +174,6 @@ static Ws make_ws(const Layout& L, void* base, int n_views) {
   w.bin_log2 = L.bin_log2;
   w.cursors = L.cursors;
   w.chunk_quads = L.chunk_quads;
-  w.ticket = 1;
   w.rec = reinterpret_cast<int4*>(b + L.rec);
   w.rec_rect = reinterpret_cast<uint2*>(b + L.rec_rect);
   w.rec_info = reinterpret_cast<uint32_t*>(b + L.rec_info);
@@ -210,6 +212,7 @@ struct lr_ctx {
   int bin_log2 = kBinLog2Default;   // from cfg.bin_size
   float light[4] = {0.f, 0.f, 1.f, 0.25f};   // LR_COLOR_LIT: unit direction toward the light, ambient
   int ovf_blocks = 1;
+  int ordered_blocks = 1;
   // last render, for lr_get_stats
   cudaStream_t last_stream = nullptr;
   void* last_ws = nullptr;
@@ -287,6 +290,7 @@ extern "C" lr_status lr_create(const lr_config* config, lr_ctx** out_ctx) {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_bin_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)kSortSmemBytes);
   if (e == cudaSuccess) e = overflow_occupancy(&c->ovf_blocks);
+  if (e == cudaSuccess) e = prepare_ordered(&c->ordered_blocks);
   if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void**>(&c->host_ctrl), sizeof(Ctrl));
   for (int i = 0; i < 9 && e == cudaSuccess; ++i) e = cudaEventCreate(&c->ev[i]);
   if (e != cudaSuccess) {
@@ -295,6 +299,8 @@ extern "C" lr_status lr_create(const lr_config* config, lr_ctx** out_ctx) {
     return s;
   }
   c->ovf_blocks = std::max(c->ovf_blocks, 1);
+  if (g.raster_ctas_per_sm > 0) c->ordered_blocks = std::min(c->ordered_blocks, g.raster_ctas_per_sm);
+  c->ordered_blocks = std::max(c->ordered_blocks, 1);
   *out_ctx = c;
   return LR_OK;
 }
@@ -543,8 +549,23 @@ static lr_status launch_sequence(lr_ctx* ctx, const Prepared& P, cudaStream_t st
     ws.grad_col = bwd->grad_colors;
     ws.bwd_mask = bwd->exact_mask;
   }
+  const bool carry = P.any_vertex || P.any_lit || (ctx->cfg.flags & LR_FLAG_CARRY_COLORS);
+  const bool ath = !bwd && (ctx->cfg.flags & LR_FLAG_ALPHA_THRESHOLD);   // no hash then (prepare)
+  // (lit views: neither hash nor threshold, see prepare)
+  const int mode = bwd ? 2 : (P.any_lit ? 17 : ((carry ? 1 : 0) | (P.any_hash ? 4 : 0) | (ath ? 8 : 0)));
+  ws.t_min = ath ? kAlphaTMin : 0.0f;
+  const VariantState& VS = ctx->vs[P.variant];
+  // the strip kernel (32-pixel bins) for forward exact renders of flat or carried colours, when
+  // asked for and built
+  const bool strip = ctx->cfg.shared_setup && VS.v->launch_strip && !bwd && !ath && !P.any_lit &&
+                     ctx->bin_log2 == kBinLog2Default;
+  long long flat_bins = 0;   // bins that k_raster_ordered may get
+  for (const ViewDev& v : P.vd)
+    if (v.color_mode == LR_COLOR_FLAT) flat_bins += (long long)v.nbx * v.nby;
+  ws.ordered = flat_bins > 0 && !bwd && !P.any_hash && !strip && !L.cursors;
   const int n_views = ws.n_views;
   const bool pdl = ctx->pdl_override >= 0 ? ctx->pdl_override != 0 : (ctx->cfg.flags & LR_FLAG_NO_PDL) == 0;
+  if (ws.ordered && pdl) ws.ordered = kOrderedOverlap;
   rec(ctx, timed, 0, st);
   // the first kViewsPerLaunch descriptors travel with k_init, further ones with k_write_views
   ViewChunk chunk;
@@ -576,26 +597,16 @@ static lr_status launch_sequence(lr_ctx* ctx, const Prepared& P, cudaStream_t st
   rec(ctx, timed, 4, st);
   launch_pdl(pdl, k_bin_sort, dim3(ctx->sms), dim3(kSortThreads), kSortSmemBytes, st, ws);
   rec(ctx, timed, 5, st);
-  const bool carry = P.any_vertex || P.any_lit || (ctx->cfg.flags & LR_FLAG_CARRY_COLORS);
-  const bool ath = !bwd && (ctx->cfg.flags & LR_FLAG_ALPHA_THRESHOLD);   // no hash then (prepare)
-  // (lit views: neither hash nor threshold, see prepare)
-  const int mode = bwd ? 2 : (P.any_lit ? 17 : ((carry ? 1 : 0) | (P.any_hash ? 4 : 0) | (ath ? 8 : 0)));
-  ws.t_min = ath ? kAlphaTMin : 0.0f;
-  const VariantState& VS = ctx->vs[P.variant];
-  // the strip kernel (32-pixel bins) for forward exact renders of flat or carried colours, when
-  // asked for and built
-  const bool strip = ctx->cfg.shared_setup && VS.v->launch_strip && !bwd && !ath && !P.any_lit &&
-                     ctx->bin_log2 == kBinLog2Default;
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
+  // (a CTA for every eight 16x8 blocks, a bin of 32 pixels, at most)
+  if (ws.ordered)
+    e = launch_ordered(ws, (int)std::min((long long)ctx->sms * ctx->ordered_blocks, flat_bins << std::max(0, 2 * (ctx->bin_log2 - 5))),
+                       st, pdl);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "raster launch");
   if (strip) {
     e = VS.v->launch_strip(mode, ws, ctx->sms * (carry ? VS.vtx_s : VS.flat_s), st);
   } else {
     const int rblocks = bwd ? VS.bwd : (P.any_lit ? VS.lit : (carry ? VS.vtx : VS.flat));
-    // two half-blocks per ticket once every warp gets at least four tickets: a bin blended in
-    // list order needs only one of the two (300k particles at 2560x1440: 106 -> 86 us); with
-    // fewer the queue's tail costs more (four 512x384 views, 35 -> 49 us)
-    const long long warps = (long long)ctx->sms * rblocks * kRasterWarps;
-    if ((long long)L.total_bins * bin_hb(ctx->bin_log2) >= 8 * warps) ws.ticket = 2;
     e = VS.v->launch(mode, ws, ctx->sms * rblocks, st);
   }
   if (e != cudaSuccess) return cuda_fail(ctx, e, "raster launch");

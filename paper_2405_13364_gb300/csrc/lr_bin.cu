@@ -10,7 +10,7 @@
 //                  large quad's bins.
 //   k_bin_scan     Phase 2: exclusive scan of the counts into list offsets, capacity
 //                  check, and a categorisation of bins by size (the paper's empty / low /
-//                  high) that orders the rasteriser's work queue, largest bins first.
+//                  high) that orders the rasterisers' work queues, largest bins first.
 //   k_bin_scatter  Phase 3: places the chunk's references, each (chunk, bin) in the range
 //                  k_bin_count reserved for it (k_bin_count's global atomic returns the
 //                  range's base, listed per chunk), slots by shared-memory atomics. A
@@ -157,6 +157,7 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_count(Ws ws)
   pdl_begin();
   __shared__ uint32_t hist[kHistSmemBins];
   __shared__ LargeList large;
+  __shared__ uint32_t flags[2][kHistSmemBins / 32];   // bins the chunk marks kBinDepths, kBinShapes
   const int v = view_of_chunk(ws.views, ws.n_views, blockIdx.x);
   const ViewDev& V = ws.views[v];
   const long long q0 = V.quad_base + (long long)(blockIdx.x - V.chunk_base) * ws.chunk_quads;
@@ -165,14 +166,22 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_count(Ws ws)
   const bool smem = nb <= kHistSmemBins;
   if (threadIdx.x == 0) large.n = 0u;
   if (smem)
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) hist[b] = 0u;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+      hist[b] = 0u;
+      flags[0][b >> 5] = flags[1][b >> 5] = 0u;
+    }
   __syncthreads();
-  // (the high half of a shared counter counts the references to quads of varying depth; a chunk
-  // makes at most kChunkQuads of either per bin)
-  static_assert(kChunkQuads < 65536, "chunk counters share a word");
   for_each_ref<true>(ws, V, q0, q1, large, [&](long long, int b, int, int, uint2, uint32_t info) {
-    if (smem) atomicAdd(&hist[b], (info & kInfoFlatDepth) ? 1u : 0x10001u);
-    else atomicAdd(&ws.bin_count[V.bin_base + b], 1u);
+    if (smem) {
+      atomicAdd(&hist[b], 1u);
+      const uint32_t bit = 1u << (b & 31);
+      uint32_t* d = &flags[0][b >> 5];
+      uint32_t* f = &flags[1][b >> 5];
+      if (!(info & kInfoFlatDepth) && !(*(volatile uint32_t*)d & bit)) atomicOr(d, bit);
+      if (!(info & kInfoRectBox) && !(*(volatile uint32_t*)f & bit)) atomicOr(f, bit);
+    } else {
+      atomicAdd(&ws.bin_count[V.bin_base + b], 1u);
+    }
   });
   __syncthreads();
   if (!smem) return;
@@ -192,9 +201,10 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_count(Ws ws)
   __syncthreads();
   uint2* list = reinterpret_cast<uint2*>(ws.refs_tmp);
   for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-    const uint32_t c = hist[b] & 0xFFFFu;
+    const uint32_t c = hist[b];
     if (!c) continue;
-    if (!ws.cursors && (hist[b] >> 16)) ws.bin_cursor[V.bin_base + b] = 1u;   // not of constant depths
+    const uint32_t fl = ((flags[0][b >> 5] >> (b & 31)) & 1u) * kBinDepths | ((flags[1][b >> 5] >> (b & 31)) & 1u) * kBinShapes;
+    if (!ws.cursors && fl) atomicOr(&ws.bin_cursor[V.bin_base + b], fl);
     const uint32_t base = atomicAdd(&ws.bin_count[V.bin_base + b], c);
     const unsigned long long at = (unsigned long long)s_start + atomicAdd(&s_pos, 1u);
     // a list past the reference capacity means the references do not fit either: the scan
@@ -203,66 +213,80 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_count(Ws ws)
   }
 }
 
-// Single CTA. Offsets (exclusive scan), capacity check, and the bin order for the
-// rasteriser: bins by decreasing size class (floor(log2(count)) + 1), empty bins last.
+// Single CTA. Offsets (exclusive scan), capacity check, and the bin order for the rasterisers:
+// k_raster's bins, then k_raster_ordered's, each by decreasing size class (class k: from 2^(k - 1)
+// references, class 0: empty). Bound by latency (one CTA): each thread takes consecutive bins, four
+// counts in flight, so that there is one scan however many bins there are (8160 bins: 20 us with a
+// scan per 1024 of them and the two orders, 16 us so; 2040 bins 12 and 8).
 __global__ __launch_bounds__(1024) void k_bin_scan(Ws ws) {
   pdl_begin();
+  constexpr int kClasses = 32;       // (a view has fewer than 2^30 quads)
   __shared__ unsigned long long warp_sums[32];
-  __shared__ uint32_t cls_count[34];
-  __shared__ uint32_t cls_base[34];
-  __shared__ unsigned long long carry;
+  __shared__ uint32_t cls_count[2 * kClasses], cls_base[2 * kClasses];
+  __shared__ uint8_t cls_of[kHistSmemBins];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int n = ws.total_bins;
-  if (tid < 34) cls_count[tid] = 0;
-  if (tid == 0) carry = 0;
+  if (tid < 2 * kClasses) cls_count[tid] = 0;
   __syncthreads();
-  unsigned long long nonempty = 0, high = 0, mx = 0;
-  for (int base = 0; base < n; base += 1024) {
-    const int i = base + tid;
-    const uint32_t c = i < n ? ws.bin_count[i] : 0u;
-    if (i < n) {
-      nonempty += c > 0;
-      high += c >= (uint32_t)kSortSmemCap;
-      mx = c > mx ? c : mx;
+  auto class_of = [&](int bin, uint32_t c, uint32_t flags) {
+    const bool ordered = ws.ordered && !(flags & kBinDepths) &&
+                         ws.views[view_of_bin(ws.views, ws.n_views, bin)].color_mode == LR_COLOR_FLAT;
+    return (c ? 32 - __clz(c) : 0) + (ordered ? kClasses : 0);
+  };
+  unsigned long long nonempty = 0, high = 0, mx = 0, sum = 0;
+  const int per = (n + 1023) >> 10, i0 = tid * per, i1 = min(n, i0 + per);
+  for (int i = i0; i < i1; i += 4) {
+    uint32_t c[4], f[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      c[u] = i + u < i1 ? ws.bin_count[i + u] : 0u;
+      f[u] = i + u < i1 ? ws.bin_cursor[i + u] : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (i + u >= i1) break;
+      sum += c[u];
+      nonempty += c[u] > 0;
+      high += c[u] >= (uint32_t)kSortSmemCap;
+      mx = c[u] > mx ? c[u] : mx;
+      const int cls = class_of(i + u, c[u], f[u]);
+      if (i + u < kHistSmemBins) cls_of[i + u] = (uint8_t)cls;
       // one shared-memory atomic per warp and size class (most bins of a warp share one)
-      const uint32_t cls = c ? 33 - __clz(c) : 0;
       const unsigned act = __activemask();
       const unsigned peers = __match_any_sync(act, cls);
       if (lane == __ffs(peers) - 1) atomicAdd(&cls_count[cls], (uint32_t)__popc(peers));
     }
-    unsigned long long x = c;
+  }
+  unsigned long long x = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) warp_sums[wid] = x;
+  __syncthreads();
+  if (wid == 0) {
+    unsigned long long s = warp_sums[lane];
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, s, o);
+      if (lane >= o) s += y;
     }
-    if (lane == 31) warp_sums[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-      unsigned long long s = warp_sums[lane];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xffffffffu, s, o);
-        if (lane >= o) s += y;
-      }
-      warp_sums[lane] = s;
-    }
-    __syncthreads();
-    const unsigned long long incl = x + (wid ? warp_sums[wid - 1] : 0ull) + carry;
-    if (i < n) {
-      const unsigned long long excl = incl - c;
-      ws.bin_off[i] = (uint32_t)min(excl, (unsigned long long)ws.refs_cap);
-      if (ws.cursors) ws.bin_cursor[i] = (uint32_t)min(excl, (unsigned long long)ws.refs_cap);
-    }
-    __syncthreads();
-    if (tid == 1023) carry = incl;
-    __syncthreads();
+    warp_sums[lane] = s;
+  }
+  __syncthreads();
+  const unsigned long long total = warp_sums[31];
+  unsigned long long excl = x - sum + (wid ? warp_sums[wid - 1] : 0ull);
+  for (int i = i0; i < i1; ++i) {
+    const uint32_t o = (uint32_t)min(excl, (unsigned long long)ws.refs_cap);
+    excl += ws.bin_count[i];
+    ws.bin_off[i] = o;
+    if (ws.cursors) ws.bin_cursor[i] = o;
   }
   if (tid == 0) {
-    ws.bin_off[n] = (uint32_t)min(carry, (unsigned long long)ws.refs_cap);
-    ws.ctrl->refs_total = carry;
-    ws.ctrl->raster_items = (unsigned long long)n * bin_hb(ws.bin_log2);
-    if (carry > (unsigned long long)ws.refs_cap) set_error(ws.ctrl, LR_ERR_OVERFLOW);
+    ws.bin_off[n] = (uint32_t)min(total, (unsigned long long)ws.refs_cap);
+    ws.ctrl->refs_total = total;
+    if (total > (unsigned long long)ws.refs_cap) set_error(ws.ctrl, LR_ERR_OVERFLOW);
   }
   // statistics
   for (int o = 16; o > 0; o >>= 1) {
@@ -276,16 +300,33 @@ __global__ __launch_bounds__(1024) void k_bin_scan(Ws ws) {
     atomicAdd(&ws.ctrl->bins_high, high);
     atomicMax(&ws.ctrl->max_bin, mx);
   }
-  __syncthreads();
-  // class bases, largest class first
-  if (tid == 0) {
-    uint32_t s = 0;
-    for (int k = 33; k >= 0; --k) { cls_base[k] = s; s += cls_count[k]; }
+  // class bases, largest class first: lane l of warp 0 has class 31 - l
+  if (wid == 0) {
+    const int k = 31 - lane;
+    const uint32_t g = cls_count[k], o = cls_count[kClasses + k];
+    uint32_t gi = g, oi = o;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, gi, d), z = __shfl_up_sync(0xffffffffu, oi, d);
+      if (lane >= d) { gi += y; oi += z; }
+    }
+    const uint32_t general = __shfl_sync(0xffffffffu, gi, 31);
+    cls_base[k] = gi - g;
+    cls_base[kClasses + k] = general + oi - o;
+    // long lists of k_raster_ordered: from 1024 references (class 11) and 3/8 of a warp's share
+    const unsigned long long share = total * 3 / 4864;
+    const uint32_t n_long = __reduce_max_sync(0xffffffffu, k >= 11 && (1ull << (k - 1)) >= share ? oi : 0u);
+    if (k == 12) ws.ctrl->high_general = gi;       // from 2048 references
+    if (k == 1) ws.ctrl->nonempty_general = gi;
+    if (lane == 0) {
+      ws.ctrl->n_general = general;
+      ws.ctrl->raster_items = (unsigned long long)general * bin_hb(ws.bin_log2);
+      ws.ctrl->n_ordered_long = n_long;
+    }
   }
   __syncthreads();
   for (int i = tid; i < n; i += 1024) {
-    const uint32_t c = ws.bin_count[i];
-    const uint32_t cls = c ? 33 - __clz(c) : 0;
+    const int cls = i < kHistSmemBins ? cls_of[i] : class_of(i, ws.bin_count[i], ws.bin_cursor[i]);
     // lanes of one class take consecutive positions from one atomic of their leader
     const unsigned act = __activemask();
     const unsigned peers = __match_any_sync(act, cls);
@@ -759,13 +800,19 @@ __global__ __launch_bounds__(kSortThreads, 1) void k_bin_sort(Ws ws) {
   __shared__ uint32_t s_red[4][64];
   if (ws.ctrl->error == LR_ERR_OVERFLOW) return;
   const unsigned long long n_big = ws.ctrl->bins_high, n_all = ws.ctrl->bins_nonempty;
+  // bin_order holds k_raster's bins, then k_raster_ordered's: the k-th dense bin, the k-th other one
+  const unsigned long long n_general = ws.ctrl->n_general, high_g = ws.ctrl->high_general, full_g = ws.ctrl->nonempty_general;
+  auto dense_bin = [&](unsigned long long k) { return (int)ws.bin_order[k < high_g ? k : n_general + (k - high_g)]; };
+  auto small_bin = [&](unsigned long long k) {
+    return (int)ws.bin_order[high_g + k < full_g ? high_g + k : n_general + (n_big - high_g) + (high_g + k - full_g)];
+  };
   const Group C{(int)threadIdx.x, kSortThreads, 0};
   unsigned long long* sbuf = reinterpret_cast<unsigned long long*>(sort_smem);
   uint32_t* stage = reinterpret_cast<uint32_t*>(sort_smem);
   while (n_big) {
     if (threadIdx.x == 0) {
       const unsigned long long k = atomicAdd(&ws.ctrl->sort_head, 1ull);
-      s_bin[0] = k < n_big ? (int)ws.bin_order[k] : -1;
+      s_bin[0] = k < n_big ? dense_bin(k) : -1;
     }
     C.sync();
     const int bin = s_bin[0];
@@ -811,15 +858,17 @@ __global__ __launch_bounds__(kSortThreads, 1) void k_bin_sort(Ws ws) {
   const int q = (int)(threadIdx.x / (kSortThreads / 4));
   const Group G{(int)(threadIdx.x % (kSortThreads / 4)), kSortThreads / 4, 1 + q};
   SmallSort& S = reinterpret_cast<SmallSort*>(sort_smem)[q];
-  auto ticket = [&]() { return (int)min(n_big + atomicAdd(&ws.ctrl->sort_small_head, 1ull), n_all); };
-  int k = 0;   // (thread 0 of the quarter; the next ticket is drawn while a bin is sorted)
+  auto ticket = [&]() {
+    const unsigned long long k = atomicAdd(&ws.ctrl->sort_small_head, 1ull);
+    return k < n_all - n_big ? small_bin(k) : -1;
+  };
+  int k = 0;   // (thread 0 of the quarter; the next bin is drawn while one is sorted)
   if (G.t == 0) s_bin[q] = ticket();
   for (;;) {
     G.sync();
-    const int item = s_bin[q];
-    if (item >= (int)n_all) return;
+    const int bin = s_bin[q];
+    if (bin < 0) return;
     if (G.t == 0) k = ticket();
-    const int bin = (int)ws.bin_order[item];
     if (bin_owned(ws, bin)) {
       const uint32_t off = ws.bin_off[bin];
       const int n = (int)(ws.bin_off[bin + 1] - off);

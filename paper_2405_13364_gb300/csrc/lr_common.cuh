@@ -76,6 +76,7 @@ constexpr uint32_t kInfoFlatDepth = 8u;     // all four vertices have the same 1
 constexpr uint32_t kInfoSwap0 = 16u;        // triangle t (bit << t): negative area, v1 <-> v2
 constexpr uint32_t kInfoSmall0 = 64u;       // triangle t (bit << t): 32-bit edge values are
                                             // exact on every half-block its box touches
+constexpr uint32_t kInfoRectBox = kInfoSmall0;   // in rec_info only (binning reads no kInfoSmall0): kRecBox
 // flags in word 15 of the record
 constexpr uint32_t kRecSmall = 1u;          // every edge value is below 2^30 on every 8x4 and
                                             // 8x8 block the quad's box touches
@@ -176,7 +177,15 @@ struct Ctrl {
   // high-density bins by the sort k_bin_sort gave them: bucket sort, merge sort in
   // shared memory alone, merge sort with runs merged through global memory
   unsigned long long sort_branch[3];
-  unsigned long long pad[4];
+  // bins that k_raster takes (first in bin_order; those of k_raster_ordered follow): all, with at
+  // least kSortSmemCap references, non-empty
+  uint32_t n_general, high_general, nonempty_general;
+  // k_raster_ordered's bins with long lists: from 1024 references, and from 3/8 of a warp's
+  // share of all lists' 16x8 blocks (4864 warps, eight blocks a bin): with one warp per block the
+  // frame would wait for them
+  uint32_t n_ordered_long;
+  unsigned long long ordered_head;      // k_raster_ordered's queue
+  unsigned long long pad;
 };
 
 // The per-quad record written by k_setup and gathered by every later stage, 64 bytes so
@@ -229,6 +238,12 @@ __device__ __forceinline__ QuadRec load_rec(const int4* rec, uint32_t i) {
   return r;
 }
 
+constexpr int kOrderedOverlap = 2;
+
+// bin_cursor: the bin holds a reference to a quad that is not of constant depth, one that is no
+// axis-parallel rectangle
+constexpr uint32_t kBinDepths = 1u, kBinShapes = 2u;
+
 // Pointers into the workspace for one render (passed by value to every kernel).
 struct Ws {
   Ctrl* ctrl;
@@ -239,7 +254,8 @@ struct Ws {
   long long total_pix;
   long long refs_cap;
   int cursors;               // a view has more bins than the shared counters hold
-  int ticket;                // half-blocks per ticket of the rasteriser's queue: 1 or 2
+  int ordered;               // k_raster_ordered runs (a forward render without hashes, with flat
+                             // views): 1, or kOrderedOverlap where k_raster may run beside it
   int chunk_quads;           // quads per binning CTA (chunk_quads_for)
   int bin_log2;              // bins of 2^bin_log2 x 2^bin_log2 pixels (the same for every view)
   int4* rec;                 // [4 * total_quads]: the 64-byte quad record (QuadRec)
@@ -248,11 +264,11 @@ struct Ws {
   float* rec_rep;            // [total_quads]: representative 1/w over the quad's whole box
   uint32_t* bin_count;       // [total_bins]
   uint32_t* bin_off;         // [total_bins + 1]
-  uint32_t* bin_cursor;      // [total_bins] with `cursors` the scatter's cursors, else 1 where the
-                             // bin holds a reference to a quad that is not of constant depth
+  uint32_t* bin_cursor;      // [total_bins] with `cursors` the scatter's cursors, else kBin* flags
   uint2* chunk_span;         // [total_chunks] (start, length) of the chunk's list of (bin, base
                              // of the chunk's range within the bin), kept in refs_tmp
-  uint32_t* bin_order;       // [total_bins]: bins by decreasing reference count
+  uint32_t* bin_order;       // [total_bins]: k_raster's bins by decreasing size class, then
+                             // k_raster_ordered's
   unsigned long long* refs;      // [refs_cap] sorted per bin: (~rep_bits << 32) | ~record
   unsigned long long* refs_tmp;  // [refs_cap] merge buffer of the high-density sort
   uint32_t* ref_hb;          // [mw * refs_cap + mrows * total_bins] per bin, the transposed

@@ -36,6 +36,8 @@ __global__ void k_bin_scatter(Ws ws);
 __global__ void k_bin_sort(Ws ws);
 cudaError_t prepare_raster_3(int* blocks_flat, int* blocks_vtx, int* blocks_bwd, int* blocks_lit);
 cudaError_t launch_raster_3(int mode, const Ws& ws, int grid, cudaStream_t st);
+cudaError_t prepare_ordered(int* blocks_per_sm);
+cudaError_t launch_ordered(const Ws& ws, int grid, cudaStream_t st, bool pdl);
 cudaError_t overflow_occupancy(int* blocks_per_sm);
 cudaError_t launch_overflow(bool bwd, const Ws& ws, int grid, cudaStream_t st, bool pdl);
 }  // namespace lr
@@ -51,7 +53,7 @@ constexpr int kMaxDevices = 64;
 struct DeviceSetup {
   bool ready = false;
   unsigned char* scratch = nullptr;   // device address of g_noalloc_scratch
-  int sms = 0, blocks_flat = 1, blocks_vtx = 1, ovf_blocks = 1;
+  int sms = 0, blocks_flat = 1, blocks_vtx = 1, ovf_blocks = 1, ordered_blocks = 1;
 };
 
 DeviceSetup g_setup[kMaxDevices];
@@ -130,7 +132,7 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
       int blocks_bwd = 1, blocks_lit = 1;
       if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
           prepare_raster_3(&d.blocks_flat, &d.blocks_vtx, &blocks_bwd, &blocks_lit) != cudaSuccess ||
-          overflow_occupancy(&d.ovf_blocks) != cudaSuccess ||
+          overflow_occupancy(&d.ovf_blocks) != cudaSuccess || prepare_ordered(&d.ordered_blocks) != cudaSuccess ||
           cudaFuncSetAttribute(k_bin_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)kSortSmemBytes) != cudaSuccess)
         return LR_ERR_CUDA;
@@ -150,6 +152,7 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
       d.blocks_flat = d.blocks_flat > 0 ? d.blocks_flat : 1;
       d.blocks_vtx = d.blocks_vtx > 0 ? d.blocks_vtx : 1;
       d.ovf_blocks = d.ovf_blocks > 0 ? d.ovf_blocks : 1;
+      d.ordered_blocks = d.ordered_blocks > 0 ? d.ordered_blocks : 1;
       d.ready = true;
     }
     ds = d;
@@ -191,7 +194,7 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
   ws.chunk_quads = chunk_quads;
   ws.bin_log2 = kBinLog2Default;
   ws.cursors = nbins > kHistSmemBins;
-  ws.ticket = 1;
+  ws.ordered = !(Q > 0 && vtx) && !ws.cursors;
   ws.rec = reinterpret_cast<int4*>(base + o_rec);
   ws.rec_rect = reinterpret_cast<uint2*>(base + o_rect);
   ws.rec_info = reinterpret_cast<uint32_t*>(base + o_info);
@@ -218,6 +221,7 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
   if (chunks > 0) k_bin_scatter<<<chunks, kBinThreads, 0, st>>>(ws);
   k_bin_sort<<<ds.sms, kSortThreads, kSortSmemBytes, st>>>(ws);
   const bool vtx_kernel = Q > 0 && vtx;
+  if (ws.ordered && launch_ordered(ws, ds.sms * ds.ordered_blocks, st, false) != cudaSuccess) return LR_ERR_CUDA;
   if (launch_raster_3(vtx_kernel ? 1 : 0, ws, ds.sms * (vtx_kernel ? ds.blocks_vtx : ds.blocks_flat), st) != cudaSuccess)
     return LR_ERR_CUDA;
   if (launch_overflow(false, ws, ds.sms * ds.ovf_blocks, st, false) != cudaSuccess) return LR_ERR_CUDA;

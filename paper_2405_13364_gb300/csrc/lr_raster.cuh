@@ -697,132 +697,6 @@ __device__ __forceinline__ float4 shade(const float4* qc, int p, bool flat_view,
   return col;
 }
 
-// A bin that holds only flat-colour quads of one depth each (camera-facing sprites and
-// particles; bin_cursor, set by the bin count): the bin's list, sorted by that depth with the
-// tie rule, is every pixel's exact fragment order, so fragments are blended as they come,
-// without depth keys, sorter or exact path. A warp takes an 8x8 block, the half-blocks hb and
-// hb_l below it, with two pixels per lane, one above the other: a record read from shared
-// memory and a step of the loop serve both, and a quad that meets both half-blocks is gathered
-// and masked once. Rectangles (kRecBox) take their masks from two spans. (Blocks of two pixels
-// per lane for quads of other depths measured slower than half-blocks, 340 against 317 us on
-// the layer frame: the pixels' triangles differ too often for the second sorter's registers.)
-// 2M particles at 1920x1080: rasteriser 496 us by half-blocks without the spans, 299 us so.
-template <bool ATH>
-__device__ __forceinline__ unsigned const_block(const Ws& ws, const ViewDev& V, const uint32_t* row_u,
-                                                const uint32_t* row_l, uint32_t off, int n, int ox, int oy, int lane,
-                                                uint16_t* cand, uint2* pend, float4* qc) {
-  const int px = ox + (lane & 7), py = oy + 2 * (lane >> 3);
-  const bool ok_a = px < V.width && py < V.height, ok_b = px < V.width && py + 1 < V.height;
-  const int Ox = 256 * ox + 128, Oy = 256 * oy + 128;
-  const uint32_t* ref_lo = reinterpret_cast<const uint32_t*>(ws.refs + off);   // low words
-  const float4* colors = reinterpret_cast<const float4*>(V.col);
-  const uint32_t quad_base = (uint32_t)V.quad_base;
-  uint32_t* pend_j = reinterpret_cast<uint32_t*>(qc + 32);   // the ring's quads; pend: their masks
-  PixelState<1, true, ATH> sa, sb;
-  sa.init();
-  sb.init();
-  uint32_t cnt_a = 0, cnt_b = 0;
-  const int nw = (n + 31) >> 5;
-  int g = -32, r0 = 0, total = 0, head = 0, tail = 0;
-  for (;;) {
-    // masks of 32 candidates, one quad per lane, until a batch of covering quads is full
-    while (tail - head < 32) {
-      if (ATH && !__any_sync(0xffffffffu, (ok_a && sa.live()) || (ok_b && sb.live()))) break;   // all finished
-      if (r0 >= total) {
-        g += 32;
-        if (g >= nw) break;
-        total = list_bits(g + lane < nw ? (__ldg(row_u + g + lane) | __ldg(row_l + g + lane)) : 0u, lane, cand);
-        r0 = 0;
-        continue;
-      }
-      // first entry m, and for triangles that overlap (concave or crossed quads) a second one:
-      // triangle 1 lies in front
-      uint32_t m[2] = {0, 0}, m2[2] = {0, 0}, j = 0;
-      if (r0 + lane < total) {
-        const uint32_t rec = ~ref_lo[2 * (32 * g + (int)cand[r0 + lane])];
-        int X[4], Y[4];
-        load_rec_xy(ws.rec, rec, X, Y);
-        const int2 fl = __ldg(reinterpret_cast<const int2*>(ws.rec + 4ull * rec + 3) + 1);   // info, record flags
-        j = rec - quad_base;
-        if (fl.y & (int)kRecBox) {
-          const BoxSpan B(X, Y, ox, oy, 8);
-          const uint32_t cols = 0x01010101u * B.columns();
-          // even rows 2 i in [y0, y1): i in [(y0 + 1) / 2, (y1 + 1) / 2); odd: [y0 / 2, y1 / 2)
-          m[0] = cols & byte_span((B.y0 + 1) >> 1, (B.y1 + 1) >> 1);
-          m[1] = cols & byte_span(B.y0 >> 1, B.y1 >> 1);
-        } else {
-          if (fl.y & (int)kRecSmall) quad_masks_small<8>(X, Y, (uint32_t)fl.x, Ox, Oy, m2, m);
-          else quad_masks_any<8>(X, Y, (uint32_t)fl.x, Ox, Oy, m2, m);
-          if (((m[0] & m2[0]) | (m[1] & m2[1])) == 0u) {
-            m[0] |= m2[0]; m[1] |= m2[1];
-            m2[0] = m2[1] = 0u;
-          }
-        }
-      }
-      r0 += 32;
-      const bool h1 = (m[0] | m[1]) != 0u, h2 = (m2[0] | m2[1]) != 0u;
-      const unsigned b1 = __ballot_sync(0xffffffffu, h1), b2 = __ballot_sync(0xffffffffu, h2);
-      const unsigned lt = (1u << lane) - 1u;
-      int at = tail + __popc(b1 & lt) + __popc(b2 & lt);
-      if (h1) {
-        pend[at & (kPendCap - 1)] = make_uint2(m[0], m[1]);
-        pend_j[at++ & (kPendCap - 1)] = j;
-      }
-      if (h2) {
-        pend[at & (kPendCap - 1)] = make_uint2(m2[0], m2[1]);
-        pend_j[at & (kPendCap - 1)] = j;
-      }
-      tail += __popc(b1) + __popc(b2);
-      __syncwarp();
-    }
-    const int nb = min(32, tail - head);
-    if (nb == 0) break;
-    // entry 31 - L of the batch goes to lane and slot L: the highest set bit is the next
-    uint2 k = make_uint2(0u, 0u);
-    if (31 - lane < nb) {
-      const int i = (head + 31 - lane) & (kPendCap - 1);
-      k = pend[i];
-      qc[lane] = __ldg(colors + pend_j[i]);
-    }
-    head += nb;
-    uint32_t m_a = warp_transpose32(k.x, lane), m_b = warp_transpose32(k.y, lane);
-    __syncwarp();
-    if (!ok_a) m_a = 0;
-    if (!ok_b) m_b = 0;
-    cnt_a += __popc(m_a);
-    cnt_b += __popc(m_b);
-    while (m_a | m_b) {
-      if (ATH) {
-        if (!sa.live()) m_a = 0;
-        if (!sb.live()) m_b = 0;
-        if (!(m_a | m_b)) break;
-      }
-      const int p = 31 - __clz(m_a | m_b);
-      const uint32_t bit = 1u << p;
-      const float4 c = qc[p];
-      if (m_a & bit) sa.blend_direct(c);
-      if (m_b & bit) sb.blend_direct(c);
-      m_a &= ~bit;
-      m_b &= ~bit;
-    }
-    __syncwarp();
-  }
-  if (V.xmask && lane < 2 && oy + lane * kHbH < V.height) {
-    const uint32_t hbw = ((uint32_t)V.width + kHbW - 1) / kHbW;
-    V.xmask[((uint32_t)oy / kHbH + lane) * hbw + (uint32_t)ox / kHbW] = 0u;
-  }
-  const long long pa = (long long)py * V.width + px;
-  if (ok_a) {
-    if (V.cnt) V.cnt[pa] = cnt_a;
-    write_pixel(V, pa, sa.r, sa.g, sa.b, sa.T);
-  }
-  if (ok_b) {
-    if (V.cnt) V.cnt[pa + V.width] = cnt_b;
-    write_pixel(V, pa + V.width, sb.r, sb.g, sb.b, sb.T);
-  }
-  return cnt_a + cnt_b;
-}
-
 // HASH: the variant that also writes the per-pixel coverage hash (a test output); the
 // others carry no code or registers for it. ATH: the alpha-threshold variant (forward
 // only, no hash), which also skips candidate quads that cannot reach in front of any
@@ -830,7 +704,11 @@ __device__ __forceinline__ unsigned const_block(const Ws& ws, const ViewDev& V, 
 // shades lit views (per-vertex normals, one directional light).
 template <int K, bool VTX, bool BWD, bool HASH, bool ATH = false, bool LIT = false>
 __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH, LIT)) void k_raster(Ws ws) {
-  pdl_begin();
+  // Behind k_raster_ordered (kOrderedOverlap) it waits at its end, not here: k_raster_ordered's CTAs
+  // let it launch once they have seen the sort complete, it reads nothing that k_raster_ordered
+  // writes and writes other pixels, and what follows still waits for both.
+  if (ws.ordered != kOrderedOverlap) asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   extern __shared__ __align__(16) unsigned char smem[];
   // the sorter carries each fragment's colour (backward: the batch holds its triangles' colours)
   constexpr bool kCarry = VTX || K == 1 || BWD;
@@ -847,18 +725,15 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
   // others keep ea
   unsigned long long* dkey = reinterpret_cast<unsigned long long*>(&geo);
   uint32_t* did = reinterpret_cast<uint32_t*>(&geo);
-  if (ws.ctrl->error == LR_ERR_OVERFLOW) return;
-  const uint32_t nitems = (uint32_t)ws.ctrl->raster_items;   // (a batch has less than 2^32 pixels)
+  // (a batch has less than 2^32 pixels)
+  const uint32_t nitems = ws.ctrl->error == LR_ERR_OVERFLOW ? 0u : (uint32_t)ws.ctrl->raster_items;
   unsigned long long frag_total = 0;
 
-  // the next item: the one after i, or the first of a new ticket (of 1 or 2 items)
-  auto next_item = [&](uint32_t i) {
-    if (i & (uint32_t)(ws.ticket - 1)) return i;
+  for (;;) {
     unsigned long long k = 0;
-    if (lane == 0) k = atomicAdd(&ws.ctrl->raster_head, (unsigned long long)ws.ticket);
-    return (uint32_t)__shfl_sync(0xffffffffu, (uint32_t)min(k, 0xFFFFFFF0ull), 0);
-  };
-  for (uint32_t item = next_item(0u); item < nitems; item = next_item(item + 1u)) {
+    if (lane == 0) k = atomicAdd(&ws.ctrl->raster_head, 1ull);
+    const uint32_t item = __shfl_sync(0xffffffffu, (uint32_t)min(k, 0xFFFFFFF0ull), 0);
+    if (item >= nitems) break;
     const int lg = ws.bin_log2, hl = bin_hb_log2(lg), cl = bin_hb_cols_log2(lg);
     const int bin_g = (int)ws.bin_order[item >> hl];
     // items 2 i and 2 i + 1 of a bin: the upper and the lower half-block of its 8x8 block i
@@ -874,13 +749,6 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
     const bool pix_ok = px < V.width && py < V.height;
     const uint32_t off = ws.bin_off[bin_g];
     const int n = (int)(ws.bin_off[bin_g + 1] - off);
-    if (!HASH && !BWD && !ws.cursors && V.color_mode == LR_COLOR_FLAT && ws.bin_cursor[bin_g] == 0u) {
-      // an 8x8 block at its upper half-block; nothing at its lower one
-      if (item & 1u) continue;
-      frag_total += const_block<ATH>(ws, V, hb_row(ws, off, bin_g, n, hb), hb_row(ws, off, bin_g, n, hb + (1 << cl)), off, n,
-                                     ox, oy, lane, cand, pend, reinterpret_cast<float4*>(&geo));
-      continue;
-    }
     const bool flat_view = V.color_mode == LR_COLOR_FLAT, lit_view = LIT && V.color_mode == LR_COLOR_LIT;
     const bool hashing = HASH && V.hash != nullptr;
     const int Ox = 256 * ox + 128, Oy = 256 * oy + 128;   // first pixel centre, 1/256 px
@@ -1140,6 +1008,7 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) frag_total += __shfl_xor_sync(0xffffffffu, frag_total, o);
   if (lane == 0 && frag_total) atomicAdd(&ws.ctrl->fragments, frag_total);
+  if (ws.ordered == kOrderedOverlap) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace lr
@@ -1183,21 +1052,21 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
      + 8: alpha threshold (modes 8 and 9 only); 17: colours in the sorter with lit views */   \
   cudaError_t launch_raster_##KK(int mode, const Ws& ws, int grid, cudaStream_t st) {         \
     const size_t sf = raster_smem_bytes(false), sv = raster_smem_bytes(true);                 \
-    /* a plain launch: with programmatic serialisation the persistent CTAs, placed early  \
-       next to the bin sort's, measured slower on the particle frame */                       \
+    /* a plain launch but behind k_raster_ordered: with programmatic serialisation the        \
+       persistent CTAs, placed early next to the bin sort's, measured slower */                \
+    const bool pdl = ws.ordered == kOrderedOverlap;                                           \
+    const dim3 g(grid), t(kRasterThreads);                                                    \
     switch (mode) {                                                                           \
-      case 1: k_raster<KK, true, false, false><<<grid, kRasterThreads, sv, st>>>(ws); break;  \
-      case 2: k_raster<KK, false, true, false><<<grid, kRasterThreads, raster_smem_bytes(false, true), st>>>(ws); break; \
-      case 4: k_raster<KK, false, false, true><<<grid, kRasterThreads, sf, st>>>(ws); break;  \
-      case 5: k_raster<KK, true, false, true><<<grid, kRasterThreads, sv, st>>>(ws); break;   \
-      case 8: k_raster<KK, false, false, false, true><<<grid, kRasterThreads, sf, st>>>(ws); break; \
-      case 9: k_raster<KK, true, false, false, true><<<grid, kRasterThreads, sv, st>>>(ws); break; \
+      case 1: return launch_pdl(pdl, k_raster<KK, true, false, false>, g, t, sv, st, ws);     \
+      case 2: return launch_pdl(pdl, k_raster<KK, false, true, false>, g, t, raster_smem_bytes(false, true), st, ws); \
+      case 4: return launch_pdl(pdl, k_raster<KK, false, false, true>, g, t, sf, st, ws);     \
+      case 5: return launch_pdl(pdl, k_raster<KK, true, false, true>, g, t, sv, st, ws);      \
+      case 8: return launch_pdl(pdl, k_raster<KK, false, false, false, true>, g, t, sf, st, ws); \
+      case 9: return launch_pdl(pdl, k_raster<KK, true, false, false, true>, g, t, sv, st, ws); \
       case 17:                                                                                \
-        k_raster<KK, true, false, false, false, true>                                         \
-            <<<grid, kRasterThreads, raster_smem_bytes(true, false, true), st>>>(ws);         \
-        break;                                                                                \
-      default: k_raster<KK, false, false, false><<<grid, kRasterThreads, sf, st>>>(ws); break; \
+        return launch_pdl(pdl, k_raster<KK, true, false, false, false, true>, g, t,           \
+                          raster_smem_bytes(true, false, true), st, ws);                      \
+      default: return launch_pdl(pdl, k_raster<KK, false, false, false>, g, t, sf, st, ws);   \
     }                                                                                         \
-    return cudaGetLastError();                                                                \
   }                                                                                           \
   }

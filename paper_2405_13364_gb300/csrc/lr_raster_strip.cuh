@@ -142,7 +142,7 @@ __global__ __launch_bounds__(kRasterThreads, 3) void k_raster_strip(Ws ws) {
   const int hx = warp & 3, hyl = warp >> 2;          // this warp's half-block in the strip
   uint32_t* my_slot = s_slot + warp * 32;
   if (ws.ctrl->error == LR_ERR_OVERFLOW) return;
-  const unsigned long long nitems = ws.ctrl->raster_items >> 3;   // 8 half-blocks per strip
+  const unsigned long long nitems = ((unsigned long long)ws.total_bins * bin_hb(ws.bin_log2)) >> 3;   // 8 half-blocks per strip
   unsigned long long frag_total = 0;
 
   for (;;) {

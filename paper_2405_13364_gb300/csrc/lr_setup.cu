@@ -193,7 +193,8 @@ __global__ __launch_bounds__(256) void k_setup(Ws ws) {
       ws.rec_rep[g] = rep;
     }
     ws.rec_rect[g] = rect;
-    ws.rec_info[g] = info | (worst << 8);
+    // (binning reads the rectangle flag where the rasteriser's record has kInfoSmall0)
+    ws.rec_info[g] = (info & ~(3u * kInfoSmall0)) | ((rflags & kRecBox) && worst == kVisible ? kInfoRectBox : 0u) | (worst << 8);
     if (bad) set_error(ws.ctrl, LR_ERR_INVALID_ARG);
   }
   // statistics: culled quads per reason, one atomic per reason present in the warp, by its
