@@ -373,21 +373,22 @@ __device__ __forceinline__ void batch_gradients(uint32_t done, uint32_t j, float
   uint32_t m = warp_transpose32(done, lane);   // (its shuffles precede the reads below)
   __syncwarp();
   if (!m) return;
-  float r = 0.f, g = 0.f, b = 0.f, s = 0.f;
+  // (dL/da pixel by pixel: its two terms nearly cancel, so their sums would round worse)
+  const float4 c = qc[lane];
+  const float om = 1.0f - c.w, inv = om > 1e-6f ? rcp_approx(om) : 0.f;
+  float r = 0.f, g = 0.f, b = 0.f, da = 0.f;
   while (m) {
     const int px = __ffs(m) - 1;
     m &= m - 1;
     const float4 p = G.g[px];
     const float2 ts = G.ts[__popc((__float_as_uint(p.w) >> lane) >> 1)][px];
-    r += ts.x * p.x;
-    g += ts.x * p.y;
-    b += ts.x * p.z;
-    s += ts.y;
+    const float w = ts.x * c.w;
+    r += w * p.x;
+    g += w * p.y;
+    b += w * p.z;
+    da += ts.x * (p.x * c.x + p.y * c.y + p.z * c.z) - ts.y * inv;
   }
-  const float4 c = qc[lane];
-  const float om = 1.0f - c.w;
-  const float da = r * c.x + g * c.y + b * c.z - (om > 1e-6f ? s * rcp_approx(om) : 0.f);
-  atomicAdd(reinterpret_cast<float4*>(grad) + j, make_float4(r * c.w, g * c.w, b * c.w, da));
+  atomicAdd(reinterpret_cast<float4*>(grad) + j, make_float4(r, g, b, da));
 }
 
 __device__ __forceinline__ void write_pixel(const ViewDev& V, long long pidx, float r, float g, float b,
