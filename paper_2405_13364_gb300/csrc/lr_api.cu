@@ -919,10 +919,11 @@ extern "C" lr_status lr_render_msaa(lr_ctx* ctx, const lr_quads* quads, const lr
 extern "C" lr_status lr_get_stats(lr_ctx* ctx, lr_stats* stats) {
   if (!ctx) return LR_ERR_INVALID_ARG;
   if (!ctx->have_last) return fail(ctx, LR_ERR_INVALID_ARG, "no render issued on this context%s");
-  cudaError_t e = cudaStreamSynchronize(ctx->last_stream);
+  // the copy queued behind the render, so that the host waits once
+  cudaError_t e = cudaMemcpyAsync(ctx->host_ctrl, ctx->last_ws, sizeof(Ctrl), cudaMemcpyDeviceToHost, ctx->last_stream);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemcpyAsync(ctrl)");
+  e = cudaStreamSynchronize(ctx->last_stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaStreamSynchronize");
-  e = cudaMemcpy(ctx->host_ctrl, ctx->last_ws, sizeof(Ctrl), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemcpy(ctrl)");
   const Ctrl& h = *ctx->host_ctrl;
   if (stats) {
     memset(stats, 0, sizeof(*stats));

@@ -91,6 +91,18 @@ static void finish(lr_server* s, uint64_t t, int status) {
   if (status != LR_OK) s->stats.failed++;
 }
 
+// A small frame is bound by its launches' latency: two rendered together take hardly longer than
+// one. So a lone small request waits for company while a batch runs, until the batch ends but at
+// most two poll intervals.
+static bool hold_back(const lr_server* s) {
+  if (s->queue.size() != 1 || s->cfg.max_batch_views < 2 || s->stopping) return false;
+  bool busy = false;
+  for (const Slot& sl : s->slots) busy |= sl.busy;
+  const Req& r = s->reqs.at(s->queue.front());
+  return busy && !r.alone && r.view.quads.num_quads <= 32768 && (long long)r.view.width * r.view.height <= 262144 &&
+         now_ns() - r.t_submit < 2000ull * (uint64_t)s->cfg.poll_interval_us;
+}
+
 static void serve_loop(lr_server* s) {
   std::unique_lock<std::mutex> lk(s->mu);
   std::vector<lr_view> views;
@@ -120,8 +132,9 @@ static void serve_loop(lr_server* s) {
     if (progressed) s->done_cv.notify_all();
     // ---- admission -----------------------------------------------------------------
     s->submitted.store(false);
+    const bool hold = hold_back(s);
     for (Slot& sl : s->slots) {
-      if (sl.busy || s->queue.empty()) continue;
+      if (sl.busy || s->queue.empty() || hold) continue;
       views.clear();
       std::vector<uint64_t> batch;
       int batch_k = 0;
