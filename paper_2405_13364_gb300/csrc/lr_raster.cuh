@@ -112,13 +112,18 @@ __device__ __forceinline__ uint32_t row_cover(int r, int sx) {
 // ATH: the alpha-threshold variant. Once the transmittance drops to kAlphaTMin nothing
 // more is blended and `last` stays at the key of the fragment that got it there, so the
 // misorder test below only flags fragments that belong in front of that one.
-template <int K, bool VTX, bool ATH = false>
+// PARK: the held fragments' colours stay where they were put, in shared memory, and only their places
+// move with the keys, where moving a colour through a slot takes eight selects (K = 3: 250k layers
+// at 1024x768 148 us with colours in the sorter's registers, 139 so; six mixed views 737 and 692).
+template <int K, bool VTX, bool ATH = false, bool PARK = false>
 struct PixelState {
   // K = 1 with flat colours gathered at blend time: the colour of the fragment held in the
   // slot is loaded when it enters, so the gather overlaps the next fragment's work
   static constexpr bool kPrefetch = !VTX && K == 1;
   unsigned long long s[K];
-  float4 c[VTX || kPrefetch ? K : 1];
+  float4 c[(VTX || kPrefetch) && !PARK ? K : 1];
+  uint32_t sl[PARK ? K : 1];         // place of slot i's colour
+  float4* park;                      // the lane's places, 32 apart
   unsigned long long last;
   float r, g, b, T;
   bool flagged;
@@ -132,6 +137,8 @@ struct PixelState {
   __device__ __forceinline__ void init() {
 #pragma unroll
     for (int i = 0; i < K; ++i) s[i] = kSent;
+#pragma unroll
+    for (int i = 0; i < (PARK ? K : 0); ++i) sl[i] = (uint32_t)i;
     if (kNullSlot) c[0] = make_float4(0.f, 0.f, 0.f, 0.f);
     last = kSent;
     r = g = b = 0.f;
@@ -227,7 +234,15 @@ struct PixelState {
     const unsigned long long ev = xfirst ? x : s[0];
     const unsigned long long y = xfirst ? s[0] : x;
     float4 evc = xc, yc = xc;
-    if (VTX) {
+    uint32_t ys = 0;
+    if (PARK) {
+      // the fragment that is kept takes (or already has) the evicted one's place
+      ys = sl[0];
+      if (!xfirst) {
+        evc = park[32 * ys];
+        park[32 * ys] = xc;
+      }
+    } else if (VTX) {
       evc = xfirst ? xc : c[0];
       yc = xfirst ? c[0] : xc;
     }
@@ -238,7 +253,10 @@ struct PixelState {
       const bool take_y = (i == 0) || (s[i] > y);
       const unsigned long long nxt = s[i + 1 < K ? i + 1 : i];
       s[i] = take_next ? nxt : (take_y ? y : s[i]);
-      if (VTX) {
+      if (PARK) {
+        const uint32_t ns = sl[i + 1 < K ? i + 1 : i];
+        sl[i] = take_next ? ns : (take_y ? ys : sl[i]);
+      } else if (VTX) {
         const float4 nc = c[i + 1 < K ? i + 1 : i];
         c[i] = take_next ? nc : (take_y ? yc : c[i]);
       }
@@ -252,7 +270,10 @@ struct PixelState {
   __device__ __forceinline__ void flush(const ViewDev& V) {
 #pragma unroll
     for (int i = 0; i < K; ++i)
-      if (s[i] != kSent && live()) blend(s[i], VTX || kPrefetch ? c[i] : make_float4(0.f, 0.f, 0.f, 0.f), V);
+      if (s[i] != kSent && live()) {
+        if (PARK) blend(s[i], park[32 * sl[i]], V);
+        else blend(s[i], VTX || kPrefetch ? c[i] : make_float4(0.f, 0.f, 0.f, 0.f), V);
+      }
   }
 };
 
@@ -577,9 +598,10 @@ __device__ __forceinline__ uint32_t byte_span(int a, int b) {
 // Per warp: the candidates of a 1024-reference window, a ring of covering triangles waiting for
 // a batch, and the records of the batch the fragment loop reads, one 16-byte array per field so that a slot's fields lie at one address
 // plus constants and eight neighbouring slots never share a bank.
-// references per bitmap window (a word per lane; half of them in the backward, whose shared memory
-// leaves room for three CTAs then)
-__host__ __device__ constexpr int win_refs(bool bwd) { return bwd ? 512 : 1024; }
+// references per bitmap window (a word per lane; half of them in the backward and for lit views at
+// K = 3, whose shared memory leaves room for three CTAs then)
+__host__ __device__ constexpr int win_refs(bool half) { return half ? 512 : 1024; }
+__host__ __device__ constexpr bool half_window(int k, bool bwd, bool lit) { return bwd || (lit && k == 3); }
 constexpr int kPendCap = 128;      // at most 31 left over + 64 pushed per candidate round
 constexpr uint32_t kPendConst = 0x80000000u;   // pending id: flat colour and constant depth
 struct BatchGeo {
@@ -590,12 +612,16 @@ struct BatchGeo {
   int2 hi[32];                     // high words of 64-bit e1, e2
 };
 __host__ __device__ constexpr int batch_cols(bool vtx, bool lit) { return vtx ? (lit ? 6 : 3) : 1; }
-__host__ __device__ constexpr size_t batch_smem_warp(bool vtx, bool bwd, bool lit) {
-  return win_refs(bwd) * sizeof(uint16_t) + kPendCap * sizeof(uint2) + sizeof(BatchGeo) +
-         (size_t)batch_cols(vtx, lit) * 32 * sizeof(float4) + (bwd ? sizeof(GradShared) : 0);
+// sorters whose colours are parked in shared memory (which then still holds three CTAs). Not flat
+// colours, which are gathered as they are blended (layers at K = 3: 121 us, parked 123).
+__host__ __device__ constexpr bool parked(int k, bool vtx, bool bwd) { return vtx && !bwd && (k == 2 || k == 3); }
+__host__ __device__ constexpr size_t batch_smem_warp(bool vtx, bool bwd, bool lit, int k) {
+  return win_refs(half_window(k, bwd, lit)) * sizeof(uint16_t) + kPendCap * sizeof(uint2) + sizeof(BatchGeo) +
+         (size_t)batch_cols(vtx, lit) * 32 * sizeof(float4) + (bwd ? sizeof(GradShared) : 0) +
+         (parked(k, vtx, bwd) ? (size_t)k * 32 * sizeof(float4) : 0);
 }
-__host__ __device__ constexpr size_t raster_smem_bytes(bool vtx, bool bwd = false, bool lit = false) {
-  return (size_t)kRasterWarps * batch_smem_warp(vtx, bwd, lit);
+__host__ __device__ constexpr size_t raster_smem_bytes(bool vtx, bool bwd = false, bool lit = false, int k = 1) {
+  return (size_t)kRasterWarps * batch_smem_warp(vtx, bwd, lit, k);
 }
 
 // The record of covering triangle id (2 * quad + triangle of view V) into slot `lane` of the
@@ -713,10 +739,11 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
   extern __shared__ __align__(16) unsigned char smem[];
   // the sorter carries each fragment's colour (backward: the batch holds its triangles' colours)
   constexpr bool kCarry = VTX || K == 1 || BWD;
-  constexpr int kWin = win_refs(BWD);
+  constexpr int kWin = win_refs(half_window(K, BWD, LIT));
+  constexpr bool kPark = parked(K, VTX, BWD);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lx = lane & (kHbW - 1), ly = lane >> 3;
-  unsigned char* wbase = smem + (size_t)warp * batch_smem_warp(VTX, BWD, LIT);
+  unsigned char* wbase = smem + (size_t)warp * batch_smem_warp(VTX, BWD, LIT, K);
   uint16_t* cand = reinterpret_cast<uint16_t*>(wbase);
   uint2* pend = reinterpret_cast<uint2*>(wbase + kWin * sizeof(uint16_t));
   BatchGeo& geo = *reinterpret_cast<BatchGeo*>(pend + kPendCap);
@@ -757,12 +784,13 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
     const float4 light = LIT ? make_float4(V.light[0], V.light[1], V.light[2], V.light[3])
                              : make_float4(0.f, 0.f, 0.f, 0.f);
 
-    typename std::conditional<BWD, GradState<K>, PixelState<K, kCarry, ATH>>::type st;
+    typename std::conditional<BWD, GradState<K>, PixelState<K, kCarry, ATH, kPark>>::type st;
     if constexpr (BWD) {
       st.gp = GradPixel();
       if (pix_ok) st.gp.load(ws.grad_out, ws.fwd, (long long)py * V.width + px);
     } else {
       st.init();
+      if (kPark) st.park = qc + batch_cols(VTX, LIT) * 32 + lane;
     }
     uint32_t cnt = 0;
     unsigned long long hsh = 0;
@@ -1023,7 +1051,7 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
   static cudaError_t raster_attr_##KK() {                                                     \
     return cudaFuncSetAttribute(k_raster<KK, VTX, BWD, HASH, ATH, LIT>,                       \
                                 cudaFuncAttributeMaxDynamicSharedMemorySize,                  \
-                                (int)raster_smem_bytes(VTX, BWD, LIT));                       \
+                                (int)raster_smem_bytes(VTX, BWD, LIT, KK));                       \
   }                                                                                           \
   cudaError_t prepare_raster_##KK(int* blocks_flat, int* blocks_vtx, int* blocks_bwd,         \
                                   int* blocks_lit) {                                          \
@@ -1038,21 +1066,21 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
     if (e != cudaSuccess) return e;                                                           \
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(                                        \
         blocks_lit, k_raster<KK, true, false, false, false, true>, kRasterThreads,            \
-        raster_smem_bytes(true, false, true));                                                \
+        raster_smem_bytes(true, false, true, KK));                                                \
     if (e != cudaSuccess) return e;                                                           \
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_flat, k_raster<KK, false, false, false>, \
-                                                      kRasterThreads, raster_smem_bytes(false)); \
+                                                      kRasterThreads, raster_smem_bytes(false, false, false, KK)); \
     if (e != cudaSuccess) return e;                                                           \
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_bwd, k_raster<KK, false, true, false>, \
                                                       kRasterThreads, raster_smem_bytes(false, true)); \
     if (e != cudaSuccess) return e;                                                           \
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_vtx, k_raster<KK, true, false, false>, \
-                                                         kRasterThreads, raster_smem_bytes(true)); \
+                                                         kRasterThreads, raster_smem_bytes(true, false, false, KK)); \
   }                                                                                           \
   /* mode: 0 flat colours, 1 colours in the sorter, 2 backward; + 4: coverage hash;        \
      + 8: alpha threshold (modes 8 and 9 only); 17: colours in the sorter with lit views */   \
   cudaError_t launch_raster_##KK(int mode, const Ws& ws, int grid, cudaStream_t st) {         \
-    const size_t sf = raster_smem_bytes(false), sv = raster_smem_bytes(true);                 \
+    const size_t sf = raster_smem_bytes(false, false, false, KK), sv = raster_smem_bytes(true, false, false, KK);                 \
     /* a plain launch but behind k_raster_ordered: with programmatic serialisation the        \
        persistent CTAs, placed early next to the bin sort's, measured slower */                \
     const bool pdl = ws.ordered == kOrderedOverlap;                                           \
@@ -1066,7 +1094,7 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH,
       case 9: return launch_pdl(pdl, k_raster<KK, true, false, false, true>, g, t, sv, st, ws); \
       case 17:                                                                                \
         return launch_pdl(pdl, k_raster<KK, true, false, false, false, true>, g, t,           \
-                          raster_smem_bytes(true, false, true), st, ws);                      \
+                          raster_smem_bytes(true, false, true, KK), st, ws);                      \
       default: return launch_pdl(pdl, k_raster<KK, false, false, false>, g, t, sf, st, ws);   \
     }                                                                                         \
   }                                                                                           \
