@@ -285,14 +285,13 @@ struct PixelState {
 // record them per batch in shared memory, rank of the fragment in its pixel by pixel, and
 // batch_gradients sums them with one lane per triangle and one vector atomic each. Only fragments
 // blended after their batch (the K last of it) or beyond kGradRanks of a pixel are added one by
-// one. 25M fragments at 1024x1024, K = 1: 435 us and 384M warp instructions when each blended
-// fragment searched the warp for lanes with the same quad and issued four atomics per group;
-// 289 us and 215M so.
+// one, each with a vector atomic. 25M fragments at 1024x1024, K = 1: 435 us when each blended
+// fragment searched the warp for lanes with the same quad and issued four atomics per group, 291
+// when only the late ones did, 258 so.
 constexpr uint32_t kOldSlot = 32u;
 constexpr int kGradRanks = 12;     // (eight fragments per pixel and batch are ordinary)
 struct GradShared {
   float4 g[32];                    // per pixel: dL/d(R, G, B), its batch coverage (bits)
-  float4 agg[32];                  // combines lanes' gradients of late fragments
   float2 ts[kGradRanks][32];       // (T, S) by rank and pixel
 };
 template <int K>
@@ -333,23 +332,9 @@ struct GradState {
     } else {
       const float om = 1.0f - c.w;
       const float da = T * (gp.gr * c.x + gp.gg * c.y + gp.gb * c.z) - (om > 1e-6f ? S * rcp_approx(om) : 0.f);
-      // lanes blending a fragment of the same quad at this point add their contributions
-      // in shared memory first, and one of them issues the global atomic
-      const unsigned act = __activemask();
-      const unsigned grp = __match_any_sync(act, j);
-      G.agg[lane] = make_float4(gp.gr * w, gp.gg * w, gp.gb * w, da);
-      __syncwarp(act);
-      if (lane == __ffs(grp) - 1) {
-        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (unsigned m = grp; m; m &= m - 1) {
-          const float4 x = G.agg[__ffs(m) - 1];
-          sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
-        }
-        atomicAdd(reinterpret_cast<float4*>(gp.grad) + j, sum);
-      }
-      __syncwarp(act);
+      atomicAdd(reinterpret_cast<float4*>(gp.grad) + j, make_float4(gp.gr * w, gp.gg * w, gp.gb * w, da));
     }
-    T *= 1.0f - c.w;
+    T = __fmaf_rn(-T, c.w, T);   // as the forward, so that r, g, b are its own and S their difference
   }
 
   // without a gradient (gp.grad null) the order is tested, nothing is blended
