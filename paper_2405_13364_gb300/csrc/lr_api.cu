@@ -589,11 +589,11 @@ static lr_status launch_sequence(lr_ctx* ctx, const Prepared& P, cudaStream_t st
              (unsigned long long)L.refs_cap, chunk, P.views_dev);
   if (L.total_quads > 0) launch_pdl(pdl, k_setup, dim3((unsigned)((L.total_quads + 255) / 256)), dim3(256), 0, st, ws);
   rec(ctx, timed, 1, st);
-  if (L.total_chunks > 0) launch_pdl(pdl, k_bin_count, dim3(L.total_chunks), dim3(kBinThreads), 0, st, ws);
+  if (L.total_chunks > 0) launch_pdl(pdl, k_bin_count, dim3(L.total_chunks), dim3(bin_threads_for(L.chunk_quads)), 0, st, ws);
   rec(ctx, timed, 2, st);
   launch_pdl(pdl, k_bin_scan, dim3(1), dim3(1024), 0, st, ws);
   rec(ctx, timed, 3, st);
-  if (L.total_chunks > 0) launch_pdl(pdl, k_bin_scatter, dim3(L.total_chunks), dim3(kBinThreads), 0, st, ws);
+  if (L.total_chunks > 0) launch_pdl(pdl, k_bin_scatter, dim3(L.total_chunks), dim3(bin_threads_for(L.chunk_quads)), 0, st, ws);
   rec(ctx, timed, 4, st);
   launch_pdl(pdl, k_bin_sort, dim3(ctx->sms), dim3(kSortThreads), kSortSmemBytes, st, ws);
   rec(ctx, timed, 5, st);

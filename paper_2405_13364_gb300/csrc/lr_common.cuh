@@ -45,21 +45,21 @@ constexpr int kMaxBucket = 64;
 constexpr size_t kSortSmemBytes = (size_t)kBucketBigCap * 8 + (size_t)kBucketsBig * 2;
 static_assert(kSortSmemBytes >= 2 * (size_t)kSortBigCap * 8, "two merge buffers");
 constexpr int kHistSmemBins = 8192;         // shared-memory bin counters per CTA (Sec. 2 Stage 2)
-#ifndef LR_CHUNK_QUADS
-#define LR_CHUNK_QUADS 2048
-#endif
-constexpr int kChunkQuads = LR_CHUNK_QUADS;  // quads per binning CTA, at most
-constexpr int kChunkQuadsMin = 256;
-// ... and of a render of `quads` quads: halved until there are two CTAs for each of the 152 SMs
-// (the count and the scatter are bound by latency, and 2048 quads each left most SMs idle below
-// 600,000 quads)
+// Quads per binning CTA: 4096 (from 1.6M quads on: 2M particles 35 us against 29 for the count, 41
+// against 39 for the scatter; a batch of 1.4M quads with large ones among them 47 against 57), else
+// 2048, halved until there are two CTAs for each of the 152 SMs (both kernels are bound by latency, and
+// 2048 quads each left most SMs idle below 600,000 quads). One thread per quad where that is fewer
+// than 512 (100,000 quads: 14 us each with 512 threads, 12 with 256; with 256 for 2048 quads the
+// layer frame took 31 and 37 us instead of 20 and 25).
+constexpr int kChunkQuads = 4096, kChunkQuadsMin = 256;
 __host__ __forceinline__ int chunk_quads_for(long long quads) {
-  int c = kChunkQuads;
+  if (quads >= 400LL * kChunkQuads) return kChunkQuads;
+  int c = kChunkQuads / 2;
   while (c > kChunkQuadsMin && quads < 304LL * c) c >>= 1;
   return c;
 }
-constexpr int kBinThreads = kChunkQuads / 4 < 1024 ? kChunkQuads / 4 : 1024;   // threads per binning CTA
-constexpr int kBinMinBlocks = kBinThreads >= 1024 ? 1 : (kBinThreads >= 512 ? 2 : 5);
+constexpr int kBinThreads = 512, kBinMinBlocks = 2;   // threads per binning CTA at most, CTAs per SM
+__host__ __forceinline__ int bin_threads_for(int chunk_quads) { return chunk_quads < kBinThreads ? chunk_quads : kBinThreads; }
 constexpr int kSmallBins = 4;               // AABB-counted up to kSmallBins x kSmallBins bins
 
 // cull reasons (stats and rec_info bits 8..11)

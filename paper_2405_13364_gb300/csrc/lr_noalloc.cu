@@ -216,9 +216,9 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
   memset(&no_views, 0, sizeof(no_views));
   k_init<<<(int)((nbins + 255) / 256), 256, 0, st>>>(ws, (unsigned long long)cap, no_views, nullptr);
   if (Q > 0) k_setup<<<(unsigned)((Q + 255) / 256), 256, 0, st>>>(ws);
-  if (chunks > 0) k_bin_count<<<chunks, kBinThreads, 0, st>>>(ws);
+  if (chunks > 0) k_bin_count<<<chunks, bin_threads_for(chunk_quads), 0, st>>>(ws);
   k_bin_scan<<<1, 1024, 0, st>>>(ws);
-  if (chunks > 0) k_bin_scatter<<<chunks, kBinThreads, 0, st>>>(ws);
+  if (chunks > 0) k_bin_scatter<<<chunks, bin_threads_for(chunk_quads), 0, st>>>(ws);
   k_bin_sort<<<ds.sms, kSortThreads, kSortSmemBytes, st>>>(ws);
   const bool vtx_kernel = Q > 0 && vtx;
   if (ws.ordered && launch_ordered(ws, ds.sms * ds.ordered_blocks, st, false) != cudaSuccess) return LR_ERR_CUDA;
