@@ -263,6 +263,7 @@ struct OrderedBlock {
   const uint32_t *row_u, *row_l;
   int n, ox, oy;
   bool shapes;               // the bin holds other shapes than axis-parallel rectangles
+  bool bytes;                // the view wants 8-bit values
   __device__ __forceinline__ OrderedBlock(const Ws& ws, uint32_t n_general, uint32_t item) {
     const int lg = ws.bin_log2, bl = bin_hb_log2(lg) - 2, cl = bin_hb_cols_log2(lg) - 1, cols = bin_hb_cols(lg);
     const int bin_g = (int)ws.bin_order[n_general + (item >> bl)], blk = (int)(item & ((1u << bl) - 1u));
@@ -277,6 +278,7 @@ struct OrderedBlock {
     row_u = hb_row(ws, off, bin_g, n, hb);
     row_l = hb_row(ws, off, bin_g, n, hb + cols);
     shapes = (ws.bin_cursor[bin_g] & kBinShapes) != 0u;
+    bytes = V->out8 != nullptr;
     if (ox >= V->width || oy >= V->height || !tile_owned(*V, ox, oy)) V = nullptr;
   }
 };
@@ -287,7 +289,8 @@ struct OrderedBlock {
 // bin's list took longer than all the rest of the frame (400,000 particles at 960x540: 168 us
 // against 61 us, 2M at 1920x1080 295 against 207; cut from 4096 references on they took 231, since
 // the longest uncut lists then start late). Then a warp per block. With the alpha
-// threshold, whose stop is defined on the running product, always a warp per block.
+// threshold, whose stop is defined on the running product, and for views with 8-bit values, whose
+// rounding would show where a list was cut, always a warp per block.
 template <bool ATH>
 __global__ __launch_bounds__(kRasterThreads, LR_ORDERED_MIN_BLOCKS) void k_raster_ordered(Ws ws) {
   pdl_begin();
@@ -305,6 +308,17 @@ __global__ __launch_bounds__(kRasterThreads, LR_ORDERED_MIN_BLOCKS) void k_raste
   const uint32_t nlong = ATH || !run ? 0u : ws.ctrl->n_ordered_long << bl;
   unsigned long long frag_total = 0;
   auto draw = [&]() { return (uint32_t)min(atomicAdd(&ws.ctrl->ordered_head, 1ull), 0xFFFFFFF0ull); };
+  auto whole_block = [&](const OrderedBlock& B) {   // rectangles, by one warp
+    const int nw = (B.n + 31) >> 5;
+    BoxPixels<ATH> P;
+    P.init();
+    box_block<ATH>(P, ws.rec, B.refs, *B.V, B.row_u, B.row_l, nw, 0, nw, B.ox, B.oy, lane, cand, qc);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      frag_total += box_write(*B.V, B.ox + 2 * (lane & 7) + (i & 1), B.oy + 2 * (lane >> 3) + (i >> 1), P.st[i].r, P.st[i].g, P.st[i].b,
+                              P.st[i].T, P.cnt[i]);
+    box_xmask(*B.V, B.ox, B.oy, lane);
+  };
   uint32_t item = 0xFFFFFFFFu;         // warp 0: the first item past the CTA's
   while (nlong) {
     if (threadIdx.x == 0) s_item = draw();
@@ -312,7 +326,15 @@ __global__ __launch_bounds__(kRasterThreads, LR_ORDERED_MIN_BLOCKS) void k_raste
     item = s_item;
     if (item >= nlong) break;
     const OrderedBlock B(ws, n_general, item);
-    if (B.V && !B.shapes) {
+    const uint32_t blk = item & ((1u << bl) - 1u);
+    if (!B.shapes && B.bytes) {
+      // eight blocks of the bin (two of a 16-pixel bin), a warp each
+      const uint32_t it = item + warp;
+      if ((blk & 7u) == 0u && it >> bl == item >> bl) {
+        const OrderedBlock W(ws, n_general, it);
+        if (W.V) whole_block(W);
+      }
+    } else if (B.V && !B.shapes) {
       const int nw = (B.n + 31) >> 5, per = (nw + kRasterWarps - 1) / kRasterWarps;
       BoxPixels<ATH> P;
       P.init();
@@ -344,7 +366,7 @@ __global__ __launch_bounds__(kRasterThreads, LR_ORDERED_MIN_BLOCKS) void k_raste
         frag_total += box_write(*B.V, px, py, r, g, b, T, c);
         if (warp == 0) box_xmask(*B.V, B.ox, B.oy, lane);
       }
-    } else if (B.shapes && (item & ((1u << bl) - 1u) & 3u) == 0u) {
+    } else if (B.shapes && (blk & 3u) == 0u) {
       // four blocks of the bin (two of a 16-pixel bin) as eight 8x8 blocks, a warp each
       const uint32_t it = item + (warp >> 1);
       if (it >> bl == item >> bl) {
@@ -367,14 +389,7 @@ __global__ __launch_bounds__(kRasterThreads, LR_ORDERED_MIN_BLOCKS) void k_raste
     if (!B.V) continue;
     const int nw = (B.n + 31) >> 5;
     if (!B.shapes) {
-      BoxPixels<ATH> P;
-      P.init();
-      box_block<ATH>(P, ws.rec, B.refs, *B.V, B.row_u, B.row_l, nw, 0, nw, B.ox, B.oy, lane, cand, qc);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        frag_total += box_write(*B.V, B.ox + 2 * (lane & 7) + (i & 1), B.oy + 2 * (lane >> 3) + (i >> 1), P.st[i].r, P.st[i].g, P.st[i].b,
-                                P.st[i].T, P.cnt[i]);
-      box_xmask(*B.V, B.ox, B.oy, lane);
+      whole_block(B);
     } else {
 #pragma unroll 1
       for (int h = 0; h < 2 && B.ox + 8 * h < B.V->width; ++h)

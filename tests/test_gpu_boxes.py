@@ -100,3 +100,20 @@ def test_long_lists_of_other_shapes(lr, n, bin_size):
     xy = rng.uniform(0, [w, h], (n, 1, 2)) + rng.uniform(2.0, 9.0, (n, 1, 1)) * np.array([[0, -1], [1, 0], [0, 1], [-1, 0]])
     xy[: n // 2] = rng.uniform(0, 30, (n // 2, 1, 2)) + rng.uniform(2.0, 30.0, (n // 2, 1, 2)) * np.array([[0, 0], [1, 0], [1, 1], [0, 1]])
     check(lr, scene(xy, rng.uniform(1.0, 2.0, (n, 1)), rgba(rng, n, 0.01, 0.05), w, h), 1, bin_size=bin_size)
+
+
+@pytest.mark.parametrize("n", [900, 3000, 30000])
+@pytest.mark.parametrize("bin_size", [16, 32, 64])
+def test_long_lists_bytes(lr, n, bin_size):
+    # 8-bit values are those of the list blended in one go, as the hashing rasteriser blends it
+    rng = np.random.default_rng(n)
+    w, h = 75, 67
+    xy = boxes(rng, n, w, h, 1.0, 30.0)
+    s = scene(xy, rng.uniform(1.0, 2.0, (n, 1)), rgba(rng, n, 0.005, 0.05), w, h)
+    r = lr.Renderer(sorter_k=1, bin_size=bin_size)
+    d = lr.DeviceScene.from_scene(s)
+    a = r.render(d, w, h, rgba8=True, count=True)
+    b = r.render(d, w, h, rgba8=True, count=True, hash=True)
+    assert torch.equal(a["rgba8"], b["rgba8"]) and torch.equal(a["count"], b["count"])
+    assert torch.equal(a["rgba"], b["rgba"])
+    r.close()
