@@ -609,6 +609,13 @@ __host__ __device__ constexpr size_t raster_smem_bytes(bool vtx, bool bwd = fals
   return (size_t)kRasterWarps * batch_smem_warp(vtx, bwd, lit, k);
 }
 
+// q c - p with both operations rounded, as each corner's product has to be for the 8-bit values to be
+// those of corners weighted before they are subtracted.
+__device__ __forceinline__ float4 weighted_difference(float q, float4 c, float4 p) {
+  return make_float4(__fsub_rn(__fmul_rn(q, c.x), p.x), __fsub_rn(__fmul_rn(q, c.y), p.y),
+                     __fsub_rn(__fmul_rn(q, c.z), p.z), __fsub_rn(__fmul_rn(q, c.w), p.w));
+}
+
 // The record of covering triangle id (2 * quad + triangle of view V) into slot `lane` of the
 // batch: the depth key's two edge values at the block's first pixel centre (Ox, Oy), their
 // steps, its plane, and with colours carried (CARRY) the flat colour or the corner colours
@@ -654,14 +661,14 @@ __device__ __forceinline__ void setup_batch(const Ws& ws, const ViewDev& V, bool
     const float4 c0 = __ldg(cv + (size_t)cs * vi.x), c1 = __ldg(cv + (size_t)cs * vb), c2 = __ldg(cv + (size_t)cs * vc);
     const float4 p0 = make_float4(q_a * c0.x, q_a * c0.y, q_a * c0.z, q_a * c0.w);
     qc[lane] = p0;
-    qc[32 + lane] = make_float4(q_b * c1.x - p0.x, q_b * c1.y - p0.y, q_b * c1.z - p0.z, q_b * c1.w - p0.w);
-    qc[64 + lane] = make_float4(q_c * c2.x - p0.x, q_c * c2.y - p0.y, q_c * c2.z - p0.z, q_c * c2.w - p0.w);
+    qc[32 + lane] = weighted_difference(q_b, c1, p0);
+    qc[64 + lane] = weighted_difference(q_c, c2, p0);
     if (LIT && lit) {
       const float4 n0 = __ldg(cv + 2ull * vi.x + 1), n1 = __ldg(cv + 2ull * vb + 1), n2 = __ldg(cv + 2ull * vc + 1);
       const float4 o0 = make_float4(q_a * n0.x, q_a * n0.y, q_a * n0.z, 0.f);
       qc[96 + lane] = o0;
-      qc[128 + lane] = make_float4(q_b * n1.x - o0.x, q_b * n1.y - o0.y, q_b * n1.z - o0.z, 0.f);
-      qc[160 + lane] = make_float4(q_c * n2.x - o0.x, q_c * n2.y - o0.y, q_c * n2.z - o0.z, 0.f);
+      qc[128 + lane] = weighted_difference(q_b, make_float4(n1.x, n1.y, n1.z, 0.f), o0);
+      qc[160 + lane] = weighted_difference(q_c, make_float4(n2.x, n2.y, n2.z, 0.f), o0);
     }
   } else if (CARRY) {
     qc[lane] = __ldg(reinterpret_cast<const float4*>(V.col) + jl);
