@@ -103,7 +103,8 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
   const size_t o_cnt = o; o = up256(o + 4 * (size_t)nbins);
   const size_t o_off = o; o = up256(o + 4 * ((size_t)nbins + 1));
   const size_t o_cur = o; o = up256(o + 4 * (size_t)nbins);
-  const int chunk_quads = chunk_quads_for(Q), chunks = (int)((Q + chunk_quads - 1) / chunk_quads);
+  // (one chunk size, so that what fits the fixed array does not depend on how the binning splits)
+  const int chunk_quads = 2048, chunks = (int)((Q + chunk_quads - 1) / chunk_quads);
   const size_t o_span = o; o = up256(o + 8 * (size_t)chunks);
   const size_t o_ord = o; o = up256(o + 4 * (size_t)nbins);
   const size_t o_ovf = o; o = up256(o + 4 * (size_t)npix);
