@@ -36,33 +36,36 @@ WORKLOAD = "layers-1080p: 1920x1080, 32 wavy layers x 256x128 = 1,048,576 indexe
 # multiplies + 2 adds = 8, sorter = K compare/selects, blend = 8 fp32 ops
 OPS_PER_FRAG_BASE = 25
 # kernels launched per frame (one view): k_init (which also writes the view descriptor),
-# k_setup, k_bin_count, k_bin_scan, k_bin_scatter, k_bin_sort, k_bin_sort_big, k_raster,
-# k_overflow
-LAUNCHES_PER_FRAME = 9
+# k_setup, k_bin_count, k_bin_scan, k_bin_scatter, k_bin_sort, k_raster, k_overflow; flat views
+# also k_raster_ordered, before k_raster
+LAUNCHES_PER_FRAME = 8
 # DRAM bytes (read + write) per k_raster launch from ncu captures (profiles/), keyed by
 # (workload, K, carried colours), with the hash of the rasteriser sources they were taken
 # on: the figure is reported only while the kernel is unchanged.
 RASTER_TRAFFIC = {
     # (DRAM read + write bytes per launch, ncu smsp__issue_active, ncu smsp__inst_executed,
     #  source hash of the captured build)
-    ("layers", 1, False): (101_893_120, 0.7544, 348_696_989, "3e9f8ff852bad3aa"),      # profiles/k_raster_layers1080p.md
-    ("particles", 1, False): (383_102_464, 0.6758, 847_920_159, "3e9f8ff852bad3aa"),  # profiles/k_raster_particles1080p.md
+    ("layers", 1, False): (101_276_000, 0.7009, 265_736_245, "b9ecf6cfba2fb4fc"),      # profiles/k_raster_layers1080p.md
+    # (k_raster_ordered, which does not depend on K: profiles/k_raster_ordered_particles1080p.md)
+    ("particles", 1, False): (360_786_000, 0.6195, 151_340_566, "b9ecf6cfba2fb4fc"),
+    ("particles", 2, False): (360_786_000, 0.6195, 151_340_566, "b9ecf6cfba2fb4fc"),
+    ("particles", 3, False): (360_786_000, 0.6195, 151_340_566, "b9ecf6cfba2fb4fc"),
 }
 # the same for the rasteriser's variants and the multisample resolve on the layer frame
 # (K = 1): (DRAM bytes per launch, issue-slot share, warp instructions, kernel us, hash)
 VARIANT_CAPTURES = {
-    "alpha_threshold": (93_937_920, 0.7421, 273_373_076, 300.6, "3e9f8ff852bad3aa"),   # profiles/k_raster_alpha_layers1080p.md
-    "lit": (116_687_360, 0.5619, 422_811_933, 605.7, "3e9f8ff852bad3aa"),               # profiles/k_raster_lit_layers1080p.md
-    "msaa_resolve": (149_222_923, 0.2601, 7_452_000, 26.6, "3e9f8ff852bad3aa"),         # profiles/k_resolve_msaa4_layers1080p.md
+    "alpha_threshold": (94_906_000, 0.6501, 225_990_913, 283.4, "b9ecf6cfba2fb4fc"),   # profiles/k_raster_alpha_layers1080p.md
+    "lit": (115_487_000, 0.6383, 319_002_729, 406.4, "b9ecf6cfba2fb4fc"),               # profiles/k_raster_lit_layers1080p.md
+    "msaa_resolve": (149_758_000, 0.2631, 7_452_000, 27.0, "b9ecf6cfba2fb4fc"),         # profiles/k_resolve_msaa4_layers1080p.md
 }
-RASTER_SOURCES = ("lr_raster.cuh", "lr_common.cuh")
+RASTER_SOURCES = ("lr_raster.cuh", "lr_ordered.cu", "lr_common.cuh")
 LANES_PER_SM_CLK = 128
 # the autotuner's candidates for the timed workloads: sorter capacity, bin size, rasteriser
 # CTAs per SM (0 = the occupancy limit)
 TUNE_KS = (1, 2, 3)
 TUNE_BINS = (16, 32, 64)
 TUNE_CTAS = (0, 2)
-TUNE_BLOCKS = (4, 8)
+TUNE_BLOCKS = (4,)
 TUNE_SHARED = (False, True)
 
 
@@ -808,7 +811,7 @@ def run_gpu(args):
                 "serial_ms_per_step": round(e2e_serial_ms, 4)},
         "served_stream": serving,
         "differentiable": differentiable,
-        "gpu_launches": LAUNCHES_PER_FRAME * args.steps,
+        "gpu_launches": (LAUNCHES_PER_FRAME + (scene.color_mode == P.LR_COLOR_FLAT)) * args.steps,
         "clocks": clocks,
     }
     if peaks:
@@ -823,8 +826,8 @@ def run_profile(args):
     baseline. --variant picks the rasteriser form: exact (the benchmark's), alpha (the
     opt-in alpha threshold), lit (lit per-vertex colours on the layer scene) or msaa (4
     samples per pixel, ending in k_resolve). Kernel launch order per exact frame: k_init,
-    k_setup, k_bin_count, k_bin_scan, k_bin_scatter, k_bin_sort, k_bin_sort_big, k_raster,
-    k_overflow."""
+    k_setup, k_bin_count, k_bin_scan, k_bin_scatter, k_bin_sort, k_raster_ordered (flat views),
+    k_raster, k_overflow."""
     import torch
 
     import paper_2405_13364_gb300 as P

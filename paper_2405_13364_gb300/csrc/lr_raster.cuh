@@ -34,14 +34,13 @@
 // Sort keys are (float bits of key) << 32 | (2 * quad + triangle): distinct per pixel, so
 // the per-pixel order is total and the result is unique.
 //
-// What bounds it and what it took (K = 1, 1920x1080, kernel times): on 1M wavy quads with
-// vertex colours the shared-memory and gather wavefronts (80% of the L1 data pipe; a 16-byte
-// load per lane costs four), 62% of issue slots; against setting up both triangles of each
-// candidate with a binary search per edge and row, 349M -> 253M warp instructions and
-// 375 -> 328 us. On 2M particles, 60% of issue slots and the gathers of scattered records;
-// 848M -> 372M instructions, 1005 -> 506 us. With normals 602 -> 416 us, with the alpha
-// threshold on the particles 389 -> 268 us, a batch of mixed views at K = 3 2040 -> 911 us,
-// 100k scattered parallelograms with a few screen-filling ones 117 -> 66 us.
+// What bounds it and what it took (1920x1080, kernel times): at K = 1 on 1M wavy quads with vertex
+// colours the shared-memory and gather wavefronts (81% of the L1 data pipe; a 16-byte load per lane
+// costs four) and 70% of issue slots together; against setting up both triangles of each candidate
+// with a binary search per edge and row, 349M -> 266M warp instructions and 375 -> 307 us. With
+// normals 602 -> 402 us, six mixed views at K = 3 2040 -> 692, 100k
+// scattered parallelograms with a few screen-filling ones 117 -> 58. Bins whose list is already in
+// every pixel's order are left to k_raster_ordered.
 #pragma once
 
 #include "lr_common.cuh"
@@ -56,8 +55,8 @@ constexpr unsigned long long kSent = ~0ull;
 constexpr int kRasterThreads = 256;
 // Resident CTAs per SM requested from the compiler: 3 caps registers at 80 per thread (24 warps
 // per SM), 4 at 64. Neither spills in the forward kernels up to K = 3. With four the layer frame
-// took 307 instead of 315 us, flat layers at K = 3 154 instead of 168; with three the particle frame 275 instead of 309, the batch of mixed views at
-// K = 3 833 instead of 868, lit layers 406 instead of 422, flat layers with the alpha threshold
+// took 307 instead of 315 us, flat layers at K = 3 154 instead of 168; with three the batch of mixed
+// views at K = 3 833 instead of 868, lit layers 406 instead of 422, flat layers with the alpha threshold
 // 217 instead of 225. The backward's shared memory holds three.
 __host__ __device__ constexpr int raster_min_blocks(int k, bool vtx, bool bwd, bool ath, bool lit) {
   if (lit || ath || k > 3) return 3;
