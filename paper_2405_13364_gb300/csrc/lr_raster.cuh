@@ -54,14 +54,14 @@ constexpr uint32_t kTriWide = 256u;
 constexpr unsigned long long kSent = ~0ull;
 constexpr int kRasterThreads = 256;
 // Resident CTAs per SM requested from the compiler: 3 caps registers at 80 per thread (24 warps
-// per SM), 4 at 64. Neither spills in the forward kernels up to K = 3. With four the layer frame
-// took 307 instead of 315 us, flat layers at K = 3 154 instead of 168; with three the batch of mixed
-// views at K = 3 833 instead of 868, lit layers 406 instead of 422, flat layers with the alpha threshold
-// 217 instead of 225. The backward's shared memory holds three.
-__host__ __device__ constexpr int raster_min_blocks(int k, bool vtx, bool bwd, bool ath, bool lit) {
-  if (lit || ath || k > 3) return 3;
-  if (bwd) return 3;
-  return vtx ? (k == 1 ? 4 : 3) : (k == 1 ? 3 : 4);
+// per SM), 4 at 64; neither spills in the forward kernels up to K = 3. Four where they fit: against
+// three the layer frame took 307 instead of 315 us, 200,000 parallelograms at K = 1 143 instead of 148,
+// flat layers at K = 3 154 instead of 168, with the alpha threshold at K = 1, 2, 3 135, 156, 172 instead of
+// 145, 174, 184, layers with it 164 instead of 172. With three the batch of mixed views at K = 3 took 833
+// instead of 868, lit layers 406 instead of 422; the shared memory of the parked colours, of lit
+// colours and of the backward holds three.
+__host__ __device__ constexpr int raster_min_blocks(int k, bool vtx, bool bwd, bool lit) {
+  return lit || bwd || k > 3 || (vtx && k > 1) ? 3 : 4;
 }
 constexpr int kRasterWarps = kRasterThreads / 32;
 constexpr int kOvfThreads = 128;
@@ -721,7 +721,7 @@ __device__ __forceinline__ float4 shade(const float4* qc, int p, bool flat_view,
 // pixel of the half-block still blending. LIT: the colour-carrying variant that also
 // shades lit views (per-vertex normals, one directional light).
 template <int K, bool VTX, bool BWD, bool HASH, bool ATH = false, bool LIT = false>
-__global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, ATH, LIT)) void k_raster(Ws ws) {
+__global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, LIT)) void k_raster(Ws ws) {
   // Behind k_raster_ordered (kOrderedOverlap) it waits at its end, not here: k_raster_ordered's CTAs
   // let it launch once they have seen the sort complete, it reads nothing that k_raster_ordered
   // writes and writes other pixels, and what follows still waits for both.
