@@ -54,7 +54,7 @@ RASTER_TRAFFIC = {
 # the same for the rasteriser's variants and the multisample resolve on the layer frame
 # (K = 1): (DRAM bytes per launch, issue-slot share, warp instructions, kernel us, hash)
 VARIANT_CAPTURES = {
-    "alpha_threshold": (94_906_000, 0.6501, 225_990_913, 283.4, "7cb1aac2c7011f52"),   # profiles/k_raster_alpha_layers1080p.md
+    "alpha_threshold": (95_037_000, 0.7181, 234_664_928, 268.4, "7cb1aac2c7011f52"),   # profiles/k_raster_alpha_layers1080p.md
     "lit": (115_487_000, 0.6383, 319_002_729, 406.4, "7cb1aac2c7011f52"),               # profiles/k_raster_lit_layers1080p.md
     "msaa_resolve": (149_758_000, 0.2631, 7_452_000, 27.0, "7cb1aac2c7011f52"),         # profiles/k_resolve_msaa4_layers1080p.md
 }
