@@ -40,7 +40,7 @@ cudaError_t launch_overflow(bool bwd, const Ws& ws, int grid, cudaStream_t st, b
 
 #define LR_DECLARE_RASTER(KK)                                                                     \
   cudaError_t prepare_raster_##KK(int* blocks_flat, int* blocks_vtx, int* blocks_bwd, int* blocks_lit); \
-  cudaError_t launch_raster_##KK(int mode, const Ws& ws, int grid, cudaStream_t st);
+  cudaError_t launch_raster_##KK(int mode, const Ws& ws, int grid, cudaStream_t st, bool pdl);
 LR_DECLARE_RASTER(1)
 LR_DECLARE_RASTER(2)
 LR_DECLARE_RASTER(3)
@@ -62,8 +62,9 @@ __global__ void k_write_views(ViewChunk chunk, ViewDev* dst) {
 }
 
 typedef cudaError_t (*PrepareFn)(int*, int*, int*, int*);
-typedef cudaError_t (*LaunchFn)(int, const Ws&, int, cudaStream_t);   // mode 0 flat, 1 colours, 2 backward
+typedef cudaError_t (*LaunchFn)(int, const Ws&, int, cudaStream_t, bool);   // mode 0 flat, 1 colours, 2 backward
 typedef cudaError_t (*PrepareStripFn)(int*, int*);
+typedef cudaError_t (*LaunchStripFn)(int, const Ws&, int, cudaStream_t);
 
 // A sorter capacity's rasterisers: the one of lr_raster.cuh (every mode) and, for K <= 3, the
 // strip form (forward exact renders, flat or carried colours, with or without the hash).
@@ -72,7 +73,7 @@ struct RasterVariant {
   PrepareFn prepare;
   LaunchFn launch;
   PrepareStripFn prepare_strip;   // the per-strip shared set-up (lr_raster_strip.cuh)
-  LaunchFn launch_strip;
+  LaunchStripFn launch_strip;
 };
 
 static const RasterVariant kVariants[] = {
@@ -565,7 +566,6 @@ static lr_status launch_sequence(lr_ctx* ctx, const Prepared& P, cudaStream_t st
   ws.ordered = flat_bins > 0 && !bwd && !P.any_hash && !strip && !L.cursors;
   const int n_views = ws.n_views;
   const bool pdl = ctx->pdl_override >= 0 ? ctx->pdl_override != 0 : (ctx->cfg.flags & LR_FLAG_NO_PDL) == 0;
-  if (ws.ordered && pdl) ws.ordered = kOrderedOverlap;
   rec(ctx, timed, 0, st);
   // the first kViewsPerLaunch descriptors travel with k_init, further ones with k_write_views
   ViewChunk chunk;
@@ -607,7 +607,9 @@ static lr_status launch_sequence(lr_ctx* ctx, const Prepared& P, cudaStream_t st
     e = VS.v->launch_strip(mode, ws, ctx->sms * (carry ? VS.vtx_s : VS.flat_s), st);
   } else {
     const int rblocks = bwd ? VS.bwd : (P.any_lit ? VS.lit : (carry ? VS.vtx : VS.flat));
-    e = VS.v->launch(mode, ws, ctx->sms * rblocks, st);
+    // programmatic only behind k_raster_ordered: its persistent CTAs, placed early next to the bin
+    // sort's, measured slower
+    e = VS.v->launch(mode, ws, ctx->sms * rblocks, st, pdl && ws.ordered);
   }
   if (e != cudaSuccess) return cuda_fail(ctx, e, "raster launch");
   rec(ctx, timed, 6, st);

@@ -127,11 +127,13 @@ struct ViewChunk {
   int first, count;
 };
 
-// Programmatic dependent launch (sm_90 and later). The pipeline's kernels (all but the
-// rasteriser) are launched with programmatic stream serialisation (launch_pdl), so each
-// may be scheduled while its predecessor in the stream drains; every kernel first waits
+// Programmatic dependent launch (sm_90 and later). The pipeline's kernels (k_raster only
+// behind k_raster_ordered) are launched with programmatic stream serialisation (launch_pdl), so
+// each may be scheduled while its predecessor in the stream drains; every kernel first waits
 // for its predecessor's completion and memory (griddepcontrol.wait: nothing of the kernel
-// touches memory before it), then lets its own successor begin launching. A kernel
+// touches memory before it), then lets its own successor begin launching. The wait is what
+// makes an earlier grid's writes visible: a successor is let go before its predecessor's
+// memory is flushed, whatever the predecessor itself has waited for. A kernel
 // launched without the attribute passes both instructions at once. Contexts that render
 // on several streams at once turn it off (LR_FLAG_NO_PDL): early-placed waiting CTAs would
 // hold resources the other streams' kernels need.
@@ -238,8 +240,6 @@ __device__ __forceinline__ QuadRec load_rec(const int4* rec, uint32_t i) {
   return r;
 }
 
-constexpr int kOrderedOverlap = 2;
-
 // bin_cursor: the bin holds a reference to a quad that is not of constant depth, one that is no
 // axis-parallel rectangle
 constexpr uint32_t kBinDepths = 1u, kBinShapes = 2u;
@@ -254,8 +254,7 @@ struct Ws {
   long long total_pix;
   long long refs_cap;
   int cursors;               // a view has more bins than the shared counters hold
-  int ordered;               // k_raster_ordered runs (a forward render without hashes, with flat
-                             // views): 1, or kOrderedOverlap where k_raster may run beside it
+  int ordered;               // k_raster_ordered runs (a forward render without hashes, with flat views)
   int chunk_quads;           // quads per binning CTA (chunk_quads_for)
   int bin_log2;              // bins of 2^bin_log2 x 2^bin_log2 pixels (the same for every view)
   int4* rec;                 // [4 * total_quads]: the 64-byte quad record (QuadRec)

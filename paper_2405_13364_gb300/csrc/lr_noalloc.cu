@@ -35,7 +35,7 @@ __global__ void k_bin_scan(Ws ws);
 __global__ void k_bin_scatter(Ws ws);
 __global__ void k_bin_sort(Ws ws);
 cudaError_t prepare_raster_3(int* blocks_flat, int* blocks_vtx, int* blocks_bwd, int* blocks_lit);
-cudaError_t launch_raster_3(int mode, const Ws& ws, int grid, cudaStream_t st);
+cudaError_t launch_raster_3(int mode, const Ws& ws, int grid, cudaStream_t st, bool pdl);
 cudaError_t prepare_ordered(int* blocks_per_sm);
 cudaError_t launch_ordered(const Ws& ws, int grid, cudaStream_t st, bool pdl);
 cudaError_t overflow_occupancy(int* blocks_per_sm);
@@ -223,7 +223,7 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
   k_bin_sort<<<ds.sms, kSortThreads, kSortSmemBytes, st>>>(ws);
   const bool vtx_kernel = Q > 0 && vtx;
   if (ws.ordered && launch_ordered(ws, ds.sms * ds.ordered_blocks, st, false) != cudaSuccess) return LR_ERR_CUDA;
-  if (launch_raster_3(vtx_kernel ? 1 : 0, ws, ds.sms * (vtx_kernel ? ds.blocks_vtx : ds.blocks_flat), st) != cudaSuccess)
+  if (launch_raster_3(vtx_kernel ? 1 : 0, ws, ds.sms * (vtx_kernel ? ds.blocks_vtx : ds.blocks_flat), st, false) != cudaSuccess)
     return LR_ERR_CUDA;
   if (launch_overflow(false, ws, ds.sms * ds.ovf_blocks, st, false) != cudaSuccess) return LR_ERR_CUDA;
   if (device_status) k_noalloc_status<<<1, 1, 0, st>>>(ws.ctrl, device_status);

@@ -722,11 +722,7 @@ __device__ __forceinline__ float4 shade(const float4* qc, int p, bool flat_view,
 // shades lit views (per-vertex normals, one directional light).
 template <int K, bool VTX, bool BWD, bool HASH, bool ATH = false, bool LIT = false>
 __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, LIT)) void k_raster(Ws ws) {
-  // Behind k_raster_ordered (kOrderedOverlap) it waits at its end, not here: k_raster_ordered's CTAs
-  // let it launch once they have seen the sort complete, it reads nothing that k_raster_ordered
-  // writes and writes other pixels, and what follows still waits for both.
-  if (ws.ordered != kOrderedOverlap) asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char smem[];
   // the sorter carries each fragment's colour (backward: the batch holds its triangles' colours)
   constexpr bool kCarry = VTX || K == 1 || BWD;
@@ -1028,7 +1024,6 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, LIT)
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) frag_total += __shfl_xor_sync(0xffffffffu, frag_total, o);
   if (lane == 0 && frag_total) atomicAdd(&ws.ctrl->fragments, frag_total);
-  if (ws.ordered == kOrderedOverlap) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace lr
@@ -1070,11 +1065,8 @@ __global__ __launch_bounds__(kRasterThreads, raster_min_blocks(K, VTX, BWD, LIT)
   }                                                                                           \
   /* mode: 0 flat colours, 1 colours in the sorter, 2 backward; + 4: coverage hash;        \
      + 8: alpha threshold (modes 8 and 9 only); 17: colours in the sorter with lit views */   \
-  cudaError_t launch_raster_##KK(int mode, const Ws& ws, int grid, cudaStream_t st) {         \
+  cudaError_t launch_raster_##KK(int mode, const Ws& ws, int grid, cudaStream_t st, bool pdl) { \
     const size_t sf = raster_smem_bytes(false, false, false, KK), sv = raster_smem_bytes(true, false, false, KK);                 \
-    /* a plain launch but behind k_raster_ordered: with programmatic serialisation the        \
-       persistent CTAs, placed early next to the bin sort's, measured slower */                \
-    const bool pdl = ws.ordered == kOrderedOverlap;                                           \
     const dim3 g(grid), t(kRasterThreads);                                                    \
     switch (mode) {                                                                           \
       case 1: return launch_pdl(pdl, k_raster<KK, true, false, false>, g, t, sv, st, ws);     \
