@@ -563,7 +563,9 @@ static lr_status launch_sequence(lr_ctx* ctx, const Prepared& P, cudaStream_t st
   long long flat_bins = 0;   // bins that k_raster_ordered may get
   for (const ViewDev& v : P.vd)
     if (v.color_mode == LR_COLOR_FLAT) flat_bins += (long long)v.nbx * v.nby;
-  ws.ordered = flat_bins > 0 && !bwd && !P.any_hash && !strip && !L.cursors;
+  // (a CTA for every eight 16x8 blocks, a bin of 32 pixels, at most)
+  const int ordered_grid = (int)std::min((long long)ctx->sms * ctx->ordered_blocks, flat_bins << std::max(0, 2 * (ctx->bin_log2 - 5)));
+  ws.ordered = !bwd && !P.any_hash && !strip && !L.cursors ? ordered_grid * kRasterWarps : 0;
   const int n_views = ws.n_views;
   const bool pdl = ctx->pdl_override >= 0 ? ctx->pdl_override != 0 : (ctx->cfg.flags & LR_FLAG_NO_PDL) == 0;
   rec(ctx, timed, 0, st);
@@ -598,10 +600,7 @@ static lr_status launch_sequence(lr_ctx* ctx, const Prepared& P, cudaStream_t st
   launch_pdl(pdl, k_bin_sort, dim3(ctx->sms), dim3(kSortThreads), kSortSmemBytes, st, ws);
   rec(ctx, timed, 5, st);
   cudaError_t e = cudaSuccess;
-  // (a CTA for every eight 16x8 blocks, a bin of 32 pixels, at most)
-  if (ws.ordered)
-    e = launch_ordered(ws, (int)std::min((long long)ctx->sms * ctx->ordered_blocks, flat_bins << std::max(0, 2 * (ctx->bin_log2 - 5))),
-                       st, pdl);
+  if (ws.ordered) e = launch_ordered(ws, ordered_grid, st, pdl);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "raster launch");
   if (strip) {
     e = VS.v->launch_strip(mode, ws, ctx->sms * (carry ? VS.vtx_s : VS.flat_s), st);

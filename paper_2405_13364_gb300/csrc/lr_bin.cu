@@ -221,6 +221,7 @@ __global__ __launch_bounds__(1024) void k_bin_scan(Ws ws) {
   pdl_begin();
   constexpr int kClasses = 32;       // (a view has fewer than 2^30 quads)
   __shared__ unsigned long long warp_sums[32];
+  __shared__ uint32_t warp_ordered[32];   // references of k_raster_ordered's bins
   __shared__ uint32_t cls_count[2 * kClasses], cls_base[2 * kClasses];
   __shared__ uint8_t cls_of[kHistSmemBins];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -233,6 +234,7 @@ __global__ __launch_bounds__(1024) void k_bin_scan(Ws ws) {
     return (c ? 32 - __clz(c) : 0) + (ordered ? kClasses : 0);
   };
   unsigned long long nonempty = 0, high = 0, mx = 0, sum = 0;
+  uint32_t ordered_sum = 0;            // (32 bits: more references than that overflow)
   const int per = (n + 1023) >> 10, i0 = tid * per, i1 = min(n, i0 + per);
   for (int i = i0; i < i1; i += 4) {
     uint32_t c[4], f[4];
@@ -249,6 +251,7 @@ __global__ __launch_bounds__(1024) void k_bin_scan(Ws ws) {
       high += c[u] >= (uint32_t)kSortSmemCap;
       mx = c[u] > mx ? c[u] : mx;
       const int cls = class_of(i + u, c[u], f[u]);
+      if (cls >= kClasses) ordered_sum += c[u];
       if (i + u < kHistSmemBins) cls_of[i + u] = (uint8_t)cls;
       // one shared-memory atomic per warp and size class (most bins of a warp share one)
       const unsigned act = __activemask();
@@ -262,7 +265,8 @@ __global__ __launch_bounds__(1024) void k_bin_scan(Ws ws) {
     const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
-  if (lane == 31) warp_sums[wid] = x;
+  ordered_sum = __reduce_add_sync(0xffffffffu, ordered_sum);
+  if (lane == 31) { warp_sums[wid] = x; warp_ordered[wid] = ordered_sum; }
   __syncthreads();
   if (wid == 0) {
     unsigned long long s = warp_sums[lane];
@@ -312,15 +316,20 @@ __global__ __launch_bounds__(1024) void k_bin_scan(Ws ws) {
     const uint32_t general = __shfl_sync(0xffffffffu, gi, 31);
     cls_base[k] = gi - g;
     cls_base[kClasses + k] = general + oi - o;
-    // long lists of k_raster_ordered: from 1024 references (class 11) and 3/8 of a warp's share
-    const unsigned long long share = total * 3 / 4864;
-    const uint32_t n_long = __reduce_max_sync(0xffffffffu, k >= 11 && (1ull << (k - 1)) >= share ? oi : 0u);
+    // long lists of k_raster_ordered
+    const unsigned long long blocks = (unsigned long long)__reduce_add_sync(0xffffffffu, warp_ordered[lane]) * (unsigned)(bin_hb(ws.bin_log2) / 4);
+    const unsigned long long warps8 = 8ull * (unsigned)max(ws.ordered, 1), least = k > 0 ? 1ull << (k - 1) : 0ull;
+    const bool is_long = least >= kOrderedLong && least * warps8 >= blocks * kOrderedLongShare8;
+    const bool is_longest = is_long && least >= kOrderedLongest && least * warps8 >= blocks * kOrderedLongestShare8;
+    const uint32_t n_long = __reduce_max_sync(0xffffffffu, is_long ? oi : 0u);
+    const uint32_t n_longest = __reduce_max_sync(0xffffffffu, is_longest ? oi : 0u);
     if (k == 12) ws.ctrl->high_general = gi;       // from 2048 references
     if (k == 1) ws.ctrl->nonempty_general = gi;
     if (lane == 0) {
       ws.ctrl->n_general = general;
       ws.ctrl->raster_items = (unsigned long long)general * bin_hb(ws.bin_log2);
       ws.ctrl->n_ordered_long = n_long;
+      ws.ctrl->n_ordered_longest = n_longest;
     }
   }
   __syncthreads();

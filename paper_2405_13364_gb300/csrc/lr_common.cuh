@@ -182,12 +182,11 @@ struct Ctrl {
   // bins that k_raster takes (first in bin_order; those of k_raster_ordered follow): all, with at
   // least kSortSmemCap references, non-empty
   uint32_t n_general, high_general, nonempty_general;
-  // k_raster_ordered's bins with long lists: from 1024 references, and from 3/8 of a warp's
-  // share of all lists' 16x8 blocks (4864 warps, eight blocks a bin): with one warp per block the
-  // frame would wait for them
+  // k_raster_ordered's bins with long lists (kOrderedLong), taken by smaller blocks
   uint32_t n_ordered_long;
   unsigned long long ordered_head;      // k_raster_ordered's queue
-  unsigned long long pad;
+  uint32_t n_ordered_longest;           // of the n_ordered_long, those taken by half-blocks
+  uint32_t pad;
 };
 
 // The per-quad record written by k_setup and gathered by every later stage, 64 bytes so
@@ -240,6 +239,14 @@ __device__ __forceinline__ QuadRec load_rec(const int4* rec, uint32_t i) {
   return r;
 }
 
+// k_raster_ordered's blocks by the length of a bin's list (in powers of two): long from 1024 references
+// and 3/8 of a warp's share of its bins' 16x8 blocks, longest from 2048 and twice a share. 2M particles
+// at 1920x1080: 205 us from 3/8, 207 from 1/4; with half-blocks from 3/8 on 238, without the limit of
+// 1024 300,000 at 2560x1440 take 67 instead of 63. 400,000 at 960x540 with half-blocks from two shares 78
+// us, from three 84, from six 98.
+constexpr int kOrderedLong = 1024, kOrderedLongShare8 = 3;
+constexpr int kOrderedLongest = 2048, kOrderedLongestShare8 = 16;
+
 // bin_cursor: the bin holds a reference to a quad that is not of constant depth, one that is no
 // axis-parallel rectangle
 constexpr uint32_t kBinDepths = 1u, kBinShapes = 2u;
@@ -254,7 +261,8 @@ struct Ws {
   long long total_pix;
   long long refs_cap;
   int cursors;               // a view has more bins than the shared counters hold
-  int ordered;               // k_raster_ordered runs (a forward render without hashes, with flat views)
+  int ordered;               // k_raster_ordered runs (a forward render without hashes, with flat views):
+                             // its warps, else 0
   int chunk_quads;           // quads per binning CTA (chunk_quads_for)
   int bin_log2;              // bins of 2^bin_log2 x 2^bin_log2 pixels (the same for every view)
   int4* rec;                 // [4 * total_quads]: the 64-byte quad record (QuadRec)

@@ -195,7 +195,8 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
   ws.chunk_quads = chunk_quads;
   ws.bin_log2 = kBinLog2Default;
   ws.cursors = nbins > kHistSmemBins;
-  ws.ordered = !(Q > 0 && vtx) && !ws.cursors;
+  const int ordered_grid = ds.sms * ds.ordered_blocks;
+  ws.ordered = !(Q > 0 && vtx) && !ws.cursors ? ordered_grid * kRasterWarps : 0;
   ws.rec = reinterpret_cast<int4*>(base + o_rec);
   ws.rec_rect = reinterpret_cast<uint2*>(base + o_rect);
   ws.rec_info = reinterpret_cast<uint32_t*>(base + o_info);
@@ -222,7 +223,7 @@ extern "C" lr_status lr_render_noalloc(const lr_quads* quads, const lr_camera* c
   if (chunks > 0) k_bin_scatter<<<chunks, bin_threads_for(chunk_quads), 0, st>>>(ws);
   k_bin_sort<<<ds.sms, kSortThreads, kSortSmemBytes, st>>>(ws);
   const bool vtx_kernel = Q > 0 && vtx;
-  if (ws.ordered && launch_ordered(ws, ds.sms * ds.ordered_blocks, st, false) != cudaSuccess) return LR_ERR_CUDA;
+  if (ws.ordered && launch_ordered(ws, ordered_grid, st, false) != cudaSuccess) return LR_ERR_CUDA;
   if (launch_raster_3(vtx_kernel ? 1 : 0, ws, ds.sms * (vtx_kernel ? ds.blocks_vtx : ds.blocks_flat), st, false) != cudaSuccess)
     return LR_ERR_CUDA;
   if (launch_overflow(false, ws, ds.sms * ds.ovf_blocks, st, false) != cudaSuccess) return LR_ERR_CUDA;

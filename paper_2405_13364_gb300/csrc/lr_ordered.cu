@@ -8,7 +8,6 @@
 #include "lr_raster.cuh"
 
 namespace lr {
-
 // Bins that hold only flat-colour quads of one depth each: the bin's list, sorted by that depth with the tie
 // rule, is every pixel's exact fragment order. A warp takes an 8x8 block, the half-blocks hb and
 // hb_l below it, with two pixels per lane, one above the other: a record read from shared
@@ -125,41 +124,54 @@ __device__ __forceinline__ unsigned const_block(const int4* recs, const unsigned
 }
 
 // A bin of such quads that are axis-parallel rectangles too (kRecBox: particles, upright
-// billboards). A warp takes 16x8 pixels, four half-blocks, with 2x2 pixels per lane. Coverage is
-// separable: a candidate's columns and rows are one word, one transpose across the warp turns 32
-// of them into a word per column and per row, and a pixel's candidates are the intersection of
-// two. The loop runs over the candidates of a lane's four pixels together, so that its overhead and
-// the colour's load serve up to four fragments. Records' corners and colours are loaded one round
-// ahead, the references two. Nearly every candidate covers a pixel, so there is no ring.
-// 2M particles at 1920x1080: 274 us by 8x8 blocks with a mask per candidate, 295 us so as a branch of
-// k_raster.
-// The four pixels of a lane, (cx, cy), (cx + 1, cy) and the two below.
-template <bool ATH>
+// billboards). A warp takes 16x8 pixels, four half-blocks, with 2x2 pixels per lane (NP = 4), an 8x8
+// block with 1x2 (NP = 2) or a half-block (NP = 1). Coverage is separable: a candidate's columns and
+// rows are one word, one transpose across the warp turns 32 of them into a word per column and per
+// row, and a pixel's candidates are the intersection of two. The loop runs over the candidates of a
+// lane's pixels together, so that its overhead and the colour's load serve up to four fragments.
+// Records' corners and colours are loaded one round ahead, the references two (further ahead measured
+// no faster). Nearly every candidate covers a pixel, so there is no ring.
+template <bool ATH, int NP>
 struct BoxPixels {
-  PixelState<1, true, ATH> st[4];
-  uint32_t cnt[4];
+  PixelState<1, true, ATH> st[NP];
+  uint32_t cnt[NP];
+  // the lane's pixel i in the block
+  static __device__ __forceinline__ int px(int lane, int i) { return NP == 4 ? 2 * (lane & 7) + (i & 1) : lane & 7; }
+  static __device__ __forceinline__ int py(int lane, int i) {
+    return NP == 4 ? 2 * (lane >> 3) + (i >> 1) : (NP == 2 ? 2 * (lane >> 3) + i : lane >> 3);
+  }
   __device__ __forceinline__ void init() {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < NP; ++i) {
       st[i].init();
       cnt[i] = 0;
     }
   }
 };
-// Blends the references of bitmap words [w0, w1).
-template <bool ATH>
-__device__ __forceinline__ void box_block(BoxPixels<ATH>& P, const int4* recs, const unsigned long long* refs, const ViewDev& V,
-                                          const uint32_t* row_u, const uint32_t* row_l, int nw, int w0, int w1, int ox,
-                                          int oy, int lane, uint16_t* cand, float4* qc) {
-  const int cx = 2 * (lane & 7), cy = 2 * (lane >> 3);
+// With this many candidates of a round on one lane, the round's 32 colours are all read in turn, by the
+// whole warp from one address and ahead of their use, instead of each lane finding its own: no
+// chain from bit search to load to blend. 2M particles at 1920x1080: 264 us without for NP = 1, 235 so;
+// 225 and 205 for NP = 2. (Where a lane has four pixels, too few of the 32 meet any.)
+__host__ __device__ constexpr int box_dense(int np) { return np == 1 ? 10 : 14; }
+// Blends the bin's references that the bitmap rows list: row_u and the one behind it the upper two
+// half-blocks, row_l and the one behind it the lower two; NP = 2: row_u and row_l; NP = 1: row_u.
+template <bool ATH, int NP>
+__device__ __forceinline__ void box_block(BoxPixels<ATH, NP>& P, const int4* recs, const unsigned long long* refs, const ViewDev& V,
+                                          const uint32_t* row_u, const uint32_t* row_l, int nw, int ox, int oy, int lane,
+                                          uint16_t* cand, float4* qc) {
+  constexpr int BW = NP == 4 ? 16 : 8, BH = NP == 1 ? 4 : 8;
+  const int cx = P.px(lane, 0), cy = P.py(lane, 0);
   const uint32_t* ref_lo = reinterpret_cast<const uint32_t*>(refs);   // low words
   const float4* colors = reinterpret_cast<const float4*>(V.col);
   const uint32_t quad_base = (uint32_t)V.quad_base;
-  // (row_u, row_l: the left half-blocks of the upper and the lower pair)
-  int g = w0 - 32, r0 = 0, total = 0;
+  int g = -32, r0 = 0, total = 0;
   uint32_t words = 0;                 // the next window's bitmap words
   auto load_words = [&](int w) {
-    words = w < w1 ? (__ldg(row_u + w) | __ldg(row_u + nw + w) | __ldg(row_l + w) | __ldg(row_l + nw + w)) : 0u;
+    words = 0u;
+    if (w >= nw) return;
+    words = __ldg(row_u + w);
+    if (NP > 1) words |= __ldg(row_l + w);
+    if (NP == 4) words |= __ldg(row_u + nw + w) | __ldg(row_l + nw + w);
   };
   load_words(g + 32 + lane);
   constexpr uint32_t kNone = 0xFFFFFFFFu;
@@ -167,7 +179,7 @@ __device__ __forceinline__ void box_block(BoxPixels<ATH>& P, const int4* recs, c
     rec = kNone;
     while (r0 >= total) {
       g += 32;
-      if (g >= w1) return false;
+      if (g >= nw) return false;
       const uint32_t cur = words;
       load_words(g + 32 + lane);
       total = list_bits(cur, lane, cand);
@@ -187,9 +199,8 @@ __device__ __forceinline__ void box_block(BoxPixels<ATH>& P, const int4* recs, c
     rec = rec_n;
     has = has_n;
     if (rec != kNone) {
-      const int2 a = __ldg(reinterpret_cast<const int2*>(recs + 4ull * rec));
-      const int2 b = __ldg(reinterpret_cast<const int2*>(recs + 4ull * rec + 1));
-      xy = make_int4(a.x, a.y, b.x, b.y);
+      const Int8 a = ldg32(recs + 4ull * rec);
+      xy = make_int4(a.v[0], a.v[1], a.v[4], a.v[5]);
       col = __ldg(colors + (rec - quad_base));
     }
     if (has) has_n = next_refs(rec_n);
@@ -199,33 +210,46 @@ __device__ __forceinline__ void box_block(BoxPixels<ATH>& P, const int4* recs, c
     if (ATH) {   // all finished
       bool live = false;
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        live |= ox + cx + (i & 1) < V.width && oy + cy + (i >> 1) < V.height && P.st[i].live();
+      for (int i = 0; i < NP; ++i) live |= ox + P.px(lane, i) < V.width && oy + P.py(lane, i) < V.height && P.st[i].live();
       if (!__any_sync(0xffffffffu, live)) break;
     }
     // under the top-left rule a centre is covered iff xmin <= x < xmax and ymin <= y < ymax
-    const int c0 = min(max(((min(xy.x, xy.z) + 127) >> 8) - ox, 0), 16), c1 = min(max(((max(xy.x, xy.z) + 127) >> 8) - ox, 0), 16);
-    const int y0 = min(max(((min(xy.y, xy.w) + 127) >> 8) - oy, 0), 8), y1 = min(max(((max(xy.y, xy.w) + 127) >> 8) - oy, 0), 8);
-    const uint32_t word = rec != kNone ? (0xFFFFu & (0xFFFFu << c0) & ~(0xFFFFFFFFu << c1)) |
-                                             ((0xFFu & (0xFFu << y0) & ~(0xFFFFFFFFu << y1)) << 16)
+    const int c0 = min(max(((min(xy.x, xy.z) + 127) >> 8) - ox, 0), BW), c1 = min(max(((max(xy.x, xy.z) + 127) >> 8) - ox, 0), BW);
+    const int y0 = min(max(((min(xy.y, xy.w) + 127) >> 8) - oy, 0), BH), y1 = min(max(((max(xy.y, xy.w) + 127) >> 8) - oy, 0), BH);
+    constexpr uint32_t kCols = (1u << BW) - 1u, kRows = (1u << BH) - 1u;
+    const uint32_t word = rec != kNone ? (kCols & (kCols << c0) & ~(0xFFFFFFFFu << c1)) |
+                                             ((kRows & (kRows << y0) & ~(0xFFFFFFFFu << y1)) << BW)
                                        : 0u;
     qc[lane] = col;
     advance();
-    // lane x < 16: the candidates covering column x; lane 16 + y: row y
+    // lane x < BW: the candidates covering column x; lane BW + y: row y
     const uint32_t t = warp_transpose32(word, lane);
-    const uint32_t mx0 = __shfl_sync(0xffffffffu, t, cx), mx1 = __shfl_sync(0xffffffffu, t, cx + 1);
-    const uint32_t my0 = __shfl_sync(0xffffffffu, t, 16 + cy), my1 = __shfl_sync(0xffffffffu, t, 17 + cy);
+    const uint32_t mx0 = __shfl_sync(0xffffffffu, t, cx), mx1 = NP == 4 ? __shfl_sync(0xffffffffu, t, cx + 1) : mx0;
+    const uint32_t my0 = __shfl_sync(0xffffffffu, t, BW + cy), my1 = NP > 1 ? __shfl_sync(0xffffffffu, t, BW + cy + 1) : my0;
     __syncwarp();
-    const uint32_t m[4] = {mx0 & my0, mx1 & my0, mx0 & my1, mx1 & my1};
+    uint32_t m[NP], u = 0u;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) P.cnt[i] += __popc(m[i]);
-    uint32_t u = (mx0 | mx1) & (my0 | my1);
+    for (int i = 0; i < NP; ++i) {
+      m[i] = (NP == 4 && (i & 1) ? mx1 : mx0) & ((NP == 4 ? i >> 1 : i) ? my1 : my0);
+      u |= m[i];
+      P.cnt[i] += __popc(m[i]);
+    }
+    if (NP <= 2 && !ATH && __reduce_max_sync(0xffffffffu, __popc(u)) >= box_dense(NP)) {
+#pragma unroll
+      for (int p = 31; p >= 0; --p) {
+        const float4 c = qc[p];
+#pragma unroll
+        for (int i = 0; i < NP; ++i)
+          if (m[i] & (1u << p)) P.st[i].blend_direct(c);
+      }
+      u = 0u;
+    }
     while (u) {
       const int p = 31 - __clz(u);
       const uint32_t bit = 1u << p;
       const float4 c = qc[p];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < NP; ++i)
         if ((m[i] & bit) && P.st[i].live()) P.st[i].blend_direct(c);
       u ^= bit;
     }
@@ -233,167 +257,127 @@ __device__ __forceinline__ void box_block(BoxPixels<ATH>& P, const int4* recs, c
   }
 }
 
-// Writes pixel (px, py) of the block, if it is in the image, and returns its fragments.
-__device__ __forceinline__ uint32_t box_write(const ViewDev& V, int px, int py, float r, float g, float b, float T, uint32_t cnt) {
-  if (px >= V.width || py >= V.height) return 0u;
-  const long long pidx = (long long)py * V.width + px;
-  if (V.cnt) V.cnt[pidx] = cnt;
-  write_pixel(V, pidx, r, g, b, T);
-  return cnt;
-}
-// The block's half-blocks have no pixel for the exact path.
-__device__ __forceinline__ void box_xmask(const ViewDev& V, int ox, int oy, int lane) {
-  const int x = ox + (lane & 1) * kHbW, y = oy + (lane >> 1) * kHbH;
-  if (V.xmask && lane < 4 && x < V.width && y < V.height)
-    V.xmask[((uint32_t)y / kHbH) * (((uint32_t)V.width + kHbW - 1) / kHbW) + (uint32_t)x / kHbW] = 0u;
-}
-
 constexpr size_t kOrderedSmemWarp = win_refs(false) * sizeof(uint16_t) + kPendCap * sizeof(uint2) +
                                    32 * sizeof(float4) + kPendCap * sizeof(uint32_t);
-// (two CTAs per SM 266 us on the 2M particles, three 209, four 213 and 45 instead of 41 on four small
-// mixed views, five 262)
-#ifndef LR_ORDERED_MIN_BLOCKS
-#define LR_ORDERED_MIN_BLOCKS 3
-#endif
 
-// One 16x8 block of a bin (an item of the queue).
-struct OrderedBlock {
-  const ViewDev* V;          // null: nothing to do
+// A bin as the queue's items see it.
+struct OrderedBin {
+  const ViewDev* V;
   const unsigned long long* refs;
-  const uint32_t *row_u, *row_l;
-  int n, ox, oy;
-  bool shapes;               // the bin holds other shapes than axis-parallel rectangles
-  bool bytes;                // the view wants 8-bit values
-  __device__ __forceinline__ OrderedBlock(const Ws& ws, uint32_t n_general, uint32_t item) {
-    const int lg = ws.bin_log2, bl = bin_hb_log2(lg) - 2, cl = bin_hb_cols_log2(lg) - 1, cols = bin_hb_cols(lg);
-    const int bin_g = (int)ws.bin_order[n_general + (item >> bl)], blk = (int)(item & ((1u << bl) - 1u));
-    V = ws.views + view_of_bin(ws.views, ws.n_views, bin_g);
-    const int b = bin_g - V->bin_base, bx = blk & ((1 << cl) - 1), by = blk >> cl;
-    ox = ((b % V->nbx) << lg) + 16 * bx;
-    oy = ((b / V->nbx) << lg) + 8 * by;
-    const uint32_t off = ws.bin_off[bin_g];
-    n = (int)(ws.bin_off[bin_g + 1] - off);
+  const uint32_t* rows;      // of its bitmap, nw words each
+  int n, nw, x0, y0;
+  bool shapes;               // it holds other shapes than axis-parallel rectangles
+  __device__ __forceinline__ OrderedBin(const Ws& ws, int bin) {
+    V = ws.views + view_of_bin(ws.views, ws.n_views, bin);
+    const int b = bin - V->bin_base;
+    x0 = (b % V->nbx) << ws.bin_log2;
+    y0 = (b / V->nbx) << ws.bin_log2;
+    const uint32_t off = ws.bin_off[bin];
+    n = (int)(ws.bin_off[bin + 1] - off);
+    nw = (n + 31) >> 5;
     refs = ws.refs + off;
-    const int hb = 2 * by * cols + 2 * bx;   // upper left half-block
-    row_u = hb_row(ws, off, bin_g, n, hb);
-    row_l = hb_row(ws, off, bin_g, n, hb + cols);
-    shapes = (ws.bin_cursor[bin_g] & kBinShapes) != 0u;
-    bytes = V->out8 != nullptr;
-    if (ox >= V->width || oy >= V->height || !tile_owned(*V, ox, oy)) V = nullptr;
+    rows = hb_row(ws, off, bin, n, 0);
+    shapes = (ws.bin_cursor[bin] & kBinShapes) != 0u;
   }
 };
 
-// Persistent CTAs over the 16x8 blocks of these bins, longest lists first. Bins with long lists
-// (n_ordered_long): the CTA's eight warps take an eighth of a block's list each and their composites are
-// combined in order (consecutive segments combine as C1 + T1 C2, T1 T2): one warp through a dense
-// bin's list took longer than all the rest of the frame (400,000 particles at 960x540: 168 us
-// against 61 us, 2M at 1920x1080 295 against 207; cut from 4096 references on they took 231, since
-// the longest uncut lists then start late). Then a warp per block. With the alpha
-// threshold, whose stop is defined on the running product, and for views with 8-bit values, whose
-// rounding would show where a list was cut, always a warp per block.
+// Persistent warps over these bins, longest lists first, an item each: a 16x8 block, of a bin with a
+// long list (n_ordered_long) an 8x8 block, of the longest (n_ordered_longest) a half-block. One warp
+// through a dense bin's list for 16x8 pixels takes longer than all the rest of the frame (2M particles at
+// 1920x1080: 277 us, 203 with the smaller blocks; 400,000 at 960x540 201 and 78), while smaller blocks
+// everywhere repeat the candidates' work and are bound by the L1 data pipe (265 us with half-blocks
+// alone). Every pixel blends its list from the front in all of them, so an image depends neither on
+// the form nor on what else is in the batch or asked for. (Lists cut into segments whose composites are
+// then combined take 213 and 65 us, but round differently wherever one is cut.) The alpha
+// threshold, which ends most lists early, has 16x8 blocks only (70 us on the 2M, 80 with the others).
+// Bins of other shapes than rectangles: 8x8 blocks always.
 template <bool ATH>
-__global__ __launch_bounds__(kRasterThreads, LR_ORDERED_MIN_BLOCKS) void k_raster_ordered(Ws ws) {
+__global__ __launch_bounds__(kRasterThreads, 3) void k_raster_ordered(Ws ws) {
   pdl_begin();
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ uint32_t s_item;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned char* wbase = smem + (size_t)warp * kOrderedSmemWarp;
   uint16_t* cand = reinterpret_cast<uint16_t*>(wbase);
   uint2* pend = reinterpret_cast<uint2*>(wbase + win_refs(false) * sizeof(uint16_t));
   float4* qc = reinterpret_cast<float4*>(pend + kPendCap);
-  const bool run = ws.ctrl->error != LR_ERR_OVERFLOW;
-  const uint32_t n_general = ws.ctrl->n_general;
-  const int bl = bin_hb_log2(ws.bin_log2) - 2;
-  const uint32_t nitems = run ? ((uint32_t)ws.total_bins - n_general) << bl : 0u;   // (a batch has less than 2^32 pixels)
-  const uint32_t nlong = ATH || !run ? 0u : ws.ctrl->n_ordered_long << bl;
+  if (ws.ctrl->error == LR_ERR_OVERFLOW) return;
+  const uint32_t n_general = ws.ctrl->n_general, n_longest = ATH ? 0u : ws.ctrl->n_ordered_longest, n_long = ATH ? 0u : ws.ctrl->n_ordered_long;
+  const int lg = ws.bin_log2, hl = bin_hb_log2(lg), cl = bin_hb_cols_log2(lg), bl = hl - 2;
+  // (a batch has less than 2^32 pixels)
+  const uint32_t items1 = n_longest << hl, items2 = items1 + ((n_long - n_longest) << (hl - 1));
+  const uint32_t nitems = items2 + (((uint32_t)ws.total_bins - n_general - n_long) << bl);
   unsigned long long frag_total = 0;
-  auto draw = [&]() { return (uint32_t)min(atomicAdd(&ws.ctrl->ordered_head, 1ull), 0xFFFFFFF0ull); };
-  auto whole_block = [&](const OrderedBlock& B) {   // rectangles, by one warp
-    const int nw = (B.n + 31) >> 5;
-    BoxPixels<ATH> P;
-    P.init();
-    box_block<ATH>(P, ws.rec, B.refs, *B.V, B.row_u, B.row_l, nw, 0, nw, B.ox, B.oy, lane, cand, qc);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      frag_total += box_write(*B.V, B.ox + 2 * (lane & 7) + (i & 1), B.oy + 2 * (lane >> 3) + (i >> 1), P.st[i].r, P.st[i].g, P.st[i].b,
-                              P.st[i].T, P.cnt[i]);
-    box_xmask(*B.V, B.ox, B.oy, lane);
+  // a lane's pixel, if it is in the image
+  auto write = [&](const ViewDev& V, int px, int py, const PixelState<1, true, ATH>& st, uint32_t cnt) {
+    if (px >= V.width || py >= V.height) return;
+    const long long pidx = (long long)py * V.width + px;
+    if (V.cnt) V.cnt[pidx] = cnt;
+    write_pixel(V, pidx, st.r, st.g, st.b, st.T);
+    frag_total += cnt;
   };
-  uint32_t item = 0xFFFFFFFFu;         // warp 0: the first item past the CTA's
-  while (nlong) {
-    if (threadIdx.x == 0) s_item = draw();
-    __syncthreads();
-    item = s_item;
-    if (item >= nlong) break;
-    const OrderedBlock B(ws, n_general, item);
-    const uint32_t blk = item & ((1u << bl) - 1u);
-    if (!B.shapes && B.bytes) {
-      // eight blocks of the bin (two of a 16-pixel bin), a warp each
-      const uint32_t it = item + warp;
-      if ((blk & 7u) == 0u && it >> bl == item >> bl) {
-        const OrderedBlock W(ws, n_general, it);
-        if (W.V) whole_block(W);
-      }
-    } else if (B.V && !B.shapes) {
-      const int nw = (B.n + 31) >> 5, per = (nw + kRasterWarps - 1) / kRasterWarps;
-      BoxPixels<ATH> P;
-      P.init();
-      box_block<ATH>(P, ws.rec, B.refs, *B.V, B.row_u, B.row_l, nw, warp * per, min(nw, (warp + 1) * per), B.ox, B.oy, lane, cand, qc);
-      // the warp's composite in place of its candidates, its counts in place of the ring
-      float4* part = reinterpret_cast<float4*>(cand);
-      uint32_t* pcnt = reinterpret_cast<uint32_t*>(pend);
-      __syncwarp();
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        part[32 * i + lane] = make_float4(P.st[i].r, P.st[i].g, P.st[i].b, P.st[i].T);
-        pcnt[32 * i + lane] = P.cnt[i];
-      }
-      __syncthreads();
-      if (threadIdx.x < 128) {
-        float r = 0.f, g = 0.f, b = 0.f, T = 1.f;
-        uint32_t c = 0;
-#pragma unroll
-        for (int w = 0; w < kRasterWarps; ++w) {
-          const unsigned char* wb = smem + (size_t)w * kOrderedSmemWarp;
-          const float4 p = reinterpret_cast<const float4*>(wb)[threadIdx.x];
-          r += T * p.x;
-          g += T * p.y;
-          b += T * p.z;
-          T *= p.w;
-          c += reinterpret_cast<const uint32_t*>(wb + win_refs(false) * sizeof(uint16_t))[threadIdx.x];
-        }
-        const int px = B.ox + 2 * (lane & 7) + (warp & 1), py = B.oy + 2 * (lane >> 3) + (warp >> 1);
-        frag_total += box_write(*B.V, px, py, r, g, b, T, c);
-        if (warp == 0) box_xmask(*B.V, B.ox, B.oy, lane);
-      }
-    } else if (B.shapes && (blk & 3u) == 0u) {
-      // four blocks of the bin (two of a 16-pixel bin) as eight 8x8 blocks, a warp each
-      const uint32_t it = item + (warp >> 1);
-      if (it >> bl == item >> bl) {
-        const OrderedBlock W(ws, n_general, it);
-        const int h = warp & 1, nw = (W.n + 31) >> 5;
-        if (W.V && W.ox + 8 * h < W.V->width)
-          frag_total += const_block<ATH>(ws.rec, W.refs, *W.V, W.row_u + h * nw, W.row_l + h * nw, W.n, W.ox + 8 * h, W.oy, lane, cand, pend, qc);
-      }
-    }
-    __syncthreads();
-  }
-  for (bool drawn = nlong != 0u && warp == 0; run; drawn = false) {
-    if (!drawn) {
-      uint32_t k = 0;
-      if (lane == 0) k = draw();
-      item = __shfl_sync(0xffffffffu, k, 0);
+  // half-block (x, y) has no pixel for the exact path
+  auto no_exact = [&](const ViewDev& V, int x, int y) {
+    if (V.xmask && x < V.width && y < V.height)
+      V.xmask[((uint32_t)y / kHbH) * (((uint32_t)V.width + kHbW - 1) / kHbW) + (uint32_t)x / kHbW] = 0u;
+  };
+  // The first items are spread so that every SM gets long and shorter lists alike: warp 0 of every CTA
+  // takes the longest, warp 1 the next, and so on
+  const uint32_t warps = gridDim.x * kRasterWarps;
+  for (bool first = true;; first = false) {
+    uint32_t item = warp * gridDim.x + blockIdx.x;
+    if (!first) {
+      if (lane == 0) item = warps + (uint32_t)min(atomicAdd(&ws.ctrl->ordered_head, 1ull), 0xFFF00000ull);
+      item = __shfl_sync(0xffffffffu, item, 0);
     }
     if (item >= nitems) break;
-    const OrderedBlock B(ws, n_general, item);
-    if (!B.V) continue;
-    const int nw = (B.n + 31) >> 5;
-    if (!B.shapes) {
-      whole_block(B);
+    const int form = item < items1 ? 1 : (item < items2 ? 2 : 4);   // pixels per lane
+    const uint32_t i = item - (form == 1 ? 0u : (form == 2 ? items1 : items2));
+    const int shift = form == 1 ? hl : (form == 2 ? hl - 1 : bl);
+    const OrderedBin B(ws, (int)ws.bin_order[n_general + (form == 1 ? 0u : (form == 2 ? n_longest : n_long)) + (i >> shift)]);
+    const ViewDev& V = *B.V;
+    if (form <= 2) {
+      // of the half-blocks, 2 j and 2 j + 1 are the upper and the lower one of 8x8 block j
+      const int blk = (int)(i & ((1u << shift) - 1u)) >> (form == 1), lower = form == 1 ? (int)(i & 1u) : 0;
+      const int bx = blk & ((1 << cl) - 1), by = 2 * (blk >> cl) + lower;
+      const int ox = B.x0 + kHbW * bx, oy = B.y0 + kHbH * by;
+      if (ox >= V.width || oy >= V.height || !tile_owned(V, ox, oy)) continue;
+      const uint32_t* row_u = B.rows + (size_t)((by << cl) + bx) * B.nw;
+      const uint32_t* row_l = row_u + ((size_t)B.nw << cl);   // (not read for a half-block)
+      if (B.shapes) {
+        if (!lower) frag_total += const_block<ATH>(ws.rec, B.refs, V, row_u, row_l, B.n, ox, oy, lane, cand, pend, qc);
+      } else if (form == 1) {
+        BoxPixels<ATH, 1> P;
+        P.init();
+        box_block<ATH, 1>(P, ws.rec, B.refs, V, row_u, row_u, B.nw, ox, oy, lane, cand, qc);
+        write(V, ox + (lane & 7), oy + (lane >> 3), P.st[0], P.cnt[0]);
+        if (lane == 0) no_exact(V, ox, oy);
+      } else {
+        BoxPixels<ATH, 2> P;
+        P.init();
+        box_block<ATH, 2>(P, ws.rec, B.refs, V, row_u, row_l, B.nw, ox, oy, lane, cand, qc);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) write(V, ox + (lane & 7), oy + 2 * (lane >> 3) + k, P.st[k], P.cnt[k]);
+        if (lane < 2) no_exact(V, ox, oy + lane * kHbH);
+      }
     } else {
+      const int blk = (int)(i & ((1u << bl) - 1u)), bx = blk & ((1 << (cl - 1)) - 1), by = blk >> (cl - 1);
+      const int ox = B.x0 + 2 * kHbW * bx, oy = B.y0 + 2 * kHbH * by;
+      if (ox >= V.width || oy >= V.height || !tile_owned(V, ox, oy)) continue;
+      const uint32_t* row_u = B.rows + (size_t)((2 * by << cl) + 2 * bx) * B.nw;   // the upper left half-block's
+      const uint32_t* row_l = row_u + ((size_t)B.nw << cl);
+      if (!B.shapes) {
+        BoxPixels<ATH, 4> P;
+        P.init();
+        box_block<ATH, 4>(P, ws.rec, B.refs, V, row_u, row_l, B.nw, ox, oy, lane, cand, qc);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          write(V, ox + 2 * (lane & 7) + (k & 1), oy + 2 * (lane >> 3) + (k >> 1), P.st[k], P.cnt[k]);
+        if (lane < 4) no_exact(V, ox + (lane & 1) * kHbW, oy + (lane >> 1) * kHbH);
+      } else {
 #pragma unroll 1
-      for (int h = 0; h < 2 && B.ox + 8 * h < B.V->width; ++h)
-        frag_total += const_block<ATH>(ws.rec, B.refs, *B.V, B.row_u + h * nw, B.row_l + h * nw, B.n, B.ox + 8 * h, B.oy, lane, cand, pend, qc);
+        for (int h = 0; h < 2 && ox + 8 * h < V.width; ++h)
+          frag_total += const_block<ATH>(ws.rec, B.refs, V, row_u + h * B.nw, row_l + h * B.nw, B.n, ox + 8 * h, oy, lane, cand, pend, qc);
+      }
     }
   }
 #pragma unroll
