@@ -156,7 +156,7 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_count(Ws ws)
   pdl_begin();
   __shared__ uint32_t hist[kHistSmemBins];
   __shared__ LargeList large;
-  __shared__ uint32_t flags[2][kHistSmemBins / 32];   // bins the chunk marks kBinDepths, kBinShapes
+  __shared__ uint32_t depths[kHistSmemBins / 32];   // bins the chunk marks kBinDepths
   const int v = view_of_chunk(ws.views, ws.n_views, blockIdx.x);
   const ViewDev& V = ws.views[v];
   const long long q0 = V.quad_base + (long long)(blockIdx.x - V.chunk_base) * ws.chunk_quads;
@@ -167,17 +167,15 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_count(Ws ws)
   if (smem)
     for (int b = threadIdx.x; b < nb; b += blockDim.x) {
       hist[b] = 0u;
-      flags[0][b >> 5] = flags[1][b >> 5] = 0u;
+      depths[b >> 5] = 0u;
     }
   __syncthreads();
   for_each_ref<true>(ws, V, q0, q1, large, [&](long long, int b, int, int, uint2, uint32_t info) {
     if (smem) {
       atomicAdd(&hist[b], 1u);
       const uint32_t bit = 1u << (b & 31);
-      uint32_t* d = &flags[0][b >> 5];
-      uint32_t* f = &flags[1][b >> 5];
+      uint32_t* d = &depths[b >> 5];
       if (!(info & kInfoFlatDepth) && !(*(volatile uint32_t*)d & bit)) atomicOr(d, bit);
-      if (!(info & kInfoRectBox) && !(*(volatile uint32_t*)f & bit)) atomicOr(f, bit);
     } else {
       atomicAdd(&ws.bin_count[V.bin_base + b], 1u);
     }
@@ -202,8 +200,7 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_count(Ws ws)
   for (int b = threadIdx.x; b < nb; b += blockDim.x) {
     const uint32_t c = hist[b];
     if (!c) continue;
-    const uint32_t fl = ((flags[0][b >> 5] >> (b & 31)) & 1u) * kBinDepths | ((flags[1][b >> 5] >> (b & 31)) & 1u) * kBinShapes;
-    if (!ws.cursors && fl) atomicOr(&ws.bin_cursor[V.bin_base + b], fl);
+    if (!ws.cursors && ((depths[b >> 5] >> (b & 31)) & 1u)) atomicOr(&ws.bin_cursor[V.bin_base + b], kBinDepths);
     const uint32_t base = atomicAdd(&ws.bin_count[V.bin_base + b], c);
     const unsigned long long at = (unsigned long long)s_start + atomicAdd(&s_pos, 1u);
     // a list past the reference capacity means the references do not fit either: the scan
@@ -350,6 +347,7 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_scatter(Ws w
   pdl_begin();
   __shared__ uint32_t hist[kHistSmemBins];
   __shared__ LargeList large;
+  __shared__ uint32_t shapes[kHistSmemBins / 32];   // bins the chunk has marked kBinShapes
   if (ws.ctrl->error == LR_ERR_OVERFLOW) return;
   const int v = view_of_chunk(ws.views, ws.n_views, blockIdx.x);
   const ViewDev& V = ws.views[v];
@@ -359,6 +357,7 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_scatter(Ws w
   const bool smem = nb <= kHistSmemBins;
   if (threadIdx.x == 0) large.n = 0u;
   if (smem) {
+    for (int b = threadIdx.x; b < kHistSmemBins / 32; b += blockDim.x) shapes[b] = 0u;
     // the chunk's range in each bin it touches, reserved by k_bin_count
     const uint2 sp = ws.chunk_span[blockIdx.x];
     const uint2* list = reinterpret_cast<const uint2*>(ws.refs_tmp) + sp.x;
@@ -379,8 +378,14 @@ __global__ __launch_bounds__(kBinThreads, kBinMinBlocks) void k_bin_scatter(Ws w
     // box clipped to this bin
     const bool one_bin = ((rect.x & 0xffff) >> lg) == ((rect.x >> 16) >> lg) &&
                          ((rect.y & 0xffff) >> lg) == ((rect.y >> 16) >> lg);
-    const float rep = (one_bin || (info & kInfoFlatDepth)) ? ws.rec_rep[q] : rep_depth(ws, q, info, x0, x1, y0, y1);
-    if (slot < (uint32_t)ws.refs_cap) ws.refs[slot] = ref_key(rep, q);
+    const bool flat = (info & kInfoFlatDepth) != 0u;
+    const float rep = one_bin || flat ? ws.rec_rep[q] : rep_depth(ws, q, info, x0, x1, y0, y1);
+    if (ws.ordered && flat && rep > 0.f) {   // (no rectangle; the views' bins then have shared counters)
+      const uint32_t bit = 1u << (b & 31);
+      uint32_t* s = &shapes[b >> 5];
+      if (!(*(volatile uint32_t*)s & bit) && !(atomicOr(s, bit) & bit)) atomicOr(&ws.bin_cursor[V.bin_base + b], kBinShapes);
+    }
+    if (slot < (uint32_t)ws.refs_cap) ws.refs[slot] = ref_key(fabsf(rep), q);
   });
 }
 

@@ -76,7 +76,6 @@ constexpr uint32_t kInfoFlatDepth = 8u;     // all four vertices have the same 1
 constexpr uint32_t kInfoSwap0 = 16u;        // triangle t (bit << t): negative area, v1 <-> v2
 constexpr uint32_t kInfoSmall0 = 64u;       // triangle t (bit << t): 32-bit edge values are
                                             // exact on every half-block its box touches
-constexpr uint32_t kInfoRectBox = kInfoSmall0;   // in rec_info only (binning reads no kInfoSmall0): kRecBox
 // flags in word 15 of the record
 constexpr uint32_t kRecSmall = 1u;          // every edge value is below 2^30 on every 8x4 and
                                             // 8x8 block the quad's box touches
@@ -247,8 +246,8 @@ __device__ __forceinline__ QuadRec load_rec(const int4* rec, uint32_t i) {
 constexpr int kOrderedLong = 1024, kOrderedLongShare8 = 3;
 constexpr int kOrderedLongest = 2048, kOrderedLongestShare8 = 16;
 
-// bin_cursor: the bin holds a reference to a quad that is not of constant depth, one that is no
-// axis-parallel rectangle
+// bin_cursor: the bin holds a reference to a quad that is not of constant depth (k_bin_count), one of
+// constant depth that is no axis-parallel rectangle (k_bin_scatter)
 constexpr uint32_t kBinDepths = 1u, kBinShapes = 2u;
 
 // Pointers into the workspace for one render (passed by value to every kernel).
@@ -268,7 +267,8 @@ struct Ws {
   int4* rec;                 // [4 * total_quads]: the 64-byte quad record (QuadRec)
   uint2* rec_rect;           // [total_quads]: pixel AABB (px0 | px1 << 16, py0 | py1 << 16)
   uint32_t* rec_info;        // [total_quads]: kInfo* bits | cull reason << 8
-  float* rec_rep;            // [total_quads]: representative 1/w over the quad's whole box
+  float* rec_rep;            // [total_quads]: representative 1/w over the quad's whole box, negative
+                             // for an axis-parallel rectangle (kRecBox)
   uint32_t* bin_count;       // [total_bins]
   uint32_t* bin_off;         // [total_bins + 1]
   uint32_t* bin_cursor;      // [total_bins] with `cursors` the scatter's cursors, else kBin* flags

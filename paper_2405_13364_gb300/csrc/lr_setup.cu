@@ -190,11 +190,10 @@ __global__ __launch_bounds__(256) void k_setup(Ws ws) {
       stg32(rp, X[0], Y[0], X[1], Y[1], X[2], Y[2], X[3], Y[3]);
       stg32(rp + 2, __float_as_int(q[0]), __float_as_int(q[1]), __float_as_int(q[2]), __float_as_int(q[3]),
             __float_as_int(inv.x), __float_as_int(inv.y), (int)info, (int)rflags);
-      ws.rec_rep[g] = rep;
+      ws.rec_rep[g] = (rflags & kRecBox) ? -rep : rep;
     }
     ws.rec_rect[g] = rect;
-    // (binning reads the rectangle flag where the rasteriser's record has kInfoSmall0)
-    ws.rec_info[g] = (info & ~(3u * kInfoSmall0)) | ((rflags & kRecBox) && worst == kVisible ? kInfoRectBox : 0u) | (worst << 8);
+    ws.rec_info[g] = info | (worst << 8);
     if (bad) set_error(ws.ctrl, LR_ERR_INVALID_ARG);
   }
   // statistics: culled quads per reason, one atomic per reason present in the warp, by its
