@@ -380,7 +380,8 @@ __device__ __forceinline__ void batch_gradients(uint32_t done, uint32_t j, float
   if (!m) return;
   // (dL/da pixel by pixel: its two terms nearly cancel, so their sums would round worse)
   const float4 c = qc[lane];
-  const float om = 1.0f - c.w, inv = om > 1e-6f ? rcp_approx(om) : 0.f;
+  const float om = 1.0f - c.w, inv = rcp_approx(om);
+  const bool thin = om > 1e-6f;   // (an opaque quad's S may be 0 times infinity)
   float r = 0.f, g = 0.f, b = 0.f, da = 0.f;
   while (m) {
     const int px = __ffs(m) - 1;
@@ -391,7 +392,8 @@ __device__ __forceinline__ void batch_gradients(uint32_t done, uint32_t j, float
     r += w * p.x;
     g += w * p.y;
     b += w * p.z;
-    da += ts.x * (p.x * c.x + p.y * c.y + p.z * c.z) - ts.y * inv;
+    const float front = ts.x * (p.x * c.x + p.y * c.y + p.z * c.z);
+    da += thin ? front - ts.y * inv : front;
   }
   atomicAdd(reinterpret_cast<float4*>(grad) + j, make_float4(r, g, b, da));
 }
