@@ -124,7 +124,7 @@ static Layout make_layout(int n, const long long* Q, const int* W, const int* H,
   L.bin_count = take(sizeof(uint32_t) * (size_t)L.total_bins);
   L.bin_off = take(sizeof(uint32_t) * ((size_t)L.total_bins + 1));
   L.bin_cursor = take(sizeof(uint32_t) * (size_t)L.total_bins);
-  L.chunk_span = take(sizeof(uint2) * (size_t)L.total_chunks);
+  L.chunk_span = take(sizeof(uint2) * (size_t)chunks_reserved(L.total_quads, n));
   L.bin_order = take(sizeof(uint32_t) * (size_t)L.total_bins);
   L.ovf_list = take(sizeof(uint32_t) * (size_t)L.total_pix);
   L.refs = o;      // refs and refs_tmp follow; see set_capacity

@@ -58,6 +58,12 @@ __host__ __forceinline__ int chunk_quads_for(long long quads) {
   while (c > kChunkQuadsMin && quads < 304LL * c) c >>= 1;
   return c;
 }
+// At least as many chunks as these quads in `views` views make, growing with the quads: what the
+// workspace reserves, so that one for more quads also holds a render of fewer.
+__host__ __forceinline__ long long chunks_reserved(long long quads, int views) {
+  const long long few = (quads + kChunkQuadsMin - 1) / kChunkQuadsMin, large = quads / (kChunkQuads / 2);
+  return views + (large > 608 ? large : (few < 608 ? few : 608));
+}
 constexpr int kBinThreads = 512, kBinMinBlocks = 2;   // threads per binning CTA at most, CTAs per SM
 __host__ __forceinline__ int bin_threads_for(int chunk_quads) { return chunk_quads < kBinThreads ? chunk_quads : kBinThreads; }
 constexpr int kSmallBins = 4;               // AABB-counted up to kSmallBins x kSmallBins bins
