@@ -7,7 +7,7 @@
 //                  Quads whose bin rectangle is at most 4x4 bins are counted from their
 //                  AABB; larger quads are tested bin by bin with a conservative
 //                  per-triangle edge test (trivial reject), the whole warp sharing one
-//                  large quad's bins.
+//                  large quad's bins and the whole CTA those of one over 128 bins.
 //   k_bin_scan     Phase 2: exclusive scan of the counts into list offsets, capacity
 //                  check, and a categorisation of bins by size (the paper's empty / low /
 //                  high) that orders the rasterisers' work queues, largest bins first.

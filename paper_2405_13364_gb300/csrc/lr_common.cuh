@@ -45,12 +45,12 @@ constexpr int kMaxBucket = 64;
 constexpr size_t kSortSmemBytes = (size_t)kBucketBigCap * 8 + (size_t)kBucketsBig * 2;
 static_assert(kSortSmemBytes >= 2 * (size_t)kSortBigCap * 8, "two merge buffers");
 constexpr int kHistSmemBins = 8192;         // shared-memory bin counters per CTA (Sec. 2 Stage 2)
-// Quads per binning CTA: 4096 (from 1.6M quads on: 2M particles 35 us against 29 for the count, 41
-// against 39 for the scatter; a batch of 1.4M quads with large ones among them 47 against 57), else
-// 2048, halved until there are two CTAs for each of the 152 SMs (both kernels are bound by latency, and
-// 2048 quads each left most SMs idle below 600,000 quads). One thread per quad where that is fewer
-// than 512 (100,000 quads: 14 us each with 512 threads, 12 with 256; with 256 for 2048 quads the
-// layer frame took 31 and 37 us instead of 20 and 25).
+// Quads per binning CTA: 4096 from 1.6M quads on (count + scatter at 2M quads with 4096 and with 2048:
+// particles 70 and 78 us, scattered parallelograms 127 and 137, layers 66 and 68; at 1.6M, 390 chunks of
+// 4096 for 304 places, 66 and 66, 119 and 111, 59 and 57), else 2048, halved until there are two CTAs for
+// each of the 152 SMs (both kernels are bound by latency, and 2048 quads each left most SMs idle below
+// 600,000 quads). One thread per quad where that is fewer than 512 (100,000 quads: 14 us each with 512
+// threads, 12 with 256; with 256 for 2048 quads the layer frame took 31 and 37 us instead of 20 and 25).
 constexpr int kChunkQuads = 4096, kChunkQuadsMin = 256;
 __host__ __forceinline__ int chunk_quads_for(long long quads) {
   if (quads >= 400LL * kChunkQuads) return kChunkQuads;

@@ -1,13 +1,14 @@
 // lr_ordered.cu -- the rasteriser of the bins whose sorted list is every pixel's exact fragment
 // order: bins that hold only flat-colour quads of one depth each (camera-facing sprites and
 // particles; kBinDepths, set by the bin count). Fragments are blended as they come, without depth
-// keys, sorter or exact path, in blocks of several pixels per lane. k_bin_scan puts these bins
-// behind the others in bin_order; k_raster, launched next, takes the others. (As a branch of k_raster the two block
-// forms cost its own loops registers: the layer frame 309 -> 317 us, mixed views at K = 3 743 ->
+// keys, sorter or exact path, in blocks of one to four pixels per lane. k_bin_scan puts these bins
+// behind the others in bin_order; k_raster, launched next, takes the others. (As branches of k_raster the
+// block forms cost its own loops registers: the layer frame 309 -> 317 us, mixed views at K = 3 743 ->
 // 774.)
 #include "lr_raster.cuh"
 
 namespace lr {
+
 // Bins that hold only flat-colour quads of one depth each: the bin's list, sorted by that depth with the tie
 // rule, is every pixel's exact fragment order. A warp takes an 8x8 block, the half-blocks hb and
 // hb_l below it, with two pixels per lane, one above the other: a record read from shared
