@@ -45,18 +45,18 @@ LAUNCHES_PER_FRAME = 8
 RASTER_TRAFFIC = {
     # (DRAM read + write bytes per launch, ncu smsp__issue_active, ncu smsp__inst_executed,
     #  source hash of the captured build)
-    ("layers", 1, False): (101_276_000, 0.7009, 265_736_245, "7cb1aac2c7011f52"),      # profiles/k_raster_layers1080p.md
+    ("layers", 1, False): (100_988_000, 0.6995, 265_697_333, "573345bbe27ccebf"),      # profiles/k_raster_layers1080p.md
     # (k_raster_ordered, which does not depend on K: profiles/k_raster_ordered_particles1080p.md)
-    ("particles", 1, False): (360_786_000, 0.6195, 151_340_566, "7cb1aac2c7011f52"),
-    ("particles", 2, False): (360_786_000, 0.6195, 151_340_566, "7cb1aac2c7011f52"),
-    ("particles", 3, False): (360_786_000, 0.6195, 151_340_566, "7cb1aac2c7011f52"),
+    ("particles", 1, False): (358_161_000, 0.7011, 160_297_054, "573345bbe27ccebf"),
+    ("particles", 2, False): (358_161_000, 0.7011, 160_297_054, "573345bbe27ccebf"),
+    ("particles", 3, False): (358_161_000, 0.7011, 160_297_054, "573345bbe27ccebf"),
 }
 # the same for the rasteriser's variants and the multisample resolve on the layer frame
 # (K = 1): (DRAM bytes per launch, issue-slot share, warp instructions, kernel us, hash)
 VARIANT_CAPTURES = {
-    "alpha_threshold": (95_037_000, 0.7181, 234_664_928, 268.4, "7cb1aac2c7011f52"),   # profiles/k_raster_alpha_layers1080p.md
-    "lit": (115_487_000, 0.6383, 319_002_729, 406.4, "7cb1aac2c7011f52"),               # profiles/k_raster_lit_layers1080p.md
-    "msaa_resolve": (149_758_000, 0.2631, 7_452_000, 27.0, "7cb1aac2c7011f52"),         # profiles/k_resolve_msaa4_layers1080p.md
+    "alpha_threshold": (94_735_000, 0.7134, 234_626_016, 270.3, "573345bbe27ccebf"),   # profiles/k_raster_alpha_layers1080p.md
+    "lit": (115_462_000, 0.6365, 318_973_545, 406.4, "573345bbe27ccebf"),               # profiles/k_raster_lit_layers1080p.md
+    "msaa_resolve": (149_445_000, 0.2664, 7_452_000, 27.1, "573345bbe27ccebf"),         # profiles/k_resolve_msaa4_layers1080p.md
 }
 RASTER_SOURCES = ("lr_raster.cuh", "lr_ordered.cu", "lr_common.cuh")
 LANES_PER_SM_CLK = 128
